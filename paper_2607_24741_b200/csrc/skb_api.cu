@@ -175,6 +175,7 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, char *
     d.guard_bad = (int *)take(4);
     d.state = (int *)take(W * 4); d.flag = (int *)take(W * 4); d.verdict = (int *)take(W * 4);
     d.nonfinite = (int *)take(W * 4);
+    d.absorbed = (int *)take(W * 4); d.cyc_log = (int *)take(W * 4);
     d.ret_at = (int *)take(W * 4); d.n_checks = (int *)take(W * 4);
     d.rsum_row64 = (unsigned long long *)take(W * 8); d.esc = (int *)take(W * 4);
     d.rsum_row = (unsigned long long *)take(W * 8); d.rsum_col = (unsigned long long *)take(W * 8);
@@ -208,6 +209,10 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, char *
     d.wa = (double *)take(W * np * 8); d.wb = (double *)take(W * mp * 8);
     d.phi[0] = (double *)take(W * np * 8); d.phi[1] = (double *)take(W * np * 8);
     d.gam = (double *)take(W * mp * 8);
+    if (var->xf && var->DP && scaling_fits(c->n, c->m)) {
+        d.phi0 = (double *)take(W * np * 8); d.gam0 = (double *)take(W * mp * 8);
+        d.uu[0] = (double *)take(W * np * 8); d.uu[1] = (double *)take(W * np * 8); d.vv = (double *)take(W * mp * 8);
+    }
     d.f_out = (double *)take(L * n * 8); d.g_out = (double *)take(L * m * 8);
     // guard band: raw copies of the inputs (the float64 re-evaluation reads nothing but these and the potentials)
     d.guard = guard_width(c);
@@ -473,13 +478,17 @@ extern "C" skb_status sinkhorn_batch_set_profiling(skb_batch *h, int on)
 static int launch_leg(skb_batch *h, int leg, int w)
 {
     if (h->tensor) { launch_update_tc(h->dev, h->maps, leg, w, h->stream); return 0; }
+    if (h->dev.phi0) { launch_scaling(h->dev, leg, 0, w, h->stream); return 0; }
     return h->var->launch(h->dev, leg, w, h->stream);
 }
 
-// ACTIVE batches whose lanes have few row blocks run several whole cycles per launch, one
-// thread-block cluster per lane (lane_cycles_kernel), followed by one planner for all of them.
+// Batches whose lanes have few row blocks run several whole cycles per launch, one thread-block cluster
+// per lane (scaling_kernel, lane_resident_kernel or lane_cycles_kernel), followed by one planner for all
+// of them.  A mask can be kept inside such a launch by the scaling kernel only; a STATIC batch cannot be
+// run that way at all, because the cycle at which all of its lanes stop is not known beforehand.
 static bool cycles_in_one_launch(const skb_batch *h)
 {
+    if (h->dev.phi0) return h->cfg.mode != SKB_STATIC && !h->profiling && !h->no_multi_cycle;
     if (h->cfg.mode != SKB_ACTIVE || h->tensor || h->profiling || !h->var->launch_cycles || h->no_multi_cycle) return false;
     const int mx = h->cfg.n > h->cfg.m ? h->cfg.n : h->cfg.m;
     const int nc = (mx + h->var->rows_per_cta - 1) / h->var->rows_per_cta;
@@ -496,7 +505,8 @@ static bool cycles_in_one_launch(const skb_batch *h)
 static void enqueue_cycles_launch(skb_batch *h, int cycles)
 {
     const int w = h->known_width;
-    h->var->launch_cycles(h->dev, cycles, w, h->stream);
+    if (h->dev.phi0) launch_scaling(h->dev, LEG_F, cycles, w, h->stream);
+    else h->var->launch_cycles(h->dev, cycles, w, h->stream);
     int nk = 1;
     nk += launch_plan_cycles(h->dev, w, cycles, h->stream);
     nk += launch_emit_move(h->dev, w, h->stream);
@@ -611,13 +621,15 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
         skb_status st0 = poll_snapshot(h, true);
         if (st0 != SKB_OK) { cudaStreamSynchronize(h->stream); return st0; }
     }
-    int chunk = 2, snap = 0, rounds = 0;
+    // lanes that finish inside a launch leave it, so a long first launch costs nothing; on the scaling
+    // kernel it saves forming the kernel matrices again
+    int chunk = h->dev.phi0 && cycles_in_one_launch(h) ? 16 : 2, snap = 0, rounds = 0;
     bool have_prev = false;
     // every lane is retired by the audit that follows cycle max_iter; STATIC needs one more pass
     const long long hard_cap = (long long)h->cfg.max_iter + 4;
     while (!h->finished) {
         const bool multi = cycles_in_one_launch(h);      // may become true as the batch narrows
-        const int chunk_max = multi ? 32 : 16;
+        const int chunk_max = h->dev.phi0 && multi ? (h->cfg.mode == SKB_ACTIVE ? MAX_CYCLES_IN_LAUNCH : 64) : (multi ? 32 : 16);
         NvtxRange nvtx_chunk(multi ? "skb:chunk (cycles in one launch)" : "skb:chunk (launch per leg)");
         if (multi) enqueue_cycles_launch(h, chunk);
         else for (int i = 0; i < chunk; ++i) enqueue_cycle(h);
@@ -635,7 +647,7 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
         // grow the chunk every other round: cycles enqueued past completion are empty launches that
         // still have to drain, which matters for batches that finish within a dozen cycles
         if (chunk < chunk_max && (++rounds & 1) == 0) chunk *= 2;
-        if (h->enqueued - h->enqueued_at_refill > hard_cap + 64) break;
+        if (h->enqueued - h->enqueued_at_refill > hard_cap + 64 + 2 * MAX_CYCLES_IN_LAUNCH) break;
     }
     if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "drain");
     if ((e = cudaMemcpy(&h->h_ctl[0], h->dev.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost)) != cudaSuccess)
@@ -718,7 +730,7 @@ extern "C" skb_status sinkhorn_batch_apply_plan(skb_batch *h, const void *x, con
 extern "C" skb_status sinkhorn_batch_last_audit(skb_batch *h, float *r_row, float *r_col, int *flagged)
 {
     if (!h) return SKB_ERR_NULL;
-    if (cycles_in_one_launch(h)) return fail(h, SKB_ERR_STATE, "per-audit values are kept by the one-launch-per-leg path only (MASKED, STATIC, tensor or profiled batches)");
+    if (cycles_in_one_launch(h) && h->cfg.mode == SKB_ACTIVE) return fail(h, SKB_ERR_STATE, "per-audit values are kept by the one-launch-per-leg path only (MASKED, STATIC, tensor or profiled batches)");
     launch_gather_audit(h->dev, r_row, r_col, flagged, h->stream);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? SKB_OK : cuda_fail(h, e, "last_audit");

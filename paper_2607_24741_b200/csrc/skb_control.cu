@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(256) lane_stats_kernel(const Dev P, const void
         P.nonfinite[slot] = 0; P.state[slot] = 0; P.flag[slot] = 0; P.verdict[slot] = 0;
         P.rsum_row[slot] = 0ull; P.rsum_col[slot] = 0ull; P.rsum_row64[slot] = 0ull; P.esc[slot] = 0;
         P.ret_at[slot] = 0; P.n_checks[slot] = 0;
+        P.absorbed[slot] = 0; P.cyc_log[slot] = 0;
         int form = P.cost_form == 1 ? FORM_DOT : (P.cost_form == 2 ? FORM_DIFF : (s * red[0] > P.form_threshold ? FORM_DIFF : FORM_DOT));
         P.form[slot] = form;
         atomicMax(&P.ctl->max_radius_bits, (unsigned long long)__double_as_longlong(eps_ok ? s * red[0] : 0.0));
@@ -310,6 +311,8 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_kernel(const Dev P)
         P.start[dst] = P.start[src];
         P.scale[dst] = P.scale[src];
         P.form[dst] = P.form[src];
+        P.absorbed[dst] = P.absorbed[src];
+        P.cyc_log[dst] = P.cyc_log[src];
         P.nonfinite[dst] = 0;
     }
     if (tid == 0) {
@@ -380,11 +383,12 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
     __syncthreads();
     int nret = 0;
     for (int j = 0; j < K; ++j) nret += left_at[j];
-    const int Anew = A - nret;
+    const bool compact = P.mode == MODE_ACTIVE;      // MASKED: lanes stay where they are, frozen or not
+    const int Anew = compact ? A - nret : A;
     const int parity_new = c.parity ^ (K & 1);       // survivors ran all K cycles
     // ordered lists: holes below the new width, survivors at or above it
     int base[3] = {0, 0, 0};
-    for (int s0 = 0; s0 < (nret > 0 ? A : 0); s0 += NT) {
+    for (int s0 = 0; s0 < (nret > 0 && compact ? A : 0); s0 += NT) {
         const int s = s0 + tid;
         const int r = (s < A && P.ret_at[s] > 0) ? 1 : 0;
         const int hole = r && s < Anew;
@@ -406,6 +410,8 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
         P.start[dst] = P.start[src];
         P.scale[dst] = P.scale[src];
         P.form[dst] = P.form[src];
+        P.absorbed[dst] = P.absorbed[src];
+        P.cyc_log[dst] = P.cyc_log[src];
         P.nonfinite[dst] = 0;
     }
     for (int s = tid; s < A; s += NT) { P.ret_at[s] = 0; P.n_checks[s] = 0; }
@@ -413,24 +419,26 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
         Ctl *g = P.ctl;
         const long long nm = (long long)P.n * P.m;
         long long slots = 0, terms = (long long)checks_s * nm;
-        int w = A, ran = 0;
+        int w = c.n_running, ran = 0;                // running lanes; the launch's width is theirs, or W under a mask
+        const bool full = P.mode == MODE_MASKED && !P.early_exit;
         for (int j = 0; j < K; ++j) {
-            terms += (long long)w * nm;              // the f-leg whose epilogue screened the state after k0 + j cycles
+            terms += (long long)(full ? A : w) * nm; // the f-leg whose epilogue screened the state after k0 + j cycles
             w -= left_at[j];
             if (w == 0) break;
-            if (k0 + j < P.widths_cap) P.widths[k0 + j] = w;      // cycle k0 + j + 1 ran at width w
-            slots += w;
-            terms += (long long)w * nm;              // its g-leg
+            const int width = full ? A : w;
+            if (k0 + j < P.widths_cap) P.widths[k0 + j] = width;      // cycle k0 + j + 1 ran at this width
+            slots += width;
+            terms += (long long)width * nm;          // its g-leg
             ++ran;
         }
         g->cycle = k0 + ran;
         g->parity = parity_new;
         g->emit_parity = parity_new ^ 1;             // the move copies the OTHER buffer: the survivors' current row potentials
-        g->n_phys = Anew; g->n_running = Anew;
+        g->n_phys = Anew; g->n_running = c.n_running - nret;
         g->n_retire = FUSE ? 0 : nholes;
         g->slots += slots;
         g->pair_terms += terms;
-        if (Anew == 0) g->done = 1;
+        if (c.n_running == nret) g->done = 1;
     }
     if (FUSE && nholes > 0) {
         __syncthreads();
@@ -483,9 +491,9 @@ __device__ __forceinline__ void emit_move_one(const Dev &P, const Ctl &c, const 
     // Move the survivor in slot `src` into the hole `slot`: all of its slot-indexed arrays as ONE list
     // of 16-byte vectors, so that a thread's loads in flight span arrays (array after array, each
     // with its own loop, cost one DRAM round trip per array: ~15 us for any lane size).
-    __shared__ const uint4 *seg_src[16];
-    __shared__ uint4 *seg_dst[16];
-    __shared__ unsigned seg_end[16];          // running total of vectors up to and including the segment
+    __shared__ const uint4 *seg_src[24];
+    __shared__ uint4 *seg_dst[24];
+    __shared__ unsigned seg_end[24];          // running total of vectors up to and including the segment
     __shared__ int seg_n;
     __syncthreads();                          // the table may still be in use by this block's previous retiree
     if (threadIdx.x == 0) {
@@ -514,10 +522,15 @@ __device__ __forceinline__ void emit_move_one(const Dev &P, const Ctl &c, const 
         add(P.la2, (size_t)P.np * 8); add(P.lb2, (size_t)P.mp * 8);
         add(P.wa, (size_t)P.np * 8); add(P.wb, (size_t)P.mp * 8);
         add(P.phi[np_], (size_t)P.np * 8);
-        add(P.ft[np_], (size_t)P.np * sizeof(T));
-        add(P.fl[np_], (size_t)P.np * sizeof(T));
-        add(P.gt, (size_t)P.mp * sizeof(T));
-        add(P.gl, (size_t)P.mp * sizeof(T));
+        if (P.phi0) {                                                 // lanes on the scaling kernel have no streamed terms
+            add(P.phi0, (size_t)P.np * 8); add(P.gam0, (size_t)P.mp * 8);
+            add(P.uu[np_], (size_t)P.np * 8); add(P.vv, (size_t)P.mp * 8);
+        } else {
+            add(P.ft[np_], (size_t)P.np * sizeof(T));
+            add(P.fl[np_], (size_t)P.np * sizeof(T));
+            add(P.gt, (size_t)P.mp * sizeof(T));
+            add(P.gl, (size_t)P.mp * sizeof(T));
+        }
         seg_n = ns;
     }
     __syncthreads();
@@ -675,7 +688,7 @@ static size_t lane_state_bytes(const Dev &P)
     size_t coords = (size_t)P.DP * (P.np + P.mp) * ts;
     if (P.tensor) coords = ((size_t)((P.n + 127) / 128) + (size_t)((P.m + 127) / 128)) * P.d * 256;
     if (P.guard > 0.0) coords += P.xraw_stride + P.yraw_stride;
-    return coords + (size_t)(P.np + P.mp) * (4 * 8 + 2 * ts + 8);
+    return coords + (size_t)(P.np + P.mp) * (4 * 8 + (P.phi0 ? 16 : 2 * ts) + 8);
 }
 // When even the retirement of every lane at once would move little (narrow batches of small
 // lanes), the planner's own block emits and moves, and the emit/move kernel is not launched:

@@ -72,6 +72,9 @@ struct Dev {
     double *wa, *wb;          // a, b
     double *phi[2];           // [W][np]
     double *gam;              // [W][mp]
+    // lanes whose kernel matrix is kept on chip (scaling_kernel; null otherwise): potentials absorbed
+    // into the matrix and the scalings relative to them
+    double *phi0, *gam0, *uu[2], *vv;
     // per-slot scalars
     double *scale;            // s
     int *lane_id;
@@ -81,6 +84,7 @@ struct Dev {
     int *flag;                // screen-positive at this audit
     int *verdict;             // two-sided check passed
     int *nonfinite;
+    int *absorbed, *cyc_log;  // scaling_kernel: phi0 .. vv are valid; the last f-leg ran in the log domain
     // multi-cycle launches: cycle count + 1 at which the lane in the slot left inside the launch
     // (0 = still running), and the column checks it ran
     int *ret_at, *n_checks;

@@ -44,7 +44,7 @@ struct Variant {
     bool (*lane_fits_shared)(int n, int m);
 };
 constexpr int MAX_CLUSTER_BLOCKS = MAX_CLUSTER_RANKS;   // a lane needs at most this many row blocks
-constexpr int MAX_CYCLES_IN_LAUNCH = 64;    // upper bound on the cycles one multi-cycle launch runs
+constexpr int MAX_CYCLES_IN_LAUNCH = 256;   // upper bound on the cycles one multi-cycle launch runs
 // Picks the variant for a shape (depends on the static shape only, so that every mode
 // and every run of the same batch uses the same reduction order).  Null if unsupported.
 const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_exp, int force_cs);
@@ -66,6 +66,10 @@ void launch_guard_pool(const Dev &P, cudaStream_t st);
 void launch_guard_strips(void *base, const GuardList &gl, bool fill, int *bad, cudaStream_t st);
 void launch_update_tc(const Dev &P, const void *maps, int leg, int width, cudaStream_t st);
 int launch_emit_move(const Dev &P, int width, cudaStream_t st);
+// lanes of mixed arithmetic small enough for their kernel matrix to stay on chip: whole cycles
+// (cycles > 0), or one leg as a launch of its own (cycles == 0)
+bool scaling_fits(int n, int m);
+void launch_scaling(const Dev &P, int leg, int cycles, int width, cudaStream_t st);
 int launch_plan_cycles(const Dev &P, int width, int cycles, cudaStream_t st);
 void launch_gather(const Dev &P, void *f, void *g, bool f64, cudaStream_t st);
 void launch_gather_audit(const Dev &P, float *rrow, float *rcol, int *flagged, cudaStream_t st);

@@ -1,0 +1,990 @@
+// Small lanes in mixed arithmetic: the lane's kernel matrix is formed once and kept in registers.
+//
+// With potentials (phi0, gam0) absorbed into the matrix,
+//     K_ij = 2^(phi0_i + gam0_j - s C_ij) / a_i,      phi = phi0 + log2 u,   gam = gam0 + log2 v,
+// the two legs of Eq. 3 are the scaling updates
+//     u_i = 1 / sum_j K_ij v_j,        v_j = b_j / sum_i K_ij a_i u_i,
+// one fp32 multiply-add per pair and leg instead of a d-term float64 distance and an exponential.
+// Exponents are float64 (rounded once, after the integer part has been split off), K is fp32, sums are
+// fp32 over at most 32 terms and float64 beyond, u, v and the potentials are float64: what the
+// log-domain kernels of the mixed arithmetic hold in 32 and in 64 bits is held so here.
+//
+// Range.  fp32 K has no entries below 2^-124.  An update that would take a u or v out of 2^+-60 is not
+// taken: the leg is done again in the log domain (log_rows / log_cols: per-row or per-column maximum,
+// then the sum, both passes over the distances), after which the new potentials are absorbed and K is
+// formed anew.  A lane whose u or v has left 2^+-30 after a cycle is absorbed too, so an entry that K
+// does not hold is below 2^(-124 + 30 + 60) = 2^-34 of its row or column sum.  The first cycle of a cold or
+// warm start is a log-domain cycle.  All of these decisions are taken per lane from the lane's own values, and K is a function of
+// (phi0, gam0) alone, which are part of the lane's state: a lane's bits depend neither on how its cycles
+// were shared out among launches nor on the mode.
+//
+// Work layout.  A cluster of NC blocks owns the lane; a block of NW warps owns NW * RW rows, a warp RW of
+// them, and a thread the entries of its warp's rows in CL columns, in registers: E = RW * CL values.  Row
+// sums are reduced by a halving exchange over the 32 threads; column sums go through shared memory (and
+// to the other blocks through distributed shared memory), every block forming all of v by itself.  One
+// cluster barrier and two block barriers per cycle: the column sums of the next state are formed before
+// the row residual has been decided on, and dropped where the lane leaves.
+//
+// What bounds it: the chain of dependent steps of a cycle (two rounds of multiply-adds, the exchange of row
+// sums, two float64 reciprocals, the column parts through shared memory, the exchange between blocks), not a
+// unit: the multiply-adds of a 256 x 256 lane are 256 clk of packed fp32 per scheduler, a cycle is 3700.
+// Measured per cycle in long launches, before (cost and exponential recomputed in every leg by a cluster of
+// eight blocks) -> now: 8 lanes of 64 x 64, d = 2: 5.3 -> 0.93 us; one lane of 256 x 256, d = 8: 1.9 us; all 1024
+// lanes of the sweep workload at tol 1e-3: 112 -> 24 ms per solve; the masked control at 96 lanes of
+// 100 x 77: 105 -> 5.7 ms (it ran one launch per leg).  Forming K costs 25 to 40 us per launch.
+// The exchange between blocks through remote stores that report to a barrier of the receiver, instead of a
+// cluster barrier: 2.9 -> 2.4 us; 128-thread blocks (two of different lanes per SM) instead of 256: 58 -> 47 us
+// per cycle of 1024 lanes, together with the rows' order that spares the selects of the exchange.
+#include "skb_update.cuh"
+#include "skb_host.h"
+
+namespace skb {
+
+enum ScalingWhat : int { SC_CYCLES = 3 };               // besides LEG_F, LEG_G, LEG_V: whole cycles
+constexpr int SC_TAKE = 60, SC_KEEP = 30;               // bands of log2 u and log2 v: update taken / K kept
+constexpr int SC_BAD = 1, SC_DRIFT = 2, SC_NF = 4;
+
+// 2^arg for a float64 argument: integer part split off in float64, the remainder (|.| <= 1/2) rounded
+// to fp32 and put through the Taylor series of e^(x ln 2) (degree 7: truncation 5e-9), so the result is
+// good to about an ulp whatever the size of the argument.  Zero below 2^-124.
+__device__ __forceinline__ float exp2_split(const double arg)
+{
+    const double x = fmin(fmax(arg, -200.0), 100.0);
+    const double magic = 6755399441055744.0;             // 1.5 * 2^52: the sum's low word is the integer part
+    const double t = x + magic;
+    const int ni = __double2loint(t);
+    const float f = (float)(x - (t - magic));
+    float q = 1.5252734e-5f;
+    q = fmaf(q, f, 1.5403530e-4f);
+    q = fmaf(q, f, 1.3333558e-3f);
+    q = fmaf(q, f, 9.6181291e-3f);
+    q = fmaf(q, f, 5.5504109e-2f);
+    q = fmaf(q, f, 2.4022651e-1f);
+    q = fmaf(q, f, 6.9314718e-1f);
+    const float p = fmaf(q, f, 1.0f);
+    return ni >= -124 ? __int_as_float(__float_as_int(p) + (ni << 23)) : 0.0f;
+}
+
+__device__ __forceinline__ u64 mul2(u64 a, u64 b)
+{
+    u64 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// 1 / s to float64 accuracy for s within the range of normal fp32 numbers: two Newton steps on the fp32
+// approximation.  Outside that range the result is 0, infinite or NaN, which out_of_band() reports.
+__device__ __forceinline__ double rcp64(const double s)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)s));
+    double x = (double)r;
+    x = fma(x, fma(-s, x, 1.0), x);
+    return fma(x, fma(-s, x, 1.0), x);
+}
+// x (u or v) is not within 2^+-BAND: negative, zero, infinite and NaN included
+template <int BAND>
+__device__ __forceinline__ bool out_of_band(const double x)
+{
+    return ((unsigned)__double2hiint(x) >> 20) - (unsigned)(1023 - BAND) >= (unsigned)(2 * BAND);
+}
+
+template <int NW_, int CL_, int RW_>
+struct ScalingShape {
+    static constexpr int NW = NW_, CL = CL_, RW = RW_;
+    static constexpr int THREADS = 32 * NW, COLS = 32 * CL, RB = NW * RW;
+    static constexpr int NQ = (COLS + THREADS - 1) / THREADS;        // columns a thread owns in the column steps
+    static constexpr int G = (CL >= 16 || CL * RW == 64) ? 2 : 4;    // rows whose distances are formed together
+    static constexpr int SHARE = 32 / RW;                            // threads that end up with the same row's sum
+    static constexpr int BLOCKS = (CL * RW >= 128 ? 256 : 512) / THREADS;   // registers: 255 / 128 a thread
+    static constexpr int FP32_COLS = CL <= 4 ? 8 : 32;               // columns a row's sum holds before it becomes float64
+    static constexpr int FP32_WARPS = CL >= 8 && RW <= 16 ? 2 : 1;   // warps' column parts added in fp32 (at most 32 rows)
+    static_assert(RW >= 8 && RW <= 32 && CL >= 2 && CL <= 16, "unsupported tile");
+    static size_t smem(int nc) { return sizeof(double) * 2 * (size_t)nc * COLS; }        // the exchange buffers
+};
+
+// x_i . y_j of the scaled coordinates for G consecutive rows and this thread's CL columns
+// (2 lane, 2 lane + 1, + 64, ...).  Rows and columns past the end read row / column 0; their results are
+// masked by the additive terms.
+template <int CL, int G>
+__device__ __forceinline__ void dot_tile(const double *xs, const double *ys, const int np, const int mp, const int d,
+                                         const int i0, const int lane, double (&acc)[G][CL])
+{
+#pragma unroll
+    for (int r = 0; r < G; ++r)
+#pragma unroll
+        for (int e = 0; e < CL; ++e) acc[r][e] = 0.0;
+    const double *xp = xs + (i0 < np ? i0 : 0);
+    int yo[CL / 2];
+#pragma unroll
+    for (int h = 0; h < CL / 2; ++h) { const int j = h * 64 + 2 * lane; yo[h] = j < mp ? j : 0; }
+#pragma unroll 1
+    for (int k = 0; k < d; ++k) {
+        double x[G];
+#pragma unroll
+        for (int r = 0; r < G; r += 2) {
+            const double2 t = *reinterpret_cast<const double2 *>(xp + (size_t)k * np + r);
+            x[r] = t.x; x[r + 1] = t.y;
+        }
+#pragma unroll
+        for (int h = 0; h < CL / 2; ++h) {
+            const double2 y = *reinterpret_cast<const double2 *>(ys + (size_t)k * mp + yo[h]);
+#pragma unroll
+            for (int r = 0; r < G; ++r) {
+                acc[r][2 * h] = fma(x[r], y.x, acc[r][2 * h]);
+                acc[r][2 * h + 1] = fma(x[r], y.y, acc[r][2 * h + 1]);
+            }
+        }
+    }
+}
+
+// Halving exchange: RW per-thread partial sums (one per row of the warp) -> the sum over the 32 threads of
+// row lane / SHARE.  Sums are fp32 while they hold at most LIM columns, float64 from there on.
+// PERM: threads hold the rows in an order of their own - local row r is row r ^ (lane / SHARE & ~3) - in
+// which the half to keep always comes first, so that the wide steps need no selects.
+template <int CL, int LIM, bool PERM, int OFF, int CNT, typename V>
+__device__ __forceinline__ double row_exchange(V (&s)[CNT], const int lane)
+{
+    constexpr int COLS_IN = CL * (32 / (2 * OFF));                 // columns a partial sum holds already
+    if constexpr (sizeof(V) == 4 && COLS_IN >= LIM) {
+        double t[CNT];
+#pragma unroll
+        for (int r = 0; r < CNT; ++r) t[r] = (double)s[r];
+        return row_exchange<CL, LIM, PERM, OFF, CNT, double>(t, lane);
+    } else {
+        if constexpr (CNT > 1) {
+            V h[CNT / 2];
+            const bool up = (lane & OFF) != 0;
+#pragma unroll
+            for (int r = 0; r < CNT / 2; ++r) {
+                const bool swap = !(PERM && CNT / 2 >= 4) && up;
+                const V keep = swap ? s[r + CNT / 2] : s[r], give = swap ? s[r] : s[r + CNT / 2];
+                h[r] = keep + __shfl_xor_sync(0xffffffffu, give, OFF);
+            }
+            if constexpr (OFF == 1) return (double)h[0];
+            else return row_exchange<CL, LIM, PERM, OFF / 2, CNT / 2, V>(h, lane);
+        } else {
+            V h[1] = {s[0] + __shfl_xor_sync(0xffffffffu, s[0], OFF)};
+            if constexpr (OFF == 1) return (double)h[0];
+            else return row_exchange<CL, LIM, PERM, OFF / 2, 1, V>(h, lane);
+        }
+    }
+}
+
+// Log-domain row step for the RW rows of a warp: integer-valued reference M >= every argument - 1 and
+// S = sum_j 2^(arg_ij - M), arg_ij = colB_j + x_i . y_j, of row lane / SHARE.  Two passes over the
+// distances; runs in the first cycle and where an update leaves the range of K.
+template <int NW, int CL, int RW>
+__device__ __noinline__ void log_rows(const double *xs, const double *ys, const int np, const int mp, const int d, const int i0,
+                                      const double *colB, double *S, double *M)
+{
+    typedef ScalingShape<NW, CL, RW> L;
+    const int lane = threadIdx.x & 31;
+    double mine = 0.0;
+    float part[RW];
+#pragma unroll
+    for (int g = 0; g < RW / L::G; ++g) {
+        double acc[L::G][CL], mr[L::G];
+        dot_tile<CL, L::G>(xs, ys, np, mp, d, i0 + g * L::G, lane, acc);
+#pragma unroll
+        for (int r = 0; r < L::G; ++r) {
+            double t = -1.0e300;
+#pragma unroll
+            for (int e = 0; e < CL; ++e) {
+                acc[r][e] += colB[(e / 2) * 64 + 2 * lane + (e & 1)];
+                t = fmax(t, acc[r][e]);
+            }
+            for (int off = 16; off > 0; off >>= 1) t = fmax(t, __shfl_xor_sync(0xffffffffu, t, off));
+            mr[r] = ceil(t);
+            if (lane / L::SHARE == g * L::G + r) mine = mr[r];
+            float s = 0.f;
+#pragma unroll
+            for (int e = 0; e < CL; ++e) s += exp2_split(acc[r][e] - mr[r]);
+            part[g * L::G + r] = s;
+        }
+    }
+    *S = row_exchange<CL, L::FP32_COLS, false, 16, RW, float>(part, lane);
+    *M = mine;
+}
+
+// Column counterpart of log_rows, first half: the maximum of rowA_i + x_i . y_j over the warp's rows.
+template <int NW, int CL, int RW>
+__device__ __noinline__ void log_cols_max(const double *xs, const double *ys, const int np, const int mp, const int d, const int i0,
+                                          const double *rowA, double *out)
+{
+    typedef ScalingShape<NW, CL, RW> L;
+    const int lane = threadIdx.x & 31;
+    double mc[CL];
+#pragma unroll
+    for (int e = 0; e < CL; ++e) mc[e] = -1.0e300;
+#pragma unroll 1
+    for (int g = 0; g < RW / L::G; ++g) {
+        double acc[L::G][CL];
+        dot_tile<CL, L::G>(xs, ys, np, mp, d, i0 + g * L::G, lane, acc);
+#pragma unroll
+        for (int r = 0; r < L::G; ++r)
+#pragma unroll
+            for (int e = 0; e < CL; ++e) mc[e] = fmax(mc[e], rowA[g * L::G + r] + acc[r][e]);
+    }
+#pragma unroll
+    for (int e = 0; e < CL; ++e) out[(e / 2) * 64 + 2 * lane + (e & 1)] = mc[e];
+}
+// ... second half: sums of 2^(rowA_i + x_i . y_j - M_j) over the warp's rows.
+template <int NW, int CL, int RW>
+__device__ __noinline__ void log_cols_sum(const double *xs, const double *ys, const int np, const int mp, const int d, const int i0,
+                                          const double *rowA, const double *colM, float *out)
+{
+    typedef ScalingShape<NW, CL, RW> L;
+    const int lane = threadIdx.x & 31;
+    float s[CL];
+#pragma unroll
+    for (int e = 0; e < CL; ++e) s[e] = 0.f;
+#pragma unroll 1
+    for (int g = 0; g < RW / L::G; ++g) {
+        double acc[L::G][CL];
+        dot_tile<CL, L::G>(xs, ys, np, mp, d, i0 + g * L::G, lane, acc);
+#pragma unroll
+        for (int r = 0; r < L::G; ++r)
+#pragma unroll
+            for (int e = 0; e < CL; ++e) s[e] += exp2_split(rowA[g * L::G + r] + acc[r][e] - colM[(e / 2) * 64 + 2 * lane + (e & 1)]);
+    }
+#pragma unroll
+    for (int e = 0; e < CL; ++e) out[(e / 2) * 64 + 2 * lane + (e & 1)] = s[e];
+}
+
+// Float64 re-evaluation of a block's rows (guard band); out of line so that its registers stay out of the
+// cycle loop's allocation.
+template <int NW>
+__device__ __noinline__ unsigned long long scaling_reeval(const Dev *P, const int slot, const int r0, const int r1, const double *pot,
+                                                          unsigned long long *red, int *bad)
+{
+    return direct_rows_block<NW>(*P, slot, r0, NW, r1, pot, r0, red, bad);
+}
+
+// Exchange between the blocks of a cluster without a cluster barrier: remote stores that report their bytes
+// to a barrier in the receiver's shared memory, which the receiver waits on.  (A cluster barrier's release
+// waits until all of the block's remote stores have been acknowledged: about 850 clk per cycle at four
+// blocks; measured.)  The wait is bounded like every wait of this library.
+constexpr long long SC_WAIT_CLOCKS = 2000000000LL;
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ unsigned peer_addr(const unsigned a, const unsigned rank)
+{
+    unsigned x;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(x) : "r"(a), "r"(rank));
+    return x;
+}
+__device__ __forceinline__ void st_async(const unsigned addr, const unsigned long long v, const unsigned bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr), "l"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async2(const unsigned addr, const unsigned long long v0, const unsigned long long v1, const unsigned bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(addr), "l"(v0), "l"(v1), "r"(bar) : "memory");
+}
+__device__ __forceinline__ bool bar_try_wait(const unsigned a, const unsigned parity)
+{
+    unsigned ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(a), "r"(parity) : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool bar_wait(const unsigned a, const unsigned parity)
+{
+    if (bar_try_wait(a, parity)) return true;
+    const long long t0 = clock64();
+    while (!bar_try_wait(a, parity))
+        if (clock64() - t0 > SC_WAIT_CLOCKS) return false;
+    return true;
+}
+
+template <bool CLU>
+__device__ __forceinline__ void scaling_barrier()
+{
+    if constexpr (CLU) cluster_sync_all();
+    else __syncthreads();
+}
+
+// what = SC_CYCLES: up to `cycles` whole cycles of every lane; LEG_F / LEG_V / LEG_G: one leg as a launch of its
+// own, for STATIC batches (whose common last cycle only the planner knows), phase timing and dry runs.
+// CLU = 0: a lane has one block (its rows fit), and nothing of the cluster machinery is in the way.
+template <int NW, int CL, int RW, bool CLU>
+__global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) scaling_kernel(const __grid_constant__ Dev P, const int what, const int cycles)
+{
+    typedef ScalingShape<NW, CL, RW> L;
+    constexpr int THREADS = L::THREADS, COLS = L::COLS, RB = L::RB, NQ = L::NQ, SHARE = L::SHARE;
+
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ unsigned long long swr[NW];
+    __shared__ unsigned long long xw[2][MAX_CLUSTER_RANKS * NW];    // residual part and flags of every warp of the cluster
+    __shared__ int sflag;                                // column flags
+    __shared__ __align__(16) double partd[NW * COLS];    // column parts of every warp
+    float *partf = reinterpret_cast<float *>(partd);
+    __shared__ __align__(16) double colB[COLS], rowA[RB];       // additive terms of columns / own rows
+    __shared__ __align__(16) float vs[COLS];             // v of all columns
+    __shared__ __align__(16) float2 uas[RB];             // a u of own rows, in both halves
+    __shared__ __align__(8) unsigned long long xbar[2];  // arrival of an exchange's stores, one per buffer
+
+    pdl_enter();
+    const Ctl c = *P.ctl;
+    const int slot = blockIdx.y;
+    if (c.done || slot >= c.n_phys) return;              // every exit here is taken by the whole cluster
+    if (P.early_exit && P.state[slot] != 0) return;
+    if (what != SC_CYCLES) {
+        if (what != LEG_V && c.static_final) return;
+        if (what == LEG_V && !(c.static_final || lane_needs_column_check(P, c, slot))) return;
+    }
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b = CLU ? (int)blockIdx.x : 0, NC = CLU ? (int)gridDim.x : 1;
+    double *xbuf = reinterpret_cast<double *>(smem_raw);                 // [2][NC][COLS] column parts of every block
+    int xch = 0;                                                         // exchanges so far: their buffer alternates
+
+    const double *xs = reinterpret_cast<const double *>(P.xs) + (size_t)slot * P.DP * P.np;
+    const double *ys = reinterpret_cast<const double *>(P.ys) + (size_t)slot * P.DP * P.mp;
+    const int i0 = b * RB + warp * RW;                   // first row of this warp
+    const int lr = warp * RW + lane / SHARE;             // this thread's row (SHARE threads hold the same one)
+    const int perm = lane / SHARE & ~3;                  // order of the rows in K (see row_exchange)
+    const int i = b * RB + lr;
+    const bool rok = i < P.n, rown = rok && lane % SHARE == 0;
+    const int j0 = tid * NQ;                             // this thread's columns in the column steps: NQ adjacent ones
+    const bool cown = COLS >= THREADS || tid < COLS;
+    const size_t ro = (size_t)slot * P.np + (rok ? i : 0), co = (size_t)slot * P.mp;
+    const int lane_id = P.lane_id[slot], start = P.start[slot];
+    const double inv_s = 1.0 / P.scale[slot];
+    const double a_i = rok ? P.wa[ro] : 0.0, a_fix = a_i * RSUM_SCALE;
+    bool frozen = P.mode == MODE_MASKED && P.state[slot] != 0;
+
+    // state: `us`, `vsd` are u and v while `ab` (potentials absorbed into K), the potentials themselves before
+    bool ab = P.absorbed[slot] != 0;
+    // (the absorbed potentials stay in registers: every block holds all columns', and global memory gets them
+    // back only at the end, when no block of the cluster can still be reading)
+    double us = ab ? 1.0 : 0.0, phi0 = 0.0, vsd[NQ], gam0[NQ], bq[NQ];
+    if (rok) { us = ab ? P.uu[c.parity][ro] : P.phi[c.parity][ro]; phi0 = P.phi0[ro]; }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        const int j = j0 + q;
+        const bool has = cown && j < P.m;
+        vsd[q] = has ? (ab ? P.vv[co + j] : P.gam[co + j]) : 0.0;
+        gam0[q] = has ? P.gam0[co + j] : 0.0;
+        bq[q] = has ? P.wb[co + j] : 0.0;
+    }
+    // residual totals above this (fixed point) can neither pass the screen nor lie in the guard band
+    unsigned long long near_tot;
+    {
+        double t = P.tol_screen;
+        if (P.guard > 0.0) {
+            t = fmax(t, P.tol_screen + fmax(P.guard * P.tol_screen, GUARD_ABS_FLOOR));
+            t = fmax(t, P.tol_stop + fmax(P.guard * P.tol_stop, GUARD_ABS_FLOOR));
+        }
+        near_tot = (unsigned long long)fmin(t * 1.000001 * RSUM_SCALE, 1.0e18) + 2ull;
+    }
+    if (tid == 0) {
+        sflag = 0;
+        if constexpr (CLU) {
+            for (int e = 0; e < 2; ++e) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&xbar[e])) : "memory");
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+    }
+    unsigned xphase = 0u;                                // phase of each buffer's barrier
+    bool dead = false;                                   // a bounded wait ran out
+    scaling_barrier<CLU>();                              // every block's shared memory is there
+
+    u64 K[RW][CL / 2];                                   // pairs of columns
+    auto row_phi = [&](const double x) -> double { return ab ? phi0 + log2(x) : x; };
+    auto col_gam = [&](const int q) -> double { return ab ? gam0[q] + log2(vsd[q]) : vsd[q]; };
+    // column parts of sum_i K_ij w_i, w in uas: one row of partf per warp
+    auto col_parts = [&]() {
+        u64 acc[CL / 2];
+#pragma unroll
+        for (int r = 0; r < RW; r += 4) {
+            const ulonglong2 w0 = *reinterpret_cast<const ulonglong2 *>(uas + warp * RW + (r ^ perm));
+            const ulonglong2 w1 = *reinterpret_cast<const ulonglong2 *>(uas + warp * RW + (r ^ perm) + 2);
+            const u64 wr[4] = {w0.x, w0.y, w1.x, w1.y};
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int h = 0; h < CL / 2; ++h) acc[h] = r + q ? fma2(K[r + q][h], wr[q], acc[h]) : mul2(K[0][h], wr[0]);
+        }
+#pragma unroll
+        for (int h = 0; h < CL / 2; ++h) *reinterpret_cast<u64 *>(partf + warp * COLS + h * 64 + 2 * lane) = acc[h];
+    };
+    // this block's part of column j: fp32 up to 32 rows, float64 beyond
+    auto block_col = [&](const int j) -> double {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < NW; w += L::FP32_WARPS) {
+            if constexpr (L::FP32_WARPS == 2) t += (double)(partf[w * COLS + j] + partf[(w + 1) * COLS + j]);
+            else t += (double)partf[w * COLS + j];
+        }
+        return t;
+    };
+    // exact sum over a warp of fixed-point terms below 2^47, valid in every thread
+    auto warp_fixed = [&](const unsigned long long x) -> unsigned long long {
+        const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)x & 0x3ffffffu);
+        const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 26));
+        return (unsigned long long)lo + ((unsigned long long)hi << 26);
+    };
+    // a term of a residual, scaled to the fixed point and clamped (never NaN), as an integer
+    auto to_fixed = [&](const double t) -> unsigned long long {
+        const double z = fmin(t, RSUM_ROW_MAX * RSUM_SCALE) + 0x1p52;
+        return ((unsigned long long)(__double2hiint(z) & 0xfffff) << 32) | (unsigned)__double2loint(z);
+    };
+    // hands `val` (one per owned column) to every block, then the barrier; in column order of the blocks
+    auto send_cols = [&](const double (&val)[NQ]) {
+        double *dst = xbuf + ((size_t)(xch & 1) * NC + b) * COLS;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int j = j0 + q;
+            if (cown) {
+                if constexpr (!CLU) dst[j] = val[q];
+                else for (int rk = 0; rk < NC; ++rk) st_cluster<double>(dst + j, rk, val[q]);
+            }
+        }
+    };
+    // every warp's residual part and flags (bits 60 and up) go to every block ...
+    auto rows_word = [&](const unsigned long long fx, const int flags) -> unsigned long long {
+        unsigned long long word = warp_fixed(fx);
+        if (__any_sync(0xffffffffu, flags)) word |= (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)flags) << 60;
+        return word;
+    };
+    auto send_rows = [&](const unsigned long long fx, const int flags) {
+        const unsigned long long word = rows_word(fx, flags);
+        if constexpr (CLU) { if (lane < NC) st_cluster<unsigned long long>(&xw[xch & 1][b * NW + warp], lane, word); }
+        else if (lane == 0) xw[xch & 1][warp] = word;
+    };
+    // ... and are added up by everyone, after the exchange's barrier
+    auto recv_rows = [&](int &flags) -> unsigned long long {
+        const unsigned long long low = (1ull << 60) - 1ull;
+        if constexpr (!CLU) {
+            unsigned long long t = 0ull, f = 0ull;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) { const unsigned long long x = xw[xch & 1][w]; t += x & low; f |= x; }
+            flags = (int)(f >> 60);
+            return t;
+        } else {
+            unsigned lo = 0u, hi = 0u, f = 0u;
+            for (int e = lane; e < NC * NW; e += 32) {
+                const unsigned long long w = xw[xch & 1][e];
+                lo += (unsigned)w & 0x3ffffffu;
+                hi += (unsigned)((w & low) >> 26);
+                f |= (unsigned)(w >> 60);
+            }
+            lo = __reduce_add_sync(0xffffffffu, lo);
+            hi = __reduce_add_sync(0xffffffffu, hi);
+            flags = __any_sync(0xffffffffu, f) ? (int)__reduce_or_sync(0xffffffffu, f) : 0;
+            return (unsigned long long)lo + ((unsigned long long)hi << 26);
+        }
+    };
+    auto recv_col = [&](const int j, const bool is_max) -> double {
+        const double *src = xbuf + (size_t)(xch & 1) * NC * COLS + j;
+        double t = src[0];
+        for (int rk = 1; rk < NC; ++rk) { const double o = src[(size_t)rk * COLS]; t = is_max ? fmax(t, o) : t + o; }
+        return t;
+    };
+    // log-domain column step from row potentials `phi`: the potential of every owned column that makes its
+    // marginal equal to its weight
+    auto log_cols = [&](const double phi, double (&pnew)[NQ]) {
+        if (lane % SHARE == 0) rowA[lr] = rok ? phi - P.sqx[ro] : -1.0e30;
+        __syncwarp();
+        log_cols_max<NW, CL, RW>(xs, ys, P.np, P.mp, P.d, i0, rowA + warp * RW, partd + warp * COLS);
+        __syncthreads();
+        double val[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int j = j0 + q;
+            val[q] = -1.0e300;
+            if (cown) for (int w = 0; w < NW; ++w) val[q] = fmax(val[q], partd[w * COLS + j]);
+        }
+        send_cols(val);
+        scaling_barrier<CLU>();
+        double mc[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int j = j0 + q;
+            mc[q] = 0.0;
+            if (cown) { mc[q] = ceil(recv_col(j, true)); colB[j] = mc[q]; }
+        }
+        ++xch;
+        __syncthreads();
+        log_cols_sum<NW, CL, RW>(xs, ys, P.np, P.mp, P.d, i0, rowA + warp * RW, colB, partf + warp * COLS);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) { const int j = j0 + q; val[q] = cown ? block_col(j) : 0.0; }
+        send_cols(val);
+        scaling_barrier<CLU>();
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int j = j0 + q;
+            pnew[q] = 0.0;
+            if (cown && j < P.m) pnew[q] = P.lb2[co + j] + P.sqy[co + j] - (mc[q] + log2(recv_col(j, false)));
+        }
+        ++xch;
+        __syncthreads();
+    };
+
+    int par = c.parity, k = c.cycle, it = 0, checks = 0, retired_at = 0, fl = 0;
+    int nf = what == SC_CYCLES && !frozen ? P.nonfinite[slot] : 0;
+    double rr = 0.0, rc = 0.0;
+    bool need_build = true, near = false;
+    for (;;) {
+        if (need_build && ab) {
+            if (lane % SHARE == 0) rowA[lr] = rok ? phi0 - P.la2[ro] - P.sqx[ro] : -1.0e30;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const int j = j0 + q;
+                if (cown) {
+                    colB[j] = j < P.m ? gam0[q] - P.sqy[co + j] : -1.0e30;
+                    vs[j] = (float)vsd[q];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int g = 0; g < RW / L::G; ++g) {
+                double acc[L::G][CL];
+                dot_tile<CL, L::G>(xs, ys, P.np, P.mp, P.d, i0 + ((g * L::G) ^ perm), lane, acc);
+#pragma unroll
+                for (int r = 0; r < L::G; ++r) {
+                    const double ra = rowA[warp * RW + ((g * L::G) ^ perm) + r];
+#pragma unroll
+                    for (int h = 0; h < CL / 2; ++h)
+                        K[g * L::G + r][h] = pack2(exp2_split(ra + colB[h * 64 + 2 * lane] + acc[r][2 * h]),
+                                                   exp2_split(ra + colB[h * 64 + 2 * lane + 1] + acc[r][2 * h + 1]));
+                }
+            }
+            __syncthreads();
+        }
+        need_build = false;
+
+        // ---------------- whole cycles on K while nothing needs a decision; the f-leg yields the row residual
+        // of the state before it, and the column sums of the state after it are formed beside it
+        bool scal = ab, done = false;
+        double unew = 0.0, T[NQ];
+        unsigned long long tot = 0ull;
+        int all = SC_BAD;                            // "the f-leg is still to be done, in the log domain"
+        if (ab && (what == SC_CYCLES || what == LEG_F)) {
+#pragma unroll 1
+            for (;;) {
+                {
+                    u64 v[CL / 2];
+                    float s[RW];
+#pragma unroll
+                    for (int h = 0; h < CL / 2; ++h) v[h] = *reinterpret_cast<const u64 *>(vs + h * 64 + 2 * lane);
+#pragma unroll
+                    for (int r = 0; r < RW; ++r) {
+                        u64 t = mul2(K[r][0], v[0]);
+#pragma unroll
+                        for (int h = 1; h < CL / 2; ++h) t = fma2(K[r][h], v[h], t);
+                        float s0, s1;
+                        unpack2(t, s0, s1);
+                        s[r] = s0 + s1;
+                    }
+                    const double S = row_exchange<CL, L::FP32_COLS, true, 16, RW, float>(s, lane);
+                    unew = rok ? rcp64(S) : 1.0;
+                    const double term = rown ? a_fix * fabs(fma(us, S, -1.0)) : 0.0;
+                    const int flags = (out_of_band<SC_TAKE>(unew) ? SC_BAD : 0) | (out_of_band<SC_KEEP>(unew) ? SC_DRIFT : 0);
+                    if (lane % SHARE == 0) { const float w = (float)(a_i * unew); uas[lr] = make_float2(w, w); }
+                    __syncwarp();
+                    col_parts();
+                    const unsigned long long word = rows_word(to_fixed(term), flags);
+                    if constexpr (CLU) {
+                        if (lane < NC) st_async(peer_addr(smem_addr(&xw[xch & 1][b * NW + warp]), lane), word, peer_addr(smem_addr(&xbar[xch & 1]), lane));
+                    } else if (lane == 0) xw[xch & 1][warp] = word;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) { const int j = j0 + q; T[q] = cown ? block_col(j) : 0.0; }
+                if constexpr (CLU) {
+                    const unsigned bar = smem_addr(&xbar[xch & 1]);
+                    if (tid == 0)
+                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((unsigned)(NC * (COLS + NW) * 8)) : "memory");
+                    const unsigned dst = smem_addr(xbuf + ((size_t)(xch & 1) * NC + b) * COLS + j0);
+                    if (cown) {
+#pragma unroll
+                        for (int rk = 0; rk < MAX_CLUSTER_RANKS; ++rk) {
+                            if (rk >= NC) continue;
+                            if constexpr (NQ == 2) st_async2(peer_addr(dst, rk), (unsigned long long)__double_as_longlong(T[0]), (unsigned long long)__double_as_longlong(T[1]), peer_addr(bar, rk));
+                            else st_async(peer_addr(dst, rk), (unsigned long long)__double_as_longlong(T[0]), peer_addr(bar, rk));
+                        }
+                    }
+                    const bool ok = bar_wait(bar, (xphase >> (xch & 1)) & 1u);
+                    xphase ^= 1u << (xch & 1);
+                    if (__syncthreads_or(!ok)) { dead = true; break; }
+                }
+                tot = recv_rows(all);
+                if constexpr (CLU) {
+                    if (cown) {
+                        const double *src = xbuf + (size_t)(xch & 1) * NC * COLS + j0;
+#pragma unroll
+                        for (int rk = 0; rk < MAX_CLUSTER_RANKS; ++rk) {
+                            if (rk >= NC) continue;
+                            if constexpr (NQ == 2) {
+                                const double2 t = *reinterpret_cast<const double2 *>(src + rk * COLS);
+                                T[0] = rk ? T[0] + t.x : t.x; T[1] = rk ? T[1] + t.y : t.y;
+                            } else T[0] = rk ? T[0] + src[rk * COLS] : src[rk * COLS];
+                        }
+                    }
+                }
+                ++xch;
+                if (all || (tot <= near_tot && !frozen) || nf || k - start >= P.max_iter || what == LEG_F) break;
+                // g-leg
+                double vn[NQ];
+                int flags = 0;
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const int j = j0 + q;
+                    vn[q] = 0.0;
+                    if (cown) {
+                        if (j < P.m) {
+                            vn[q] = bq[q] * rcp64(T[q]);
+                            flags |= out_of_band<SC_KEEP>(vn[q]);
+                        }
+                        if (!frozen) vs[j] = (float)vn[q];
+                    }
+                }
+                if (__syncthreads_or(flags)) break;
+                if (!frozen) {
+                    us = unew;
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) vsd[q] = vn[q];
+                }
+                ++k;
+                par ^= 1;
+                if (++it >= cycles) { done = true; break; }
+            }
+        }
+        if (dead) {
+            if (tid == 0) atomicOr(&P.ctl->error, ERR_WAIT);
+            break;
+        }
+        if (done) {
+            rr = (double)tot * (1.0 / RSUM_SCALE);
+            break;
+        }
+
+        // ---------------- f-leg in the log domain, where K cannot be used
+        if (what != LEG_V && what != LEG_G) {
+            if (all & SC_BAD) {
+                scal = false;
+                double term = 0.0;                       // in units of the fixed point
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const int j = j0 + q;
+                    if (cown) colB[j] = j < P.m ? col_gam(q) - P.sqy[co + j] : -1.0e30;
+                }
+                __syncthreads();
+                double S, M;
+                log_rows<NW, CL, RW>(xs, ys, P.np, P.mp, P.d, i0, colB, &S, &M);
+                unew = 0.0;
+                if (rok) row_math((int)FORM_DOT, true, P.la2[ro], P.sqx[ro], a_i, row_phi(us), (float)M, S, 0.f, unew, term);
+                const int flags = !isfinite(unew) || !isfinite(term) ? SC_NF : 0;
+                send_rows(rown && !flags ? to_fixed(term * RSUM_SCALE) : 0ull, flags);
+                scaling_barrier<CLU>();
+                tot = recv_rows(all);
+                ++xch;
+            }
+            if (all & SC_NF) nf = 1;
+            near = tot <= near_tot;
+            rr = (double)tot * (1.0 / RSUM_SCALE);
+            if (scal && (all & SC_DRIFT)) need_build = true;
+            {
+                if (what == LEG_F && !P.dry_run) {
+                    if (rown && !frozen) {
+                        P.phi[par ^ 1][ro] = scal ? phi0 + log2(unew) : unew;
+                        P.uu[par ^ 1][ro] = unew;
+                    }
+                    if (b == 0 && tid == 0) {
+                        P.rsum_row[slot] += tot;
+                        P.cyc_log[slot] = scal ? 0 : 1;
+                        if (nf && !frozen) P.nonfinite[slot] = 1;
+                    }
+                }
+            }
+            if (what == LEG_F) break;
+        }
+
+        // ---------------- audit of the state before the f-leg
+        if (what == SC_CYCLES) { fl = 0; rc = 0.0; }
+        if (what == SC_CYCLES && near && !frozen) {
+            const bool audited = lane_audited(P, k, start);
+            if (audited && !nf && in_guard_band(P, rr)) {
+                // guard band: decide from a float64 re-evaluation of the row residual; it reads the column
+                // potentials from global memory
+                if (lane % SHARE == 0) rowA[lr] = rok ? row_phi(us) : 0.0;
+                if (b == 0) {
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) { const int j = j0 + q; if (cown && j < P.m) P.gam[co + j] = col_gam(q); }
+                }
+                scaling_barrier<CLU>();
+                __syncthreads();
+                int bad;
+                const unsigned long long mine = scaling_reeval<NW>(&P, slot, b * RB, min(b * RB + RB, P.n), rowA, swr, &bad);
+                send_rows(tid == 0 ? mine : 0ull, bad ? SC_NF : 0);
+                scaling_barrier<CLU>();
+                int all;
+                const unsigned long long tot = recv_rows(all);
+                ++xch;
+                rr = (double)tot * (1.0 / RSUM_SCALE);
+                if (all & SC_NF) nf = 1;
+            }
+            fl = audited && !nf && rr <= P.tol_screen;
+        }
+        if (what == LEG_V || (what == SC_CYCLES && fl)) {
+            // column half of the two-sided check: the marginals of the audited state, genuinely measured
+            double term[NQ];
+            if (ab) {
+                if (lane % SHARE == 0) { const float w = (float)(a_i * us); uas[lr] = make_float2(w, w); }
+                __syncwarp();
+                col_parts();
+                __syncthreads();
+                double val[NQ];
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) { const int j = j0 + q; val[q] = cown ? block_col(j) : 0.0; }
+                send_cols(val);
+                scaling_barrier<CLU>();
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const int j = j0 + q;
+                    term[q] = (cown && j < P.m) ? fabs(vsd[q] * recv_col(j, false) - bq[q]) : 0.0;
+                }
+                ++xch;
+            } else {
+                double pn[NQ];
+                log_cols(us, pn);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const int j = j0 + q;
+                    term[q] = (cown && j < P.m) ? bq[q] * fabs(expm1((vsd[q] - pn[q]) * 0.6931471805599453)) : 0.0;
+                }
+            }
+            unsigned long long fx = 0ull;
+            int bad = 0;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                if (!isfinite(term[q])) bad = 1;
+                else fx += to_fixed(term[q] * RSUM_SCALE);
+            }
+            bad = __syncthreads_or(bad);
+            const unsigned long long ws = warp_fixed(fx);
+            if (lane == 0) swr[warp] = ws;
+            __syncthreads();
+            unsigned long long totc = 0ull;                           // every block has all columns: the same total
+            for (int w = 0; w < NW; ++w) totc += swr[w];
+            __syncthreads();
+            if (bad) nf = 1;
+            rc = (double)totc * (1.0 / RSUM_SCALE);
+            ++checks;
+            if (what == LEG_V) {
+                if (b == 0 && tid == 0 && !P.dry_run) { P.rsum_col[slot] += totc; if (bad) P.nonfinite[slot] = 1; }
+                break;
+            }
+        }
+        if (what == SC_CYCLES && !frozen && (near || nf || k - start >= P.max_iter)) {
+            const bool vd = !nf && fmax(rr, rc) <= P.tol_stop;
+            const bool limit = k - start >= P.max_iter;
+            int st = LANE_RUNNING;
+            if (nf) st = LANE_NONFINITE;
+            else if (fl && vd) st = LANE_DONE;
+            else if (limit) st = LANE_ITER_LIMIT;
+            if (st != LANE_RUNNING) {
+                if (rown) P.f_out[(size_t)lane_id * P.n + i] = row_phi(us) * inv_s;
+                if (b == 0) {
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) { const int j = j0 + q; if (cown && j < P.m) P.g_out[(size_t)lane_id * P.m + j] = col_gam(q) * inv_s; }
+                    if (tid == 0) {
+                        P.res_row[lane_id] = rr;
+                        P.res_col[lane_id] = fl ? rc : __longlong_as_double(0x7ff8000000000000LL);
+                        P.depth[lane_id] = (limit && st != LANE_DONE) ? P.max_iter : k - start;
+                        P.status[lane_id] = st;
+                        P.emitted[lane_id] = 1;
+                        if (P.mode == MODE_MASKED) P.state[slot] = 1;
+                    }
+                }
+                retired_at = k + 1;
+                if (P.mode == MODE_ACTIVE || P.early_exit) break;
+                frozen = true;                           // logical mask: the work goes on, nothing is stored
+            }
+        }
+
+        // ---------------- g-leg
+        double vnew[NQ];
+        bool log_g = false;
+        if (what == LEG_G) {
+            // us is what the f-leg left (u, or the row potential where it ran in the log domain)
+            log_g = !ab || P.cyc_log[slot] != 0;
+            unew = us;
+            scal = !log_g;
+            if (scal) {
+                if (lane % SHARE == 0) { const float w = rok ? (float)(a_i * unew) : 0.f; uas[lr] = make_float2(w, w); }
+                __syncwarp();
+                col_parts();
+                send_rows(0ull, rok && out_of_band<SC_KEEP>(unew) ? SC_DRIFT : 0);
+                __syncthreads();
+                double val[NQ];
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) { const int j = j0 + q; val[q] = cown ? block_col(j) : 0.0; }
+                send_cols(val);
+                scaling_barrier<CLU>();
+                int all;
+                recv_rows(all);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) { const int j = j0 + q; T[q] = cown ? recv_col(j, false) : 0.0; }
+                ++xch;
+                need_build = (all & SC_DRIFT) != 0;
+            }
+        }
+        if (scal) {
+            int flags = 0;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const int j = j0 + q;
+                vnew[q] = 0.0;
+                if (cown) {
+                    if (j < P.m) {
+                        vnew[q] = bq[q] * rcp64(T[q]);
+                        flags |= (out_of_band<SC_TAKE>(vnew[q]) ? SC_BAD : 0) | (out_of_band<SC_KEEP>(vnew[q]) ? SC_DRIFT : 0);
+                    }
+                    if (!frozen) vs[j] = (float)vnew[q];
+                }
+            }
+            if (flags) atomicOr(&sflag, flags);
+            __syncthreads();
+            const int all = sflag;
+            if (all) { __syncthreads(); if (tid == 0) sflag = 0; }
+            if (all & SC_DRIFT) need_build = true;
+            if (all & SC_BAD) log_g = true;
+        } else log_g = true;
+        double phinew = unew;                            // row potential, where the column step needs it
+        if (log_g) {
+            if (scal) phinew = rok ? phi0 + log2(unew) : 0.0;
+            log_cols(phinew, vnew);
+            need_build = true;
+            bool bad = false;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) bad = bad || !isfinite(vnew[q]);
+            if (__syncthreads_or(bad ? 1 : 0) && !frozen) nf = 1;
+        }
+        if (!frozen) {
+            if (need_build) {
+                // absorb the new potentials: K is formed anew from them
+                if (!log_g) {
+                    phinew = rok ? phi0 + log2(unew) : 0.0;
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) { const int j = j0 + q; if (cown && j < P.m) vnew[q] = gam0[q] + log2(vnew[q]); }
+                }
+                ab = true;
+                us = 1.0;
+                phi0 = phinew;
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) gam0[q] = vnew[q];
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) { const int j = j0 + q; vsd[q] = (cown && j < P.m) ? 1.0 : 0.0; }
+            } else {
+                us = unew;
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) vsd[q] = vnew[q];
+            }
+        } else need_build = false;
+        if (what == LEG_G) {
+            if (!P.dry_run && !frozen) {
+                if (nf && b == 0 && tid == 0) P.nonfinite[slot] = 1;
+                if (need_build && rown) { P.uu[par][ro] = 1.0; P.phi0[ro] = phi0; }
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const int j = j0 + q;
+                    if (b == 0 && cown && j < P.m) {
+                        P.vv[co + j] = vsd[q];
+                        P.gam0[co + j] = gam0[q];
+                        P.gam[co + j] = col_gam(q);
+                    }
+                }
+                if (b == 0 && tid == 0) P.absorbed[slot] = 1;
+            }
+            break;
+        }
+        ++k;
+        par ^= 1;
+        if (++it >= cycles) break;
+    }
+    if (what == SC_CYCLES) {
+        if (b == 0 && tid == 0) {
+            P.ret_at[slot] = retired_at;
+            P.n_checks[slot] = checks;
+            P.rrow[slot] = rr; P.rcol[slot] = rc; P.flag[slot] = fl;
+        }
+        if (!retired_at || P.mode == MODE_MASKED) {
+            // the lane goes back out; a frozen one keeps the state it froze with
+            if (rown) {
+                P.phi[par][ro] = row_phi(us);
+                P.uu[par][ro] = us;
+                P.phi0[ro] = phi0;
+            }
+            if (b == 0) {
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const int j = j0 + q;
+                    if (cown && j < P.m) { P.gam[co + j] = col_gam(q); P.vv[co + j] = vsd[q]; P.gam0[co + j] = gam0[q]; }
+                }
+                if (tid == 0) { P.absorbed[slot] = ab ? 1 : 0; if (nf) P.nonfinite[slot] = 1; }
+            }
+        }
+    }
+    if constexpr (CLU) cluster_sync_all();               // no block leaves while another may still write into its memory
+}
+
+// ---------------------------------------------------------------- host side
+struct ScalingVariant {
+    int threads, cols, rb;
+    bool cluster;                                        // lanes of several blocks
+    const void *kernel;
+    size_t (*smem)(int nc);
+};
+#define SKB_SC(NW, CL, RW, CLU) { 32 * NW, 32 * CL, NW * RW, CLU, (const void *)&scaling_kernel<NW, CL, RW, CLU>, &ScalingShape<NW, CL, RW>::smem }
+// narrowest column count first, then fewest rows per block
+static const ScalingVariant g_scaling[] = {
+    SKB_SC(2, 2, 8, false), SKB_SC(4, 2, 16, false), SKB_SC(4, 2, 32, false), SKB_SC(4, 2, 32, true),
+    SKB_SC(4, 4, 16, false), SKB_SC(4, 4, 32, false), SKB_SC(4, 4, 32, true),
+    SKB_SC(4, 8, 16, false), SKB_SC(4, 8, 16, true),
+    SKB_SC(8, 16, 8, true),
+};
+
+// The variant of a lane shape: the narrowest column tile that holds the columns; of its row tiles the
+// smallest that needs the fewest blocks.  Depends on the shape alone (the order of the sums follows from
+// it), so every mode and every launch of a batch uses the same one.  Null: the lane is too large.
+static const ScalingVariant *scaling_variant(int n, int m)
+{
+    const ScalingVariant *best = nullptr;
+    int best_nc = MAX_CLUSTER_RANKS + 1;
+    for (const ScalingVariant &v : g_scaling) {
+        if (m > v.cols || (best && v.cols > best->cols)) continue;
+        const int nc = (n + v.rb - 1) / v.rb;
+        if (nc > 1 && !v.cluster) continue;
+        if (nc < best_nc) { best = &v; best_nc = nc; }
+    }
+    return best;
+}
+
+bool scaling_fits(int n, int m) { return scaling_variant(n, m) != nullptr; }
+
+void launch_scaling(const Dev &P, int leg, int cycles, int width, cudaStream_t st)
+{
+    const ScalingVariant *v = scaling_variant(P.n, P.m);
+    const int nc = (P.n + v->rb - 1) / v->rb;
+    const size_t smem = v->smem(nc);
+    // (with the fixed arrays some variants are beyond the 48 KB that need no permission; the attribute belongs
+    // to the current device, so it is set with every launch)
+    if (v->cluster) cudaFuncSetAttribute(v->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nc, width < 1 ? 1 : width);
+    cfg.blockDim = dim3(v->threads);
+    cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = nc; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = v->cluster ? 2 : 1;
+    Dev dev = P;
+    int w = cycles > 0 ? (int)SC_CYCLES : leg, cy = cycles;
+    void *args[3] = {&dev, &w, &cy};
+    cudaLaunchKernelExC(&cfg, v->kernel, args);
+}
+
+}  // namespace skb

@@ -1185,3 +1185,32 @@ def test_plan_application_against_the_oracle(oracle, case):
 def want_row(oracle, w, k, f, g):
     row, _ = oracle.marginals(oracle.cost_matrix(w.x[k], w.y[k]), f, g, float(w.eps[k]))
     return row
+
+
+# ---- lanes whose kernel matrix stays on chip (mixed arithmetic) --------------------------------------
+@pytest.mark.parametrize("n,m", [(16, 64), (17, 63), (64, 2), (65, 64), (128, 33), (129, 64), (64, 65), (65, 128), (129, 100),
+                                 (64, 129), (65, 256), (512, 200), (513, 200), (64, 257), (300, 512), (513, 512)])
+def test_kernel_matrix_lanes_at_the_edges_of_their_tiles(oracle, n, m):
+    # first and last sizes of every tile shape and of the lanes that fit at all; one launch of many cycles
+    # (drain), one of one cycle each (step), a logical mask and the one-launch-per-leg path (phase timing)
+    # must give the same bits, whatever the lanes' K was formed from
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("sweep", W=3, n=n, m=m, d=5, max_iter=120)
+    r = run_gpu(w, compute="mixed")
+    check_against_oracle(oracle, w, r, range(3), pot_tol=POT_TOL_F32, exact_depth=False, floor=MARGIN_AUTO, max_iter=120,
+                         label=f"kernel matrix on chip, {n} x {m}")
+    check_accounting(oracle, r, 3, "active")
+    rm = run_gpu(w, compute="mixed", mode="masked")
+    np.testing.assert_array_equal(rm["f"], r["f"]); np.testing.assert_array_equal(rm["r_row"], r["r_row"])
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    for profiling in (False, True):
+        sb = B.SinkhornBatch(t(w.x), t(w.y), t(w.a), t(w.b), t(w.eps), w.tol, compute="mixed", max_iter=120)
+        sb.set_profiling(profiling)
+        for _ in range(121):
+            sb.step(1)
+        assert sb.active() == 0
+        f, g = sb.potentials(f64=True)
+        np.testing.assert_array_equal(f.cpu().numpy(), r["f"]); np.testing.assert_array_equal(g.cpu().numpy(), r["g"])
+        assert sb.check_guards() == -1
+        sb.close()
