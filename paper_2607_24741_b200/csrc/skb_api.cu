@@ -108,6 +108,13 @@ static double mixed_radius(double tol)
     return MIXED_RADIUS * (tol < 1.0e-3 ? tol / 1.0e-3 : 1.0);
 }
 
+// Large low-dimensional fp32 lanes go into spatial order (skb_near.cu) up to this tolerance.  Its arithmetic is also
+// the more accurate one: the expanded form's rounding, M * 8e-8 in every plan entry, is 3.5 % of a tolerance of
+// 1e-3 at the M = 430 of the registration workload.  Looser solves, where that is below a per cent or two, stay on
+// the expanded form and on the results they have always had: plans applied from them agree with earlier ones
+// to 1e-6, the other path's differ by as much as the expanded form's own error, 1.2e-6.
+static const double SPATIAL_TOL = 2.0e-3;
+
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 static bool config_ok(const skb_config *c, std::string &why)
@@ -142,7 +149,8 @@ static double guard_width(const skb_config *c)
 // Lays the batch's arrays out in the workspace (base may be null: size query only).
 // Every array is followed by a guard strip (GUARD_STRIP_BYTES of a known pattern, see
 // sinkhorn_batch_check_guards); their offsets are listed in *guards.
-static size_t carve(const skb_config *c, const Variant *var, bool tensor, char *base, Dev *D, size_t *zero_end_out = nullptr,
+// spatial: the batch may keep its lanes in spatial order (SPATIAL_TOL).
+static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool spatial, char *base, Dev *D, size_t *zero_end_out = nullptr,
                     GuardList *guards = nullptr)
 {
     size_t off = 0;
@@ -157,7 +165,9 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, char *
     };
     const size_t W = c->W, n = c->n, m = c->m;
     const size_t L = c->lane_capacity > c->W ? c->lane_capacity : c->W;      // lanes the result buffers hold
-    const size_t np = align_up(n, 4), mp = align_up(m, 4), DP = var->DP ? var->DP : padded_dim(c->d);
+    const size_t DP = var->DP ? var->DP : padded_dim(c->d);
+    const bool near = spatial && !tensor && near_shape(var->f64, var->DP, var->CS, c->n, c->m);      // lanes in spatial order: whole boxes
+    const size_t np = align_up(n, near ? BOX_COLS : 4), mp = align_up(m, near ? BOX_COLS : 4);
     const size_t ts = var->f64 ? 8 : 4;
     Dev d;
     memset(&d, 0, sizeof(d));
@@ -175,6 +185,7 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, char *
     d.guard_bad = (int *)take(4);
     d.state = (int *)take(W * 4); d.flag = (int *)take(W * 4); d.verdict = (int *)take(W * 4);
     d.nonfinite = (int *)take(W * 4);
+    d.radius = (double *)take(W * 8);
     d.absorbed = (int *)take(W * 4); d.cyc_log = (int *)take(W * 4);
     d.ret_at = (int *)take(W * 4); d.n_checks = (int *)take(W * 4);
     d.rsum_row64 = (unsigned long long *)take(W * 8); d.esc = (int *)take(W * 4);
@@ -209,6 +220,12 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, char *
     d.wa = (double *)take(W * np * 8); d.wb = (double *)take(W * mp * 8);
     d.phi[0] = (double *)take(W * np * 8); d.phi[1] = (double *)take(W * np * 8);
     d.gam = (double *)take(W * mp * 8);
+    if (near) {
+        d.nbx = (int)align_up((n + BOX_COLS - 1) / BOX_COLS, 4); d.nby = (int)align_up((m + BOX_COLS - 1) / BOX_COLS, 4);
+        d.permx = (int *)take(L * np * 4); d.permy = (int *)take(L * mp * 4);
+        d.boxx = (float *)take(W * 2 * DP * d.nbx * 4); d.boxy = (float *)take(W * 2 * DP * d.nby * 4);
+        d.topx[0] = (float *)take(W * d.nbx * 4); d.topx[1] = (float *)take(W * d.nbx * 4); d.topy = (float *)take(W * d.nby * 4);
+    }
     if (var->xf && var->DP && scaling_fits(c->n, c->m)) {
         d.phi0 = (double *)take(W * np * 8); d.gam0 = (double *)take(W * mp * 8);
         d.uu[0] = (double *)take(W * np * 8); d.uu[1] = (double *)take(W * np * 8); d.vv = (double *)take(W * mp * 8);
@@ -227,11 +244,11 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, char *
     return off;
 }
 
-static const Variant *variant_for(const skb_config *c, int compute)
+static const Variant *variant_for(const skb_config *c, int compute, bool spatial)
 {
     if (compute == SKB_COMPUTE_TENSOR) compute = SKB_COMPUTE_F32;     // fp32 epilogue, same scratch shapes
     const bool f64 = compute == SKB_COMPUTE_F64 || compute == SKB_COMPUTE_MIXED;
-    return choose_variant(c->W, c->n, c->m, c->d, f64, compute == SKB_COMPUTE_MIXED, c->column_split);
+    return choose_variant(c->W, c->n, c->m, c->d, f64, compute == SKB_COMPUTE_MIXED, c->column_split, spatial);
 }
 
 extern "C" size_t sinkhorn_batch_workspace_bytes(const skb_config *cfg)
@@ -240,12 +257,18 @@ extern "C" size_t sinkhorn_batch_workspace_bytes(const skb_config *cfg)
     if (!config_ok(cfg, why)) return 0;
     // an automatic batch may end up with float64 coordinates: size for the larger layout
     if (cfg->compute == SKB_COMPUTE_TENSOR && !tc_eligible(cfg->d, cfg->xy_dtype == SKB_BF16)) return 0;
-    const Variant *v = variant_for(cfg, cfg->compute == SKB_COMPUTE_AUTO ? SKB_COMPUTE_MIXED : cfg->compute);
+    const Variant *v = variant_for(cfg, cfg->compute == SKB_COMPUTE_AUTO ? SKB_COMPUTE_MIXED : cfg->compute, false);
     if (!v) return 0;
-    size_t need = carve(cfg, v, cfg->compute == SKB_COMPUTE_TENSOR, nullptr, nullptr);
+    size_t need = carve(cfg, v, cfg->compute == SKB_COMPUTE_TENSOR, false, nullptr, nullptr);
     if (cfg->compute == SKB_COMPUTE_AUTO && tc_eligible(cfg->d, cfg->xy_dtype == SKB_BF16)) {
-        const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32), true, nullptr, nullptr);
+        const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, false), true, false, nullptr, nullptr);
         if (t > need) need = t;
+    }
+    if (cfg->compute == SKB_COMPUTE_AUTO || cfg->compute == SKB_COMPUTE_F32) {
+        for (const bool spatial : {false, true}) {           // the tolerance, which decides, is not known here
+            const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, spatial), false, spatial, nullptr, nullptr);
+            if (t > need) need = t;
+        }
     }
     return need;
 }
@@ -275,8 +298,9 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     }
     if (!(tol > 0.0f) || !std::isfinite(tol)) return fail(nullptr, SKB_ERR_VALUE, "tol must be positive and finite");
     const bool automatic = cfg->compute == SKB_COMPUTE_AUTO;
-    const Variant *var = variant_for(cfg, automatic ? SKB_COMPUTE_F32 : cfg->compute);
-    const Variant *var_big = variant_for(cfg, automatic ? SKB_COMPUTE_MIXED : cfg->compute);
+    const bool spatial = (double)tol <= SPATIAL_TOL;
+    const Variant *var = variant_for(cfg, automatic ? SKB_COMPUTE_F32 : cfg->compute, spatial);
+    const Variant *var_big = variant_for(cfg, automatic ? SKB_COMPUTE_MIXED : cfg->compute, spatial);
     if (!var || !var_big) return fail(nullptr, SKB_ERR_SHAPE, "dimension d is not supported by any update kernel");
     const int mx = cfg->n > cfg->m ? cfg->n : cfg->m;
     // a lane's residual is a 64-bit fixed-point sum of per-row terms clamped at RSUM_ROW_MAX
@@ -287,7 +311,7 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     if (cfg->compute == SKB_COMPUTE_TENSOR && !can_tensor)
         return fail(nullptr, SKB_ERR_SHAPE, "the tensor-core path needs bf16 x, y and d a multiple of 64 with 64 <= d <= 512");
     size_t zero_end = 0;
-    carve(cfg, var_big, false, nullptr, nullptr, &zero_end);
+    carve(cfg, var_big, false, spatial, nullptr, nullptr, &zero_end);
     const size_t need = sinkhorn_batch_workspace_bytes(cfg);
     if (!cfg->workspace) return fail(nullptr, SKB_ERR_WORKSPACE, "workspace is null");
     if (((uintptr_t)cfg->workspace & 255u) != 0) return fail(nullptr, SKB_ERR_WORKSPACE, "workspace must be 256-byte aligned");
@@ -306,7 +330,7 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     h->lanes_used = cfg->W; h->enqueued_at_refill = 0;
     for (int i = 0; i < SKB_N_PHASES; ++i) h->phase_ms[i] = 0.f;
     h->guards.count = 0;
-    carve(cfg, var, h->tensor, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+    carve(cfg, var, h->tensor, spatial, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
     h->dev.tol_stop = (double)tol;
     h->dev.tol_screen = cfg->tol_screen > 0.0f ? (double)cfg->tol_screen : (double)tol;
     cudaError_t e;
@@ -345,10 +369,10 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
         const double ts = h->dev.tol_stop, tsc = h->dev.tol_screen;
         if (radius > mixed_radius(ts < tsc ? ts : tsc)) {
             h->var = var_big;
-            carve(cfg, var_big, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+            carve(cfg, var_big, false, spatial, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
         } else if (can_tensor) {
             h->tensor = true;
-            carve(cfg, var, true, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+            carve(cfg, var, true, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
         }
         h->dev.tol_stop = ts; h->dev.tol_screen = tsc;
     }
@@ -367,8 +391,9 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
             return st;
         }
     }
+    if (h->dev.permx) { launch_spatial_sort(h->dev, x, y, 0, cfg->W, h->stream); h->launches += 1; }
     launch_prep(h->dev, x, y, a, b, 0, cfg->W, h->stream);
-    if (h->dev.guard > 0.0) {
+    if (h->dev.guard > 0.0 && !h->dev.permx) {            // (lanes in spatial order: the layout kernel writes them)
         const size_t es = cfg->xy_dtype == SKB_BF16 ? 2 : 4;
         const size_t xb = (size_t)cfg->n * cfg->d * es, yb = (size_t)cfg->m * cfg->d * es;
         if ((e = cudaMemcpy2DAsync(h->dev.xraw, h->dev.xraw_stride, x, xb, xb, cfg->W, cudaMemcpyDeviceToDevice, h->stream)) != cudaSuccess ||
@@ -398,7 +423,11 @@ extern "C" skb_status sinkhorn_batch_warm_start(skb_batch *h, const double *f0, 
 {
     if (!h) return SKB_ERR_NULL;
     if (h->enqueued != 0) return fail(h, SKB_ERR_STATE, "a warm proposal must be given before the first step or drain");
-    if (f0 || g0) { launch_warm(h->dev, f0, g0, h->stream); h->launches += 1; }
+    if (f0 || g0) {
+        launch_warm(h->dev, f0, g0, h->stream);
+        h->launches += 1;
+        if (h->dev.permx) { launch_near_tops(h->dev, h->stream); h->launches += 1; }
+    }
     h->dev.audit_initial = audit_initial ? 1 : 0;
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? SKB_OK : cuda_fail(h, e, "warm_start");
@@ -438,8 +467,9 @@ extern "C" skb_status sinkhorn_batch_refill(skb_batch *h, const void *x, const v
         launch_retile(y, (char *)D.yb + (size_t)width * yt, count, h->cfg.m, h->cfg.d, h->stream);
         h->launches += 2;
     }
+    if (D.permx) { launch_spatial_sort(D, x, y, width, count, h->stream); h->launches += 1; }
     launch_prep(D, x, y, a, b, width, count, h->stream);
-    if (D.guard > 0.0) {
+    if (D.guard > 0.0 && !D.permx) {
         const size_t xb = (size_t)h->cfg.n * h->cfg.d * es, yb = (size_t)h->cfg.m * h->cfg.d * es;
         e = cudaMemcpy2DAsync((char *)D.xraw + (size_t)width * D.xraw_stride, D.xraw_stride, x, xb, xb, count, cudaMemcpyDeviceToDevice, h->stream);
         if (e == cudaSuccess)
@@ -479,6 +509,7 @@ static int launch_leg(skb_batch *h, int leg, int w)
 {
     if (h->tensor) { launch_update_tc(h->dev, h->maps, leg, w, h->stream); return 0; }
     if (h->dev.phi0) { launch_scaling(h->dev, leg, 0, w, h->stream); return 0; }
+    if (h->dev.permx) return launch_near(h->dev, leg, w, h->stream);
     return h->var->launch(h->dev, leg, w, h->stream);
 }
 
@@ -490,6 +521,7 @@ static bool cycles_in_one_launch(const skb_batch *h)
 {
     if (h->dev.phi0) return h->cfg.mode != SKB_STATIC && !h->profiling && !h->no_multi_cycle;
     if (h->cfg.mode != SKB_ACTIVE || h->tensor || h->profiling || !h->var->launch_cycles || h->no_multi_cycle) return false;
+    if (h->dev.permx) return false;
     const int mx = h->cfg.n > h->cfg.m ? h->cfg.n : h->cfg.m;
     const int nc = (mx + h->var->rows_per_cta - 1) / h->var->rows_per_cta;
     if (nc > MAX_CLUSTER_BLOCKS) return false;

@@ -69,7 +69,9 @@ __global__ void __launch_bounds__(256) lane_stats_kernel(const Dev P, const void
         P.rsum_row[slot] = 0ull; P.rsum_col[slot] = 0ull; P.rsum_row64[slot] = 0ull; P.esc[slot] = 0;
         P.ret_at[slot] = 0; P.n_checks[slot] = 0;
         P.absorbed[slot] = 0; P.cyc_log[slot] = 0;
-        int form = P.cost_form == 1 ? FORM_DOT : (P.cost_form == 2 ? FORM_DIFF : (s * red[0] > P.form_threshold ? FORM_DIFF : FORM_DOT));
+        P.radius[slot] = sqrt(red[0]);
+        // (lanes in spatial order have a form of their own, which shares the expanded form's scale and terms)
+        int form = P.permx ? FORM_DOT : P.cost_form == 1 ? FORM_DOT : (P.cost_form == 2 ? FORM_DIFF : (s * red[0] > P.form_threshold ? FORM_DIFF : FORM_DOT));
         P.form[slot] = form;
         atomicMax(&P.ctl->max_radius_bits, (unsigned long long)__double_as_longlong(eps_ok ? s * red[0] : 0.0));
     }
@@ -143,7 +145,8 @@ __global__ void warm_kernel(const Dev P, const double *f0, const double *g0)
     if (i >= npts) return;
     const double *src = side ? g0 : f0;
     if (!src) return;
-    const double v = src[(size_t)slot * npts + i];
+    const int *perm = side ? P.permy : P.permx;
+    const double v = src[(size_t)slot * npts + (perm ? perm[(size_t)P.lane_id[slot] * pp + i] : i)];
     if (!isfinite(v)) { atomicOr(&P.ctl->error, ERR_VALUE); return; }
     const int form = (sizeof(T) == 8) ? (int)FORM_DOT : P.form[slot];
     const size_t o = (size_t)slot * pp + i;
@@ -480,10 +483,10 @@ __device__ __forceinline__ void emit_move_one(const Dev &P, const Ctl &c, const 
     // in the hole wrote its own outputs when it left (multi-cycle launches), only the move is left
     if (lane >= 0)
         for (int i = tid; i < P.n; i += nth)
-            P.f_out[(size_t)lane * P.n + i] = P.phi[ep][(size_t)slot * P.np + i] * inv_s;
+            P.f_out[(size_t)lane * P.n + (P.permx ? P.permx[(size_t)lane * P.np + i] : i)] = P.phi[ep][(size_t)slot * P.np + i] * inv_s;
     for (int j = tid; j < P.m; j += nth) {
         // the hole's own g is read before the survivor's g is copied over it (same thread)
-        if (lane >= 0) P.g_out[(size_t)lane * P.m + j] = P.gam[(size_t)slot * P.mp + j] * inv_s;
+        if (lane >= 0) P.g_out[(size_t)lane * P.m + (P.permy ? P.permy[(size_t)lane * P.mp + j] : j)] = P.gam[(size_t)slot * P.mp + j] * inv_s;
         if (src >= 0) P.gam[(size_t)slot * P.mp + j] = P.gam[(size_t)src * P.mp + j];
     }
     if (tid == 0 && lane >= 0) P.emitted[lane] = 1;
@@ -531,6 +534,10 @@ __device__ __forceinline__ void emit_move_one(const Dev &P, const Ctl &c, const 
             add(P.gt, (size_t)P.mp * sizeof(T));
             add(P.gl, (size_t)P.mp * sizeof(T));
         }
+        if (P.topy) {                                                 // lanes in spatial order (the order itself is kept by lane)
+            add(P.boxx, (size_t)2 * P.DP * P.nbx * 4); add(P.boxy, (size_t)2 * P.DP * P.nby * 4);
+            add(P.topx[np_], (size_t)P.nbx * 4); add(P.topy, (size_t)P.nby * 4);
+        }
         seg_n = ns;
     }
     __syncthreads();
@@ -576,9 +583,9 @@ __global__ void gather_kernel(const Dev P, O *f, O *g)
         if (P.emitted[lane]) return;
         const double inv_s = 1.0 / P.scale[slot];
         if (f) for (int i = tid; i < P.n; i += nth)
-            f[(size_t)lane * P.n + i] = (O)(P.phi[c.parity][(size_t)slot * P.np + i] * inv_s);
+            f[(size_t)lane * P.n + (P.permx ? P.permx[(size_t)lane * P.np + i] : i)] = (O)(P.phi[c.parity][(size_t)slot * P.np + i] * inv_s);
         if (g) for (int j = tid; j < P.m; j += nth)
-            g[(size_t)lane * P.m + j] = (O)(P.gam[(size_t)slot * P.mp + j] * inv_s);
+            g[(size_t)lane * P.m + (P.permy ? P.permy[(size_t)lane * P.mp + j] : j)] = (O)(P.gam[(size_t)slot * P.mp + j] * inv_s);
     }
 }
 
@@ -664,7 +671,8 @@ void launch_prep(const Dev &P, const void *x, const void *y, const float *a, con
 {
     const int pp = P.np > P.mp ? P.np : P.mp;
     dim3 grid((pp + 127) / 128, count, 2);
-    if (P.compute_f64) prep_kernel<double><<<grid, 128, 0, st>>>(P, x, y, a, b, slot0);
+    if (P.permx) launch_prep_near(P, x, y, a, b, slot0, count, st);
+    else if (P.compute_f64) prep_kernel<double><<<grid, 128, 0, st>>>(P, x, y, a, b, slot0);
     else prep_kernel<float><<<grid, 128, 0, st>>>(P, x, y, a, b, slot0);
 }
 // New lanes have come in: the control block takes them into the width (between cycles, ACTIVE only).

@@ -26,6 +26,7 @@ enum Form : int { FORM_DOT = 0, FORM_DIFF = 1 };
 
 constexpr float NEG_BIG = -1.0e30f;   // "minus infinity" for padded columns (finite: no NaNs)
 constexpr int UPD_THREADS = 128;
+constexpr int BOX_COLS = 32;          // points per bounding box of lanes in spatial order
 constexpr int TC_MAX_SPLIT = 8;      // a row block's columns go to at most this many clusters
 constexpr int MAX_CLUSTER_RANKS = 8;  // blocks per cluster (portable limit): row blocks of a lane in the multi-cycle kernels
 constexpr double RSUM_SCALE = 17592186044416.0;     // 2^44: unit of the fixed-point residual sums
@@ -75,6 +76,11 @@ struct Dev {
     // lanes whose kernel matrix is kept on chip (scaling_kernel; null otherwise): potentials absorbed
     // into the matrix and the scalings relative to them
     double *phi0, *gam0, *uu[2], *vv;
+    // lanes in spatial order (update_near_kernel; null otherwise): point i of a lane is input point perm[lane][i];
+    // bounding boxes of every 32 points [2 DP][nb]; the largest potential of every 32 points, rounded up
+    int *permx, *permy;
+    float *boxx, *boxy, *topx[2], *topy;
+    int nbx, nby;             // boxes of 32 points, padded to a multiple of 4
     // per-slot scalars
     double *scale;            // s
     int *lane_id;
@@ -84,6 +90,7 @@ struct Dev {
     int *flag;                // screen-positive at this audit
     int *verdict;             // two-sided check passed
     int *nonfinite;
+    double *radius;           // largest distance of a point from the centre, in the inputs' units
     int *absorbed, *cyc_log;  // scaling_kernel: phi0 .. vv are valid; the last f-leg ran in the log domain
     // multi-cycle launches: cycle count + 1 at which the lane in the slot left inside the launch
     // (0 = still running), and the column checks it ran

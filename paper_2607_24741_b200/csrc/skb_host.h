@@ -47,7 +47,7 @@ constexpr int MAX_CLUSTER_BLOCKS = MAX_CLUSTER_RANKS;   // a lane needs at most 
 constexpr int MAX_CYCLES_IN_LAUNCH = 256;   // upper bound on the cycles one multi-cycle launch runs
 // Picks the variant for a shape (depends on the static shape only, so that every mode
 // and every run of the same batch uses the same reduction order).  Null if unsupported.
-const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_exp, int force_cs);
+const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_exp, int force_cs, bool spatial);
 int padded_dim(int d);
 
 void launch_lane_stats(const Dev &P, const void *x, const void *y, const float *eps, int slot0, int lane0, int count,
@@ -66,6 +66,13 @@ void launch_guard_pool(const Dev &P, cudaStream_t st);
 void launch_guard_strips(void *base, const GuardList &gl, bool fill, int *bad, cudaStream_t st);
 void launch_update_tc(const Dev &P, const void *maps, int leg, int width, cudaStream_t st);
 int launch_emit_move(const Dev &P, int width, cudaStream_t st);
+// lanes kept in spatial order, whose legs skip the boxes of columns that are too far away to matter
+bool near_shape(int f64, int DP, int CS, int n, int m);
+void launch_spatial_sort(const Dev &P, const void *x, const void *y, int slot0, int count, cudaStream_t st);
+void launch_prep_near(const Dev &P, const void *x, const void *y, const float *a, const float *b, int slot0, int count, cudaStream_t st);
+void launch_near_tops(const Dev &P, cudaStream_t st);
+int launch_near(const Dev &P, int leg, int width, cudaStream_t st);     // 1: the guard band's pool rode in a column-check launch
+int guard_pool_rows(int per_row, bool on, int lanes);
 // lanes of mixed arithmetic small enough for their kernel matrix to stay on chip: whole cycles
 // (cycles > 0), or one leg as a launch of its own (cycles == 0)
 bool scaling_fits(int n, int m);

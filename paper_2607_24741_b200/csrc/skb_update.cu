@@ -13,7 +13,7 @@ constexpr long long NARROW_BLOCKS = 148 * 4;      // below this many blocks some
 // Grid rows (of `per_row` blocks each) that hold the guard band's pool of about two blocks per SM.
 // None when the launch has no room for them (grid.y is 16 bits): the caller then runs the pool as
 // a launch of its own.
-static int pool_rows(int per_row, bool on, int lanes)
+int guard_pool_rows(int per_row, bool on, int lanes)
 {
     const int rows = on ? (2 * 148 + per_row - 1) / per_row : 0;
     return lanes + rows <= 65535 ? rows : 0;
@@ -45,7 +45,7 @@ static int launch_update(const Dev &P, int leg, int width, cudaStream_t st)   //
         const int rbw = (UPD_THREADS / 32) * RW * (32 / CS);
         const long long ctas = (long long)((nrows + rbw - 1) / rbw) * lanes;
         if (ctas >= 2 * 148 * 4) {
-            const int pool = pool_rows((nrows + rbw - 1) / rbw, guard_pool, lanes);
+            const int pool = guard_pool_rows((nrows + rbw - 1) / rbw, guard_pool, lanes);
             launch_pdl(update_kernel<T, DP, CS, XF, RW>, dim3((nrows + rbw - 1) / rbw, lanes + pool), dim3(UPD_THREADS), smem, st, P, leg, lanes);
             return pool > 0;
         }
@@ -61,13 +61,13 @@ static int launch_update(const Dev &P, int leg, int width, cudaStream_t st)   //
         const int rb2 = (UPD_THREADS / 32) * Tune<T, DP>::R * (32 / CS);
         if ((long long)((nrows + rb2 - 1) / rb2) * lanes < NARROW_BLOCKS) {
             const int rbr = (UPD_THREADS / 32) * 1 * (32 / CS);
-            const int pool = pool_rows((nrows + rbr - 1) / rbr, guard_pool, lanes);
+            const int pool = guard_pool_rows((nrows + rbr - 1) / rbr, guard_pool, lanes);
             launch_pdl(update_kernel<T, DP, CS, XF, 1>, dim3((nrows + rbr - 1) / rbr, lanes + pool), dim3(UPD_THREADS), smem, st, P, leg, lanes);
             return pool > 0;
         }
     }
     const int rb = (UPD_THREADS / 32) * Tune<T, DP>::R * (32 / CS);
-    const int pool = pool_rows((nrows + rb - 1) / rb, guard_pool, lanes);
+    const int pool = guard_pool_rows((nrows + rb - 1) / rb, guard_pool, lanes);
     launch_pdl(update_kernel<T, DP, CS, XF>, dim3((nrows + rb - 1) / rb, lanes + pool), dim3(UPD_THREADS), smem, st, P, leg, lanes);
     return pool > 0;
 }
@@ -153,7 +153,7 @@ int padded_dim(int d)
     return -1;
 }
 
-const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_exp, int force_cs)
+const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_exp, int force_cs, bool spatial)
 {
     const int DP = padded_dim(d);
     if (DP < 0) return nullptr;
@@ -184,6 +184,7 @@ const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_ex
         const double score = (util_n < util_m ? util_n : util_m) * fill * (c == 32 ? 0.6 : (c == 1 ? 0.85 : 1.0));
         if (score > best + 1e-9) { best = score; cs = c; }
     }
+    if (spatial && near_shape(f64 ? 1 : 0, DP, 4, n, m)) cs = 4;             // far columns are skipped: few steps are left to split
     if (force_cs == 1 || force_cs == 4 || force_cs == 32) cs = force_cs;
     for (const Variant &v : g_variants)
         if (v.f64 == (f64 ? 1 : 0) && v.xf == ((f64 && fast_exp) ? 1 : 0) && v.DP == DP && v.CS == cs) return &v;

@@ -501,7 +501,8 @@ __device__ __forceinline__ void split_potential(const int form, const double pne
 // term of the marginal residual (zero for the g-leg, which measures nothing).
 template <typename T>
 __device__ __forceinline__ double finish_one_row(const Dev &P, const Ctl &c, const int leg, const int slot, const int form,
-                                                 const int i, const float m, const double s, const float h, const bool writes)
+                                                 const int i, const float m, const double s, const float h, const bool writes,
+                                                 double *pot_out = nullptr)
 {
     const bool rows_x = (leg == LEG_F);
     const int rp = rows_x ? P.np : P.mp;
@@ -512,6 +513,7 @@ __device__ __forceinline__ double finish_one_row(const Dev &P, const Ctl &c, con
     const double pold = prow[i];
     double pnew, term;
     row_math(form, leg != LEG_G, lw, sq, leg != LEG_G ? (rows_x ? P.wa : P.wb)[o] : 0.0, pold, m, s, h, pnew, term);
+    if (pot_out) *pot_out = pnew;
     if (writes) {
         T hi, lo;
         split_potential<T>(form, pnew, sq, hi, lo);
@@ -549,7 +551,8 @@ __device__ __forceinline__ void finish_lane_residual(const Dev &P, const int leg
 // Float64 epilogue of a CTA's RB rows (one thread per row) and the fused residual reduction.
 // row_m / row_s hold, per CTA-local row, the integer-valued maximum and the sum of
 // 2^(arg - max) over ALL columns; row_h the fp32 shift a difference-form row carried.
-template <typename T, int RB, int THREADS = UPD_THREADS>
+// BOX: lanes in spatial order also keep the largest potential of every BOX_COLS points.
+template <typename T, int RB, int THREADS = UPD_THREADS, bool BOX = false>
 __device__ __forceinline__ void finish_rows(const Dev &P, const Ctl &c, const int leg, const int slot,
                                             const int form, const float *row_m, const double *row_s,
                                             const float *row_h, double *red, const int row_base)
@@ -562,6 +565,20 @@ __device__ __forceinline__ void finish_rows(const Dev &P, const Ctl &c, const in
     unsigned long long term_sum = 0ull;
     for (int lr = tid; lr < RB; lr += THREADS) {
         const int i = row_base + lr;
+        if constexpr (BOX) {
+            static_assert(RB % BOX_COLS == 0 && BOX_COLS == 32, "a warp's rows are one box");
+            double pot = -1.0e300, term = 0.0;
+            if (i < nrows) term = finish_one_row<T>(P, c, leg, slot, form, i, row_m[lr], row_s[lr], row_h[lr], writes, &pot);
+            if (writes) {
+                float top = __double2float_ru(pot);
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, off));
+                if (lane == 0 && i < nrows)
+                    (leg == LEG_F ? P.topx[c.parity ^ 1] + (size_t)slot * P.nbx : P.topy + (size_t)slot * P.nby)[i / BOX_COLS] = top;
+            }
+            if (leg != LEG_G && i < nrows) term_sum += residual_fixed(P, leg, slot, term, frozen);
+            continue;
+        }
         if (i >= nrows) continue;
         const double term = finish_one_row<T>(P, c, leg, slot, form, i, row_m[lr], row_s[lr], row_h[lr], writes);
         if (leg != LEG_G) term_sum += residual_fixed(P, leg, slot, term, frozen);

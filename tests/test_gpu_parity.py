@@ -1214,3 +1214,32 @@ def test_kernel_matrix_lanes_at_the_edges_of_their_tiles(oracle, n, m):
         np.testing.assert_array_equal(f.cpu().numpy(), r["f"]); np.testing.assert_array_equal(g.cpu().numpy(), r["g"])
         assert sb.check_guards() == -1
         sb.close()
+
+
+# ---- large low-dimensional lanes in spatial order ----------------------------------------------------
+@pytest.mark.parametrize("n,m,d", [(1024, 1024, 3), (1023, 1025, 3), (1055, 64, 2), (31, 1100, 4), (1024, 33, 1), (8193, 40, 3)])
+def test_lanes_in_spatial_order(oracle, n, m, d):
+    # sizes around the threshold, ragged boxes of 32, chunks of the ordering, every padded dimension; lanes of
+    # several regularisations, from one that keeps every column to one that keeps a few.  The mask control, which
+    # never changes its launch shape, must give the same bits, and a warm proposal must find its way into the order.
+    rng = np.random.default_rng(n + m + d)
+    W = 3
+    x = rng.standard_normal((W, n, d)); y = rng.standard_normal((W, m, d)) * 0.8 + 0.2
+    a = rng.uniform(0.5, 1.5, (W, n)); b = rng.uniform(0.5, 1.5, (W, m))
+    f32 = np.float32
+    w = wl.Workload("spatial", x.astype(f32), y.astype(f32), (a / a.sum(1, keepdims=True)).astype(f32),
+                    (b / b.sum(1, keepdims=True)).astype(f32), np.array([1.0, 0.2, 0.08], f32), 1e-3, 60)
+    r = run_gpu(w, compute="f32")
+    check_against_oracle(oracle, w, r, range(W), pot_tol=POT_TOL_F32, exact_depth=False, floor=MARGIN_AUTO, max_iter=60,
+                         label=f"spatial order, {n} x {m}, d {d}")
+    rm = run_gpu(w, compute="f32", mode="masked")
+    np.testing.assert_array_equal(rm["f"], r["f"]); np.testing.assert_array_equal(rm["r_row"], r["r_row"])
+    part = oracle.solve_batch(w.x, w.y, w.a, w.b, w.eps, w.tol, fixed_cycles=2)
+    rw = run_gpu(w, compute="f32", warm=(part.f, part.g))
+    check_against_oracle(oracle, w, rw, range(W), pot_tol=POT_TOL_F32, exact_depth=False, floor=MARGIN_AUTO, max_iter=60,
+                         warm=(part.f, part.g), label=f"spatial order, warm, {n} x {m}, d {d}")
+    # clouds far apart at a small eps: the first legs move potentials by far more than the estimate allows for
+    far = wl.Workload("spatial_far", w.x, (w.y + f32(6.0)).astype(f32), w.a, w.b, np.array([0.9, 0.7, 0.5], f32), 1e-3, 12)
+    rf = run_gpu(far, compute="f32")
+    ref = oracle.solve_batch(far.x, far.y, far.a, far.b, far.eps, far.tol, max_iter=12)
+    assert pot_err(rf["f"], rf["g"], ref.f, ref.g, far.eps.astype(np.float64)).max() <= POT_TOL_F32
