@@ -13,11 +13,13 @@
 //
 // It is the row screen of the update kernel in its plainest form: for every lane
 //     r_row = sum_i | sum_j exp((f_i + g_j - |x_i - y_j|^2) / eps) - a_i |,
-// float64 arithmetic, one thread per row, per-CTA partial sums combined in a fixed order by
-// the last CTA of the lane to arrive.
+// float64 arithmetic, per-CTA partial sums combined in a fixed order by the last CTA of the lane to
+// arrive; up to 32 dimensions by tiles in shared memory, beyond that one thread per row.
 #include <cuda_runtime.h>
 #include <mutex>
 #include <string>
+
+#include "skb_pairs64.cuh"
 
 #include "../../include/sinkhorn_batch.h"
 
@@ -87,6 +89,104 @@ __global__ void __launch_bounds__(NA_THREADS) row_residual_kernel(
     r_row[lane_id] = (float)tot;
 }
 
+// The same for d <= 32: a block of WPB warps takes 16 * WPB rows, column tiles come through shared memory
+// (skb_pairs64.cuh).  The entries are summed as they are; a row whose sum is not finite is redone the plain way,
+// so infinite potentials give what they always gave.  32 lanes of 1024 x 1000 points, d = 15: 1040 us with one
+// thread per row and the columns read from global memory, 150 us so.
+template <int DM, int WPB>
+__global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
+    Scratch *sc, const float *x, const float *y, const float *a, const double *f, const double *g,
+    const float *eps, int n, int m, int d, float *r_row)
+{
+    using namespace skb;
+    constexpr int R = 2, RW = 16;
+    __shared__ double tile[(DM + 1) * P64_TJ];
+    __shared__ double red[WPB];
+    __shared__ int is_last;
+    const int lane_id = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int cs = lane >> 3, i0 = blockIdx.x * (RW * WPB) + warp * RW + (lane & 7) * R;
+    const double inv_eps = 1.0 / (double)eps[lane_id], k2 = 1.4426950408889634 * inv_eps;
+    const float *xl = x + (size_t)lane_id * n * d, *yl = y + (size_t)lane_id * m * d;
+    const double *fl = f + (size_t)lane_id * n, *gl = g + (size_t)lane_id * m;
+    double xr[R][DM], ri[R], s[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = i0 + r < n ? i0 + r : n - 1;
+        double q = 0.0;
+#pragma unroll
+        for (int k = 0; k < DM; ++k) { xr[r][k] = k < d ? (double)xl[(size_t)i * d + k] : 0.0; q = fma(xr[r][k], xr[r][k], q); }
+        ri[r] = k2 * (fl[i] - q);
+        s[r] = 0.0;
+    }
+    for (int j0 = 0; j0 < m; j0 += P64_TJ) {
+        __syncthreads();
+        p64_tile<DM, 32 * WPB>(tile, j0, m, d, k2, [&](int j, int k) { return yl[(size_t)j * d + k]; }, [&](int j) { return gl[j]; });
+        __syncthreads();
+#pragma unroll 2
+        for (int jj = cs; jj < P64_TJ; jj += 4) {
+            double v[R];
+            const double c = tile[DM * P64_TJ + jj];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = c + ri[r];
+#pragma unroll
+            for (int k = 0; k < DM; ++k) {
+                const double yk = tile[k * P64_TJ + jj];
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[r] = fma(xr[r][k], yk, v[r]);
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) s[r] += exp2(v[r]);
+        }
+    }
+    double term = 0.0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        s[r] += __shfl_xor_sync(0xffffffffu, s[r], 8);
+        s[r] += __shfl_xor_sync(0xffffffffu, s[r], 16);
+        if (cs == 0 && i0 + r < n) {
+            if (!isfinite(s[r])) {
+                // the plain sum, with its running maximum
+                double mx = -1.0e300, t = 0.0;
+                for (int j = 0; j < m; ++j) {
+                    double c = 0.0;
+                    for (int k = 0; k < d; ++k) { const double e = (double)xl[(size_t)(i0 + r) * d + k] - (double)yl[(size_t)j * d + k]; c += e * e; }
+                    const double v = (fl[i0 + r] + gl[j] - c) * inv_eps;
+                    if (v > mx) { t *= exp(mx - v); mx = v; }
+                    t += exp(v - mx);
+                }
+                s[r] = exp(mx) * t;
+            }
+            term += fabs(s[r] - (double)a[(size_t)lane_id * n + i0 + r]);
+        }
+    }
+    for (int off = 4; off > 0; off >>= 1) term += __shfl_down_sync(0xffffffffu, term, off);
+    if (lane == 0) red[warp] = term;
+    __syncthreads();
+    if (tid == 0) {
+        double p = 0.0;
+        for (int w = 0; w < WPB; ++w) p += red[w];
+        sc->partial[lane_id][blockIdx.x] = p;
+        __threadfence();
+        is_last = (atomicAdd(&sc->arrived[lane_id], 1u) == gridDim.x - 1);
+    }
+    __syncthreads();
+    if (!is_last || tid != 0) return;
+    __threadfence();
+    double tot = 0.0;
+    for (unsigned b = 0; b < gridDim.x; ++b) tot += reinterpret_cast<volatile double *>(sc->partial[lane_id])[b];
+    sc->arrived[lane_id] = 0u;
+    r_row[lane_id] = (float)tot;
+}
+
+// 64 rows to a block while the scratch has a slot for every block (n <= 4096), 128 beyond
+template <int DM>
+void launch_tiled(Scratch *sc, const float *x, const float *y, const float *a, const double *f, const double *g, const float *eps,
+                  int W, int n, int m, int d, float *r_row, cudaStream_t st)
+{
+    if (n <= 64 * NA_MAX_BLOCKS) row_residual_tiled_kernel<DM, 4><<<dim3((n + 63) / 64, W), 128, 0, st>>>(sc, x, y, a, f, g, eps, n, m, d, r_row);
+    else row_residual_tiled_kernel<DM, 8><<<dim3((n + 127) / 128, W), 256, 0, st>>>(sc, x, y, a, f, g, eps, n, m, d, r_row);
+}
+
 skb_status fail(skb_status st, const std::string &msg)
 {
     g_err = msg;
@@ -123,8 +223,14 @@ extern "C" skb_status sinkhorn_row_residual_static(const float *x, const float *
     // the array keeps whatever the previous call left: the arrival counters must start at zero
     e = cudaMemsetAsync(sc->arrived, 0, sizeof(sc->arrived), st);
     if (e != cudaSuccess) return fail(SKB_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
-    dim3 grid((n + NA_THREADS - 1) / NA_THREADS, W);
-    row_residual_kernel<<<grid, NA_THREADS, 0, st>>>(sc, x, y, a, f, g, eps, n, m, d, r_row);
+    if (d <= 4) launch_tiled<4>(sc, x, y, a, f, g, eps, W, n, m, d, r_row, st);
+    else if (d <= 8) launch_tiled<8>(sc, x, y, a, f, g, eps, W, n, m, d, r_row, st);
+    else if (d <= 16) launch_tiled<16>(sc, x, y, a, f, g, eps, W, n, m, d, r_row, st);
+    else if (d <= skb::P64_MAX_D) launch_tiled<skb::P64_MAX_D>(sc, x, y, a, f, g, eps, W, n, m, d, r_row, st);
+    else {
+        dim3 grid((n + NA_THREADS - 1) / NA_THREADS, W);
+        row_residual_kernel<<<grid, NA_THREADS, 0, st>>>(sc, x, y, a, f, g, eps, n, m, d, r_row);
+    }
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(SKB_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
     g_err.clear();

@@ -1243,3 +1243,38 @@ def test_lanes_in_spatial_order(oracle, n, m, d):
     rf = run_gpu(far, compute="f32")
     ref = oracle.solve_batch(far.x, far.y, far.a, far.b, far.eps, far.tol, max_iter=12)
     assert pot_err(rf["f"], rf["g"], ref.f, ref.g, far.eps.astype(np.float64)).max() <= POT_TOL_F32
+
+
+# ---- float64 pair sums by column tiles ---------------------------------------------------------------
+@pytest.mark.parametrize("n,m,d,dv", [(1, 1, 1, 1), (63, 65, 4, 4), (64, 64, 5, 5), (65, 128, 16, 16), (130, 63, 17, 3), (40, 70, 32, 16),
+                                      (33, 50, 33, 2), (4097, 20, 3, 3)])
+def test_pair_sums_in_float64_at_the_edges_of_their_tiles(oracle, n, m, d, dv):
+    # plan application and the row residual of given potentials: tile edges, the last tiled dimension and the first
+    # beyond, both value widths, both block sizes of the residual.  Both are float64 sums rounded once to fp32:
+    # 2^-24 relative, plus the potentials' own rounding (1e-16 of C / eps = 1e3 in an exponent) far below it
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("sweep", W=2, n=n, m=m, d=d, max_iter=7)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    args = [t(v) for v in (w.x, w.y, w.a, w.b, w.eps)]
+    sb = B.SinkhornBatch(*args, w.tol, compute="f64", max_iter=7)
+    sb.drain()
+    f, g = sb.potentials(f64=True)
+    v = torch.randn(2, m, dv, device="cuda:0", generator=torch.Generator("cuda:0").manual_seed(n + m))
+    out = sb.apply_plan(v).cpu().numpy()
+    sb.close()
+    fr, gr = f.cpu().numpy(), g.cpu().numpy()
+    # the residual of potentials that are not a solution's, so that it is far from its rounding
+    f2 = f + 0.3 * args[4][:, None].double() * torch.sin(1.0 + torch.arange(n, device="cuda:0", dtype=torch.float64))
+    rr = B.sinkhorn_row_residual_static(args[0], args[1], args[2], f2, g, args[4]).cpu().numpy()
+    f2[0, n // 2] = float("inf")                       # an infinite potential: its lane's residual is not finite, the other's is
+    bad = B.sinkhorn_row_residual_static(args[0], args[1], args[2], f2, g, args[4]).cpu().numpy()
+    assert not np.isfinite(bad[0]) and bad[1] == rr[1]
+    f2[0, n // 2] = 0.0
+    for k in range(2):
+        want = oracle.apply_plan(w.x[k], w.y[k], float(w.eps[k]), fr[k], gr[k], v[k].cpu().numpy())
+        scale = np.abs(want).max()
+        np.testing.assert_allclose(out[k], want, rtol=2.0 ** -23, atol=1e-9 * scale)
+        fk = fr[k] + 0.3 * float(w.eps[k]) * np.sin(1.0 + np.arange(n))
+        res, _ = oracle.residuals(w.x[k], w.y[k], w.a[k], w.b[k], float(w.eps[k]), fk, gr[k])
+        assert abs(rr[k] - res) <= 2.0 ** -23 * res + 1e-12
