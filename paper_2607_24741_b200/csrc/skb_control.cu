@@ -25,24 +25,59 @@ namespace skb {
 // from it, and from that the cost form the lane will use.
 // Lanes come in as a block of problems: input problem q goes to slot slot0 + q as lane lane0 + q
 // (create: slot0 = lane0 = 0, all W; a refill: the first free slot, the next unused lane number).
+
+// Per-slot state of a lane that comes in; r2: largest squared distance of a point from the centre.  One thread.
+__device__ __forceinline__ void lane_enters(const Dev &P, const float *eps, const int q, const int slot, const int lane0, const int cycle0,
+                                            const double r2)
+{
+    const double e = (double)eps[q];
+    const bool eps_ok = (e > 0.0) && isfinite(e);
+    const double s = eps_ok ? 1.4426950408889634 / e : 1.0;
+    if (!eps_ok) atomicOr(&P.ctl->error, ERR_VALUE);
+    P.scale[slot] = s;
+    P.lane_id[slot] = lane0 + q;
+    P.start[slot] = cycle0;
+    // whatever an earlier lane left in the slot
+    P.nonfinite[slot] = 0; P.state[slot] = 0; P.flag[slot] = 0; P.verdict[slot] = 0;
+    P.rsum_row[slot] = 0ull; P.rsum_col[slot] = 0ull; P.rsum_row64[slot] = 0ull; P.esc[slot] = 0;
+    P.ret_at[slot] = 0; P.n_checks[slot] = 0;
+    P.absorbed[slot] = 0; P.cyc_log[slot] = 0;
+    P.radius[slot] = sqrt(r2);
+    // (lanes in spatial order have a form of their own, which shares the expanded form's scale and terms)
+    int form = P.permx ? FORM_DOT : P.cost_form == 1 ? FORM_DOT : (P.cost_form == 2 ? FORM_DIFF : (s * r2 > P.form_threshold ? FORM_DIFF : FORM_DOT));
+    P.form[slot] = form;
+    atomicMax(&P.ctl->max_radius_bits, (unsigned long long)__double_as_longlong(eps_ok ? s * r2 : 0.0));
+}
+
+// d <= 32.  Eight dimensions at a time: every thread sums its points in all of them, then one warp per dimension
+// adds the 256 partial sums up, in the order of a binary tree over the threads.  (One dimension after the other,
+// each with a tree of eight barriers, was a chain of some 15 us on the lanes of the sensor workload, d = 15.)
 __global__ void __launch_bounds__(256) lane_stats_kernel(const Dev P, const void *xin, const void *yin, const float *eps,
                                                          const int slot0, const int lane0, const int cycle0)
 {
-    __shared__ double red[256];
-    __shared__ double cen[1024];
-    const int q = blockIdx.x, slot = slot0 + q, tid = threadIdx.x;
+    __shared__ double part[8][256];
+    __shared__ double cen[32];
+    const int q = blockIdx.x, slot = slot0 + q, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tot = P.n + P.m;
-    for (int k = 0; k < P.d; ++k) {
-        double s = 0.0;
+    for (int k0 = 0; k0 < P.d; k0 += 8) {
+        double s[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[k] = 0.0;
         for (int p = tid; p < tot; p += 256) {
             const bool isx = p < P.n;
-            const size_t idx = isx ? ((size_t)q * P.n + p) * P.d + k : ((size_t)q * P.m + (p - P.n)) * P.d + k;
-            s += (double)load_raw(P, isx ? xin : yin, idx);
+            const size_t idx = (isx ? ((size_t)q * P.n + p) : ((size_t)q * P.m + (p - P.n))) * P.d + k0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) if (k0 + k < P.d) s[k] += (double)load_raw(P, isx ? xin : yin, idx + k);
         }
-        red[tid] = s;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) part[k][tid] = s[k];
         __syncthreads();
-        for (int off = 128; off > 0; off >>= 1) { if (tid < off) red[tid] += red[tid + off]; __syncthreads(); }
-        if (tid == 0) cen[k] = red[0] / (double)tot;
+        // pairs 128, 64, 32 apart, then 16 .. 1
+        const double *r = part[warp];
+        double v = ((r[lane] + r[lane + 128]) + (r[lane + 64] + r[lane + 192])) + ((r[lane + 32] + r[lane + 160]) + (r[lane + 96] + r[lane + 224]));
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+        if (lane == 0 && k0 + warp < P.d) cen[k0 + warp] = v / (double)tot;
         __syncthreads();
     }
     double mxr = 0.0;
@@ -53,28 +88,63 @@ __global__ void __launch_bounds__(256) lane_stats_kernel(const Dev P, const void
         for (int k = 0; k < P.d; ++k) { const double v = (double)load_raw(P, isx ? xin : yin, base + k) - cen[k]; r2 += v * v; }
         mxr = fmax(mxr, r2);
     }
-    red[tid] = mxr;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) mxr = fmax(mxr, __shfl_xor_sync(0xffffffffu, mxr, off));
+    if (lane == 0) part[0][warp] = mxr;
     __syncthreads();
-    for (int off = 128; off > 0; off >>= 1) { if (tid < off) red[tid] = fmax(red[tid], red[tid + off]); __syncthreads(); }
     for (int k = tid; k < P.DP; k += 256) P.center[(size_t)slot * P.DP + k] = k < P.d ? cen[k] : 0.0;
     if (tid == 0) {
-        const double e = (double)eps[q];
-        const bool eps_ok = (e > 0.0) && isfinite(e);
-        const double s = eps_ok ? 1.4426950408889634 / e : 1.0;
-        if (!eps_ok) atomicOr(&P.ctl->error, ERR_VALUE);
-        P.scale[slot] = s;
-        P.lane_id[slot] = lane0 + q;
-        P.start[slot] = cycle0;
-        // whatever an earlier lane left in the slot
-        P.nonfinite[slot] = 0; P.state[slot] = 0; P.flag[slot] = 0; P.verdict[slot] = 0;
-        P.rsum_row[slot] = 0ull; P.rsum_col[slot] = 0ull; P.rsum_row64[slot] = 0ull; P.esc[slot] = 0;
-        P.ret_at[slot] = 0; P.n_checks[slot] = 0;
-        P.absorbed[slot] = 0; P.cyc_log[slot] = 0;
-        P.radius[slot] = sqrt(red[0]);
-        // (lanes in spatial order have a form of their own, which shares the expanded form's scale and terms)
-        int form = P.permx ? FORM_DOT : P.cost_form == 1 ? FORM_DOT : (P.cost_form == 2 ? FORM_DIFF : (s * red[0] > P.form_threshold ? FORM_DIFF : FORM_DOT));
-        P.form[slot] = form;
-        atomicMax(&P.ctl->max_radius_bits, (unsigned long long)__double_as_longlong(eps_ok ? s * red[0] : 0.0));
+        for (int w = 1; w < 8; ++w) mxr = fmax(mxr, part[0][w]);
+        lane_enters(P, eps, q, slot, lane0, cycle0, mxr);
+    }
+}
+
+// Deep lanes (32 < d <= 1024): a warp takes 32 dimensions of a share of the points, so rows are read in whole
+// sectors; then a warp per point for the distances.  (One dimension after the other read two bytes of every row
+// per pass: create took 1865 us on the 64 lanes of the feature workload, d = 512, and takes 858 us with this and prep_tensor_kernel.)
+__global__ void __launch_bounds__(1024) lane_stats_deep_kernel(const Dev P, const void *xin, const void *yin, const float *eps,
+                                                               const int slot0, const int lane0, const int cycle0)
+{
+    __shared__ double part[1024];                         // [share][dimension], then the warps' maxima
+    __shared__ double cen[1024];
+    const int q = blockIdx.x, slot = slot0 + q, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tot = P.n + P.m, groups = (P.d + 31) / 32, shares = 32 / groups;
+    if (warp < groups * shares) {
+        const int k = (warp % groups) * 32 + lane, first = warp / groups;
+        const int kc = k < P.d ? k : P.d - 1;
+        double s = 0.0;
+#pragma unroll 8
+        for (int p = first; p < tot; p += shares) {
+            const bool isx = p < P.n;
+            s += (double)load_raw(P, isx ? xin : yin, (isx ? (size_t)q * P.n + p : (size_t)q * P.m + (p - P.n)) * P.d + kc);
+        }
+        part[first * groups * 32 + k] = s;
+    }
+    __syncthreads();
+    if (tid < P.d) {
+        double s = 0.0;
+        for (int h = 0; h < shares; ++h) s += part[h * groups * 32 + tid];
+        cen[tid] = s / (double)tot;
+    }
+    __syncthreads();
+    double mxr = 0.0;
+#pragma unroll 2
+    for (int p = warp; p < tot; p += 32) {
+        const bool isx = p < P.n;
+        const size_t base = (isx ? (size_t)q * P.n + p : (size_t)q * P.m + (p - P.n)) * P.d;
+        double r2 = 0.0;
+#pragma unroll 4
+        for (int k = lane; k < P.d; k += 32) { const double v = (double)load_raw(P, isx ? xin : yin, base + k) - cen[k]; r2 = fma(v, v, r2); }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, off);
+        mxr = fmax(mxr, r2);
+    }
+    if (lane == 0) part[warp] = mxr;
+    __syncthreads();
+    for (int k = tid; k < P.DP; k += 1024) P.center[(size_t)slot * P.DP + k] = k < P.d ? cen[k] : 0.0;
+    if (tid == 0) {
+        for (int w = 0; w < 32; ++w) mxr = fmax(mxr, part[w]);
+        lane_enters(P, eps, q, slot, lane0, cycle0, mxr);
     }
 }
 
@@ -95,12 +165,11 @@ __global__ void prep_kernel(const Dev P, const void *xin, const void *yin, const
     double *sq = side ? P.sqy : P.sqx, *lw = side ? P.lb2 : P.la2, *wt = side ? P.wb : P.wa;
     T hi, lo = T(0);
     if (i >= npts) {                                  // padding points
-        if (!P.tensor) for (int k = 0; k < P.DP; ++k) crd[(size_t)k * pp + i] = T(0);
+        for (int k = 0; k < P.DP; ++k) crd[(size_t)k * pp + i] = T(0);
         hi = T(NEG_BIG);
         sq[o] = 0.0; lw[o] = 0.0; wt[o] = 0.0;
     } else {
-        // tensor-core path: raw coordinates feed the MMA, the scale 2s is applied to its result
-        const double sc = P.tensor ? sqrt(2.0 * s) : sqrt(form == FORM_DOT ? 2.0 * s : s);
+        const double sc = sqrt(form == FORM_DOT ? 2.0 * s : s);
         const size_t ibase = ((size_t)q * npts + i) * P.d;
         const double *cen = P.center + (size_t)slot * P.DP;
         double nrm = 0.0;
@@ -110,10 +179,9 @@ __global__ void prep_kernel(const Dev P, const void *xin, const void *yin, const
             if (k < P.d) {
                 const float raw = load_raw(P, side ? yin : xin, ibase + k);
                 ok = ok && isfinite(raw);
-                v = P.tensor ? (T)0 : (T)(sc * ((double)raw - cen[k]));
-                if (P.tensor) nrm += (sc * (double)raw) * (sc * (double)raw);
+                v = (T)(sc * ((double)raw - cen[k]));
             }
-            if (!P.tensor) crd[(size_t)k * pp + i] = v;
+            crd[(size_t)k * pp + i] = v;
             nrm += (double)v * (double)v;
         }
         nrm = form == FORM_DOT ? 0.5 * nrm : 0.0;
@@ -131,6 +199,49 @@ __global__ void prep_kernel(const Dev P, const void *xin, const void *yin, const
         P.phi[0][o] = 0.0; P.phi[1][o] = 0.0;
     } else {
         P.gam[o] = 0.0;
+    }
+}
+
+// Layout of tensor-core lanes: their coordinates stay raw (the tiled bf16 copies), so a point leaves only its
+// scaled squared norm, weight and cold potentials here.  One warp per point reads its row in whole sectors.
+__global__ void __launch_bounds__(256) prep_tensor_kernel(const Dev P, const void *xin, const void *yin, const float *a, const float *b, const int slot0)
+{
+    const int q = blockIdx.y, slot = slot0 + q, side = blockIdx.z, lane = threadIdx.x & 31;
+    const int npts = side ? P.m : P.n, pp = side ? P.mp : P.np;
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= pp) return;
+    const size_t o = (size_t)slot * pp + i;
+    float hi = NEG_BIG;                                    // padding points
+    double nrm = 0.0, lw = 0.0, wt = 0.0;
+    if (i < npts) {
+        const size_t ibase = ((size_t)q * npts + i) * P.d;
+        const double sc = sqrt(2.0 * P.scale[slot]);
+        bool ok = true;
+#pragma unroll 4
+        for (int k = lane; k < P.d; k += 32) {
+            const float raw = load_raw(P, side ? yin : xin, ibase + k);
+            ok = ok && isfinite(raw);
+            const double v = sc * (double)raw;
+            nrm = fma(v, v, nrm);
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
+        nrm *= 0.5;
+        const float w = (side ? b : a)[(size_t)q * npts + i];
+        ok = __all_sync(0xffffffffu, ok) && (w > 0.0f) && isfinite(w);
+        if (!ok && lane == 0) atomicOr(&P.ctl->error, ERR_VALUE);
+        lw = ok ? log2((double)w) : 0.0;
+        wt = ok ? (double)w : 0.0;
+        hi = (float)(-nrm);                                // cold start: phi = gam = 0
+    }
+    if (lane != 0) return;
+    (side ? P.sqy : P.sqx)[o] = nrm; (side ? P.lb2 : P.la2)[o] = lw; (side ? P.wb : P.wa)[o] = wt;
+    if (side) {
+        reinterpret_cast<float *>(P.gt)[o] = hi; reinterpret_cast<float *>(P.gl)[o] = 0.f; P.gam[o] = 0.0;
+    } else {
+        for (int e = 0; e < 2; ++e) {
+            reinterpret_cast<float *>(P.ft[e])[o] = hi; reinterpret_cast<float *>(P.fl[e])[o] = 0.f; P.phi[e][o] = 0.0;
+        }
     }
 }
 
@@ -742,13 +853,15 @@ void launch_apply_plan(const Dev &P, const void *x, const void *y, const float *
 void launch_lane_stats(const Dev &P, const void *x, const void *y, const float *eps, int slot0, int lane0, int count,
                        int cycle0, cudaStream_t st)
 {
-    lane_stats_kernel<<<count, 256, 0, st>>>(P, x, y, eps, slot0, lane0, cycle0);
+    if (P.d <= 32) lane_stats_kernel<<<count, 256, 0, st>>>(P, x, y, eps, slot0, lane0, cycle0);
+    else lane_stats_deep_kernel<<<count, 1024, 0, st>>>(P, x, y, eps, slot0, lane0, cycle0);
 }
 void launch_prep(const Dev &P, const void *x, const void *y, const float *a, const float *b, int slot0, int count, cudaStream_t st)
 {
     const int pp = P.np > P.mp ? P.np : P.mp;
     dim3 grid((pp + 127) / 128, count, 2);
     if (P.permx) launch_prep_near(P, x, y, a, b, slot0, count, st);
+    else if (P.tensor) prep_tensor_kernel<<<dim3((pp + 7) / 8, count, 2), 256, 0, st>>>(P, x, y, a, b, slot0);
     else if (P.compute_f64) prep_kernel<double><<<grid, 128, 0, st>>>(P, x, y, a, b, slot0);
     else prep_kernel<float><<<grid, 128, 0, st>>>(P, x, y, a, b, slot0);
 }
