@@ -191,6 +191,7 @@ __global__ void prep_kernel(const Dev P, const void *xin, const void *yin, const
         sq[o] = nrm;
         lw[o] = ok ? log2((double)w) : 0.0;
         wt[o] = ok ? (double)w : 0.0;
+        if (P.phi0 && ok && w < SC_MIN_WEIGHT) P.absorbed[slot] = SC_NO_MATRIX;      // (every writer stores the same value)
         hi = (T)(-nrm);                                // cold start: phi = gam = 0
     }
     hi0[o] = hi; lo0[o] = lo;

@@ -26,6 +26,8 @@ enum Form : int { FORM_DOT = 0, FORM_DIFF = 1 };
 
 constexpr float NEG_BIG = -1.0e30f;   // "minus infinity" for padded columns (finite: no NaNs)
 constexpr int UPD_THREADS = 128;
+constexpr int SC_NO_MATRIX = -1;      // scaling_kernel: a weight below SC_MIN_WEIGHT, the lane stays in the log domain
+constexpr float SC_MIN_WEIGHT = 0x1p-80f;
 constexpr int BOX_COLS = 32;          // points per bounding box of lanes in spatial order
 constexpr int TC_MAX_SPLIT = 8;      // a row block's columns go to at most this many clusters
 constexpr int MAX_CLUSTER_RANKS = 8;  // blocks per cluster (portable limit): row blocks of a lane in the multi-cycle kernels
@@ -91,7 +93,7 @@ struct Dev {
     int *verdict;             // two-sided check passed
     int *nonfinite;
     double *radius;           // largest distance of a point from the centre, in the inputs' units
-    int *absorbed, *cyc_log;  // scaling_kernel: phi0 .. vv are valid; the last f-leg ran in the log domain
+    int *absorbed, *cyc_log;  // scaling_kernel: phi0 .. vv are valid (or SC_NO_MATRIX); the last f-leg ran in the log domain
     // multi-cycle launches: cycle count + 1 at which the lane in the slot left inside the launch
     // (0 = still running), and the column checks it ran
     int *ret_at, *n_checks;

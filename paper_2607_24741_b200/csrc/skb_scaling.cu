@@ -1,19 +1,24 @@
 // Small lanes in mixed arithmetic: the lane's kernel matrix is formed once and kept in registers.
 //
 // With potentials (phi0, gam0) absorbed into the matrix,
-//     K_ij = 2^(phi0_i + gam0_j - s C_ij) / a_i,      phi = phi0 + log2 u,   gam = gam0 + log2 v,
+//     K_ij = 2^(phi0_i + gam0_j - s C_ij) / (a_i b_j),      phi = phi0 + log2 u,   gam = gam0 + log2 v,
 // the two legs of Eq. 3 are the scaling updates
-//     u_i = 1 / sum_j K_ij v_j,        v_j = b_j / sum_i K_ij a_i u_i,
+//     u_i = 1 / sum_j K_ij b_j v_j,        v_j = 1 / sum_i K_ij a_i u_i,
 // one fp32 multiply-add per pair and leg instead of a d-term float64 distance and an exponential.
 // Exponents are float64 (rounded once, after the integer part has been split off), K is fp32, sums are
 // fp32 over at most 32 terms and float64 beyond, u, v and the potentials are float64: what the
 // log-domain kernels of the mixed arithmetic hold in 32 and in 64 bits is held so here.
 //
-// Range.  fp32 K has no entries below 2^-124.  An update that would take a u or v out of 2^+-60 is not
+// Range.  fp32 K has no entries below 2^-124.  An update that would take a u or v out of 2^+-45 is not
 // taken: the leg is done again in the log domain (log_rows / log_cols: per-row or per-column maximum,
 // then the sum, both passes over the distances), after which the new potentials are absorbed and K is
-// formed anew.  A lane whose u or v has left 2^+-30 after a cycle is absorbed too, so an entry that K
-// does not hold is below 2^(-124 + 30 + 60) = 2^-34 of its row or column sum.  The first cycle of a cold or
+// formed anew.  A lane whose u or v has left 2^+-30 after a cycle is absorbed too.  So what K does not hold is
+// below 2^-124 sum_j b_j v_j <= 2^(-124 + 30) of a row sum 1 / u_i >= 2^-45, and below 2^-124 sum_i a_i u_i <=
+// 2^(-124 + 45) of a column sum 1 / v_j >= 2^-45: at most 2^-34 of the sum, whatever the weights (K divided by both
+// of them: with a_i alone the column bound would carry a factor a_i / b_j).  The operands a u and b v stay normal
+// fp32 numbers, and K = P / (a_i b_j) <= 1 / a_i within its range, while no weight is below 2^-80: a lane with a
+// smaller one (SC_NO_MATRIX, found when its layout is written) stays in the log domain for all of its cycles.
+// The first cycle of a cold or
 // warm start is a log-domain cycle.  All of these decisions are taken per lane from the lane's own values, and K is a function of
 // (phi0, gam0) alone, which are part of the lane's state: a lane's bits depend neither on how its cycles
 // were shared out among launches nor on the mode.
@@ -41,7 +46,7 @@
 namespace skb {
 
 enum ScalingWhat : int { SC_CYCLES = 3 };               // besides LEG_F, LEG_G, LEG_V: whole cycles
-constexpr int SC_TAKE = 60, SC_KEEP = 30;               // bands of log2 u and log2 v: update taken / K kept
+constexpr int SC_TAKE = 45, SC_KEEP = 30;               // bands of log2 u and log2 v: update taken / K kept
 constexpr int SC_BAD = 1, SC_DRIFT = 2, SC_NF = 4;
 
 // 2^arg for a float64 argument: integer part split off in float64, the remainder (|.| <= 1/2) rounded
@@ -319,7 +324,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
     __shared__ __align__(16) double partd[NW * COLS];    // column parts of every warp
     float *partf = reinterpret_cast<float *>(partd);
     __shared__ __align__(16) double colB[COLS], rowA[RB];       // additive terms of columns / own rows
-    __shared__ __align__(16) float vs[COLS];             // v of all columns
+    __shared__ __align__(16) float vs[COLS];             // b v of all columns
     __shared__ __align__(16) float2 uas[RB];             // a u of own rows, in both halves
     __shared__ __align__(8) unsigned long long xbar[2];  // arrival of an exchange's stores, one per buffer
 
@@ -353,7 +358,8 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
     bool frozen = P.mode == MODE_MASKED && P.state[slot] != 0;
 
     // state: `us`, `vsd` are u and v while `ab` (potentials absorbed into K), the potentials themselves before
-    bool ab = P.absorbed[slot] != 0;
+    bool ab = P.absorbed[slot] > 0;
+    const bool no_matrix = P.absorbed[slot] < 0;
     // (the absorbed potentials stay in registers: every block holds all columns', and global memory gets them
     // back only at the end, when no block of the cluster can still be reading)
     double us = ab ? 1.0 : 0.0, phi0 = 0.0, vsd[NQ], gam0[NQ], bq[NQ];
@@ -531,8 +537,8 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
             for (int q = 0; q < NQ; ++q) {
                 const int j = j0 + q;
                 if (cown) {
-                    colB[j] = j < P.m ? gam0[q] - P.sqy[co + j] : -1.0e30;
-                    vs[j] = (float)vsd[q];
+                    colB[j] = j < P.m ? gam0[q] - P.lb2[co + j] - P.sqy[co + j] : -1.0e30;
+                    vs[j] = (float)(bq[q] * vsd[q]);
                 }
             }
             __syncthreads();
@@ -633,10 +639,10 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
                     vn[q] = 0.0;
                     if (cown) {
                         if (j < P.m) {
-                            vn[q] = bq[q] * rcp64(T[q]);
+                            vn[q] = rcp64(T[q]);
                             flags |= out_of_band<SC_KEEP>(vn[q]);
                         }
-                        if (!frozen) vs[j] = (float)vn[q];
+                        if (!frozen) vs[j] = (float)(bq[q] * vn[q]);
                     }
                 }
                 if (__syncthreads_or(flags)) break;
@@ -742,7 +748,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) {
                     const int j = j0 + q;
-                    term[q] = (cown && j < P.m) ? fabs(vsd[q] * recv_col(j, false) - bq[q]) : 0.0;
+                    term[q] = (cown && j < P.m) ? bq[q] * fabs(fma(vsd[q], recv_col(j, false), -1.0)) : 0.0;
                 }
                 ++xch;
             } else {
@@ -838,10 +844,10 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
                 vnew[q] = 0.0;
                 if (cown) {
                     if (j < P.m) {
-                        vnew[q] = bq[q] * rcp64(T[q]);
+                        vnew[q] = rcp64(T[q]);
                         flags |= (out_of_band<SC_TAKE>(vnew[q]) ? SC_BAD : 0) | (out_of_band<SC_KEEP>(vnew[q]) ? SC_DRIFT : 0);
                     }
-                    if (!frozen) vs[j] = (float)vnew[q];
+                    if (!frozen) vs[j] = (float)(bq[q] * vnew[q]);
                 }
             }
             if (flags) atomicOr(&sflag, flags);
@@ -862,7 +868,11 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
             if (__syncthreads_or(bad ? 1 : 0) && !frozen) nf = 1;
         }
         if (!frozen) {
-            if (need_build) {
+            if (need_build && no_matrix) {
+                us = phinew;                             // (every leg of such a lane has run in the log domain)
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) vsd[q] = vnew[q];
+            } else if (need_build) {
                 // absorb the new potentials: K is formed anew from them
                 if (!log_g) {
                     phinew = rok ? phi0 + log2(unew) : 0.0;
@@ -885,7 +895,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
         if (what == LEG_G) {
             if (!P.dry_run && !frozen) {
                 if (nf && b == 0 && tid == 0) P.nonfinite[slot] = 1;
-                if (need_build && rown) { P.uu[par][ro] = 1.0; P.phi0[ro] = phi0; }
+                if (need_build && ab && rown) { P.uu[par][ro] = 1.0; P.phi0[ro] = phi0; }
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) {
                     const int j = j0 + q;
@@ -895,7 +905,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
                         P.gam[co + j] = col_gam(q);
                     }
                 }
-                if (b == 0 && tid == 0) P.absorbed[slot] = 1;
+                if (b == 0 && tid == 0 && ab) P.absorbed[slot] = 1;
             }
             break;
         }
@@ -922,7 +932,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
                     const int j = j0 + q;
                     if (cown && j < P.m) { P.gam[co + j] = col_gam(q); P.vv[co + j] = vsd[q]; P.gam0[co + j] = gam0[q]; }
                 }
-                if (tid == 0) { P.absorbed[slot] = ab ? 1 : 0; if (nf) P.nonfinite[slot] = 1; }
+                if (tid == 0) { P.absorbed[slot] = ab ? 1 : (no_matrix ? SC_NO_MATRIX : 0); if (nf) P.nonfinite[slot] = 1; }
             }
         }
     }

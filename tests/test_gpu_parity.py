@@ -1216,6 +1216,47 @@ def test_kernel_matrix_lanes_at_the_edges_of_their_tiles(oracle, n, m):
         sb.close()
 
 
+@pytest.mark.parametrize("least", [2.0 ** -70, 2.0 ** -100, 2.0 ** -118])
+@pytest.mark.parametrize("n,m", [(60, 64), (150, 100), (300, 200)])
+def test_kernel_matrix_lanes_with_tiny_weights(oracle, n, m, least):
+    # weights that span 30 orders of magnitude: plan entries of a light column are far below those of the others, and
+    # a column whose entries fell out of the kernel matrix would come out wrong by O(eps)
+    rng = np.random.default_rng(n)
+    f32 = np.float32
+    W, d = 3, 3
+    a = rng.uniform(0.5, 1.5, (W, n)); b = rng.uniform(0.5, 1.5, (W, m))
+    b[:, 5:9] *= least; a[1, 3] *= least; a[2, 7:20] *= 1e-20
+    w = wl.Workload("light", rng.standard_normal((W, n, d)).astype(f32), (rng.standard_normal((W, m, d)) + 0.3).astype(f32),
+                    (a / a.sum(1, keepdims=True)).astype(f32), (b / b.sum(1, keepdims=True)).astype(f32),
+                    np.array([0.05, 0.3, 0.1], f32), 1e-4, 400)
+    for mode in ("active", "masked"):
+        r = run_gpu(w, compute="mixed", mode=mode)
+        check_against_oracle(oracle, w, r, range(W), pot_tol=POT_TOL_F32, exact_depth=False, floor=MARGIN_AUTO, max_iter=400,
+                             label=f"weights down to {least:.0e}, {n} x {m}, {mode}")
+    rl = run_gpu(w, compute="mixed", mode="static", max_iter=6)                  # one launch per leg
+    ref = oracle.solve_batch(w.x, w.y, w.a, w.b, w.eps, w.tol, max_iter=6)
+    # in units of eps: 2^-22 per exponential, a few cycles
+    err = np.abs(rl["g"] - ref.g).max(1) / w.eps
+    assert err.max() <= 1e-5, err
+
+
+@pytest.mark.parametrize("cycles", [2, 3, 5, 9, 30])
+def test_kernel_matrix_lanes_whose_potentials_move_fast(oracle, cycles):
+    # small regularisations, clouds apart: a cycle moves potentials by tens to hundreds of bits, so updates leave the
+    # bands of the scalings in every way.  In units of eps the error is 2^-22 per exponential and cycle remembered
+    rng = np.random.default_rng(5)
+    f32 = np.float32
+    W, n, m, d = 10, 100, 77, 4
+    x = rng.standard_normal((W, n, d)).astype(f32); y = (rng.standard_normal((W, m, d)) * 0.7 + 0.5).astype(f32)
+    a = rng.uniform(0.2, 1.8, (W, n)); b = rng.uniform(0.2, 1.8, (W, m))
+    w = wl.Workload("fast", x, y, (a / a.sum(1, keepdims=True)).astype(f32), (b / b.sum(1, keepdims=True)).astype(f32),
+                    np.geomspace(1e-3, 0.2, W).astype(f32), 1e-6, cycles)
+    r = run_gpu(w, compute="mixed")
+    ref = oracle.solve_batch(w.x, w.y, w.a, w.b, w.eps, w.tol, max_iter=cycles)
+    err = np.maximum(np.abs(r["f"] - ref.f).max(1), np.abs(r["g"] - ref.g).max(1)) / w.eps
+    assert err.max() <= 1e-6 * cycles + 2e-6, err
+
+
 # ---- large low-dimensional lanes in spatial order ----------------------------------------------------
 @pytest.mark.parametrize("n,m,d", [(1024, 1024, 3), (1023, 1025, 3), (1055, 64, 2), (31, 1100, 4), (1024, 33, 1), (8193, 40, 3)])
 def test_lanes_in_spatial_order(oracle, n, m, d):
