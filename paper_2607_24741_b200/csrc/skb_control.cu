@@ -768,39 +768,84 @@ __global__ void __launch_bounds__(128) apply_plan_kernel(const Dev P, const void
         }
     }
 }
+// The wide tiles' part of R rows (skb_pairs64.cuh), by differences; this thread's quarter of the columns.  Out of line:
+// its registers would come off the tiled loop's.
+template <int DM, int DV, int R>
+__device__ __noinline__ void apply_wide_tiles(const bool bf16, const int n, const int m, const int d, double *tile, const double *org, const void *x,
+                                              const void *y, const float *v, const int i0, const double k2, const double *f,
+                                              const double *g, const int dv, const int cs, const bool row_wide, double *out)
+{
+    auto raw = [bf16](const void *base, size_t i) -> float {
+        return bf16 ? __uint_as_float((unsigned)reinterpret_cast<const unsigned short *>(base)[i] << 16) : reinterpret_cast<const float *>(base)[i];
+    };
+    for (int e = 0; e < R * DV; ++e) out[e] = 0.0;
+    for (int j0 = 0; j0 < m; j0 += P64_TJ) {
+        __syncthreads();
+        P64Part<DM, 128> part;
+        p64_fetch(part, j0, m, d, [&](int j, int k) { return raw(y, (size_t)j * d + k); }, [&](int j) { return g[j]; });
+        const bool wide = p64_tile<DM, 128>(tile, org, j0, m, d, k2, part);
+        if (!__syncthreads_or(wide || row_wide)) continue;
+        for (int j = j0 + cs; j < m && j < j0 + P64_TJ; j += 4)
+            for (int r = 0; r < R; ++r) {
+                const int i = i0 + r < n ? i0 + r : n - 1;
+                const double t = p64_entry(d, k2, f[i] + g[j], [&](int k) { return raw(x, (size_t)i * d + k); }, [&](int k) { return raw(y, (size_t)j * d + k); });
+                for (int c = 0; c < dv; ++c) out[r * DV + c] = fma(t, (double)v[(size_t)j * dv + c], out[r * DV + c]);
+            }
+    }
+}
 // The same for d <= 32 by column tiles in shared memory (skb_pairs64.cuh); DV: values per point, rounded up.
-// 8 lanes of 4096 x 4096 points, d = dv = 3: 966 us with one warp per row, 411 us so.
+// 8 lanes of 4096 x 4096 points, d = dv = 3: 966 us with one warp per row, 414 us so.
 template <int DM, int DV>
 __global__ void __launch_bounds__(128) apply_plan_tiled_kernel(const Dev P, const void *x, const void *y, const float *eps,
                                                                const float *v, const int dv, float *out)
 {
     constexpr int R = 2, RW = 16;
-    __shared__ double tile[(DM + 1 + DV) * P64_TJ];
+    __shared__ double tile[P64_TILE<DM, 128>];
+    __shared__ double vals[DV * P64_TJ];                  // (a tile's values, float64)
+    __shared__ double org[DM];
     const int lane_t = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (!P.emitted[lane_t]) return;
     const int cs = lane >> 3, i0 = blockIdx.x * (4 * RW) + warp * RW + (lane & 7) * R;
     const double k2 = 1.4426950408889634 / (double)eps[lane_t];
     const double *f = P.f_out + (size_t)lane_t * P.n, *g = P.g_out + (size_t)lane_t * P.m;
     const size_t xb = (size_t)lane_t * P.n * P.d, yb = (size_t)lane_t * P.m * P.d;
+    if (threadIdx.x < DM) org[threadIdx.x] = threadIdx.x < P.d ? (double)load_raw(P, x, xb + (size_t)blockIdx.x * (4 * RW) * P.d + threadIdx.x) : 0.0;
+    __syncthreads();
     double xr[R][DM], ri[R], acc[R][DV];
+    bool row_wide = false;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int i = i0 + r < P.n ? i0 + r : P.n - 1;
         double q = 0.0;
 #pragma unroll
-        for (int k = 0; k < DM; ++k) { xr[r][k] = k < P.d ? (double)load_raw(P, x, xb + (size_t)i * P.d + k) : 0.0; q = fma(xr[r][k], xr[r][k], q); }
+        for (int k = 0; k < DM; ++k) { xr[r][k] = k < P.d ? (double)load_raw(P, x, xb + (size_t)i * P.d + k) - org[k] : 0.0; q = fma(xr[r][k], xr[r][k], q); }
         ri[r] = k2 * (f[i] - q);
+        row_wide = row_wide || p64_wide(k2, q);
 #pragma unroll
         for (int c = 0; c < DV; ++c) acc[r][c] = 0.0;
     }
-    for (int j0 = 0; j0 < P.m; j0 += P64_TJ) {
-        __syncthreads();
-        p64_tile<DM, 128>(tile, j0, P.m, P.d, k2, [&](int j, int k) { return load_raw(P, y, yb + (size_t)j * P.d + k); }, [&](int j) { return g[j]; });
-        for (int e = threadIdx.x; e < P64_TJ * DV; e += 128) {
-            const int jj = e % P64_TJ, c = e / P64_TJ;
-            tile[(DM + 1 + c) * P64_TJ + jj] = (j0 + jj < P.m && c < dv) ? (double)v[((size_t)lane_t * P.m + j0 + jj) * dv + c] : 0.0;
+    bool any_wide = false;
+    auto load = [&](int j, int k) { return load_raw(P, y, yb + (size_t)j * P.d + k); };
+    auto pot = [&](int j) { return g[j]; };
+    constexpr int NV = P64_TJ * DV / 128;
+    float vn[NV];
+    auto fetch_vals = [&](const int j0) {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const int e = threadIdx.x + 128 * q, j = j0 + e % P64_TJ, c = e / P64_TJ;
+            vn[q] = (j < P.m && c < dv) ? v[((size_t)lane_t * P.m + j) * dv + c] : 0.f;
         }
+    };
+    P64Part<DM, 128> part;
+    if (P64_AHEAD<DM>) { p64_fetch(part, 0, P.m, P.d, load, pot); fetch_vals(0); }
+    for (int j0 = 0; j0 < P.m; j0 += P64_TJ) {
+        if (!P64_AHEAD<DM>) { p64_fetch(part, j0, P.m, P.d, load, pot); fetch_vals(j0); }
         __syncthreads();
+#pragma unroll
+        for (int q = 0; q < NV; ++q) vals[threadIdx.x + 128 * q] = (double)vn[q];
+        const bool wide = p64_tile<DM, 128>(tile, org, j0, P.m, P.d, k2, part);
+        if (P64_AHEAD<DM>) { p64_fetch(part, j0 + P64_TJ, P.m, P.d, load, pot); fetch_vals(j0 + P64_TJ); }
+        if (__syncthreads_or(wide || row_wide)) { any_wide = true; continue; }
         const int end = P.m - j0 < P64_TJ ? P.m - j0 : P64_TJ;
 #pragma unroll 2
         for (int jj = cs; jj < end; jj += 4) {
@@ -818,11 +863,21 @@ __global__ void __launch_bounds__(128) apply_plan_tiled_kernel(const Dev P, cons
             for (int r = 0; r < R; ++r) t[r] = exp2(t[r]);
 #pragma unroll
             for (int c = 0; c < DV; ++c) {
-                const double vc = tile[(DM + 1 + c) * P64_TJ + jj];
+                const double vc = vals[c * P64_TJ + jj];
 #pragma unroll
                 for (int r = 0; r < R; ++r) acc[r][c] = fma(t[r], vc, acc[r][c]);
             }
         }
+    }
+    if (any_wide) {
+        double more[R][DV];
+        const size_t es = P.xy_bf16 ? 2 : 4;
+        apply_wide_tiles<DM, DV, R>(P.xy_bf16 != 0, P.n, P.m, P.d, tile, org, (const char *)x + xb * es, (const char *)y + yb * es,
+                                    v + (size_t)lane_t * P.m * dv, i0, k2, f, g, dv, cs, row_wide, &more[0][0]);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < DV; ++c) acc[r][c] += more[r][c];
     }
 #pragma unroll
     for (int r = 0; r < R; ++r)
@@ -841,13 +896,19 @@ static void launch_apply_tiled(const Dev &P, const void *x, const void *y, const
     if (dv <= 4) apply_plan_tiled_kernel<DM, 4><<<grid, 128, 0, st>>>(P, x, y, eps, v, dv, out);
     else apply_plan_tiled_kernel<DM, APPLY_MAX_DV><<<grid, 128, 0, st>>>(P, x, y, eps, v, dv, out);
 }
+// Few blocks of 64 rows leave SMs empty while the threads of the tiled kernel walk 16 times the columns: up to the
+// counts below a warp per row is faster (us, tiled -> warp per row, d = dv = 3: one lane of 1000 points 82 -> 55; of
+// 4096, 64 blocks, 257 -> 168; of 5000, 79 blocks, 340 -> 333; of 6000, 94 blocks, 404 <- 415; d = 8, dv = 1, 32 blocks
+// 152 -> 114; d = 12, 8 blocks 56 -> 46; d = 30, 5 blocks 68 -> 58).  Wide values (dv = 16, d = 4, 64 blocks 265 <- 560)
+// and more dimensions (d = dv = 15, 16 blocks 102 <- 109) want the tiles earlier.
 void launch_apply_plan(const Dev &P, const void *x, const void *y, const float *eps, const float *v, int dv, float *out,
                        int lanes, cudaStream_t st)
 {
+    const bool narrow = (long long)((P.n + 63) / 64) * lanes <= (P.d <= 8 && dv <= 8 ? 80 : 8);
+    if (P.d > P64_MAX_D || narrow) { apply_plan_kernel<<<dim3((P.n + 3) / 4, lanes), 128, 0, st>>>(P, x, y, eps, v, dv, out); return; }
     if (P.d <= 4) { launch_apply_tiled<4>(P, x, y, eps, v, dv, out, lanes, st); return; }
     if (P.d <= 16) { launch_apply_tiled<16>(P, x, y, eps, v, dv, out, lanes, st); return; }
-    if (P.d <= P64_MAX_D) { launch_apply_tiled<P64_MAX_D>(P, x, y, eps, v, dv, out, lanes, st); return; }
-    apply_plan_kernel<<<dim3((P.n + 3) / 4, lanes), 128, 0, st>>>(P, x, y, eps, v, dv, out);
+    launch_apply_tiled<P64_MAX_D>(P, x, y, eps, v, dv, out, lanes, st);
 }
 
 // ---------------------------------------------------------------- launchers

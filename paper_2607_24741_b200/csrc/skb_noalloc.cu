@@ -89,10 +89,30 @@ __global__ void __launch_bounds__(NA_THREADS) row_residual_kernel(
     r_row[lane_id] = (float)tot;
 }
 
+// The wide tiles' part of a row's sum (skb_pairs64.cuh), by differences; this thread's quarter of the columns.
+// Out of line: its registers would come off the tiled loop's.
+template <int DM, int THREADS>
+__device__ __noinline__ double wide_tiles(double *tile, const double *org, const float *xi, const float *yl, const double fi, const double *gl,
+                                          const int m, const int d, const double k2, const int cs, const bool row_wide)
+{
+    using namespace skb;
+    double s = 0.0;
+    for (int j0 = 0; j0 < m; j0 += P64_TJ) {
+        __syncthreads();
+        P64Part<DM, THREADS> part;
+        p64_fetch(part, j0, m, d, [&](int j, int k) { return yl[(size_t)j * d + k]; }, [&](int j) { return gl[j]; });
+        const bool wide = p64_tile<DM, THREADS>(tile, org, j0, m, d, k2, part);
+        if (!__syncthreads_or(wide || row_wide)) continue;
+        for (int j = j0 + cs; j < m && j < j0 + P64_TJ; j += 4)
+            s += p64_entry(d, k2, fi + gl[j], [&](int k) { return xi[k]; }, [&](int k) { return yl[(size_t)j * d + k]; });
+    }
+    return s;
+}
+
 // The same for d <= 32: a block of WPB warps takes 16 * WPB rows, column tiles come through shared memory
 // (skb_pairs64.cuh).  The entries are summed as they are; a row whose sum is not finite is redone the plain way,
 // so infinite potentials give what they always gave.  32 lanes of 1024 x 1000 points, d = 15: 1040 us with one
-// thread per row and the columns read from global memory, 150 us so.
+// thread per row and the columns read from global memory, 145 us so.
 template <int DM, int WPB>
 __global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
     Scratch *sc, const float *x, const float *y, const float *a, const double *f, const double *g,
@@ -100,7 +120,8 @@ __global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
 {
     using namespace skb;
     constexpr int R = 2, RW = 16;
-    __shared__ double tile[(DM + 1) * P64_TJ];
+    __shared__ double tile[P64_TILE<DM, 32 * WPB>];
+    __shared__ double org[DM];
     __shared__ double red[WPB];
     __shared__ int is_last;
     const int lane_id = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -108,20 +129,31 @@ __global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
     const double inv_eps = 1.0 / (double)eps[lane_id], k2 = 1.4426950408889634 * inv_eps;
     const float *xl = x + (size_t)lane_id * n * d, *yl = y + (size_t)lane_id * m * d;
     const double *fl = f + (size_t)lane_id * n, *gl = g + (size_t)lane_id * m;
+    if (tid < DM) org[tid] = tid < d ? (double)xl[(size_t)blockIdx.x * (RW * WPB) * d + tid] : 0.0;
+    __syncthreads();
     double xr[R][DM], ri[R], s[R];
+    bool row_wide = false;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int i = i0 + r < n ? i0 + r : n - 1;
         double q = 0.0;
 #pragma unroll
-        for (int k = 0; k < DM; ++k) { xr[r][k] = k < d ? (double)xl[(size_t)i * d + k] : 0.0; q = fma(xr[r][k], xr[r][k], q); }
+        for (int k = 0; k < DM; ++k) { xr[r][k] = k < d ? (double)xl[(size_t)i * d + k] - org[k] : 0.0; q = fma(xr[r][k], xr[r][k], q); }
         ri[r] = k2 * (fl[i] - q);
+        row_wide = row_wide || p64_wide(k2, q);
         s[r] = 0.0;
     }
+    bool any_wide = false;
+    auto load = [&](int j, int k) { return yl[(size_t)j * d + k]; };
+    auto pot = [&](int j) { return gl[j]; };
+    P64Part<DM, 32 * WPB> part;
+    if (P64_AHEAD<DM>) p64_fetch(part, 0, m, d, load, pot);
     for (int j0 = 0; j0 < m; j0 += P64_TJ) {
+        if (!P64_AHEAD<DM>) p64_fetch(part, j0, m, d, load, pot);
         __syncthreads();
-        p64_tile<DM, 32 * WPB>(tile, j0, m, d, k2, [&](int j, int k) { return yl[(size_t)j * d + k]; }, [&](int j) { return gl[j]; });
-        __syncthreads();
+        const bool wide = p64_tile<DM, 32 * WPB>(tile, org, j0, m, d, k2, part);
+        if (P64_AHEAD<DM>) p64_fetch(part, j0 + P64_TJ, m, d, load, pot);
+        if (__syncthreads_or(wide || row_wide)) { any_wide = true; continue; }
 #pragma unroll 2
         for (int jj = cs; jj < P64_TJ; jj += 4) {
             double v[R];
@@ -138,6 +170,11 @@ __global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
             for (int r = 0; r < R; ++r) s[r] += exp2(v[r]);
         }
     }
+    if (any_wide)
+        for (int r = 0; r < R; ++r) {
+            const int i = i0 + r < n ? i0 + r : n - 1;
+            s[r] += wide_tiles<DM, 32 * WPB>(tile, org, xl + (size_t)i * d, yl, fl[i], gl, m, d, k2, cs, row_wide);
+        }
     double term = 0.0;
 #pragma unroll
     for (int r = 0; r < R; ++r) {

@@ -1319,3 +1319,37 @@ def test_pair_sums_in_float64_at_the_edges_of_their_tiles(oracle, n, m, d, dv):
         fk = fr[k] + 0.3 * float(w.eps[k]) * np.sin(1.0 + np.arange(n))
         res, _ = oracle.residuals(w.x[k], w.y[k], w.a[k], w.b[k], float(w.eps[k]), fk, gr[k])
         assert abs(rr[k] - res) <= 2.0 ** -23 * res + 1e-12
+
+
+@pytest.mark.parametrize("eps", [1e-2, 1e-3])
+@pytest.mark.parametrize("offset,outlier", [(0.0, 0.0), (1e2, 0.0), (1e4, 0.0), (1e5, 0.0), (1e4, 1e2)])
+def test_pair_sums_do_not_depend_on_where_the_clouds_lie(oracle, offset, outlier, eps):
+    # clouds far from the origin, and a block whose first point is far from all others: the cost is a difference,
+    # so both calls must be as tight as for centred clouds.  Bound: the fp32 result's 2^-24, and arguments good to
+    # 2^-32 (k f is below 2^21 here: its own rounding, 2^-32, is of that size too)
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    rng = np.random.default_rng(11)
+    W, n, m, d = 2, 130, 150, 3
+    f32 = np.float32
+    x = (offset + 0.3 * rng.standard_normal((W, n, d))).astype(f32)
+    y = (offset + 0.3 * rng.standard_normal((W, m, d))).astype(f32)
+    x[:, 0] += f32(outlier)
+    y[:, 70] -= f32(outlier)
+    a, b = np.full((W, n), 1.0 / n, f32), np.full((W, m), 1.0 / m, f32)
+    e = np.full(W, eps, f32)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    args = [t(v) for v in (x, y, a, b, e)]
+    sb = B.SinkhornBatch(*args, 1e-9, compute="f64", max_iter=9)
+    sb.drain()
+    f, g = sb.potentials(f64=True)
+    v = (0.5 + rng.random((W, m, 2))).astype(f32)
+    out = sb.apply_plan(t(v)).cpu().numpy()
+    sb.close()
+    f2 = f + 0.3 * eps * torch.sin(1.0 + torch.arange(n, device="cuda:0", dtype=torch.float64))
+    rr = B.sinkhorn_row_residual_static(args[0], args[1], args[2], f2, g, args[4]).cpu().numpy()
+    for k in range(W):
+        want = oracle.apply_plan(x[k], y[k], float(e[k]), f[k].cpu().numpy(), g[k].cpu().numpy(), v[k])
+        np.testing.assert_allclose(out[k], want, rtol=2.0 ** -23, atol=0.0)
+        res, _ = oracle.residuals(x[k], y[k], a[k], b[k], float(e[k]), f2[k].cpu().numpy(), g[k].cpu().numpy())
+        assert abs(rr[k] - res) <= 2.0 ** -23 * res + 2.0 ** -31
