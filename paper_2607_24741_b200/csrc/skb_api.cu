@@ -227,8 +227,9 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
         d.topx[0] = (float *)take(W * d.nbx * 4); d.topx[1] = (float *)take(W * d.nbx * 4); d.topy = (float *)take(W * d.nby * 4);
     }
     if (var->xf && var->DP && scaling_fits(c->n, c->m)) {
-        d.phi0 = (double *)take(W * np * 8); d.gam0 = (double *)take(W * mp * 8);
-        d.uu[0] = (double *)take(W * np * 8); d.uu[1] = (double *)take(W * np * 8); d.vv = (double *)take(W * mp * 8);
+        // (these lanes have no streamed terms: what the set-up kernels write there is not read)
+        d.phi0 = (double *)d.ft[0]; d.uu[0] = (double *)d.ft[1]; d.uu[1] = (double *)d.fl[0];
+        d.gam0 = (double *)d.gt; d.vv = (double *)d.gl;
     }
     d.f_out = (double *)take(L * n * 8); d.g_out = (double *)take(L * m * 8);
     // guard band: raw copies of the inputs (the float64 re-evaluation reads nothing but these and the potentials)
