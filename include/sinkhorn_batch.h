@@ -223,8 +223,9 @@ skb_status sinkhorn_batch_apply_plan(skb_batch *h, const void *x, const void *y,
  * whether the lane was screen-positive.  After step(k) these belong to the state after k-1
  * cycles: the screen of a state is a by-product of the NEXT f-leg.  For shadow replays of the
  * audit (Section 5's attribution: does the screen ever hold back a lane the full check would
- * release?).  Kept by the one-launch-per-leg path only: MASKED, STATIC, tensor-core or profiled
- * batches (SKB_ERR_STATE otherwise).  Enqueues one kernel.
+ * release?).  The values do not depend on how the cycles were shared out among calls.  Not kept by
+ * ACTIVE batches that run several cycles per launch (SKB_ERR_STATE): MASKED, STATIC, tensor-core
+ * or profiled batches have them.  Enqueues one kernel.
  */
 skb_status sinkhorn_batch_last_audit(skb_batch *h, float *r_row, float *r_col, int *flagged);
 

@@ -509,18 +509,18 @@ extern "C" skb_status sinkhorn_batch_set_profiling(skb_batch *h, int on)
 static int launch_leg(skb_batch *h, int leg, int w)
 {
     if (h->tensor) { launch_update_tc(h->dev, h->maps, leg, w, h->stream); return 0; }
-    if (h->dev.phi0) { launch_scaling(h->dev, leg, 0, w, h->stream); return 0; }
+    if (h->dev.phi0) { launch_scaling(h->dev, SC_LEG, leg, 0, w, h->stream); return 0; }
     if (h->dev.permx) return launch_near(h->dev, leg, w, h->stream);
     return h->var->launch(h->dev, leg, w, h->stream);
 }
 
 // Batches whose lanes have few row blocks run several whole cycles per launch, one thread-block cluster
 // per lane (scaling_kernel, lane_resident_kernel or lane_cycles_kernel), followed by one planner for all
-// of them.  A mask can be kept inside such a launch by the scaling kernel only; a STATIC batch cannot be
-// run that way at all, because the cycle at which all of its lanes stop is not known beforehand.
+// of them.  A mask can be kept inside such a launch by the scaling kernel only, and only that one can run STATIC
+// batches so: the cycle at which all of their lanes stop is not known beforehand (plan_static_kernel).
 static bool cycles_in_one_launch(const skb_batch *h)
 {
-    if (h->dev.phi0) return h->cfg.mode != SKB_STATIC && !h->profiling && !h->no_multi_cycle;
+    if (h->dev.phi0) return !h->profiling && !h->no_multi_cycle;
     if (h->cfg.mode != SKB_ACTIVE || h->tensor || h->profiling || !h->var->launch_cycles || h->no_multi_cycle) return false;
     if (h->dev.permx) return false;
     const int mx = h->cfg.n > h->cfg.m ? h->cfg.n : h->cfg.m;
@@ -538,7 +538,15 @@ static bool cycles_in_one_launch(const skb_batch *h)
 static void enqueue_cycles_launch(skb_batch *h, int cycles)
 {
     const int w = h->known_width;
-    if (h->dev.phi0) launch_scaling(h->dev, LEG_F, cycles, w, h->stream);
+    if (h->cfg.mode == SKB_STATIC) {
+        launch_scaling(h->dev, SC_CYCLES, 0, cycles, w, h->stream);
+        launch_plan_static(h->dev, cycles, h->stream);
+        launch_scaling(h->dev, SC_CATCH_UP, 0, 0, w, h->stream);
+        h->enqueued += cycles;
+        h->launches += 3;
+        return;
+    }
+    if (h->dev.phi0) launch_scaling(h->dev, SC_CYCLES, 0, cycles, w, h->stream);
     else h->var->launch_cycles(h->dev, cycles, w, h->stream);
     int nk = 1;
     nk += launch_plan_cycles(h->dev, w, cycles, h->stream);
@@ -662,7 +670,7 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
     const long long hard_cap = (long long)h->cfg.max_iter + 4;
     while (!h->finished) {
         const bool multi = cycles_in_one_launch(h);      // may become true as the batch narrows
-        const int chunk_max = h->dev.phi0 && multi ? (h->cfg.mode == SKB_ACTIVE ? MAX_CYCLES_IN_LAUNCH : 64) : (multi ? 32 : 16);
+        const int chunk_max = h->dev.phi0 && multi ? (h->cfg.mode == SKB_MASKED || h->cfg.mode == SKB_MASKED_EXIT ? 64 : MAX_CYCLES_IN_LAUNCH) : (multi ? 32 : 16);
         NvtxRange nvtx_chunk(multi ? "skb:chunk (cycles in one launch)" : "skb:chunk (launch per leg)");
         if (multi) enqueue_cycles_launch(h, chunk);
         else for (int i = 0; i < chunk; ++i) enqueue_cycle(h);

@@ -530,7 +530,22 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
         P.cyc_log[dst] = P.cyc_log[src];
         P.nonfinite[dst] = 0;
     }
-    for (int s = tid; s < A; s += NT) { P.ret_at[s] = 0; P.n_checks[s] = 0; }
+    // the audit that counts as the most recent one: the launch's last, or the one at which the last lane left.  A lane
+    // that froze at that very audit shows what it was decided from; one that froze before shows a frozen lane's values
+    int jl = K - 1;
+    if (nret == c.n_running) while (jl > 0 && left_at[jl] == 0) --jl;
+    for (int s = tid; s < A; s += NT) {
+        if (P.mode == MODE_MASKED) {
+            const int r = P.ret_at[s];
+            if (r > 0 && r - 1 - k0 == jl) {
+                const double rc = P.res_col[P.lane_id[s]];
+                P.rrow[s] = P.res_row[P.lane_id[s]];
+                P.flag[s] = !isnan(rc);
+                P.rcol[s] = isnan(rc) ? 0.0 : rc;
+            } else if (P.early_exit && P.state[s]) { P.rrow[s] = 0.0; P.rcol[s] = 0.0; P.flag[s] = 0; }
+        }
+        P.ret_at[s] = 0; P.n_checks[s] = 0;
+    }
     if (tid == 0) {
         Ctl *g = P.ctl;
         const long long nm = (long long)P.n * P.m;
@@ -562,6 +577,58 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
         cc.emit_parity = parity_new ^ 1;
         for (int r = 0; r < nholes; ++r) emit_move_one<T>(P, cc, r, tid, NT);
     }
+}
+
+// Planner of a STATIC batch between the two halves of a multi-cycle launch (scaling_kernel).  In the first half the
+// lanes that had not passed ran up to K cycles, each stopping at the state it passed at.  If some lane has still
+// not passed, every lane goes on to cycle k0 + K; otherwise the batch ends at the cycle of the last one to pass.  The
+// second half (SC_CATCH_UP) takes the passed lanes there, and in the end writes everyone's outputs.  Whole lanes
+// are independent problems, so the order in which their cycles run changes no bit, and each runs every cycle once.
+__global__ void __launch_bounds__(PLAN_THREADS) plan_static_kernel(const Dev P, const int K)
+{
+    __shared__ int nret_s, checks_s, last_s;
+    pdl_enter();
+    const Ctl c = *P.ctl;
+    const int tid = threadIdx.x, NT = blockDim.x;
+    if (c.done) return;
+    const int k0 = c.cycle;
+    if (tid == 0) nret_s = checks_s = last_s = 0;
+    __syncthreads();
+    int nret = 0, nchk = 0, last = 0;
+    for (int s = tid; s < P.W; s += NT) {
+        const int r = P.ret_at[s];                       // (left for SC_CATCH_UP, which clears it)
+        if (r > 0) { ++nret; last = max(last, r - 1 - k0); }
+        nchk += P.n_checks[s];
+        P.n_checks[s] = 0;
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+        nret += __shfl_down_sync(0xffffffffu, nret, off);
+        nchk += __shfl_down_sync(0xffffffffu, nchk, off);
+        last = max(last, __shfl_down_sync(0xffffffffu, last, off));
+    }
+    if ((tid & 31) == 0) { atomicAdd(&nret_s, nret); atomicAdd(&checks_s, nchk); atomicMax(&last_s, last); }
+    __syncthreads();
+    const bool all = c.n_passed + nret_s == P.W;
+    const int ran = all ? last_s : K;
+    for (int j = tid; j < ran; j += NT) if (k0 + j < P.widths_cap) P.widths[k0 + j] = P.W;
+    if (tid == 0) {
+        Ctl *g = P.ctl;
+        const long long nm = (long long)P.n * P.m;
+        g->prev_cycle = k0;
+        g->cycle = k0 + ran;
+        g->parity = c.parity ^ (ran & 1);
+        g->n_passed = c.n_passed + nret_s;
+        g->n_retire = 0;
+        g->slots += (long long)ran * P.W;
+        // both legs of every cycle, the f-leg that screened the last state, the column checks, the closing one
+        g->pair_terms += ((2ll * ran + (all ? 2 : 0)) * P.W + checks_s) * nm;
+        if (all) { g->static_final = 1; g->n_running = 0; g->done = 1; }
+    }
+}
+void launch_plan_static(const Dev &P, int cycles, cudaStream_t st)
+{
+    const int nt = P.W >= PLAN_THREADS ? PLAN_THREADS : (P.W + 31) / 32 * 32;
+    launch_pdl(plan_static_kernel, dim3(1), dim3(nt), 0, st, P, cycles);
 }
 
 // ---------------------------------------------------------------- emit + move

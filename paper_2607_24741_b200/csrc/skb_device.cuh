@@ -47,7 +47,8 @@ struct Ctl {
     int static_final;  // STATIC: every lane has passed, next audit emits all lanes
     int error;         // sticky ErrBits
     int n_passed;      // STATIC: lanes that have recorded a depth
-    int pad0, pad1;
+    int prev_cycle;    // STATIC, launches of whole cycles: `cycle` before the launch just run
+    int pad0;
     unsigned long long max_radius_bits;   // largest scaled squared radius over lanes (double bits)
     long long slots;       // lane-cycles physically executed
     long long pair_terms;  // exp terms evaluated by update launches

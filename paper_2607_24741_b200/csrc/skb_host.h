@@ -73,11 +73,13 @@ void launch_prep_near(const Dev &P, const void *x, const void *y, const float *a
 void launch_near_tops(const Dev &P, cudaStream_t st);
 int launch_near(const Dev &P, int leg, int width, cudaStream_t st);     // 1: the guard band's pool rode in a column-check launch
 int guard_pool_rows(int per_row, bool on, int lanes);
-// lanes of mixed arithmetic small enough for their kernel matrix to stay on chip: whole cycles
-// (cycles > 0), or one leg as a launch of its own (cycles == 0)
+// lanes of mixed arithmetic small enough for their kernel matrix to stay on chip: whole cycles, or one leg as a
+// launch of its own
 bool scaling_fits(int n, int m);
-void launch_scaling(const Dev &P, int leg, int cycles, int width, cudaStream_t st);
+enum ScalingKind : int { SC_CYCLES, SC_CATCH_UP, SC_LEG };      // see scaling_kernel; `leg` counts for SC_LEG only
+void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int width, cudaStream_t st);
 int launch_plan_cycles(const Dev &P, int width, int cycles, cudaStream_t st);
+void launch_plan_static(const Dev &P, int cycles, cudaStream_t st);
 void launch_gather(const Dev &P, void *f, void *g, bool f64, cudaStream_t st);
 void launch_gather_audit(const Dev &P, float *rrow, float *rcol, int *flagged, cudaStream_t st);
 void launch_apply_plan(const Dev &P, const void *x, const void *y, const float *eps, const float *v, int dv, float *out,

@@ -45,16 +45,19 @@
 
 namespace skb {
 
-enum ScalingWhat : int { SC_CYCLES = 3 };               // besides LEG_F, LEG_G, LEG_V: whole cycles
 constexpr int SC_TAKE = 45, SC_KEEP = 30;               // bands of log2 u and log2 v: update taken / K kept
 constexpr int SC_BAD = 1, SC_DRIFT = 2, SC_NF = 4;
 
 // 2^arg for a float64 argument: integer part split off in float64, the remainder (|.| <= 1/2) rounded
 // to fp32 and put through the Taylor series of e^(x ln 2) (degree 7: truncation 5e-9), so the result is
-// good to about an ulp whatever the size of the argument.  Zero below 2^-124.
+// good to about an ulp whatever the size of the argument.  Zero below 2^-124, 2^100 from there on.
+// WORDS: the range tested on the argument's high word, by integers, instead of by two float64 comparisons and
+// selects.  Same results; the launches of one leg are faster so, the launches of whole cycles slower (96 lanes of
+// 100 x 77: 4.1 -> 5.1 ms a solve: it changes what the cycle loop keeps in registers).
+template <bool WORDS = false>
 __device__ __forceinline__ float exp2_split(const double arg)
 {
-    const double x = fmin(fmax(arg, -200.0), 100.0);
+    const double x = WORDS ? arg : fmin(fmax(arg, -200.0), 100.0);
     const double magic = 6755399441055744.0;             // 1.5 * 2^52: the sum's low word is the integer part
     const double t = x + magic;
     const int ni = __double2loint(t);
@@ -67,7 +70,13 @@ __device__ __forceinline__ float exp2_split(const double arg)
     q = fmaf(q, f, 2.4022651e-1f);
     q = fmaf(q, f, 6.9314718e-1f);
     const float p = fmaf(q, f, 1.0f);
-    return ni >= -124 ? __int_as_float(__float_as_int(p) + (ni << 23)) : 0.0f;
+    const float r = __int_as_float(__float_as_int(p) + (ni << 23));
+    if constexpr (!WORDS) return ni >= -124 ? r : 0.0f;
+    else {
+        const int hi = __double2hiint(arg);
+        const float z = (unsigned)hi <= 0xc05f4000u && ni >= -124 ? r : 0.0f;         // -125
+        return hi < 0x40590000 ? z : 0x1p100f;                                        // 100
+    }
 }
 
 __device__ __forceinline__ u64 mul2(u64 a, u64 b)
@@ -101,23 +110,20 @@ struct ScalingShape {
     static constexpr int G = (CL >= 16 || CL * RW == 64) ? 2 : 4;    // rows whose distances are formed together
     static constexpr int SHARE = 32 / RW;                            // threads that end up with the same row's sum
     static constexpr int BLOCKS = (CL * RW >= 128 ? 256 : 512) / THREADS;   // registers: 255 / 128 a thread
+    static constexpr int LEG_BLOCKS = 512 / THREADS;                 // launches of one leg do not hold K: 128
     static constexpr int FP32_COLS = CL <= 4 ? 8 : 32;               // columns a row's sum holds before it becomes float64
     static constexpr int FP32_WARPS = CL >= 8 && RW <= 16 ? 2 : 1;   // warps' column parts added in fp32 (at most 32 rows)
     static_assert(RW >= 8 && RW <= 32 && CL >= 2 && CL <= 16, "unsupported tile");
     static size_t smem(int nc) { return sizeof(double) * 2 * (size_t)nc * COLS; }        // the exchange buffers
 };
 
-// x_i . y_j of the scaled coordinates for G consecutive rows and this thread's CL columns
+// acc += x_i . y_j of the scaled coordinates for G consecutive rows and this thread's CL columns
 // (2 lane, 2 lane + 1, + 64, ...).  Rows and columns past the end read row / column 0; their results are
 // masked by the additive terms.
 template <int CL, int G>
 __device__ __forceinline__ void dot_tile(const double *xs, const double *ys, const int np, const int mp, const int d,
                                          const int i0, const int lane, double (&acc)[G][CL])
 {
-#pragma unroll
-    for (int r = 0; r < G; ++r)
-#pragma unroll
-        for (int e = 0; e < CL; ++e) acc[r][e] = 0.0;
     const double *xp = xs + (i0 < np ? i0 : 0);
     int yo[CL / 2];
 #pragma unroll
@@ -189,15 +195,16 @@ __device__ __noinline__ void log_rows(const double *xs, const double *ys, const 
 #pragma unroll
     for (int g = 0; g < RW / L::G; ++g) {
         double acc[L::G][CL], mr[L::G];
+#pragma unroll
+        for (int r = 0; r < L::G; ++r)
+#pragma unroll
+            for (int e = 0; e < CL; ++e) acc[r][e] = colB[(e / 2) * 64 + 2 * lane + (e & 1)];
         dot_tile<CL, L::G>(xs, ys, np, mp, d, i0 + g * L::G, lane, acc);
 #pragma unroll
         for (int r = 0; r < L::G; ++r) {
             double t = -1.0e300;
 #pragma unroll
-            for (int e = 0; e < CL; ++e) {
-                acc[r][e] += colB[(e / 2) * 64 + 2 * lane + (e & 1)];
-                t = fmax(t, acc[r][e]);
-            }
+            for (int e = 0; e < CL; ++e) t = fmax(t, acc[r][e]);
             for (int off = 16; off > 0; off >>= 1) t = fmax(t, __shfl_xor_sync(0xffffffffu, t, off));
             mr[r] = ceil(t);
             if (lane / L::SHARE == g * L::G + r) mine = mr[r];
@@ -224,11 +231,15 @@ __device__ __noinline__ void log_cols_max(const double *xs, const double *ys, co
 #pragma unroll 1
     for (int g = 0; g < RW / L::G; ++g) {
         double acc[L::G][CL];
+#pragma unroll
+        for (int r = 0; r < L::G; ++r)
+#pragma unroll
+            for (int e = 0; e < CL; ++e) acc[r][e] = rowA[g * L::G + r];
         dot_tile<CL, L::G>(xs, ys, np, mp, d, i0 + g * L::G, lane, acc);
 #pragma unroll
         for (int r = 0; r < L::G; ++r)
 #pragma unroll
-            for (int e = 0; e < CL; ++e) mc[e] = fmax(mc[e], rowA[g * L::G + r] + acc[r][e]);
+            for (int e = 0; e < CL; ++e) mc[e] = fmax(mc[e], acc[r][e]);
     }
 #pragma unroll
     for (int e = 0; e < CL; ++e) out[(e / 2) * 64 + 2 * lane + (e & 1)] = mc[e];
@@ -246,11 +257,15 @@ __device__ __noinline__ void log_cols_sum(const double *xs, const double *ys, co
 #pragma unroll 1
     for (int g = 0; g < RW / L::G; ++g) {
         double acc[L::G][CL];
+#pragma unroll
+        for (int r = 0; r < L::G; ++r)
+#pragma unroll
+            for (int e = 0; e < CL; ++e) acc[r][e] = rowA[g * L::G + r] - colM[(e / 2) * 64 + 2 * lane + (e & 1)];
         dot_tile<CL, L::G>(xs, ys, np, mp, d, i0 + g * L::G, lane, acc);
 #pragma unroll
         for (int r = 0; r < L::G; ++r)
 #pragma unroll
-            for (int e = 0; e < CL; ++e) s[e] += exp2_split(rowA[g * L::G + r] + acc[r][e] - colM[(e / 2) * 64 + 2 * lane + (e & 1)]);
+            for (int e = 0; e < CL; ++e) s[e] += exp2_split(acc[r][e]);
     }
 #pragma unroll
     for (int e = 0; e < CL; ++e) out[(e / 2) * 64 + 2 * lane + (e & 1)] = s[e];
@@ -308,13 +323,16 @@ __device__ __forceinline__ void scaling_barrier()
     else __syncthreads();
 }
 
-// what = SC_CYCLES: up to `cycles` whole cycles of every lane; LEG_F / LEG_V / LEG_G: one leg as a launch of its
-// own, for STATIC batches (whose common last cycle only the planner knows), phase timing and dry runs.
+// KIND = SC_CYCLES: up to `cycles` whole cycles of every lane.  SC_CATCH_UP: the passed lanes of a STATIC batch go on to
+// the cycle that the others have reached (plan_static_kernel).  SC_LEG: leg = LEG_F / LEG_V / LEG_G as a launch of its
+// own, for phase timing and dry runs: an entry of K is formed where it is used, with the same bits, and never kept.
 // CLU = 0: a lane has one block (its rows fit), and nothing of the cluster machinery is in the way.
-template <int NW, int CL, int RW, bool CLU>
-__global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) scaling_kernel(const __grid_constant__ Dev P, const int what, const int cycles)
+template <int NW, int CL, int RW, bool CLU, int KIND>
+__global__ void __launch_bounds__(32 * NW, (KIND == SC_LEG ? ScalingShape<NW, CL, RW>::LEG_BLOCKS : ScalingShape<NW, CL, RW>::BLOCKS))
+scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
 {
     typedef ScalingShape<NW, CL, RW> L;
+    constexpr bool LEG = KIND == SC_LEG, catch_up = KIND == SC_CATCH_UP;
     constexpr int THREADS = L::THREADS, COLS = L::COLS, RB = L::RB, NQ = L::NQ, SHARE = L::SHARE;
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -331,12 +349,27 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
     pdl_enter();
     const Ctl c = *P.ctl;
     const int slot = blockIdx.y;
-    if (c.done || slot >= c.n_phys) return;              // every exit here is taken by the whole cluster
+    // every exit here is taken by the whole cluster
+    const int lane_id = P.lane_id[slot < c.n_phys ? slot : 0];
+    if ((c.done && !catch_up) || slot >= c.n_phys) return;
     if (P.early_exit && P.state[slot] != 0) return;
-    if (what != SC_CYCLES) {
-        if (what != LEG_V && c.static_final) return;
-        if (what == LEG_V && !(c.static_final || lane_needs_column_check(P, c, slot))) return;
+    int par = c.parity, k = c.cycle, todo = cycles;
+    bool just_passed = false;
+    if constexpr (LEG) {
+        if (leg != LEG_V && c.static_final) return;
+        if (leg == LEG_V && !(c.static_final || lane_needs_column_check(P, c, slot))) return;
+    } else if (P.mode == MODE_STATIC) {
+        if ((P.state[slot] != 0) != catch_up) return;
+        if (catch_up) {
+            if (P.emitted[lane_id]) return;
+            const int left = P.ret_at[slot];             // passed in the launch just run, or before it
+            k = left > 0 ? left - 1 : c.prev_cycle;
+            todo = c.cycle - k;
+            just_passed = left > 0 && todo == 0;         // at the state that is the last one: its audit stands
+            par = c.parity ^ (todo & 1);
+        }
     }
+    const bool closing = catch_up && c.static_final;     // every lane has passed: this one's outputs are written at c.cycle
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = CLU ? (int)blockIdx.x : 0, NC = CLU ? (int)gridDim.x : 1;
     double *xbuf = reinterpret_cast<double *>(smem_raw);                 // [2][NC][COLS] column parts of every block
@@ -352,7 +385,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
     const int j0 = tid * NQ;                             // this thread's columns in the column steps: NQ adjacent ones
     const bool cown = COLS >= THREADS || tid < COLS;
     const size_t ro = (size_t)slot * P.np + (rok ? i : 0), co = (size_t)slot * P.mp;
-    const int lane_id = P.lane_id[slot], start = P.start[slot];
+    const int start = P.start[slot];
     const double inv_s = 1.0 / P.scale[slot];
     const double a_i = rok ? P.wa[ro] : 0.0, a_fix = a_i * RSUM_SCALE;
     bool frozen = P.mode == MODE_MASKED && P.state[slot] != 0;
@@ -363,7 +396,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
     // (the absorbed potentials stay in registers: every block holds all columns', and global memory gets them
     // back only at the end, when no block of the cluster can still be reading)
     double us = ab ? 1.0 : 0.0, phi0 = 0.0, vsd[NQ], gam0[NQ], bq[NQ];
-    if (rok) { us = ab ? P.uu[c.parity][ro] : P.phi[c.parity][ro]; phi0 = P.phi0[ro]; }
+    if (rok) { us = ab ? P.uu[par][ro] : P.phi[par][ro]; phi0 = P.phi0[ro]; }
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         const int j = j0 + q;
@@ -393,21 +426,41 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
     bool dead = false;                                   // a bounded wait ran out
     scaling_barrier<CLU>();                              // every block's shared memory is there
 
-    u64 K[RW][CL / 2];                                   // pairs of columns
+    u64 K[LEG ? 1 : RW][CL / 2];                         // pairs of columns
+    // entries of K for G of the warp's rows, from rowA and colB
+    auto form = [&](const int g, u64 (&kk)[L::G][CL / 2]) {
+        double acc[L::G][CL];
+#pragma unroll
+        for (int r = 0; r < L::G; ++r) {
+            const double ra = rowA[warp * RW + ((g * L::G) ^ perm) + r];
+#pragma unroll
+            for (int e = 0; e < CL; ++e) acc[r][e] = ra + colB[(e / 2) * 64 + 2 * lane + (e & 1)];
+        }
+        dot_tile<CL, L::G>(xs, ys, P.np, P.mp, P.d, i0 + ((g * L::G) ^ perm), lane, acc);
+#pragma unroll
+        for (int r = 0; r < L::G; ++r)
+#pragma unroll
+            for (int h = 0; h < CL / 2; ++h) kk[r][h] = pack2(exp2_split<LEG>(acc[r][2 * h]), exp2_split<LEG>(acc[r][2 * h + 1]));
+    };
     auto row_phi = [&](const double x) -> double { return ab ? phi0 + log2(x) : x; };
     auto col_gam = [&](const int q) -> double { return ab ? gam0[q] + log2(vsd[q]) : vsd[q]; };
     // column parts of sum_i K_ij w_i, w in uas: one row of partf per warp
     auto col_parts = [&]() {
         u64 acc[CL / 2];
 #pragma unroll
-        for (int r = 0; r < RW; r += 4) {
-            const ulonglong2 w0 = *reinterpret_cast<const ulonglong2 *>(uas + warp * RW + (r ^ perm));
-            const ulonglong2 w1 = *reinterpret_cast<const ulonglong2 *>(uas + warp * RW + (r ^ perm) + 2);
-            const u64 wr[4] = {w0.x, w0.y, w1.x, w1.y};
+        for (int r = 0; r < RW; r += L::G) {
+            u64 kk[L::G][CL / 2];
+            if constexpr (LEG) form(r / L::G, kk);
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
+            for (int q = 0; q < L::G; q += 2) {
+                const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(uas + warp * RW + ((r + q) ^ perm));
 #pragma unroll
-                for (int h = 0; h < CL / 2; ++h) acc[h] = r + q ? fma2(K[r + q][h], wr[q], acc[h]) : mul2(K[0][h], wr[0]);
+                for (int h = 0; h < CL / 2; ++h) {
+                    const u64 k0 = LEG ? kk[q][h] : K[LEG ? 0 : r + q][h], k1 = LEG ? kk[q + 1][h] : K[LEG ? 0 : r + q + 1][h];
+                    acc[h] = r + q ? fma2(k0, w.x, acc[h]) : mul2(k0, w.x);
+                    acc[h] = fma2(k1, w.y, acc[h]);
+                }
+            }
         }
 #pragma unroll
         for (int h = 0; h < CL / 2; ++h) *reinterpret_cast<u64 *>(partf + warp * COLS + h * 64 + 2 * lane) = acc[h];
@@ -526,8 +579,8 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
         __syncthreads();
     };
 
-    int par = c.parity, k = c.cycle, it = 0, checks = 0, retired_at = 0, fl = 0;
-    int nf = what == SC_CYCLES && !frozen ? P.nonfinite[slot] : 0;
+    int it = 0, checks = 0, retired_at = 0, fl = 0;
+    int nf = !LEG && !frozen ? P.nonfinite[slot] : 0;
     double rr = 0.0, rc = 0.0;
     bool need_build = true, near = false;
     for (;;) {
@@ -542,20 +595,18 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
                 }
             }
             __syncthreads();
+            if constexpr (!LEG) {
 #pragma unroll
-            for (int g = 0; g < RW / L::G; ++g) {
-                double acc[L::G][CL];
-                dot_tile<CL, L::G>(xs, ys, P.np, P.mp, P.d, i0 + ((g * L::G) ^ perm), lane, acc);
+                for (int g = 0; g < RW / L::G; ++g) {
+                    u64 kk[L::G][CL / 2];
+                    form(g, kk);
 #pragma unroll
-                for (int r = 0; r < L::G; ++r) {
-                    const double ra = rowA[warp * RW + ((g * L::G) ^ perm) + r];
+                    for (int r = 0; r < L::G; ++r)
 #pragma unroll
-                    for (int h = 0; h < CL / 2; ++h)
-                        K[g * L::G + r][h] = pack2(exp2_split(ra + colB[h * 64 + 2 * lane] + acc[r][2 * h]),
-                                                   exp2_split(ra + colB[h * 64 + 2 * lane + 1] + acc[r][2 * h + 1]));
+                        for (int h = 0; h < CL / 2; ++h) K[g * L::G + r][h] = kk[r][h];
                 }
+                __syncthreads();
             }
-            __syncthreads();
         }
         need_build = false;
 
@@ -565,7 +616,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
         double unew = 0.0, T[NQ];
         unsigned long long tot = 0ull;
         int all = SC_BAD;                            // "the f-leg is still to be done, in the log domain"
-        if (ab && (what == SC_CYCLES || what == LEG_F)) {
+        if (ab && (!LEG || leg == LEG_F)) {
 #pragma unroll 1
             for (;;) {
                 {
@@ -574,18 +625,30 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
 #pragma unroll
                     for (int h = 0; h < CL / 2; ++h) v[h] = *reinterpret_cast<const u64 *>(vs + h * 64 + 2 * lane);
 #pragma unroll
-                    for (int r = 0; r < RW; ++r) {
-                        u64 t = mul2(K[r][0], v[0]);
+                    for (int r = 0; r < RW; r += L::G) {
+                        u64 kk[L::G][CL / 2];
+                        if constexpr (LEG) form(r / L::G, kk);
 #pragma unroll
-                        for (int h = 1; h < CL / 2; ++h) t = fma2(K[r][h], v[h], t);
-                        float s0, s1;
-                        unpack2(t, s0, s1);
-                        s[r] = s0 + s1;
+                        for (int q = 0; q < L::G; ++q) {
+                            u64 t = mul2(LEG ? kk[q][0] : K[LEG ? 0 : r + q][0], v[0]);
+#pragma unroll
+                            for (int h = 1; h < CL / 2; ++h) t = fma2(LEG ? kk[q][h] : K[LEG ? 0 : r + q][h], v[h], t);
+                            float s0, s1;
+                            unpack2(t, s0, s1);
+                            s[r + q] = s0 + s1;
+                        }
                     }
                     const double S = row_exchange<CL, L::FP32_COLS, true, 16, RW, float>(s, lane);
                     unew = rok ? rcp64(S) : 1.0;
                     const double term = rown ? a_fix * fabs(fma(us, S, -1.0)) : 0.0;
                     const int flags = (out_of_band<SC_TAKE>(unew) ? SC_BAD : 0) | (out_of_band<SC_KEEP>(unew) ? SC_DRIFT : 0);
+                    if constexpr (LEG) {
+                        send_rows(to_fixed(term), flags);
+                        scaling_barrier<CLU>();
+                        tot = recv_rows(all);
+                        ++xch;
+                        break;
+                    }
                     if (lane % SHARE == 0) { const float w = (float)(a_i * unew); uas[lr] = make_float2(w, w); }
                     __syncwarp();
                     col_parts();
@@ -629,7 +692,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
                     }
                 }
                 ++xch;
-                if (all || (tot <= near_tot && !frozen) || nf || k - start >= P.max_iter || what == LEG_F) break;
+                if (all || (tot <= near_tot && !frozen && !catch_up) || nf || (k - start >= P.max_iter && !catch_up) || (closing && it == todo)) break;
                 // g-leg
                 double vn[NQ];
                 int flags = 0;
@@ -653,7 +716,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
                 }
                 ++k;
                 par ^= 1;
-                if (++it >= cycles) { done = true; break; }
+                if (++it >= todo && !closing) { done = true; break; }
             }
         }
         if (dead) {
@@ -661,12 +724,15 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
             break;
         }
         if (done) {
+            // (the last audit was that of the state before this launch's last cycle, and it flagged nothing)
             rr = (double)tot * (1.0 / RSUM_SCALE);
+            rc = 0.0;
+            fl = 0;
             break;
         }
 
         // ---------------- f-leg in the log domain, where K cannot be used
-        if (what != LEG_V && what != LEG_G) {
+        if (!LEG || leg == LEG_F) {
             if (all & SC_BAD) {
                 scal = false;
                 double term = 0.0;                       // in units of the fixed point
@@ -690,8 +756,8 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
             near = tot <= near_tot;
             rr = (double)tot * (1.0 / RSUM_SCALE);
             if (scal && (all & SC_DRIFT)) need_build = true;
-            {
-                if (what == LEG_F && !P.dry_run) {
+            if constexpr (LEG) {
+                if (!P.dry_run) {
                     if (rown && !frozen) {
                         P.phi[par ^ 1][ro] = scal ? phi0 + log2(unew) : unew;
                         P.uu[par ^ 1][ro] = unew;
@@ -702,13 +768,14 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
                         if (nf && !frozen) P.nonfinite[slot] = 1;
                     }
                 }
+                break;
             }
-            if (what == LEG_F) break;
         }
 
         // ---------------- audit of the state before the f-leg
-        if (what == SC_CYCLES) { fl = 0; rc = 0.0; }
-        if (what == SC_CYCLES && near && !frozen) {
+        const bool close_now = closing && it == todo;
+        if constexpr (!LEG) { fl = 0; rc = 0.0; }
+        if (!LEG && near && !frozen && !catch_up) {
             const bool audited = lane_audited(P, k, start);
             if (audited && !nf && in_guard_band(P, rr)) {
                 // guard band: decide from a float64 re-evaluation of the row residual; it reads the column
@@ -732,7 +799,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
             }
             fl = audited && !nf && rr <= P.tol_screen;
         }
-        if (what == LEG_V || (what == SC_CYCLES && fl)) {
+        if ((LEG && leg == LEG_V) || (!LEG && (fl || close_now))) {
             // column half of the two-sided check: the marginals of the audited state, genuinely measured
             double term[NQ];
             if (ab) {
@@ -777,18 +844,44 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
             if (bad) nf = 1;
             rc = (double)totc * (1.0 / RSUM_SCALE);
             ++checks;
-            if (what == LEG_V) {
+            if constexpr (LEG) {
                 if (b == 0 && tid == 0 && !P.dry_run) { P.rsum_col[slot] += totc; if (bad) P.nonfinite[slot] = 1; }
                 break;
             }
         }
-        if (what == SC_CYCLES && !frozen && (near || nf || k - start >= P.max_iter)) {
+        if (close_now) {
+            // the common last cycle of a STATIC batch.  A lane that passed at this very state keeps the row residual its
+            // decision was taken from
+            if (rown) P.f_out[(size_t)lane_id * P.n + i] = row_phi(us) * inv_s;
+            if (b == 0) {
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) { const int j = j0 + q; if (cown && j < P.m) P.g_out[(size_t)lane_id * P.m + j] = col_gam(q) * inv_s; }
+                if (tid == 0) {
+                    P.res_row[lane_id] = just_passed ? P.rrow[slot] : rr;
+                    P.res_col[lane_id] = rc;
+                    if (nf) P.status[lane_id] = LANE_NONFINITE;
+                    P.emitted[lane_id] = 1;
+                }
+            }
+            break;
+        }
+        if (!LEG && !frozen && !catch_up && (near || nf || k - start >= P.max_iter)) {
             const bool vd = !nf && fmax(rr, rc) <= P.tol_stop;
             const bool limit = k - start >= P.max_iter;
             int st = LANE_RUNNING;
             if (nf) st = LANE_NONFINITE;
             else if (fl && vd) st = LANE_DONE;
             else if (limit) st = LANE_ITER_LIMIT;
+            if (st != LANE_RUNNING && P.mode == MODE_STATIC) {
+                // the lane waits here until the others are known to go on (SC_CATCH_UP)
+                if (b == 0 && tid == 0) {
+                    P.depth[lane_id] = (limit && st != LANE_DONE) ? P.max_iter : k - start;
+                    P.status[lane_id] = st;
+                    P.state[slot] = 1;
+                }
+                retired_at = k + 1;
+                break;
+            }
             if (st != LANE_RUNNING) {
                 if (rown) P.f_out[(size_t)lane_id * P.n + i] = row_phi(us) * inv_s;
                 if (b == 0) {
@@ -812,7 +905,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
         // ---------------- g-leg
         double vnew[NQ];
         bool log_g = false;
-        if (what == LEG_G) {
+        if constexpr (LEG) {
             // us is what the f-leg left (u, or the row potential where it ran in the log domain)
             log_g = !ab || P.cyc_log[slot] != 0;
             unew = us;
@@ -892,7 +985,7 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
                 for (int q = 0; q < NQ; ++q) vsd[q] = vnew[q];
             }
         } else need_build = false;
-        if (what == LEG_G) {
+        if constexpr (LEG) {
             if (!P.dry_run && !frozen) {
                 if (nf && b == 0 && tid == 0) P.nonfinite[slot] = 1;
                 if (need_build && ab && rown) { P.uu[par][ro] = 1.0; P.phi0[ro] = phi0; }
@@ -911,15 +1004,15 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
         }
         ++k;
         par ^= 1;
-        if (++it >= cycles) break;
+        if (++it >= todo && !closing) break;
     }
-    if (what == SC_CYCLES) {
+    if constexpr (!LEG) {
         if (b == 0 && tid == 0) {
             P.ret_at[slot] = retired_at;
-            P.n_checks[slot] = checks;
-            P.rrow[slot] = rr; P.rcol[slot] = rc; P.flag[slot] = fl;
+            P.n_checks[slot] = catch_up ? 0 : checks;
+            if (!just_passed) { P.rrow[slot] = rr; P.rcol[slot] = catch_up ? 0.0 : rc; P.flag[slot] = fl; }
         }
-        if (!retired_at || P.mode == MODE_MASKED) {
+        if (!retired_at || P.mode != MODE_ACTIVE) {
             // the lane goes back out; a frozen one keeps the state it froze with
             if (rown) {
                 P.phi[par][ro] = row_phi(us);
@@ -943,10 +1036,10 @@ __global__ void __launch_bounds__(32 * NW, (ScalingShape<NW, CL, RW>::BLOCKS)) s
 struct ScalingVariant {
     int threads, cols, rb;
     bool cluster;                                        // lanes of several blocks
-    const void *kernel;
+    const void *kernel[3];                               // by ScalingKind
     size_t (*smem)(int nc);
 };
-#define SKB_SC(NW, CL, RW, CLU) { 32 * NW, 32 * CL, NW * RW, CLU, (const void *)&scaling_kernel<NW, CL, RW, CLU>, &ScalingShape<NW, CL, RW>::smem }
+#define SKB_SC(NW, CL, RW, CLU) { 32 * NW, 32 * CL, NW * RW, CLU, {(const void *)&scaling_kernel<NW, CL, RW, CLU, SC_CYCLES>, (const void *)&scaling_kernel<NW, CL, RW, CLU, SC_CATCH_UP>, (const void *)&scaling_kernel<NW, CL, RW, CLU, SC_LEG>}, &ScalingShape<NW, CL, RW>::smem }
 // narrowest column count first, then fewest rows per block
 static const ScalingVariant g_scaling[] = {
     SKB_SC(2, 2, 8, false), SKB_SC(4, 2, 16, false), SKB_SC(4, 2, 32, false), SKB_SC(4, 2, 32, true),
@@ -973,14 +1066,15 @@ static const ScalingVariant *scaling_variant(int n, int m)
 
 bool scaling_fits(int n, int m) { return scaling_variant(n, m) != nullptr; }
 
-void launch_scaling(const Dev &P, int leg, int cycles, int width, cudaStream_t st)
+void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int width, cudaStream_t st)
 {
     const ScalingVariant *v = scaling_variant(P.n, P.m);
+    const void *kernel = v->kernel[kind];
     const int nc = (P.n + v->rb - 1) / v->rb;
     const size_t smem = v->smem(nc);
     // (with the fixed arrays some variants are beyond the 48 KB that need no permission; the attribute belongs
     // to the current device, so it is set with every launch)
-    if (v->cluster) cudaFuncSetAttribute(v->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (v->cluster) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nc, width < 1 ? 1 : width);
     cfg.blockDim = dim3(v->threads);
@@ -992,9 +1086,8 @@ void launch_scaling(const Dev &P, int leg, int cycles, int width, cudaStream_t s
     attr[1].val.clusterDim.x = nc; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = v->cluster ? 2 : 1;
     Dev dev = P;
-    int w = cycles > 0 ? (int)SC_CYCLES : leg, cy = cycles;
-    void *args[3] = {&dev, &w, &cy};
-    cudaLaunchKernelExC(&cfg, v->kernel, args);
+    void *args[3] = {&dev, &leg, &cycles};
+    cudaLaunchKernelExC(&cfg, kernel, args);
 }
 
 }  // namespace skb

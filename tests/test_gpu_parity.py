@@ -1257,6 +1257,70 @@ def test_kernel_matrix_lanes_whose_potentials_move_fast(oracle, cycles):
     assert err.max() <= 1e-6 * cycles + 2e-6, err
 
 
+@pytest.mark.parametrize("kw", [dict(W=40, n=100, m=77, d=8), dict(W=24, n=64, m=64, d=2), dict(W=9, n=200, m=256, d=8), dict(W=5, n=300, m=500, d=8)])
+@pytest.mark.parametrize("every,guard", [(1, 0.0), (4, 0.3)])
+def test_static_batches_of_kernel_matrix_lanes_however_they_are_run(kw, every, guard):
+    # the whole-cycle launches (the passed lanes wait and are caught up) against one launch per leg (phase timing), in
+    # one drain, one cycle per call and a few cycles per call: same bits, same accounting; running lanes are
+    # readable in between at the common cycle
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("sweep", max_iter=150, tol=5e-3, **kw)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    args = [t(v) for v in (w.x, w.y, w.a, w.b, w.eps)]
+
+    def run(step=0, profiling=False):
+        sb = B.SinkhornBatch(*args, w.tol, mode="static", compute="mixed", max_iter=150, audit_every=every, guard_band=guard)
+        sb.set_profiling(profiling)
+        seen = {}
+        while step and sb.active():
+            sb.step(step)
+            st = sb.stats()
+            if st["cycles"] in (6, 12, 24, 48, 96):
+                seen[st["cycles"]] = [v.cpu().numpy() for v in sb.potentials(f64=True)] + [st["slots"]]
+                assert st["slots"] == w.shape[0] * st["cycles"]
+        sb.drain()
+        st = sb.stats(widths_cap=200)
+        out = [v.cpu().numpy() for v in (*sb.potentials(f64=True), *sb.depths(), *sb.residuals(), *sb.last_audit())]
+        assert sb.check_guards() == -1
+        sb.close()
+        return out + [np.array(st["widths"]), st["slots"], st["pair_terms"], st["cycles"]], seen
+    ref, seen_ref = run(1, True)
+    assert len(set(ref[2].tolist())) > 2 and (ref[3] != 0).all() and ref[-1] == ref[2].max()
+    for step in (0, 1, 3, 24):
+        got, seen = run(step)
+        for a, b in zip(got, ref):
+            np.testing.assert_array_equal(a, b)
+        for k in seen:
+            for a, b in zip(seen[k], seen_ref[k]):
+                np.testing.assert_array_equal(a, b)
+
+
+def test_last_audit_of_a_mask_does_not_depend_on_how_the_cycles_were_run():
+    # lanes that froze earlier in a launch of many cycles are not screen-positive at its last audit
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("sweep", W=40, n=100, m=77, tol=2e-2, max_iter=400)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    args = [t(v) for v in (w.x, w.y, w.a, w.b, w.eps)]
+    for mode in ("masked", "masked_exit"):
+        for cycles in (40, 160):
+            out = []
+            for step, profiling in ((1, True), (1, False), (cycles, False), (8, False)):
+                sb = B.SinkhornBatch(*args, w.tol, mode=mode, compute="mixed", max_iter=400)
+                sb.set_profiling(profiling)
+                for _ in range(cycles // step):
+                    sb.step(step)
+                running = sb.depths()[1].cpu().numpy() == 0
+                out.append([v.cpu().numpy() for v in sb.last_audit()])
+                sb.close()
+            assert 0 < running.sum() < 40 and np.isnan(out[0][1]).any()
+            for rr, rc, fl in out[1:]:
+                # (r_row of a lane that is frozen already is not a screen of anything: only the others')
+                np.testing.assert_array_equal(rr[running], out[0][0][running])
+                np.testing.assert_array_equal(rc, out[0][1]); np.testing.assert_array_equal(fl, out[0][2])
+
+
 # ---- large low-dimensional lanes in spatial order ----------------------------------------------------
 @pytest.mark.parametrize("n,m,d", [(1024, 1024, 3), (1023, 1025, 3), (1055, 64, 2), (31, 1100, 4), (1024, 33, 1), (8193, 40, 3)])
 def test_lanes_in_spatial_order(oracle, n, m, d):
