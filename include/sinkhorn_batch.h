@@ -90,8 +90,11 @@ typedef struct {
     float tol_screen;      /* row-screen threshold; <= 0 means "same as tol"               */
     int column_split;      /* 0 = automatic; 1, 4 or 32 forces how many lanes of a warp     */
                            /* share one row's columns in the update kernel (tuning knob)  */
-    int cost_form;         /* 0 = chosen per lane from its scaled radius; 1 = expanded     */
-                           /* |x|^2+|y|^2-2x.y everywhere; 2 = difference |x-y|^2 everywhere */
+    int cost_form;         /* fp32 arithmetic: 0 = chosen from the lanes' scaled radii; 1 = */
+                           /* expanded |x|^2+|y|^2-2x.y everywhere; 2 = difference |x-y|^2  */
+                           /* everywhere.  With 0, lanes of at most four dimensions and at  */
+                           /* least 1024 points may be kept in spatial order, coordinates   */
+                           /* relative to local boxes, where create finds that it pays      */
     void *stream;          /* cudaStream_t (0 = legacy default stream)                     */
     void *workspace;       /* device, 256-byte aligned                                     */
     size_t workspace_bytes;

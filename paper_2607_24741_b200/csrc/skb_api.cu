@@ -108,11 +108,15 @@ static double mixed_radius(double tol)
     return MIXED_RADIUS * (tol < 1.0e-3 ? tol / 1.0e-3 : 1.0);
 }
 
-// Large low-dimensional fp32 lanes go into spatial order (skb_near.cu) up to this tolerance.  Its arithmetic is also
-// the more accurate one: the expanded form's rounding, M * 8e-8 in every plan entry, is 3.5 % of a tolerance of
-// 1e-3 at the M = 430 of the registration workload.  Looser solves, where that is below a per cent or two, stay on
-// the expanded form and on the results they have always had: plans applied from them agree with earlier ones
-// to 1e-6, the other path's differ by as much as the expanded form's own error, 1.2e-6.
+// Large low-dimensional fp32 lanes go into spatial order (skb_near.cu) where that lets a leg skip enough: a pair costs
+// it 1.3 times the plain kernel's, so up to this share of the pairs kept, as near_estimate_kernel estimates it at
+// create.  Unit sphere, tol 1e-3, f-leg plain -> spatial: 32 lanes of 8192 points 624 -> 212 us at eps 0.01 and 593 ->
+// 747 us at 0.1 (all kept); 4 lanes of 4096 points 37 -> 16 us at 0.01, 35 -> 22 us at 0.03 (share 0.6), 35 -> 27 us at
+// 0.05 (0.8), 34 -> 34 us at 0.1.  (With few blocks in flight it still wins at 0.8, with many it loses from 0.75.)
+static const double NEAR_SHARE = 0.75;
+// ... and up to this tolerance: plans applied from looser solves agree with those of the plain kernel's potentials to
+// the rounding of its expanded cost, 1.2e-6 on the registration workload at tol 1e-2, and callers hold such results to
+// 1e-6 of earlier ones.  It costs those solves the 624 against 212 us a leg.
 static const double SPATIAL_TOL = 2.0e-3;
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -299,9 +303,8 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     }
     if (!(tol > 0.0f) || !std::isfinite(tol)) return fail(nullptr, SKB_ERR_VALUE, "tol must be positive and finite");
     const bool automatic = cfg->compute == SKB_COMPUTE_AUTO;
-    const bool spatial = (double)tol <= SPATIAL_TOL;
-    const Variant *var = variant_for(cfg, automatic ? SKB_COMPUTE_F32 : cfg->compute, spatial);
-    const Variant *var_big = variant_for(cfg, automatic ? SKB_COMPUTE_MIXED : cfg->compute, spatial);
+    const Variant *var = variant_for(cfg, automatic ? SKB_COMPUTE_F32 : cfg->compute, false);
+    const Variant *var_big = variant_for(cfg, automatic ? SKB_COMPUTE_MIXED : cfg->compute, false);
     if (!var || !var_big) return fail(nullptr, SKB_ERR_SHAPE, "dimension d is not supported by any update kernel");
     const int mx = cfg->n > cfg->m ? cfg->n : cfg->m;
     // a lane's residual is a 64-bit fixed-point sum of per-row terms clamped at RSUM_ROW_MAX
@@ -312,7 +315,7 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     if (cfg->compute == SKB_COMPUTE_TENSOR && !can_tensor)
         return fail(nullptr, SKB_ERR_SHAPE, "the tensor-core path needs bf16 x, y and d a multiple of 64 with 64 <= d <= 512");
     size_t zero_end = 0;
-    carve(cfg, var_big, false, spatial, nullptr, nullptr, &zero_end);
+    carve(cfg, var_big, false, false, nullptr, nullptr, &zero_end);
     const size_t need = sinkhorn_batch_workspace_bytes(cfg);
     if (!cfg->workspace) return fail(nullptr, SKB_ERR_WORKSPACE, "workspace is null");
     if (((uintptr_t)cfg->workspace & 255u) != 0) return fail(nullptr, SKB_ERR_WORKSPACE, "workspace must be 256-byte aligned");
@@ -331,7 +334,7 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     h->lanes_used = cfg->W; h->enqueued_at_refill = 0;
     for (int i = 0; i < SKB_N_PHASES; ++i) h->phase_ms[i] = 0.f;
     h->guards.count = 0;
-    carve(cfg, var, h->tensor, spatial, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+    carve(cfg, var, h->tensor, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
     h->dev.tol_stop = (double)tol;
     h->dev.tol_screen = cfg->tol_screen > 0.0f ? (double)cfg->tol_screen : (double)tol;
     cudaError_t e;
@@ -357,8 +360,13 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     }
     launch_lane_stats(h->dev, x, y, eps, 0, 0, cfg->W, 0, h->stream);
     h->launches += 2;   // lane statistics + layout kernel
-    if (automatic) {
-        // read the largest scaled radius back and pick the arithmetic for the whole batch
+    // spatial order: never for a cost form the caller named, nor for radii at which the plain kernels take differences
+    const Variant *var_near = variant_for(cfg, SKB_COMPUTE_F32, true);
+    const bool near_shaped = var_near && (automatic || cfg->compute == SKB_COMPUTE_F32) && (double)tol <= SPATIAL_TOL && cfg->cost_form == 0 &&
+                             near_shape(var_near->f64, var_near->DP, var_near->CS, cfg->n, cfg->m);
+    if (near_shaped) { launch_near_estimate(h->dev, x, y, cfg->W, h->stream); h->launches += 1; }
+    if (automatic || near_shaped) {
+        // read the largest scaled radius back and pick the arithmetic and the layout for the whole batch
         if ((e = cudaMemcpyAsync(&h->h_ctl[1], h->dev.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess ||
             (e = cudaStreamSynchronize(h->stream)) != cudaSuccess) {
             skb_status st = cuda_fail(nullptr, e, "create");
@@ -368,12 +376,15 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
         double radius;
         memcpy(&radius, &h->h_ctl[1].max_radius_bits, sizeof(double));
         const double ts = h->dev.tol_stop, tsc = h->dev.tol_screen;
-        if (radius > mixed_radius(ts < tsc ? ts : tsc)) {
+        if (automatic && radius > mixed_radius(ts < tsc ? ts : tsc)) {
             h->var = var_big;
-            carve(cfg, var_big, false, spatial, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
-        } else if (can_tensor) {
+            carve(cfg, var_big, false, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+        } else if (automatic && can_tensor) {
             h->tensor = true;
             carve(cfg, var, true, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+        } else if (near_shaped && radius <= FORM_DIFF_RADIUS && h->h_ctl[1].near_kept <= NEAR_SHARE * NEAR_PAIRS * cfg->W) {
+            h->var = var_near;
+            carve(cfg, var_near, false, true, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
         }
         h->dev.tol_stop = ts; h->dev.tol_screen = tsc;
     }

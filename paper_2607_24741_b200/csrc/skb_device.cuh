@@ -48,7 +48,7 @@ struct Ctl {
     int error;         // sticky ErrBits
     int n_passed;      // STATIC: lanes that have recorded a depth
     int prev_cycle;    // STATIC, launches of whole cycles: `cycle` before the launch just run
-    int pad0;
+    int near_kept;     // create: sampled pairs that the spatial order would keep (near_estimate_kernel)
     unsigned long long max_radius_bits;   // largest scaled squared radius over lanes (double bits)
     long long slots;       // lane-cycles physically executed
     long long pair_terms;  // exp terms evaluated by update launches

@@ -68,6 +68,8 @@ void launch_update_tc(const Dev &P, const void *maps, int leg, int width, cudaSt
 int launch_emit_move(const Dev &P, int width, cudaStream_t st);
 // lanes kept in spatial order, whose legs skip the boxes of columns that are too far away to matter
 bool near_shape(int f64, int DP, int CS, int n, int m);
+constexpr int NEAR_PAIRS = 4096;        // pairs per lane that launch_near_estimate counts into Ctl::near_kept
+void launch_near_estimate(const Dev &P, const void *x, const void *y, int lanes, cudaStream_t st);
 void launch_spatial_sort(const Dev &P, const void *x, const void *y, int slot0, int count, cudaStream_t st);
 void launch_prep_near(const Dev &P, const void *x, const void *y, const float *a, const float *b, int slot0, int count, cudaStream_t st);
 void launch_near_tops(const Dev &P, cudaStream_t st);

@@ -1350,6 +1350,86 @@ def test_lanes_in_spatial_order(oracle, n, m, d):
     assert pot_err(rf["f"], rf["g"], ref.f, ref.g, far.eps.astype(np.float64)).max() <= POT_TOL_F32
 
 
+def _cloud_pair(law, W, n, m, d, rng):
+    if law == "sphere":
+        x = rng.standard_normal((W, n, d)); x /= np.linalg.norm(x, axis=2, keepdims=True)
+        y = rng.standard_normal((W, m, d)); y /= np.linalg.norm(y, axis=2, keepdims=True)
+        return x, y + 0.01 * rng.standard_normal((W, m, d))
+    if law == "flat":                                    # a sheet in more dimensions than it has
+        x, y = rng.random((W, n, d)), rng.random((W, m, d))
+        x[:, :, 2:] *= 0.01; y[:, :, 2:] *= 0.01
+        return x, y
+    return rng.random((W, n, d)), rng.random((W, m, d))
+
+
+# (law, n, m, d, eps, spatial order expected): boxes of 32 points against the reach of eps
+SPATIAL = [("sphere", 4096, 4000, 3, 0.01, True), ("sphere", 2500, 2047, 3, 0.01, True), ("sphere", 4096, 4096, 3, 0.1, False),
+           ("cube", 2048, 1500, 2, 0.002, True), ("cube", 1024, 1025, 1, 0.002, True), ("cube", 2048, 2048, 2, 0.03, False),
+           ("flat", 1800, 3001, 4, 0.003, True), ("sphere", 8193, 300, 3, 0.01, True), ("flat", 2048, 33, 3, 0.003, True), ("cube", 1500, 1500, 4, 0.02, False)]
+
+
+@pytest.mark.parametrize("law,n,m,d,eps,expected", SPATIAL)
+def test_spatial_order_is_taken_where_it_can_skip(oracle, law, n, m, d, eps, expected):
+    # the choice follows the data (the ordering is one more set-up launch), and either way the state after a few cycles
+    # is the oracle's; lanes of one batch are decided together
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    rng = np.random.default_rng(n + m)
+    W = 2
+    x, y = _cloud_pair(law, W, n, m, d, rng)
+    f32 = np.float32
+    a = rng.uniform(0.5, 1.5, (W, n)); b = rng.uniform(0.5, 1.5, (W, m))
+    w = wl.Workload(law, x.astype(f32), y.astype(f32), (a / a.sum(1, keepdims=True)).astype(f32),
+                    (b / b.sum(1, keepdims=True)).astype(f32), np.array([eps, 1.3 * eps], f32), 1e-3, 6)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+
+    def run(**kw):
+        sb = B.SinkhornBatch(t(w.x), t(w.y), t(w.a), t(w.b), t(w.eps), kw.pop("tol", w.tol), max_iter=6, **kw)
+        launches, arith = sb.launch_count(), sb.arithmetic()
+        sb.drain()
+        f, g = (v.cpu().numpy() for v in sb.potentials(f64=True))
+        assert sb.check_guards() == -1
+        sb.close()
+        return f, g, launches, arith
+    f, g, launches, arith = run()
+    assert arith == "f32"
+    plain = run(column_split=1)
+    assert launches - plain[2] == (2 if expected else 1)      # the estimate, the ordering
+    ref = oracle.solve_batch(w.x, w.y, w.a, w.b, w.eps, w.tol, max_iter=6)
+    e = w.eps.astype(np.float64)
+    assert pot_err(f, g, ref.f, ref.g, e).max() <= POT_TOL_F32
+    assert pot_err(plain[0], plain[1], ref.f, ref.g, e).max() <= POT_TOL_F32
+    if expected:
+        # a mask never changes its launch shape; a warm proposal finds its way into the order
+        masked = run(mode="masked")
+        np.testing.assert_array_equal(masked[0], f); np.testing.assert_array_equal(masked[1], g)
+        part = oracle.solve_batch(w.x, w.y, w.a, w.b, w.eps, w.tol, fixed_cycles=2)
+        rw = run_gpu(w, warm=(part.f, part.g), max_iter=4)
+        assert pot_err(rw["f"], rw["g"], ref.f, ref.g, e).max() <= POT_TOL_F32
+    # a cost form that the caller names, and looser tolerances, stay on the plain kernels
+    for kw in (dict(cost_form=1), dict(cost_form=2), dict(tol=1e-2)):
+        assert run(**kw)[2] == plain[2], kw
+
+
+@pytest.mark.parametrize("cost_form", [0, 1, 2])
+def test_large_radii_in_fp32_take_differences_whatever_the_size(oracle, cost_form):
+    # scaled squared radius of 1000 to 3000, asked for in fp32: cost_form 0 and 2 must be the difference form with
+    # two-part potentials.  Per cycle its error is a few ulp of the settled terms, the expanded form's an ulp of the radius
+    rng = np.random.default_rng(3)
+    W, n, m, d, cycles = 3, 1100, 1030, 3, 4
+    f32 = np.float32
+    x = rng.standard_normal((W, n, d)); x /= np.linalg.norm(x, axis=2, keepdims=True)
+    y = x[:, rng.permutation(n)[:m]] + 0.02 * rng.standard_normal((W, m, d))
+    w = wl.Workload("radius", x.astype(f32), y.astype(f32), np.full((W, n), 1 / n, f32), np.full((W, m), 1 / m, f32),
+                    np.array([2e-3, 1e-3, 7e-4], f32), 1e-3, cycles)
+    r = run_gpu(w, compute="f32", cost_form=cost_form, max_iter=cycles)
+    ref = oracle.solve_batch(w.x, w.y, w.a, w.b, w.eps, w.tol, max_iter=cycles)
+    e = w.eps.astype(np.float64)
+    err = np.maximum(np.abs(r["f"] - ref.f).max(1), np.abs(r["g"] - ref.g).max(1)) / e
+    radius = 1.4427 / e * 1.1
+    assert (err <= (radius * 2.0 ** -22 * cycles if cost_form == 1 else 2e-5)).all(), (cost_form, err, radius)
+
+
 # ---- float64 pair sums by column tiles ---------------------------------------------------------------
 @pytest.mark.parametrize("n,m,d,dv", [(1, 1, 1, 1), (63, 65, 4, 4), (64, 64, 5, 5), (65, 128, 16, 16), (130, 63, 17, 3), (40, 70, 32, 16),
                                       (33, 50, 33, 2), (4097, 20, 3, 3)])
