@@ -189,7 +189,6 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
     d.guard_bad = (int *)take(4);
     d.state = (int *)take(W * 4); d.flag = (int *)take(W * 4); d.verdict = (int *)take(W * 4);
     d.nonfinite = (int *)take(W * 4);
-    d.radius = (double *)take(W * 8);
     d.absorbed = (int *)take(W * 4); d.cyc_log = (int *)take(W * 4);
     d.ret_at = (int *)take(W * 4); d.n_checks = (int *)take(W * 4);
     d.rsum_row64 = (unsigned long long *)take(W * 8); d.esc = (int *)take(W * 4);

@@ -42,7 +42,6 @@ __device__ __forceinline__ void lane_enters(const Dev &P, const float *eps, cons
     P.rsum_row[slot] = 0ull; P.rsum_col[slot] = 0ull; P.rsum_row64[slot] = 0ull; P.esc[slot] = 0;
     P.ret_at[slot] = 0; P.n_checks[slot] = 0;
     P.absorbed[slot] = 0; P.cyc_log[slot] = 0;
-    P.radius[slot] = sqrt(r2);
     // (lanes in spatial order have a form of their own, which shares the expanded form's scale and terms)
     int form = P.permx ? FORM_DOT : P.cost_form == 1 ? FORM_DOT : (P.cost_form == 2 ? FORM_DIFF : (s * r2 > P.form_threshold ? FORM_DIFF : FORM_DOT));
     P.form[slot] = form;

@@ -93,7 +93,6 @@ struct Dev {
     int *flag;                // screen-positive at this audit
     int *verdict;             // two-sided check passed
     int *nonfinite;
-    double *radius;           // largest distance of a point from the centre, in the inputs' units
     int *absorbed, *cyc_log;  // scaling_kernel: phi0 .. vv are valid (or SC_NO_MATRIX); the last f-leg ran in the log domain
     // multi-cycle launches: cycle count + 1 at which the lane in the slot left inside the launch
     // (0 = still running), and the column checks it ran
