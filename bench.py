@@ -41,11 +41,10 @@ ALL = ("tiny", "sensor", "feature", "registration", "sweep")
 
 # DRAM bytes (read + write) of ONE full-width f-leg launch of the dominant kernel, from the ncu
 # captures summarised in the named files under profiles/ (one launch each; they equal the lanes'
-# operands read once).  A kernel whose tiling changes needs a fresh capture: set its entry to None.
+# operands read once).  A kernel whose tiling changes needs a fresh capture and has no entry until then
+# (registration and sweep run kernels that were not captured).
 NCU_TRAFFIC = {
     "sensor": (20.5e6, "profiles/update_kernel_sensor_registration_sweep.md"),
-    "registration": (13.7e6, "profiles/update_kernel_sensor_registration_sweep.md"),
-    "sweep": (42.0e6, "profiles/update_kernel_sensor_registration_sweep.md"),
     "feature": (193.3e6, "profiles/update_tc_kernel_feature.md"),
 }
 
@@ -231,11 +230,20 @@ class Runner:
         w, args = self.w, self.args
         W, n, m, d = w.shape
         sb = self.batch("static")
+        launches = sb.launch_count()
         sb.step(2)
         k_ms = sb.profile_update(leg=0, reps=20 if W * n * m < (1 << 30) else 8)
         g_ms = sb.profile_update(leg=1, reps=3)
         arith = sb.arithmetic()
         sb.close()
+        # which kernel the legs ran: small lanes of float64 exponents keep their kernel matrix on chip; lanes in
+        # spatial order were put into it by a launch of their own at create, after one that estimated its worth
+        on_chip = arith == "mixed" and d <= 32 and m <= 512 and n <= (1024 if m <= 128 else 512)
+        spatial = False
+        if arith == "f32":
+            plain = self.batch("static", column_split=1)
+            spatial = launches - plain.launch_count() == 2
+            plain.close()
         pk = peaks()
         f_hz = pk["sm_max_mhz"] * 1e6
         pairs = float(W) * n * m
@@ -252,7 +260,41 @@ class Runner:
         traffic, traffic_from = NCU_TRAFFIC.get(self.name, (None, None))
         dtype = {"f32": "f32", "mixed": "f64 exponents / f32 exp", "f64": "f64",
                  "tensor": "bf16 (f32 accumulate, f32 exp)"}[arith]
-        if arith == "tensor":
+        if on_chip:
+            # a solve runs whole cycles in one launch: time per cycle at full width, from launches of 64 and 192
+            # cycles that no lane leaves; per pair and cycle one fp32 multiply-add in each leg
+            ms = []
+            for cycles in (64, 192):
+                best = None
+                for _ in range(4):
+                    sb = self.batch("active", tol=1e-12)
+                    sb.step(64)
+                    e0, e1 = self.torch.cuda.Event(enable_timing=True), self.torch.cuda.Event(enable_timing=True)
+                    e0.record(); sb.step(cycles); e1.record()
+                    self.torch.cuda.synchronize()
+                    sb.close()
+                    best = e0.elapsed_time(e1) if best is None else min(best, e0.elapsed_time(e1))
+                ms.append(best)
+            c_ms = (ms[1] - ms[0]) / 128
+            fma_peak = SM_COUNT * FP32_LANES * f_hz
+            fma = 2.0 * pairs / (c_ms * 1e-3)
+            r = {"bound": "latency", "kernel": "scaling_kernel (one cycle of a launch of many, full width)", "arithmetic": arith,
+                 "binding_unit": "dependent chain of a cycle", "achieved": fma / 1e12, "peak": fma_peak / 1e12, "unit": "T fp32 FMA/s",
+                 "frac": fma / fma_peak, "exp_frac": None, "pipe_frac": fma / fma_peak, "ms_per_cycle": c_ms,
+                 "ms_per_launch": k_ms, "g_leg_ms_per_launch": g_ms, "pairs_per_launch": pairs,
+                 "note": "ms_per_launch: one leg as a launch of its own (phase timing), which forms its matrix entries anew",
+                 "peak_clock_mhz": pk["sm_max_mhz"], "traffic": None, "peak_source": "nominal unit counts x max SM clock"}
+            if unit_rates:
+                r["frac_of_measured_unit_rates"] = {"pipe": fma / max(unit_rates["ffma"], unit_rates["ffma2"])}
+        elif spatial:
+            # boxes of far columns are skipped, so the pairs a launch covers are not exponentials evaluated: no
+            # fraction of a unit's rate can be formed from them
+            r = {"bound": "issue", "kernel": "update_near_kernel (f-leg, full width)", "arithmetic": arith,
+                 "binding_unit": "instruction issue and the latency of a box's chain", "achieved": achieved_exp / 1e12, "peak": None,
+                 "unit": "T pairs covered/s (far ones skipped)", "frac": None, "exp_frac": None, "pipe_frac": None,
+                 "ms_per_launch": k_ms, "g_leg_ms_per_launch": g_ms, "pairs_per_launch": pairs,
+                 "peak_clock_mhz": pk["sm_max_mhz"], "traffic": None}
+        elif arith == "tensor":
             # the cross term is a dense bf16 contraction: 2*d flops per pair against the measured
             # cuBLAS bf16 burst throughput (kernel timed alone)
             tf = 2.0 * d * pairs / (k_ms * 1e-3) / 1e12
