@@ -263,8 +263,10 @@ skb_status sinkhorn_batch_set_profiling(skb_batch *h, int on);
  *   slots      lane-cycles physically executed: sum_k A_k in ACTIVE mode, W*l_max otherwise
  *   cycles     complete cycles executed (l_max)
  *   widths     widths[k-1] = physical width of cycle k, for k = 1..min(cycles, widths_cap)
- *   pair_terms exp-terms evaluated by the update kernel, all passes (legs, look-ahead
- *              screen, column check)
+ *   pair_terms terms of the sums of Eq. 3 and Eq. 5 that were asked for, n * m per lane and pass
+ *              (legs, look-ahead screen, column check).  Lanes in spatial order skip those that
+ *              are too small to matter, lanes whose kernel matrix stays on chip spend a
+ *              multiply-add on a term instead of an exponential
  *   phase_ms   [SKB_N_PHASES] milliseconds per skb_phase summed over the solve so far;
  *              entries other than SKB_PHASE_CREATE are zero unless phase timing is on
  */
@@ -322,8 +324,10 @@ skb_status sinkhorn_batch_launch_count(skb_batch *h, long long *launches);
  * returns the mean duration per launch in milliseconds (host out).  Call it between cycles
  * (after step, before drain).  The launches are dry runs: all pair work and the row epilogue,
  * but no potential is stored and no residual term added, so a solve continued afterwards
- * gives the same bits as one that was never profiled.  Returns SKB_ERR_STATE when no lane is
- * running any more (the launch would return at once).  Synchronises.
+ * gives the same bits as one that was never profiled.  Lanes whose kernel matrix stays on chip
+ * form its entries anew in such a launch, which a solve does once per launch of many cycles: time
+ * step(k) for those.  Returns SKB_ERR_STATE when no lane is running any more (the launch would
+ * return at once).  Synchronises.
  */
 skb_status sinkhorn_batch_profile_update(skb_batch *h, int leg, int reps, float *ms_per_launch);
 

@@ -51,7 +51,7 @@ struct Ctl {
     int near_kept;     // create: sampled pairs that the spatial order would keep (near_estimate_kernel)
     unsigned long long max_radius_bits;   // largest scaled squared radius over lanes (double bits)
     long long slots;       // lane-cycles physically executed
-    long long pair_terms;  // exp terms evaluated by update launches
+    long long pair_terms;  // n * m per lane and pass of the update launches
 };
 
 struct Dev {

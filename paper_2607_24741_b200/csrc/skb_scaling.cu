@@ -36,7 +36,10 @@
 // Measured per cycle in long launches, before (cost and exponential recomputed in every leg by a cluster of
 // eight blocks) -> now: 8 lanes of 64 x 64, d = 2: 5.3 -> 0.93 us; one lane of 256 x 256, d = 8: 1.9 us; all 1024
 // lanes of the sweep workload at tol 1e-3: 112 -> 24 ms per solve; the masked control at 96 lanes of
-// 100 x 77: 105 -> 5.7 ms (it ran one launch per leg).  Forming K costs 25 to 40 us per launch.
+// 100 x 77: 105 -> 5.7 ms (it ran one launch per leg); STATIC, 1024 lanes at tol 3e-3: 249 -> 47 ms.
+// Forming K costs 25 to 40 us per launch of one wave (0.28 ms for 1024 lanes; latency: two warps per scheduler, the FP64
+// pipe at 14 %), so a caller that steps one cycle per call pays more than the recomputing kernels took - one lane of
+// 256 x 256 16 -> 25 us, 1024 lanes 176 -> 325 us - and from two (1024 lanes: four) cycles per call on less.
 // The exchange between blocks through remote stores that report to a barrier of the receiver, instead of a
 // cluster barrier: 2.9 -> 2.4 us; 128-thread blocks (two of different lanes per SM) instead of 256: 58 -> 47 us
 // per cycle of 1024 lanes, together with the rows' order that spares the selects of the exchange.
