@@ -1325,8 +1325,9 @@ def test_last_audit_of_a_mask_does_not_depend_on_how_the_cycles_were_run():
 @pytest.mark.parametrize("n,m,d", [(1024, 1024, 3), (1023, 1025, 3), (1055, 64, 2), (31, 1100, 4), (1024, 33, 1), (8193, 40, 3)])
 def test_lanes_in_spatial_order(oracle, n, m, d):
     # sizes around the threshold, ragged boxes of 32, chunks of the ordering, every padded dimension; lanes of
-    # several regularisations, from one that keeps every column to one that keeps a few.  The mask control, which
-    # never changes its launch shape, must give the same bits, and a warm proposal must find its way into the order.
+    # several regularisations.  The mask control, which never changes its launch shape, must give the same bits, and a
+    # warm proposal must find its way into the order.  (Clouds as wide as these mostly stay on the plain kernels: the
+    # next test has the batches that are put into spatial order, and says so.)
     rng = np.random.default_rng(n + m + d)
     W = 3
     x = rng.standard_normal((W, n, d)); y = rng.standard_normal((W, m, d)) * 0.8 + 0.2
