@@ -24,7 +24,10 @@
 // were shared out among launches nor on the mode.
 //
 // Work layout.  A cluster of NC blocks owns the lane; a block of NW warps owns NW * RW rows, a warp RW of
-// them, and a thread the entries of its warp's rows in CL columns, in registers: E = RW * CL values.  Row
+// them, and a thread the entries of its warp's rows in CL columns: E = RW * CL values, in registers or, where a
+// lane would otherwise need several blocks, in tensor memory, which holds as much again as the register file and is
+// read as fast as the multiply-adds go (256 words of 256 threads: 770 clk alone, 1020 with one packed
+// multiply-add per pair of words, 960 for the multiply-adds alone).  Row
 // sums are reduced by a halving exchange over the 32 threads; column sums go through shared memory (and
 // to the other blocks through distributed shared memory), every block forming all of v by itself.  One
 // cluster barrier and two block barriers per cycle: the column sums of the next state are formed before
@@ -33,18 +36,21 @@
 // What bounds it: the chain of dependent steps of a cycle (two rounds of multiply-adds, the exchange of row
 // sums, two float64 reciprocals, the column parts through shared memory, the exchange between blocks), not a
 // unit: the multiply-adds of a 256 x 256 lane are 256 clk of packed fp32 per scheduler, a cycle is 3700.
-// Measured per cycle in long launches, before (cost and exponential recomputed in every leg by a cluster of
-// eight blocks) -> now: 8 lanes of 64 x 64, d = 2: 5.3 -> 0.93 us; one lane of 256 x 256, d = 8: 1.9 us; all 1024
-// lanes of the sweep workload at tol 1e-3: 112 -> 24 ms per solve; the masked control at 96 lanes of
-// 100 x 77: 105 -> 5.7 ms (it ran one launch per leg); STATIC, 1024 lanes at tol 3e-3: 249 -> 47 ms.
-// Forming K costs 25 to 40 us per launch of one wave (0.28 ms for 1024 lanes; latency: two warps per scheduler, the FP64
-// pipe at 14 %), so a caller that steps one cycle per call pays more than the recomputing kernels took - one lane of
-// 256 x 256 16 -> 25 us, 1024 lanes 176 -> 325 us - and from two (1024 lanes: four) cycles per call on less.
+// Measured per cycle in long launches: 8 lanes of 64 x 64, d = 2: 0.82 us; 96 of 100 x 77: 0.91 us; one lane of
+// 256 x 256, d = 8, K in registers of a cluster of four blocks -> in tensor memory of one block: 1.7 -> 1.5 us; 148 of
+// them 5.4 -> 1.55 us (four blocks of a cluster per SM waited for each other's exchanges); all 1024 of the sweep workload
+// 27 -> 10 us, 24 -> 10.9 ms per solve at tol 1e-3.  512 x 512, clusters of eight blocks, registers -> of four, tensor memory:
+// 5.6 -> 3.5 us.  16 warps of 16 rows instead of 8 of 32: 2.2 us.
+// Forming K costs 10 to 20 us per launch of one wave (latency: two warps per scheduler), so a caller that steps one cycle
+// per call pays mostly for that: 25 us on one lane of 256 x 256, 155 us on 1024.  The formation is a loop in every variant:
+// unrolled, as it has to be to index registers, it was 100 KB of instructions that ran once per launch, and
+// fetching them took longer than running them (256 x 256: 43 -> 25 us per call; 96 lanes of 100 x 77: 30 -> 20 us).
 // The exchange between blocks through remote stores that report to a barrier of the receiver, instead of a
 // cluster barrier: 2.9 -> 2.4 us; 128-thread blocks (two of different lanes per SM) instead of 256: 58 -> 47 us
 // per cycle of 1024 lanes, together with the rows' order that spares the selects of the exchange.
 #include "skb_update.cuh"
 #include "skb_host.h"
+#include "skb_tmem.cuh"
 
 namespace skb {
 
@@ -105,19 +111,26 @@ __device__ __forceinline__ bool out_of_band(const double x)
     return ((unsigned)__double2hiint(x) >> 20) - (unsigned)(1023 - BAND) >= (unsigned)(2 * BAND);
 }
 
-template <int NW_, int CL_, int RW_>
+// TM: a thread's E values of K are in tensor memory, which is used as storage of its own (32x32b accesses: a warp's
+// lane and column range belong to the same threads throughout), instead of in registers.
+template <int NW_, int CL_, int RW_, bool TM_ = false>
 struct ScalingShape {
     static constexpr int NW = NW_, CL = CL_, RW = RW_;
+    static constexpr bool TM = TM_;
+    static constexpr int TM_COLS = TM ? CL * RW * NW / 4 : 32;       // tensor memory columns of a block
     static constexpr int THREADS = 32 * NW, COLS = 32 * CL, RB = NW * RW;
     static constexpr int NQ = (COLS + THREADS - 1) / THREADS;        // columns a thread owns in the column steps
     static constexpr int G = (CL >= 16 || CL * RW == 64) ? 2 : 4;    // rows whose distances are formed together
     static constexpr int SHARE = 32 / RW;                            // threads that end up with the same row's sum
-    static constexpr int BLOCKS = (CL * RW >= 128 ? 256 : 512) / THREADS;   // registers: 255 / 128 a thread
+    static constexpr int BLOCKS = TM ? 512 / TM_COLS : (CL * RW >= 128 ? 256 : 512) / THREADS;   // registers: 255 / 128 a thread
     static constexpr int LEG_BLOCKS = 512 / THREADS;                 // launches of one leg do not hold K: 128
     static constexpr int FP32_COLS = CL <= 4 ? 8 : 32;               // columns a row's sum holds before it becomes float64
     static constexpr int FP32_WARPS = CL >= 8 && RW <= 16 ? 2 : 1;   // warps' column parts added in fp32 (at most 32 rows)
     static_assert(RW >= 8 && RW <= 32 && CL >= 2 && CL <= 16, "unsupported tile");
-    static size_t smem(int nc) { return sizeof(double) * 2 * (size_t)nc * COLS; }        // the exchange buffers
+    static_assert(!TM || (NW % 4 == 0 && G * CL == 32 && TM_COLS <= 512 && BLOCKS <= 4), "unsupported tile in tensor memory");
+    __host__ __device__ static constexpr size_t exchange(int nc) { return sizeof(double) * 2 * (size_t)nc * COLS; }
+    // the exchange buffers and, where K is in registers, the words it is formed in
+    static size_t smem(int nc) { return exchange(nc) + (TM ? 0 : sizeof(float) * (size_t)RW * CL * THREADS); }
 };
 
 // acc += x_i . y_j of the scaled coordinates for G consecutive rows and this thread's CL columns
@@ -194,8 +207,8 @@ __device__ __noinline__ void log_rows(const double *xs, const double *ys, const 
     typedef ScalingShape<NW, CL, RW> L;
     const int lane = threadIdx.x & 31;
     double mine = 0.0;
-    float part[RW];
-#pragma unroll
+    float part[RW];                                      // (indexed in a rolled loop, so on the stack)
+#pragma unroll 1
     for (int g = 0; g < RW / L::G; ++g) {
         double acc[L::G][CL], mr[L::G];
 #pragma unroll
@@ -330,12 +343,12 @@ __device__ __forceinline__ void scaling_barrier()
 // the cycle that the others have reached (plan_static_kernel).  SC_LEG: leg = LEG_F / LEG_V / LEG_G as a launch of its
 // own, for phase timing and dry runs: an entry of K is formed where it is used, with the same bits, and never kept.
 // CLU = 0: a lane has one block (its rows fit), and nothing of the cluster machinery is in the way.
-template <int NW, int CL, int RW, bool CLU, int KIND>
-__global__ void __launch_bounds__(32 * NW, (KIND == SC_LEG ? ScalingShape<NW, CL, RW>::LEG_BLOCKS : ScalingShape<NW, CL, RW>::BLOCKS))
+template <int NW, int CL, int RW, bool CLU, bool TMEM, int KIND>
+__global__ void __launch_bounds__(32 * NW, (KIND == SC_LEG ? ScalingShape<NW, CL, RW, TMEM>::LEG_BLOCKS : ScalingShape<NW, CL, RW, TMEM>::BLOCKS))
 scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
 {
-    typedef ScalingShape<NW, CL, RW> L;
-    constexpr bool LEG = KIND == SC_LEG, catch_up = KIND == SC_CATCH_UP;
+    typedef ScalingShape<NW, CL, RW, TMEM> L;
+    constexpr bool LEG = KIND == SC_LEG, catch_up = KIND == SC_CATCH_UP, TM = TMEM && !LEG;
     constexpr int THREADS = L::THREADS, COLS = L::COLS, RB = L::RB, NQ = L::NQ, SHARE = L::SHARE;
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -348,6 +361,7 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
     __shared__ __align__(16) float vs[COLS];             // b v of all columns
     __shared__ __align__(16) float2 uas[RB];             // a u of own rows, in both halves
     __shared__ __align__(8) unsigned long long xbar[2];  // arrival of an exchange's stores, one per buffer
+    __shared__ uint32_t tm_holder;
 
     pdl_enter();
     const Ctl c = *P.ctl;
@@ -376,6 +390,7 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = CLU ? (int)blockIdx.x : 0, NC = CLU ? (int)gridDim.x : 1;
     double *xbuf = reinterpret_cast<double *>(smem_raw);                 // [2][NC][COLS] column parts of every block
+    u64 *kstage = reinterpret_cast<u64 *>(smem_raw + L::exchange(NC));   // K on its way into the registers
     int xch = 0;                                                         // exchanges so far: their buffer alternates
 
     const double *xs = reinterpret_cast<const double *>(P.xs) + (size_t)slot * P.DP * P.np;
@@ -427,9 +442,11 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
     }
     unsigned xphase = 0u;                                // phase of each buffer's barrier
     bool dead = false;                                   // a bounded wait ran out
+    if constexpr (TM) { if (warp == 0) tc_alloc<L::TM_COLS>(&tm_holder); tc_fence_before(); }
     scaling_barrier<CLU>();                              // every block's shared memory is there
+    uint32_t tk = 0u;                                    // this warp's part of tensor memory
+    if constexpr (TM) { tc_fence_after(); tk = tm_holder + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * (RW * CL)); }
 
-    u64 K[LEG ? 1 : RW][CL / 2];                         // pairs of columns
     // entries of K for G of the warp's rows, from rowA and colB
     auto form = [&](const int g, u64 (&kk)[L::G][CL / 2]) {
         double acc[L::G][CL];
@@ -443,30 +460,73 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
 #pragma unroll
         for (int r = 0; r < L::G; ++r)
 #pragma unroll
-            for (int h = 0; h < CL / 2; ++h) kk[r][h] = pack2(exp2_split<LEG>(acc[r][2 * h]), exp2_split<LEG>(acc[r][2 * h + 1]));
+            for (int h = 0; h < CL / 2; ++h) kk[r][h] = pack2(exp2_split<LEG || TM>(acc[r][2 * h]), exp2_split<LEG || TM>(acc[r][2 * h + 1]));
+    };
+    u64 K[LEG || TM ? 1 : RW][CL / 2];                   // pairs of columns
+    // use(r, k) for every group of G rows, k[q][h] the entries of row r + q, with the next group's on their way
+    auto each_rows = [&](auto &&use) {
+        if constexpr (TM) {
+            uint32_t ra[32], rb[32];
+            auto pass = [&](const int g, const uint32_t (&w)[32]) {
+                u64 kk[L::G][CL / 2];
+#pragma unroll
+                for (int q = 0; q < L::G; ++q)
+#pragma unroll
+                    for (int h = 0; h < CL / 2; ++h) kk[q][h] = pack2(__uint_as_float(w[q * CL + 2 * h]), __uint_as_float(w[q * CL + 2 * h + 1]));
+                use(g * L::G, kk);
+            };
+            constexpr int NG = RW / L::G;
+            static_assert(NG % 2 == 0, "groups are taken in pairs");
+            tc_ld32_issue(tk, ra);
+            tc_ld_wait(ra);
+#pragma unroll
+            for (int g = 0; g < NG; g += 2) {
+                tc_ld32_issue(tk + (uint32_t)(g + 1) * 32u, rb);
+                pass(g, ra);
+                tc_ld_wait(rb);
+                if (g + 2 < NG) tc_ld32_issue(tk + (uint32_t)(g + 2) * 32u, ra);
+                pass(g + 1, rb);
+                if (g + 2 < NG) tc_ld_wait(ra);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < RW; r += L::G) {
+                u64 kk[L::G][CL / 2];
+                if constexpr (LEG) form(r / L::G, kk);
+                else {
+#pragma unroll
+                    for (int q = 0; q < L::G; ++q)
+#pragma unroll
+                        for (int h = 0; h < CL / 2; ++h) kk[q][h] = K[r + q][h];
+                }
+                use(r, kk);
+            }
+        }
     };
     auto row_phi = [&](const double x) -> double { return ab ? phi0 + log2(x) : x; };
     auto col_gam = [&](const int q) -> double { return ab ? gam0[q] + log2(vsd[q]) : vsd[q]; };
     // column parts of sum_i K_ij w_i, w in uas: one row of partf per warp
     auto col_parts = [&]() {
-        u64 acc[CL / 2];
-#pragma unroll
-        for (int r = 0; r < RW; r += L::G) {
-            u64 kk[L::G][CL / 2];
-            if constexpr (LEG) form(r / L::G, kk);
+        // (two sums of half the rows each where a warp has 32: shorter sums, smaller errors)
+        constexpr int NA = RW > 16 ? 2 : 1;
+        u64 acc[NA][CL / 2];
+        each_rows([&](const int r, const u64 (&kk)[L::G][CL / 2]) {
+            const int e = r / (RW / NA), first = r % (RW / NA) == 0;
 #pragma unroll
             for (int q = 0; q < L::G; q += 2) {
                 const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(uas + warp * RW + ((r + q) ^ perm));
 #pragma unroll
                 for (int h = 0; h < CL / 2; ++h) {
-                    const u64 k0 = LEG ? kk[q][h] : K[LEG ? 0 : r + q][h], k1 = LEG ? kk[q + 1][h] : K[LEG ? 0 : r + q + 1][h];
-                    acc[h] = r + q ? fma2(k0, w.x, acc[h]) : mul2(k0, w.x);
-                    acc[h] = fma2(k1, w.y, acc[h]);
+                    acc[e][h] = q || !first ? fma2(kk[q][h], w.x, acc[e][h]) : mul2(kk[q][h], w.x);
+                    acc[e][h] = fma2(kk[q + 1][h], w.y, acc[e][h]);
                 }
             }
-        }
+        });
 #pragma unroll
-        for (int h = 0; h < CL / 2; ++h) *reinterpret_cast<u64 *>(partf + warp * COLS + h * 64 + 2 * lane) = acc[h];
+        for (int h = 0; h < CL / 2; ++h) {
+            if constexpr (NA == 2) acc[0][h] = add2(acc[0][h], acc[1][h]);
+            *reinterpret_cast<u64 *>(partf + warp * COLS + h * 64 + 2 * lane) = acc[0][h];
+        }
     };
     // this block's part of column j: fp32 up to 32 rows, float64 beyond
     auto block_col = [&](const int j) -> double {
@@ -599,14 +659,34 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
             }
             __syncthreads();
             if constexpr (!LEG) {
-#pragma unroll
+#pragma unroll 1
                 for (int g = 0; g < RW / L::G; ++g) {
                     u64 kk[L::G][CL / 2];
                     form(g, kk);
+                    if constexpr (TM) {
+                        uint32_t w[32];
 #pragma unroll
-                    for (int r = 0; r < L::G; ++r)
+                        for (int r = 0; r < L::G; ++r)
 #pragma unroll
-                        for (int h = 0; h < CL / 2; ++h) K[g * L::G + r][h] = kk[r][h];
+                            for (int h = 0; h < CL / 2; ++h) {
+                                float k0, k1;
+                                unpack2(kk[r][h], k0, k1);
+                                w[r * CL + 2 * h] = __float_as_uint(k0); w[r * CL + 2 * h + 1] = __float_as_uint(k1);
+                            }
+                        tc_st32_issue(tk + (uint32_t)g * 32u, w);
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < L::G; ++r)
+#pragma unroll
+                            for (int h = 0; h < CL / 2; ++h) kstage[((g * L::G + r) * (CL / 2) + h) * THREADS + tid] = kk[r][h];
+                    }
+                }
+                if constexpr (TM) tc_st_wait();
+                else {
+#pragma unroll
+                    for (int r = 0; r < RW; ++r)
+#pragma unroll
+                        for (int h = 0; h < CL / 2; ++h) K[r][h] = kstage[(r * (CL / 2) + h) * THREADS + tid];
                 }
                 __syncthreads();
             }
@@ -627,20 +707,17 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                     float s[RW];
 #pragma unroll
                     for (int h = 0; h < CL / 2; ++h) v[h] = *reinterpret_cast<const u64 *>(vs + h * 64 + 2 * lane);
-#pragma unroll
-                    for (int r = 0; r < RW; r += L::G) {
-                        u64 kk[L::G][CL / 2];
-                        if constexpr (LEG) form(r / L::G, kk);
+                    each_rows([&](const int r, const u64 (&kk)[L::G][CL / 2]) {
 #pragma unroll
                         for (int q = 0; q < L::G; ++q) {
-                            u64 t = mul2(LEG ? kk[q][0] : K[LEG ? 0 : r + q][0], v[0]);
+                            u64 t = mul2(kk[q][0], v[0]);
 #pragma unroll
-                            for (int h = 1; h < CL / 2; ++h) t = fma2(LEG ? kk[q][h] : K[LEG ? 0 : r + q][h], v[h], t);
+                            for (int h = 1; h < CL / 2; ++h) t = fma2(kk[q][h], v[h], t);
                             float s0, s1;
                             unpack2(t, s0, s1);
                             s[r + q] = s0 + s1;
                         }
-                    }
+                    });
                     const double S = row_exchange<CL, L::FP32_COLS, true, 16, RW, float>(s, lane);
                     unew = rok ? rcp64(S) : 1.0;
                     const double term = rown ? a_fix * fabs(fma(us, S, -1.0)) : 0.0;
@@ -1032,23 +1109,30 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
             }
         }
     }
+    if constexpr (TM) {
+        tc_fence_before();
+        __syncthreads();
+        if (warp == 0) { tc_fence_after(); tc_dealloc<L::TM_COLS>(tm_holder); }
+    }
     if constexpr (CLU) cluster_sync_all();               // no block leaves while another may still write into its memory
 }
 
 // ---------------------------------------------------------------- host side
+constexpr int SMEM_PER_SM = 226 << 10;                   // shared by the blocks of an SM (each is charged 1 KB more)
 struct ScalingVariant {
     int threads, cols, rb;
     bool cluster;                                        // lanes of several blocks
     const void *kernel[3];                               // by ScalingKind
+    int tm_cols;                                         // tensor memory columns (0: K in registers)
     size_t (*smem)(int nc);
 };
-#define SKB_SC(NW, CL, RW, CLU) { 32 * NW, 32 * CL, NW * RW, CLU, {(const void *)&scaling_kernel<NW, CL, RW, CLU, SC_CYCLES>, (const void *)&scaling_kernel<NW, CL, RW, CLU, SC_CATCH_UP>, (const void *)&scaling_kernel<NW, CL, RW, CLU, SC_LEG>}, &ScalingShape<NW, CL, RW>::smem }
+#define SKB_SC(NW, CL, RW, CLU, TM) { 32 * NW, 32 * CL, NW * RW, CLU, {(const void *)&scaling_kernel<NW, CL, RW, CLU, TM, SC_CYCLES>, (const void *)&scaling_kernel<NW, CL, RW, CLU, TM, SC_CATCH_UP>, (const void *)&scaling_kernel<NW, CL, RW, CLU, TM, SC_LEG>}, TM ? ScalingShape<NW, CL, RW, TM>::TM_COLS : 0, &ScalingShape<NW, CL, RW, TM>::smem }
 // narrowest column count first, then fewest rows per block
 static const ScalingVariant g_scaling[] = {
-    SKB_SC(2, 2, 8, false), SKB_SC(4, 2, 16, false), SKB_SC(4, 2, 32, false), SKB_SC(4, 2, 32, true),
-    SKB_SC(4, 4, 16, false), SKB_SC(4, 4, 32, false), SKB_SC(4, 4, 32, true),
-    SKB_SC(4, 8, 16, false), SKB_SC(4, 8, 16, true),
-    SKB_SC(8, 16, 8, true),
+    SKB_SC(2, 2, 8, false, false), SKB_SC(4, 2, 16, false, false), SKB_SC(4, 2, 32, false, false), SKB_SC(4, 2, 32, true, false),
+    SKB_SC(4, 4, 16, false, false), SKB_SC(4, 4, 32, false, false), SKB_SC(4, 4, 32, true, false),
+    SKB_SC(4, 8, 16, false, false), SKB_SC(8, 8, 16, false, true), SKB_SC(8, 8, 32, false, true), SKB_SC(4, 8, 16, true, false),
+    SKB_SC(8, 16, 16, true, true),
 };
 
 // The variant of a lane shape: the narrowest column tile that holds the columns; of its row tiles the
@@ -1074,10 +1158,19 @@ void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int wid
     const ScalingVariant *v = scaling_variant(P.n, P.m);
     const void *kernel = v->kernel[kind];
     const int nc = (P.n + v->rb - 1) / v->rb;
-    const size_t smem = v->smem(nc);
+    // Blocks that use tensor memory ask for shared memory too: in clusters in proportion, so that the blocks that fit
+    // an SM together have their tensor memory and no block waits for an allocation while its peers hold
+    // theirs; by themselves as much as keeps one block too many away (the rest is cache for the formation of K).
+    size_t smem = v->smem(nc);
+    if (v->tm_cols && kind != SC_LEG) {
+        cudaFuncAttributes fa;
+        if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;        // (the caller looks at cudaGetLastError)
+        const size_t share = v->cluster ? (size_t)SMEM_PER_SM * v->tm_cols / 512 : (size_t)SMEM_PER_SM / (512 / v->tm_cols + 1) + 1024;
+        if (share > fa.sharedSizeBytes + smem) smem = share - fa.sharedSizeBytes;
+    }
     // (with the fixed arrays some variants are beyond the 48 KB that need no permission; the attribute belongs
     // to the current device, so it is set with every launch)
-    if (v->cluster) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nc, width < 1 ? 1 : width);
     cfg.blockDim = dim3(v->threads);
