@@ -560,7 +560,7 @@ static void enqueue_cycles_launch(skb_batch *h, int cycles)
     else h->var->launch_cycles(h->dev, cycles, w, h->stream);
     int nk = 1;
     nk += launch_plan_cycles(h->dev, w, cycles, h->stream);
-    nk += launch_emit_move(h->dev, w, h->stream);
+    if (h->cfg.mode == SKB_ACTIVE) nk += launch_emit_move(h->dev, w, h->stream);       // (under a mask nothing moves)
     h->enqueued += cycles;
     h->launches += nk;
 }
@@ -672,15 +672,17 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
         skb_status st0 = poll_snapshot(h, true);
         if (st0 != SKB_OK) { cudaStreamSynchronize(h->stream); return st0; }
     }
-    // lanes that finish inside a launch leave it, so a long first launch costs nothing; on the scaling
-    // kernel it saves forming the kernel matrices again
-    int chunk = h->dev.phi0 && cycles_in_one_launch(h) ? 16 : 2, snap = 0, rounds = 0;
+    // Lanes of the scaling kernel that finish inside a launch leave it (STATIC: wait for the second half), so the longest
+    // launch costs nothing and saves forming the kernel matrices again; a mask's lanes work on until the launch
+    // ends, so its launches grow with what has been done and overshoot by an eighth at most.
+    const bool scaling = h->dev.phi0 && cycles_in_one_launch(h), masked = h->cfg.mode == SKB_MASKED;
+    int chunk = scaling ? (masked ? 16 : MAX_CYCLES_IN_LAUNCH) : 2, snap = 0, rounds = 0;
     bool have_prev = false;
     // every lane is retired by the audit that follows cycle max_iter; STATIC needs one more pass
     const long long hard_cap = (long long)h->cfg.max_iter + 4;
     while (!h->finished) {
         const bool multi = cycles_in_one_launch(h);      // may become true as the batch narrows
-        const int chunk_max = h->dev.phi0 && multi ? (h->cfg.mode == SKB_MASKED || h->cfg.mode == SKB_MASKED_EXIT ? 64 : MAX_CYCLES_IN_LAUNCH) : (multi ? 32 : 16);
+        const int chunk_max = scaling ? (masked ? 256 : MAX_CYCLES_IN_LAUNCH) : (multi ? 32 : 16);
         NvtxRange nvtx_chunk(multi ? "skb:chunk (cycles in one launch)" : "skb:chunk (launch per leg)");
         if (multi) enqueue_cycles_launch(h, chunk);
         else for (int i = 0; i < chunk; ++i) enqueue_cycle(h);
@@ -697,7 +699,7 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
         snap ^= 1;
         // grow the chunk every other round: cycles enqueued past completion are empty launches that
         // still have to drain, which matters for batches that finish within a dozen cycles
-        if (chunk < chunk_max && (++rounds & 1) == 0) chunk *= 2;
+        if (chunk < chunk_max && (scaling ? h->enqueued - h->enqueued_at_refill >= 16 * chunk : (++rounds & 1) == 0)) chunk *= 2;
         if (h->enqueued - h->enqueued_at_refill > hard_cap + 64 + 2 * MAX_CYCLES_IN_LAUNCH) break;
     }
     if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "drain");

@@ -476,19 +476,20 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
 {
     __shared__ int wsum[PLAN_THREADS / 32][3];
     __shared__ int left_at[MAX_CYCLES_IN_LAUNCH];   // lanes that left at the audit of the state after k0 + j cycles
-    __shared__ int checks_s;
+    __shared__ int checks_s, nret_s, last_s, ran_s;
+    __shared__ unsigned long long slots_s, terms_s;
     pdl_enter();
     const Ctl c = *P.ctl;
     const int tid = threadIdx.x, NT = blockDim.x;
     if (c.done) { if (tid == 0) P.ctl->n_retire = 0; return; }
     const int k0 = c.cycle, A = c.n_phys;
     for (int j = tid; j < K; j += NT) left_at[j] = 0;
-    if (tid == 0) checks_s = 0;
+    if (tid == 0) { checks_s = nret_s = ran_s = 0; last_s = 0; slots_s = terms_s = 0ull; }
     __syncthreads();
     int nchk = 0;
     for (int s = tid; s < A; s += NT) {
         const int r = P.ret_at[s];
-        if (r > 0) atomicAdd(&left_at[r - 1 - k0], 1);
+        if (r > 0) { atomicAdd(&left_at[r - 1 - k0], 1); atomicAdd(&nret_s, 1); atomicMax(&last_s, r - 1 - k0); }
         nchk += P.n_checks[s];
         P.rsum_row[s] = 0ull; P.rsum_col[s] = 0ull;      // between launches the residual sums are zero
         P.rsum_row64[s] = 0ull; P.esc[s] = 0;
@@ -496,8 +497,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
     for (int off = 16; off > 0; off >>= 1) nchk += __shfl_down_sync(0xffffffffu, nchk, off);
     if ((tid & 31) == 0 && nchk) atomicAdd(&checks_s, nchk);
     __syncthreads();
-    int nret = 0;
-    for (int j = 0; j < K; ++j) nret += left_at[j];
+    const int nret = nret_s;
     const bool compact = P.mode == MODE_ACTIVE;      // MASKED: lanes stay where they are, frozen or not
     const int Anew = compact ? A - nret : A;
     const int parity_new = c.parity ^ (K & 1);       // survivors ran all K cycles
@@ -531,8 +531,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
     }
     // the audit that counts as the most recent one: the launch's last, or the one at which the last lane left.  A lane
     // that froze at that very audit shows what it was decided from; one that froze before shows a frozen lane's values
-    int jl = K - 1;
-    if (nret == c.n_running) while (jl > 0 && left_at[jl] == 0) --jl;
+    const int jl = nret == c.n_running ? last_s : K - 1;
     for (int s = tid; s < A; s += NT) {
         if (P.mode == MODE_MASKED) {
             const int r = P.ret_at[s];
@@ -545,22 +544,38 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
         }
         P.ret_at[s] = 0; P.n_checks[s] = 0;
     }
-    if (tid == 0) {
-        Ctl *g = P.ctl;
-        const long long nm = (long long)P.n * P.m;
-        long long slots = 0, terms = (long long)checks_s * nm;
-        int w = c.n_running, ran = 0;                // running lanes; the launch's width is theirs, or W under a mask
+    // The widths of the launch's cycles and what they add up to: every thread takes a run of consecutive cycles, the
+    // lanes that left before it from a scan over the threads.
+    {
         const bool full = P.mode == MODE_MASKED && !P.early_exit;
-        for (int j = 0; j < K; ++j) {
-            terms += (long long)(full ? A : w) * nm; // the f-leg whose epilogue screened the state after k0 + j cycles
+        const int per = (K + NT - 1) / NT, j0 = tid * per, j1 = min(K, j0 + per);
+        int mine = 0;
+        for (int j = j0; j < j1; ++j) mine += left_at[j];
+        int incl = mine;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) { const int o = __shfl_up_sync(0xffffffffu, incl, off); if ((tid & 31) >= off) incl += o; }
+        if ((tid & 31) == 31) wsum[tid >> 5][0] = incl;
+        __syncthreads();
+        int w = c.n_running - (incl - mine), ran = 0;   // running lanes before cycle k0 + j0
+        for (int e = 0; e < (tid >> 5); ++e) w -= wsum[e][0];
+        unsigned long long slots = 0ull, legs = 0ull;
+        for (int j = j0; j < j1 && w > 0; ++j) {
+            legs += full ? A : w;                        // the f-leg whose epilogue screened the state after k0 + j cycles
             w -= left_at[j];
             if (w == 0) break;
-            const int width = full ? A : w;
+            const int width = full ? A : w;              // the launch's width is the running lanes', or W under a mask
             if (k0 + j < P.widths_cap) P.widths[k0 + j] = width;      // cycle k0 + j + 1 ran at this width
             slots += width;
-            terms += (long long)width * nm;          // its g-leg
+            legs += width;                               // its g-leg
             ++ran;
         }
+        if (legs) { atomicAdd(&slots_s, slots); atomicAdd(&terms_s, legs); atomicAdd(&ran_s, ran); }
+        __syncthreads();
+    }
+    if (tid == 0) {
+        Ctl *g = P.ctl;
+        const long long nm = (long long)P.n * P.m, slots = (long long)slots_s, terms = ((long long)terms_s + checks_s) * nm;
+        const int ran = ran_s;
         g->cycle = k0 + ran;
         g->parity = parity_new;
         g->emit_parity = parity_new ^ 1;             // the move copies the OTHER buffer: the survivors' current row potentials

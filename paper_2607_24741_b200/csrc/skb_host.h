@@ -44,7 +44,9 @@ struct Variant {
     bool (*lane_fits_shared)(int n, int m);
 };
 constexpr int MAX_CLUSTER_BLOCKS = MAX_CLUSTER_RANKS;   // a lane needs at most this many row blocks
-constexpr int MAX_CYCLES_IN_LAUNCH = 256;   // upper bound on the cycles one multi-cycle launch runs
+// Upper bound on the cycles one multi-cycle launch runs.  Lanes are independent and leave a launch when they pass, so a
+// long launch keeps the SMs full where a series of short ones waits for its slowest lanes after each.
+constexpr int MAX_CYCLES_IN_LAUNCH = 2048;
 // Picks the variant for a shape (depends on the static shape only, so that every mode
 // and every run of the same batch uses the same reduction order).  Null if unsupported.
 const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_exp, int force_cs, bool spatial);
