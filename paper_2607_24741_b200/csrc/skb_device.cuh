@@ -161,8 +161,8 @@ __device__ __forceinline__ bool in_guard_band(const Dev &P, const double rr)
 // One row's term |sum_j pi_ij - a_i| of the row residual (Eq. 5), from the raw inputs and the
 // float64 potentials, float64 throughout (difference-form cost, software exp2): the plain
 // definition, independent of the update kernels' layouts and arithmetic.  One WARP per row: lane l
-// takes the columns l, l + 32, ... with its own running maximum and sum, and the 32 pairs are merged
-// by xor-shuffles (every lane returns the term).  phi: the row's potential (log2 units); the column
+// takes the columns l, l + 32, ... with its own sum, and the 32 are added by xor-shuffles (every lane returns the term).
+// (With a running maximum, the merge was a chain of ten exponentials per row.)  phi: the row's potential (log2 units); the column
 // potentials are read from global memory past L1, because inside a multi-cycle launch other blocks of
 // the cluster have written them.
 template <bool VEC = false>
@@ -174,7 +174,7 @@ __device__ __forceinline__ double direct_row_term_warp(const Dev &P, const int s
     const void *xl = (const char *)P.xraw + (size_t)slot * P.xraw_stride;
     const void *yl = (const char *)P.yraw + (size_t)slot * P.yraw_stride;
     const size_t xb = (size_t)i * P.d;
-    double mx = -1.0e300, sum = 0.0;
+    double sum = 0.0;
     // four columns per lane and step: their cost chains and exponentials are independent, which is
     // what keeps the float64 pipe busy at the few warps an escalation runs on
     constexpr int U = 4;
@@ -219,27 +219,17 @@ __device__ __forceinline__ double direct_row_term_warp(const Dev &P, const int s
                 }
             }
         }
-        double v[U], mn = mx;
+        // entries of the plan: at most a weight where a g-leg has been taken, so the exponentials need no shift (a proposal
+        // whose entries leave the range has an infinite sum, which marks the lane)
+        double v[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            v[u] = (j0 + 32 * u < P.m) ? phi + gj[u] - s * c[u] : -1.0e300;
-            mn = fmax(mn, v[u]);
-        }
-        double add = 0.0;
+        for (int u = 0; u < U; ++u) v[u] = exp2(phi + gj[u] - s * c[u]);
 #pragma unroll
-        for (int u = 0; u < U; ++u) add += (j0 + 32 * u < P.m) ? exp2(v[u] - mn) : 0.0;
-        sum = sum * exp2(mx - mn) + add;
-        mx = mn;
+        for (int u = 0; u < U; ++u) sum += (j0 + 32 * u < P.m) ? v[u] : 0.0;
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const double mo = __shfl_xor_sync(0xffffffffu, mx, off);
-        const double so = __shfl_xor_sync(0xffffffffu, sum, off);
-        const double mn = fmax(mx, mo);
-        sum = sum * exp2(mx - mn) + so * exp2(mo - mn);      // a lane without columns carries (-1e300, 0): its factor underflows to 0
-        mx = mn;
-    }
-    return fabs(exp2(mx) * sum - P.wa[(size_t)slot * P.np + i]);
+    for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    return fabs(sum - P.wa[(size_t)slot * P.np + i]);
 }
 
 // Rows of a lane for one block of NW warps, one warp per row: warp w takes the rows row_first + w,
