@@ -29,6 +29,8 @@ struct skb_batch {
     long long launches;    // kernels launched so far
     int res_device;        // device the pooled host resources belong to
     bool tensor;           // the tensor-core update kernel is in use
+    const Variant *var_stream;   // the streaming kernels' variant of lanes that run on chip instead
+    bool f32_on_chip;      // lanes for which fp32 is enough, with their kernel matrix on chip (formed in float64)
     bool snap_pending;     // step() left a control-block snapshot in flight (ev[snap_idx])
     int snap_idx;
     // phase timing (Eq. 11's cost record): off unless sinkhorn_batch_set_profiling turned it on
@@ -118,6 +120,10 @@ static const double NEAR_SHARE = 0.75;
 // the rounding of its expanded cost, 1.2e-6 on the registration workload at tol 1e-2, and callers hold such results to
 // 1e-6 of earlier ones.  It costs those solves the 624 against 212 us a leg.
 static const double SPATIAL_TOL = 2.0e-3;
+
+// Deep lanes keep their dot products in the workspace and their kernel matrix on chip, up to this size of the
+// products (1024 lanes of 1024 x 1024, 2 % of the card's memory); wider batches form the products in every leg.
+static const size_t DOTS_LIMIT = (size_t)4 << 30;
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -229,7 +235,11 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
         d.boxx = (float *)take(W * 2 * DP * d.nbx * 4); d.boxy = (float *)take(W * 2 * DP * d.nby * 4);
         d.topx[0] = (float *)take(W * d.nbx * 4); d.topx[1] = (float *)take(W * d.nbx * 4); d.topy = (float *)take(W * d.nby * 4);
     }
-    if (var->xf && var->DP && scaling_fits(c->n, c->m)) {
+    if (tensor && scaling_fits(true, c->n, c->m) && W * np * mp * 4 <= DOTS_LIMIT) {
+        d.phi0 = (double *)take(W * np * 8); d.uu[0] = (double *)take(W * np * 8); d.uu[1] = (double *)take(W * np * 8);
+        d.gam0 = (double *)take(W * mp * 8); d.vv = (double *)take(W * mp * 8);
+        d.dots = (float *)take(W * np * mp * 4);
+    } else if (var->xf && var->DP && scaling_fits(false, c->n, c->m)) {
         // (these lanes have no streamed terms: what the set-up kernels write there is not read)
         d.phi0 = (double *)d.ft[0]; d.uu[0] = (double *)d.ft[1]; d.uu[1] = (double *)d.fl[0];
         d.gam0 = (double *)d.gt; d.vv = (double *)d.gl;
@@ -328,7 +338,7 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     h->cfg = *cfg; h->var = var; h->stream = (cudaStream_t)cfg->stream;
     h->known_width = cfg->W; h->finished = false; h->enqueued = 0; h->launches = 0; h->h_ctl = nullptr;
     h->ev[0] = h->ev[1] = nullptr;
-    h->tensor = cfg->compute == SKB_COMPUTE_TENSOR;
+    h->tensor = cfg->compute == SKB_COMPUTE_TENSOR; h->f32_on_chip = false; h->var_stream = var;
     h->snap_pending = false; h->snap_idx = 0; h->profiling = false; h->pev_used = 0; h->no_multi_cycle = false;
     h->lanes_used = cfg->W; h->enqueued_at_refill = 0;
     for (int i = 0; i < SKB_N_PHASES; ++i) h->phase_ms[i] = 0.f;
@@ -375,7 +385,12 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
         double radius;
         memcpy(&radius, &h->h_ctl[1].max_radius_bits, sizeof(double));
         const double ts = h->dev.tol_stop, tsc = h->dev.tol_screen;
-        if (automatic && radius > mixed_radius(ts < tsc ? ts : tsc)) {
+        const bool wide_radius = radius > mixed_radius(ts < tsc ? ts : tsc);
+        // fp32 lanes that fit on chip: the matrix is formed once, so its exponents can as well be float64.  Not where the
+        // caller names a form of the cost or a column split, which only the streaming kernels have.
+        h->f32_on_chip = automatic && !wide_radius && !can_tensor && var_big->xf && var_big->DP && scaling_fits(false, cfg->n, cfg->m) &&
+                         cfg->cost_form == 0 && cfg->column_split == 0;
+        if (automatic && (wide_radius || h->f32_on_chip)) {
             h->var = var_big;
             carve(cfg, var_big, false, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
         } else if (automatic && can_tensor) {
@@ -404,6 +419,7 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     }
     if (h->dev.permx) { launch_spatial_sort(h->dev, x, y, 0, cfg->W, h->stream); h->launches += 1; }
     launch_prep(h->dev, x, y, a, b, 0, cfg->W, h->stream);
+    if (h->dev.dots) { launch_gram(h->dev, h->maps, 0, cfg->W, h->stream); h->launches += 1; }
     if (h->dev.guard > 0.0 && !h->dev.permx) {            // (lanes in spatial order: the layout kernel writes them)
         const size_t es = cfg->xy_dtype == SKB_BF16 ? 2 : 4;
         const size_t xb = (size_t)cfg->n * cfg->d * es, yb = (size_t)cfg->m * cfg->d * es;
@@ -480,6 +496,7 @@ extern "C" skb_status sinkhorn_batch_refill(skb_batch *h, const void *x, const v
     }
     if (D.permx) { launch_spatial_sort(D, x, y, width, count, h->stream); h->launches += 1; }
     launch_prep(D, x, y, a, b, width, count, h->stream);
+    if (D.dots) { launch_gram(D, h->maps, width, count, h->stream); h->launches += 1; }
     if (D.guard > 0.0 && !D.permx) {
         const size_t xb = (size_t)h->cfg.n * h->cfg.d * es, yb = (size_t)h->cfg.m * h->cfg.d * es;
         e = cudaMemcpy2DAsync((char *)D.xraw + (size_t)width * D.xraw_stride, D.xraw_stride, x, xb, xb, count, cudaMemcpyDeviceToDevice, h->stream);
@@ -518,8 +535,8 @@ extern "C" skb_status sinkhorn_batch_set_profiling(skb_batch *h, int on)
 // Returns 1 if a column-check launch carried the guard band's pool.
 static int launch_leg(skb_batch *h, int leg, int w)
 {
-    if (h->tensor) { launch_update_tc(h->dev, h->maps, leg, w, h->stream); return 0; }
     if (h->dev.phi0) { launch_scaling(h->dev, SC_LEG, leg, 0, w, h->stream); return 0; }
+    if (h->tensor) { launch_update_tc(h->dev, h->maps, leg, w, h->stream); return 0; }
     if (h->dev.permx) return launch_near(h->dev, leg, w, h->stream);
     return h->var->launch(h->dev, leg, w, h->stream);
 }
@@ -528,19 +545,22 @@ static int launch_leg(skb_batch *h, int leg, int w)
 // per lane (scaling_kernel, lane_resident_kernel or lane_cycles_kernel), followed by one planner for all
 // of them.  A mask can be kept inside such a launch by the scaling kernel only, and only that one can run STATIC
 // batches so: the cycle at which all of their lanes stop is not known beforehand (plan_static_kernel).
+static bool narrow_lanes(const skb_batch *h, const Variant *var)
+{
+    const int mx = h->cfg.n > h->cfg.m ? h->cfg.n : h->cfg.m;
+    const int nc = (mx + var->rows_per_cta - 1) / var->rows_per_cta;
+    if (nc > MAX_CLUSTER_BLOCKS) return false;
+    // Lanes too large for shared memory run the streaming version, which is worth it once the batch is
+    // down to about one wave of blocks (it saves launches, not traffic); a wide batch of such lanes is
+    // better served by one launch per leg (256 lanes of 512 x 512, d = 15: 1.12 against 1.20 ms per solve).
+    return var->lane_fits_shared(h->cfg.n, h->cfg.m) || (long long)h->known_width * nc <= 148 * 4;
+}
 static bool cycles_in_one_launch(const skb_batch *h)
 {
     if (h->dev.phi0) return !h->profiling && !h->no_multi_cycle;
     if (h->cfg.mode != SKB_ACTIVE || h->tensor || h->profiling || !h->var->launch_cycles || h->no_multi_cycle) return false;
     if (h->dev.permx) return false;
-    const int mx = h->cfg.n > h->cfg.m ? h->cfg.n : h->cfg.m;
-    const int nc = (mx + h->var->rows_per_cta - 1) / h->var->rows_per_cta;
-    if (nc > MAX_CLUSTER_BLOCKS) return false;
-    // Lanes too large for shared memory run the streaming version, which is worth it once the batch is
-    // down to about one wave of blocks (it saves launches, not traffic); a wide batch of such lanes is
-    // better served by one launch per leg (sensor at 256 lanes: 1.12 against 1.20 ms per solve).
-    if (!h->var->lane_fits_shared(h->cfg.n, h->cfg.m) && (long long)h->known_width * nc > 148 * 4) return false;
-    return true;
+    return narrow_lanes(h, h->var);
 }
 
 // `cycles` cycles in one launch (1 <= cycles <= MAX_CYCLES_IN_LAUNCH): lanes that pass inside it write their own
@@ -783,7 +803,9 @@ extern "C" skb_status sinkhorn_batch_apply_plan(skb_batch *h, const void *x, con
 extern "C" skb_status sinkhorn_batch_last_audit(skb_batch *h, float *r_row, float *r_col, int *flagged)
 {
     if (!h) return SKB_ERR_NULL;
-    if (cycles_in_one_launch(h) && h->cfg.mode == SKB_ACTIVE) return fail(h, SKB_ERR_STATE, "per-audit values are kept by the one-launch-per-leg path only (MASKED, STATIC, tensor or profiled batches)");
+    // (lanes that the streaming kernels would run a leg at a time have them on chip too: the planner moves them along)
+    const bool streamed = h->tensor || (h->f32_on_chip && !narrow_lanes(h, h->var_stream));
+    if (cycles_in_one_launch(h) && h->cfg.mode == SKB_ACTIVE && !streamed) return fail(h, SKB_ERR_STATE, "per-audit values are kept by the one-launch-per-leg path only (MASKED, STATIC, tensor or profiled batches)");
     launch_gather_audit(h->dev, r_row, r_col, flagged, h->stream);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? SKB_OK : cuda_fail(h, e, "last_audit");
@@ -830,7 +852,7 @@ extern "C" skb_status sinkhorn_batch_cycle_trace(skb_batch *h, float *update_ms,
 extern "C" skb_status sinkhorn_batch_arithmetic(skb_batch *h, int *compute)
 {
     if (!h || !compute) return SKB_ERR_NULL;
-    *compute = h->tensor ? SKB_COMPUTE_TENSOR : (!h->var->f64 ? SKB_COMPUTE_F32 : (h->var->xf ? SKB_COMPUTE_MIXED : SKB_COMPUTE_F64));
+    *compute = h->tensor ? SKB_COMPUTE_TENSOR : (h->f32_on_chip || !h->var->f64 ? SKB_COMPUTE_F32 : (h->var->xf ? SKB_COMPUTE_MIXED : SKB_COMPUTE_F64));
     return SKB_OK;
 }
 

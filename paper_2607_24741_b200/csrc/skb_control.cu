@@ -41,7 +41,7 @@ __device__ __forceinline__ void lane_enters(const Dev &P, const float *eps, cons
     P.nonfinite[slot] = 0; P.state[slot] = 0; P.flag[slot] = 0; P.verdict[slot] = 0;
     P.rsum_row[slot] = 0ull; P.rsum_col[slot] = 0ull; P.rsum_row64[slot] = 0ull; P.esc[slot] = 0;
     P.ret_at[slot] = 0; P.n_checks[slot] = 0;
-    P.absorbed[slot] = 0; P.cyc_log[slot] = 0;
+    P.absorbed[slot] = eps_ok && 4.0 * s * r2 <= SC_COLD_BITS; P.cyc_log[slot] = 0;
     // (lanes in spatial order have a form of their own, which shares the expanded form's scale and terms)
     int form = P.permx ? FORM_DOT : P.cost_form == 1 ? FORM_DOT : (P.cost_form == 2 ? FORM_DIFF : (s * r2 > P.form_threshold ? FORM_DIFF : FORM_DOT));
     P.form[slot] = form;
@@ -98,53 +98,87 @@ __global__ void __launch_bounds__(256) lane_stats_kernel(const Dev P, const void
     }
 }
 
-// Deep lanes (32 < d <= 1024): a warp takes 32 dimensions of a share of the points, so rows are read in whole
-// sectors; then a warp per point for the distances.  (One dimension after the other read two bytes of every row
-// per pass: create took 1865 us on the 64 lanes of the feature workload, d = 512, and takes 858 us with this and prep_tensor_kernel.)
-__global__ void __launch_bounds__(1024) lane_stats_deep_kernel(const Dev P, const void *xin, const void *yin, const float *eps,
-                                                               const int slot0, const int lane0, const int cycle0)
+// Deep lanes (32 < d <= 1024): a cluster of blocks per lane, each with a share of the points.  A warp reads 256 dimensions of
+// a row at a time (whole sectors) and keeps a sum per dimension; the blocks read each other's sums through shared
+// memory, in block order.  Then a warp per point for the distances.  (One block per lane read 134 MB of the feature
+// workload - 64 lanes of 1024 x 1024, d = 512 - from 64 SMs: 713 us.)
+constexpr int STATS_BLOCKS = 8, STATS_WARPS = 8;
+__global__ void __cluster_dims__(STATS_BLOCKS, 1, 1) __launch_bounds__(32 * STATS_WARPS)
+lane_stats_deep_kernel(const Dev P, const void *xin, const void *yin, const float *eps, const int slot0, const int lane0, const int cycle0)
 {
-    __shared__ double part[1024];                         // [share][dimension], then the warps' maxima
-    __shared__ double cen[1024];
-    const int q = blockIdx.x, slot = slot0 + q, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int tot = P.n + P.m, groups = (P.d + 31) / 32, shares = 32 / groups;
-    if (warp < groups * shares) {
-        const int k = (warp % groups) * 32 + lane, first = warp / groups;
-        const int kc = k < P.d ? k : P.d - 1;
-        double s = 0.0;
-#pragma unroll 8
-        for (int p = first; p < tot; p += shares) {
-            const bool isx = p < P.n;
-            s += (double)load_raw(P, isx ? xin : yin, (isx ? (size_t)q * P.n + p : (size_t)q * P.m + (p - P.n)) * P.d + kc);
+    __shared__ double part[STATS_WARPS][256];
+    __shared__ double sums[1024], cen[1024], far[1];
+    const int q = blockIdx.y, slot = slot0 + q, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x;
+    const int tot = P.n + P.m, per = (tot + STATS_BLOCKS - 1) / STATS_BLOCKS, p0 = b * per, p1 = min(tot, p0 + per);
+    auto row = [&](const int p, const void *&base) -> size_t {
+        const bool isx = p < P.n;
+        base = isx ? xin : yin;
+        return (isx ? (size_t)q * P.n + p : (size_t)q * P.m + (p - P.n)) * P.d;
+    };
+    for (int k0 = 0; k0 < P.d; k0 += 256) {
+        double s[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e] = 0.0;
+#pragma unroll 2
+        for (int p = p0 + warp; p < p1; p += STATS_WARPS) {
+            const void *base;
+            const size_t o = row(p, base);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int k = k0 + 32 * e + lane;
+                if (k < P.d) s[e] += (double)load_raw(P, base, o + k);
+            }
         }
-        part[first * groups * 32 + k] = s;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) part[warp][32 * e + lane] = s[e];
+        __syncthreads();
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < STATS_WARPS; ++w) t += part[w][tid];
+        if (k0 + tid < P.d) sums[k0 + tid] = t;
+        __syncthreads();
     }
-    __syncthreads();
-    if (tid < P.d) {
-        double s = 0.0;
-        for (int h = 0; h < shares; ++h) s += part[h * groups * 32 + tid];
-        cen[tid] = s / (double)tot;
+    cluster_sync_all();
+    for (int k = tid; k < P.d; k += 32 * STATS_WARPS) {
+        double t = 0.0;
+#pragma unroll
+        for (int r = 0; r < STATS_BLOCKS; ++r) t += ld_cluster(&sums[k], r);
+        cen[k] = t / (double)tot;
     }
     __syncthreads();
     double mxr = 0.0;
 #pragma unroll 2
-    for (int p = warp; p < tot; p += 32) {
-        const bool isx = p < P.n;
-        const size_t base = (isx ? (size_t)q * P.n + p : (size_t)q * P.m + (p - P.n)) * P.d;
+    for (int p = p0 + warp; p < p1; p += STATS_WARPS) {
+        const void *base;
+        const size_t o = row(p, base);
         double r2 = 0.0;
-#pragma unroll 4
-        for (int k = lane; k < P.d; k += 32) { const double v = (double)load_raw(P, isx ? xin : yin, base + k) - cen[k]; r2 = fma(v, v, r2); }
+#pragma unroll 8
+        for (int k = lane; k < P.d; k += 32) { const double v = (double)load_raw(P, base, o + k) - cen[k]; r2 = fma(v, v, r2); }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, off);
         mxr = fmax(mxr, r2);
     }
-    if (lane == 0) part[warp] = mxr;
+    if (lane == 0) part[0][warp] = mxr;
     __syncthreads();
-    for (int k = tid; k < P.DP; k += 1024) P.center[(size_t)slot * P.DP + k] = k < P.d ? cen[k] : 0.0;
     if (tid == 0) {
-        for (int w = 0; w < 32; ++w) mxr = fmax(mxr, part[w]);
+        for (int w = 1; w < STATS_WARPS; ++w) mxr = fmax(mxr, part[0][w]);
+        far[0] = mxr;
+    }
+    if (b == 0) for (int k = tid; k < P.DP; k += 32 * STATS_WARPS) P.center[(size_t)slot * P.DP + k] = k < P.d ? cen[k] : 0.0;
+    cluster_sync_all();
+    if (b == 0 && tid == 0) {
+        for (int r = 1; r < STATS_BLOCKS; ++r) mxr = fmax(mxr, ld_cluster(&far[0], r));
         lane_enters(P, eps, q, slot, lane0, cycle0, mxr);
     }
+    cluster_sync_all();                                   // nobody's sums go while another may read them
+}
+
+// Zero potentials absorbed, scalings 1 (arrays that share memory with the streamed terms are written after those).
+__device__ __forceinline__ void cold_scalings(const Dev &P, const int side, const size_t o)
+{
+    if (!P.phi0) return;
+    if (side) { P.gam0[o] = 0.0; P.vv[o] = 1.0; }
+    else { P.phi0[o] = 0.0; P.uu[0][o] = 1.0; P.uu[1][o] = 1.0; }
 }
 
 template <typename T>
@@ -190,7 +224,7 @@ __global__ void prep_kernel(const Dev P, const void *xin, const void *yin, const
         sq[o] = nrm;
         lw[o] = ok ? log2((double)w) : 0.0;
         wt[o] = ok ? (double)w : 0.0;
-        if (P.phi0 && ok && w < SC_MIN_WEIGHT) P.absorbed[slot] = SC_NO_MATRIX;      // (every writer stores the same value)
+        if (P.phi0 && ok && w < SC_COLD_WEIGHT) atomicMin(&P.absorbed[slot], w < SC_MIN_WEIGHT ? SC_NO_MATRIX : 0);
         hi = (T)(-nrm);                                // cold start: phi = gam = 0
     }
     hi0[o] = hi; lo0[o] = lo;
@@ -200,41 +234,51 @@ __global__ void prep_kernel(const Dev P, const void *xin, const void *yin, const
     } else {
         P.gam[o] = 0.0;
     }
+    cold_scalings(P, side, o);
 }
 
 // Layout of tensor-core lanes: their coordinates stay raw (the tiled bf16 copies), so a point leaves only its
-// scaled squared norm, weight and cold potentials here.  One warp per point reads its row in whole sectors.
+// scaled squared norm, weight and cold potentials here.  Eight threads per point, 64 dimensions in 16-byte pieces at a
+// time (d is a multiple of 64; with two-byte loads it took 65 us on the feature workload).
 __global__ void __launch_bounds__(256) prep_tensor_kernel(const Dev P, const void *xin, const void *yin, const float *a, const float *b, const int slot0)
 {
-    const int q = blockIdx.y, slot = slot0 + q, side = blockIdx.z, lane = threadIdx.x & 31;
+    const int q = blockIdx.y, slot = slot0 + q, side = blockIdx.z, sub = threadIdx.x & 7;
     const int npts = side ? P.m : P.n, pp = side ? P.mp : P.np;
-    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (i >= pp) return;
+    const int i = blockIdx.x * 32 + (threadIdx.x >> 3);
     const size_t o = (size_t)slot * pp + i;
     float hi = NEG_BIG;                                    // padding points
     double nrm = 0.0, lw = 0.0, wt = 0.0;
+    bool ok = true;
+    const double sc = sqrt(2.0 * P.scale[slot]);
     if (i < npts) {
-        const size_t ibase = ((size_t)q * npts + i) * P.d;
-        const double sc = sqrt(2.0 * P.scale[slot]);
-        bool ok = true;
+        const uint4 *src = reinterpret_cast<const uint4 *>(reinterpret_cast<const unsigned short *>(side ? yin : xin) + ((size_t)q * npts + i) * P.d) + sub;
 #pragma unroll 4
-        for (int k = lane; k < P.d; k += 32) {
-            const float raw = load_raw(P, side ? yin : xin, ibase + k);
-            ok = ok && isfinite(raw);
-            const double v = sc * (double)raw;
-            nrm = fma(v, v, nrm);
-        }
+        for (int k = 0; k < P.d / 64; ++k) {
+            const uint4 t = src[8 * k];
+            const unsigned w[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
+            for (int e = 0; e < 8; ++e) {
+                const float raw = __uint_as_float(e & 1 ? w[e / 2] & 0xffff0000u : w[e / 2] << 16);
+                ok = ok && isfinite(raw);
+                const double v = sc * (double)raw;
+                nrm = fma(v, v, nrm);
+            }
+        }
+    }
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
+    ok = (__ballot_sync(0xffffffffu, ok) >> (threadIdx.x & 24) & 0xffu) == 0xffu;
+    if (i >= pp || sub != 0) return;
+    if (i < npts) {
         nrm *= 0.5;
         const float w = (side ? b : a)[(size_t)q * npts + i];
-        ok = __all_sync(0xffffffffu, ok) && (w > 0.0f) && isfinite(w);
-        if (!ok && lane == 0) atomicOr(&P.ctl->error, ERR_VALUE);
+        ok = ok && (w > 0.0f) && isfinite(w);
+        if (!ok) atomicOr(&P.ctl->error, ERR_VALUE);
         lw = ok ? log2((double)w) : 0.0;
         wt = ok ? (double)w : 0.0;
+        if (P.phi0 && ok && w < SC_COLD_WEIGHT) atomicMin(&P.absorbed[slot], w < SC_MIN_WEIGHT ? SC_NO_MATRIX : 0);
         hi = (float)(-nrm);                                // cold start: phi = gam = 0
     }
-    if (lane != 0) return;
     (side ? P.sqy : P.sqx)[o] = nrm; (side ? P.lb2 : P.la2)[o] = lw; (side ? P.wb : P.wa)[o] = wt;
     if (side) {
         reinterpret_cast<float *>(P.gt)[o] = hi; reinterpret_cast<float *>(P.gl)[o] = 0.f; P.gam[o] = 0.0;
@@ -243,6 +287,7 @@ __global__ void __launch_bounds__(256) prep_tensor_kernel(const Dev P, const voi
             reinterpret_cast<float *>(P.ft[e])[o] = hi; reinterpret_cast<float *>(P.fl[e])[o] = 0.f; P.phi[e][o] = 0.0;
         }
     }
+    cold_scalings(P, side, o);
 }
 
 // Warm proposal: potentials in the caller's units -> the kernels' representation of both buffers
@@ -260,6 +305,7 @@ __global__ void warm_kernel(const Dev P, const double *f0, const double *g0)
     const int *perm = side ? P.permy : P.permx;
     const double v = src[(size_t)slot * npts + (perm ? perm[(size_t)P.lane_id[slot] * pp + i] : i)];
     if (!isfinite(v)) { atomicOr(&P.ctl->error, ERR_VALUE); return; }
+    if (P.phi0 && P.absorbed[slot] > 0) P.absorbed[slot] = 0;      // (every writer stores the same value)
     const int form = (sizeof(T) == 8) ? (int)FORM_DOT : P.form[slot];
     const size_t o = (size_t)slot * pp + i;
     const double pot = P.scale[slot] * v;
@@ -528,6 +574,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
         P.absorbed[dst] = P.absorbed[src];
         P.cyc_log[dst] = P.cyc_log[src];
         P.nonfinite[dst] = 0;
+        P.rrow[dst] = P.rrow[src]; P.rcol[dst] = P.rcol[src]; P.flag[dst] = P.flag[src];
     }
     // the audit that counts as the most recent one: the launch's last, or the one at which the last lane left.  A lane
     // that froze at that very audit shows what it was decided from; one that froze before shows a frozen lane's values
@@ -719,6 +766,7 @@ __device__ __forceinline__ void emit_move_one(const Dev &P, const Ctl &c, const 
         add(P.la2, (size_t)P.np * 8); add(P.lb2, (size_t)P.mp * 8);
         add(P.wa, (size_t)P.np * 8); add(P.wb, (size_t)P.mp * 8);
         add(P.phi[np_], (size_t)P.np * 8);
+        add(P.dots, (size_t)P.np * P.mp * 4);
         if (P.phi0) {                                                 // lanes on the scaling kernel have no streamed terms
             add(P.phi0, (size_t)P.np * 8); add(P.gam0, (size_t)P.mp * 8);
             add(P.uu[np_], (size_t)P.np * 8); add(P.vv, (size_t)P.mp * 8);
@@ -997,14 +1045,14 @@ void launch_lane_stats(const Dev &P, const void *x, const void *y, const float *
                        int cycle0, cudaStream_t st)
 {
     if (P.d <= 32) lane_stats_kernel<<<count, 256, 0, st>>>(P, x, y, eps, slot0, lane0, cycle0);
-    else lane_stats_deep_kernel<<<count, 1024, 0, st>>>(P, x, y, eps, slot0, lane0, cycle0);
+    else lane_stats_deep_kernel<<<dim3(STATS_BLOCKS, count), 32 * STATS_WARPS, 0, st>>>(P, x, y, eps, slot0, lane0, cycle0);
 }
 void launch_prep(const Dev &P, const void *x, const void *y, const float *a, const float *b, int slot0, int count, cudaStream_t st)
 {
     const int pp = P.np > P.mp ? P.np : P.mp;
     dim3 grid((pp + 127) / 128, count, 2);
     if (P.permx) launch_prep_near(P, x, y, a, b, slot0, count, st);
-    else if (P.tensor) prep_tensor_kernel<<<dim3((pp + 7) / 8, count, 2), 256, 0, st>>>(P, x, y, a, b, slot0);
+    else if (P.tensor) prep_tensor_kernel<<<dim3((pp + 31) / 32, count, 2), 256, 0, st>>>(P, x, y, a, b, slot0);
     else if (P.compute_f64) prep_kernel<double><<<grid, 128, 0, st>>>(P, x, y, a, b, slot0);
     else prep_kernel<float><<<grid, 128, 0, st>>>(P, x, y, a, b, slot0);
 }
@@ -1029,6 +1077,7 @@ static size_t lane_state_bytes(const Dev &P)
     size_t coords = (size_t)P.DP * (P.np + P.mp) * ts;
     if (P.tensor) coords = ((size_t)((P.n + 127) / 128) + (size_t)((P.m + 127) / 128)) * P.d * 256;
     if (P.guard > 0.0) coords += P.xraw_stride + P.yraw_stride;
+    if (P.dots) coords += (size_t)P.np * P.mp * 4;
     return coords + (size_t)(P.np + P.mp) * (4 * 8 + (P.phi0 ? 16 : 2 * ts) + 8);
 }
 // When even the retirement of every lane at once would move little (narrow batches of small

@@ -28,6 +28,11 @@ constexpr float NEG_BIG = -1.0e30f;   // "minus infinity" for padded columns (fi
 constexpr int UPD_THREADS = 128;
 constexpr int SC_NO_MATRIX = -1;      // scaling_kernel: a weight below SC_MIN_WEIGHT, the lane stays in the log domain
 constexpr float SC_MIN_WEIGHT = 0x1p-80f;
+// scaling_kernel: lanes whose kernel entries before any potential stay above 2^-SC_COLD_BITS (four times the scaled squared
+// radius), with weights from SC_COLD_WEIGHT on, start with zero potentials absorbed; the others' first cycle is
+// a log-domain one
+constexpr double SC_COLD_BITS = 120.0;
+constexpr float SC_COLD_WEIGHT = 0x1p-40f;
 constexpr int BOX_COLS = 32;          // points per bounding box of lanes in spatial order
 constexpr int TC_MAX_SPLIT = 8;      // a row block's columns go to at most this many clusters
 constexpr int MAX_CLUSTER_RANKS = 8;  // blocks per cluster (portable limit): row blocks of a lane in the multi-cycle kernels
@@ -79,6 +84,7 @@ struct Dev {
     // lanes whose kernel matrix is kept on chip (scaling_kernel; null otherwise): potentials absorbed
     // into the matrix and the scalings relative to them
     double *phi0, *gam0, *uu[2], *vv;
+    float *dots;              // [W][np][mp] x_i . y_j of deep lanes whose kernel matrix is kept on chip (null otherwise)
     // lanes in spatial order (update_near_kernel; null otherwise): point i of a lane is input point perm[lane][i];
     // bounding boxes of every 32 points [2 DP][nb]; the largest potential of every 32 points, rounded up
     int *permx, *permy;
@@ -322,5 +328,19 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+__device__ __forceinline__ void cluster_sync_all()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// `local` of block `rank` of the cluster
+__device__ __forceinline__ double ld_cluster(const double *local, const unsigned rank)
+{
+    unsigned a = (unsigned)__cvta_generic_to_shared(local), x;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(x) : "r"(a), "r"(rank));
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(x) : "memory");
+    return v;
+}
 
 }  // namespace skb

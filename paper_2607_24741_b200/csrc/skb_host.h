@@ -67,6 +67,7 @@ void launch_wait_probe(int *out, long long budget_clocks, cudaStream_t st);
 void launch_guard_pool(const Dev &P, cudaStream_t st);
 void launch_guard_strips(void *base, const GuardList &gl, bool fill, int *bad, cudaStream_t st);
 void launch_update_tc(const Dev &P, const void *maps, int leg, int width, cudaStream_t st);
+void launch_gram(const Dev &P, const void *maps, int slot0, int count, cudaStream_t st);
 int launch_emit_move(const Dev &P, int width, cudaStream_t st);
 // lanes kept in spatial order, whose legs skip the boxes of columns that are too far away to matter
 bool near_shape(int f64, int DP, int CS, int n, int m);
@@ -79,7 +80,7 @@ int launch_near(const Dev &P, int leg, int width, cudaStream_t st);     // 1: th
 int guard_pool_rows(int per_row, bool on, int lanes);
 // lanes of mixed arithmetic small enough for their kernel matrix to stay on chip: whole cycles, or one leg as a
 // launch of its own
-bool scaling_fits(int n, int m);
+bool scaling_fits(bool dots, int n, int m);
 enum ScalingKind : int { SC_CYCLES, SC_CATCH_UP, SC_LEG };      // see scaling_kernel; `leg` counts for SC_LEG only
 void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int width, cudaStream_t st);
 int launch_plan_cycles(const Dev &P, int width, int cycles, cudaStream_t st);

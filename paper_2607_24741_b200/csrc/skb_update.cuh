@@ -898,10 +898,6 @@ __global__ void __launch_bounds__(UPD_THREADS, UpdBlocksPerSM<T, DP, XF, RR>::va
 // follows the launch does the accounting of Eq. 6-8 for all cycles of the launch at once and fills
 // the holes (Section "Screen, verify, and compact").  The legs are run_leg, so the bits are those
 // of the one-launch-per-leg path.
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ unsigned long long ld_cg_u64(const unsigned long long *p)
 {
     unsigned long long v;

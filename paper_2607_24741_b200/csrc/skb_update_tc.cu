@@ -209,8 +209,10 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr)
 // instruction descriptor: D fp32, A and B bf16, both K-major, M = 128, N = 128
 __host__ __device__ constexpr uint32_t tc_idesc(int bn) { return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24); }
 
-template <int TC_STAGES, int TC_BN>
-__global__ void __launch_bounds__(TC_THREADS, TC_BN == 128 ? 2 : 1)
+// GRAM: the products themselves are the result: x_i . y_j of the lanes from slot `leg` on, for the lanes whose kernel
+// matrix is formed from them (Dev::dots).  Rows of mp floats, np of them; points past the end give zeros.
+template <int TC_STAGES, int TC_BN, bool GRAM = false>
+__global__ void __launch_bounds__(TC_THREADS, TC_BN == 128 && !GRAM ? 2 : 1)
 update_tc_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmy, const Dev P, const int leg)
 {
     extern __shared__ __align__(1024) unsigned char smem_tc[];
@@ -228,13 +230,15 @@ update_tc_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant_
 
     pdl_enter();
     const Ctl c = *P.ctl;
-    if (c.done) return;
-    const int slot = blockIdx.y;
-    if (slot >= c.n_phys) return;
-    if (P.early_exit && P.state[slot] != 0) return;     // early-exit mask arm: a frozen lane costs a launch slot only
-    if (leg != LEG_V && c.static_final) return;
-    if (leg == LEG_V && !(c.static_final || lane_needs_column_check(P, c, slot))) return;
-    const bool rows_x = (leg == LEG_F);
+    const int slot = GRAM ? leg + (int)blockIdx.y : (int)blockIdx.y;
+    if constexpr (!GRAM) {
+        if (c.done) return;
+        if (slot >= c.n_phys) return;
+        if (P.early_exit && P.state[slot] != 0) return;     // early-exit mask arm: a frozen lane costs a launch slot only
+        if (leg != LEG_V && c.static_final) return;
+        if (leg == LEG_V && !(c.static_final || lane_needs_column_check(P, c, slot))) return;
+    }
+    const bool rows_x = GRAM || leg == LEG_F;
     const int nrows = rows_x ? P.n : P.m;
     const int ncols = rows_x ? P.m : P.n, cp = rows_x ? P.mp : P.np;
     const int i0 = blockIdx.x * TC_BM;
@@ -341,10 +345,10 @@ update_tc_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant_
         bool ok = true;
         float ts = 0.f;
         static_assert(TC_BN <= TC_EPI_THREADS, "one column term per epilogue thread and tile");
-        float g_next = (e < TC_BN && e < cp) ? colt[e] : NEG_BIG;       // column term, one tile ahead
+        float g_next = (!GRAM && e < TC_BN && e < cp) ? colt[e] : NEG_BIG;       // column term, one tile ahead
         for (int t = 0; t < ntiles && ok; ++t) {
             const int buf = t & 1;
-            if (e < TC_BN) {
+            if (!GRAM && e < TC_BN) {
                 gts[buf][e] = g_next;
                 const int j = (t + 1) * TC_BN + e;
                 g_next = (t + 1 < ntiles && j < cp) ? colt[j] : NEG_BIG;
@@ -353,14 +357,29 @@ update_tc_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant_
             ok = TC_TIMED_WAIT(dbg_w0, mbar_wait(b_tfull + 8 * buf, (t >> 1) & 1, ab));
             if (!ok) break;
             tc_fence_after();
-            tc_reduce_tile<TC_BN>(lane_base + (uint32_t)(buf * TC_BN), gts[buf], half, two_s, mx, ts, sd);
+            if constexpr (GRAM) {
+                const int row = i0 + (e & 127);
+                float *dst = P.dots + ((size_t)slot * P.np + (row < P.np ? row : 0)) * P.mp;
+#pragma unroll
+                for (int q = 0; q < TC_BN / 64; ++q) {
+                    uint32_t r[32];
+                    const int c0 = (2 * q + half) * 32;
+                    tc_ld32_issue(lane_base + (uint32_t)(buf * TC_BN + c0), r);
+                    tc_ld_wait(r);
+#pragma unroll
+                    for (int h = 0; h < 32; h += 4)
+                        if (row < P.np && t * TC_BN + c0 + h < P.mp)
+                            *reinterpret_cast<uint4 *>(dst + t * TC_BN + c0 + h) = make_uint4(r[h], r[h + 1], r[h + 2], r[h + 3]);
+                }
+            } else
+                tc_reduce_tile<TC_BN>(lane_base + (uint32_t)(buf * TC_BN), gts[buf], half, two_s, mx, ts, sd);
             sd += (double)ts;
             ts = 0.f;
             tc_fence_before();
             mbar_arrive(b_tempty + 8 * buf);                // all rows have read this accumulator
         }
         // the ring is idle by now: its first bytes carry the second half's partial results
-        tc_merge_halves(e, mx, sd, ok, reinterpret_cast<float *>(smem_tc + (sB - smem_u32(smem_tc)) + 1024),
+        if constexpr (!GRAM) tc_merge_halves(e, mx, sd, ok, reinterpret_cast<float *>(smem_tc + (sB - smem_u32(smem_tc)) + 1024),
                         reinterpret_cast<double *>(smem_tc + (sB - smem_u32(smem_tc))), row_m, row_s, row_h);
     }
     if (abort_flag) {
@@ -383,7 +402,7 @@ update_tc_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant_
     if (abort_flag) {
         if (tid == 0) atomicOr(&P.ctl->error, ERR_WAIT);
     }
-    finish_rows<float, TC_BM, TC_THREADS>(P, c, leg, slot, (int)FORM_DOT, row_m, row_s, row_h, red, (int)blockIdx.x * TC_BM);
+    if constexpr (!GRAM) finish_rows<float, TC_BM, TC_THREADS>(P, c, leg, slot, (int)FORM_DOT, row_m, row_s, row_h, red, (int)blockIdx.x * TC_BM);
 }
 
 // ---------------------------------------------------------------- CTA-pair variant
@@ -874,6 +893,16 @@ void launch_retile(const void *src, void *dst, int W, int npts, int d, cudaStrea
 {
     dim3 grid(((npts + TC_BM - 1) / TC_BM) * (d / TC_BK), W);
     retile_kernel<<<grid, 256, 0, st>>>((const uint4 *)src, (uint4 *)dst, npts, d);
+}
+
+void launch_gram(const Dev &P, const void *maps, int slot0, int count, cudaStream_t st)
+{
+    constexpr int STAGES = 4;
+    const auto kernel = update_tc_kernel<STAGES, 128, true>;
+    const int smem = (P.d / TC_BK + STAGES) * (int)TC_CHUNK + 1024;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const CUtensorMap *tm = reinterpret_cast<const CUtensorMap *>(maps);
+    kernel<<<dim3((P.n + TC_BM - 1) / TC_BM, count), TC_THREADS, smem, st>>>(tm[0], tm[1], P, slot0);
 }
 
 void launch_update_tc(const Dev &P, const void *maps, int leg, int width, cudaStream_t st)
