@@ -41,14 +41,17 @@ void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int wid
     const ScalingVariant *v = scaling_variant(P.dots != nullptr, P.n, P.m);
     const void *kernel = v->kernel[kind];
     const int nc = blocks_of(*v, P.n);
-    // Blocks that use tensor memory ask for shared memory too: in clusters in proportion, so that the blocks that fit
-    // an SM together have their tensor memory and no block waits for an allocation while its peers hold
-    // theirs; by themselves as much as keeps one block too many away (the rest is cache for the formation of K).
+    // No block may take its place on an SM and then wait there for tensor memory while blocks of its cluster hold theirs.
+    // Blocks that take the whole register file are alone anyway.  Others ask for shared memory in proportion to their tensor
+    // memory; without a cluster they may wait, and ask for as much as keeps one block too many away.  (No more
+    // than that: what is left is the cache that spilled registers live in; with all of it asked for, a solve of 64
+    // lanes of 1024 x 1024, d = 512, takes 5.9 ms instead of 5.3.)
     size_t smem = v->smem(nc);
     if (v->tm_cols && kind != SC_LEG) {
         cudaFuncAttributes fa;
         if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;        // (the caller looks at cudaGetLastError)
-        const size_t share = v->cluster ? (size_t)SMEM_PER_SM * v->tm_cols / 512 : (size_t)SMEM_PER_SM / (512 / v->tm_cols + 1) + 1024;
+        const bool alone = (fa.numRegs + 7) / 8 * 8 * v->threads >= 65536;
+        const size_t share = alone ? 0 : v->cluster ? (size_t)SMEM_PER_SM * v->tm_cols / 512 : (size_t)SMEM_PER_SM / (512 / v->tm_cols + 1) + 1024;
         if (share > fa.sharedSizeBytes + smem) smem = share - fa.sharedSizeBytes;
     }
     // (with the fixed arrays some variants are beyond the 48 KB that need no permission; the attribute belongs

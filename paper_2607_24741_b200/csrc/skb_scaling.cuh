@@ -95,15 +95,26 @@ __device__ __forceinline__ u64 mul2(u64 a, u64 b)
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
-// 1 / s to float64 accuracy for s within the range of normal fp32 numbers: two Newton steps on the fp32
-// approximation.  Outside that range the result is 0, infinite or NaN, which out_of_band() reports.
+// fp32 -> float64 and back (towards zero) by integers, for positive normal fp32 numbers: the conversion unit is slow and
+// far away.  Zero and subnormal numbers become something below 2^-125, infinities and NaN something from 2^128 on.
+__device__ __forceinline__ double widen(const float x)
+{
+    const unsigned u = __float_as_uint(x);
+    return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+}
+__device__ __forceinline__ float narrow(const double x)
+{
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), (unsigned)__double2hiint(x) - 0x38000000u, 3));
+}
+// 1 / s to float64 accuracy: a third-order step on the fp32 approximation (relative error 2^-23, cubed).  For s outside
+// 2^+-SC_SUMS the result is meaningless: the caller asks out_of_band() about s too.
+constexpr int SC_SUMS = 100;
 __device__ __forceinline__ double rcp64(const double s)
 {
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)s));
-    double x = (double)r;
-    x = fma(x, fma(-s, x, 1.0), x);
-    return fma(x, fma(-s, x, 1.0), x);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(narrow(s)));
+    const double x = widen(r), e = fma(-s, x, 1.0);
+    return fma(x * e, e, fma(x, e, x));
 }
 // x (u or v) is not within 2^+-BAND: negative, zero, infinite and NaN included
 template <int BAND>
@@ -139,10 +150,13 @@ struct ScalingShape {
     static_assert(RW >= 8 && RW <= 32 && CL >= 2 && CL <= 32, "unsupported tile");
     static_assert(!TM || (NW % 4 == 0 && GW % 32 == 0 && TM_COLS <= 512 && BLOCKS <= 4), "unsupported tile in tensor memory");
     static_assert(!TWO_STEP || COLS == 4 * THREADS, "the two-step exchange has one thread to a column where four blocks share them");
-    // dynamic shared memory: column parts of every warp; the exchange buffers (TWO_STEP: parts of the own columns,
-    // totals of all); where K is in registers, the words it is formed in
+    // dynamic shared memory: column parts of every warp; the exchange buffers: what goes out, what comes in (TWO_STEP: parts
+    // of the own columns, totals of all; totals that go out); where K is in registers, the words it is formed in
     static constexpr size_t PARTS = sizeof(double) * NW * COLS;
-    __host__ __device__ static constexpr size_t exchange(int nc) { return sizeof(double) * 2 * (TWO_STEP ? (size_t)nc * (COLS >> owner_bits(nc)) + COLS : (size_t)nc * COLS); }
+    __host__ __device__ static constexpr size_t exchange(int nc)
+    {
+        return sizeof(double) * 2 * (COLS + (TWO_STEP ? (size_t)nc * (COLS >> owner_bits(nc)) + COLS + THREADS : (size_t)nc * COLS));
+    }
     static size_t smem(int nc) { return PARTS + exchange(nc) + (TM ? 0 : sizeof(float) * (size_t)RW * CL * THREADS); }
 };
 
@@ -211,7 +225,7 @@ __device__ __forceinline__ double row_exchange(V (&s)[CNT], const int lane)
     if constexpr (sizeof(V) == 4 && COLS_IN >= LIM) {
         double t[CNT];
 #pragma unroll
-        for (int r = 0; r < CNT; ++r) t[r] = (double)s[r];
+        for (int r = 0; r < CNT; ++r) t[r] = widen(s[r]);
         return row_exchange<CL, LIM, PERM, OFF, CNT, double>(t, lane);
     } else {
         if constexpr (CNT > 1) {
@@ -332,10 +346,11 @@ __device__ __noinline__ unsigned long long scaling_reeval(const Dev *P, const in
     return direct_rows_block<NW>(*P, slot, r0, NW, r1, pot, r0, red, bad);
 }
 
-// Exchange between the blocks of a cluster without a cluster barrier: remote stores that report their bytes
-// to a barrier in the receiver's shared memory, which the receiver waits on.  (A cluster barrier's release
-// waits until all of the block's remote stores have been acknowledged: about 850 clk per cycle at four
-// blocks; measured.)  The wait is bounded like every wait of this library.
+// Exchange between the blocks of a cluster without a cluster barrier: bulk copies from shared memory to shared memory
+// that report their bytes to a barrier of the receiver, which waits on it.  (A cluster barrier's release waits until
+// all of the block's remote stores have been acknowledged, and remote stores of 16 bytes a thread go out one by one.
+// A cycle of 24 lanes of 500 x 333, four blocks: 4.2 -> 3.3 us; sent by all warps, of 64 lanes of 1024 x 1024, sixteen
+// blocks: 2.9 -> 2.4 us per four lanes.)  The wait is bounded like every wait of this library.
 constexpr long long SC_WAIT_CLOCKS = 2000000000LL;
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ unsigned peer_addr(const unsigned a, const unsigned rank)
@@ -344,14 +359,18 @@ __device__ __forceinline__ unsigned peer_addr(const unsigned a, const unsigned r
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(x) : "r"(a), "r"(rank));
     return x;
 }
-__device__ __forceinline__ void st_async(const unsigned addr, const unsigned long long v, const unsigned bar)
+// `bytes` (a multiple of 16) of this block's shared memory into a peer's, reported to the peer's barrier
+__device__ __forceinline__ void copy_to_peer(const void *dst, const void *src, const unsigned bytes, const void *bar, const unsigned rank)
 {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr), "l"(v), "r"(bar) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(peer_addr(smem_addr(dst), rank)), "r"(smem_addr(src)), "r"(bytes), "r"(peer_addr(smem_addr(bar), rank)) : "memory");
 }
-__device__ __forceinline__ void st_async2(const unsigned addr, const unsigned long long v0, const unsigned long long v1, const unsigned bar)
+__device__ __forceinline__ void expect_bytes(const void *bar, const unsigned bytes)
 {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(addr), "l"(v0), "l"(v1), "r"(bar) : "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
+// this thread's writes to shared memory become visible to copies issued after the next block barrier
+__device__ __forceinline__ void fence_for_copies() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ bool bar_try_wait(const unsigned a, const unsigned parity)
 {
     unsigned ok;
@@ -389,8 +408,10 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned long long swr[NW];
-    __shared__ unsigned long long xw[2][L::RANKS * NW];  // residual part and flags of every warp of the cluster
+    __shared__ __align__(16) unsigned long long sw[2][NW];          // ... what this block sends
+    __shared__ __align__(16) unsigned long long xw[2][L::RANKS * NW];  // residual part and flags of every warp of the cluster
     __shared__ int sflag;                                // column flags
+    __shared__ volatile int vflag;                       // 1: a column has left the band, 2: a wait ran out
     __shared__ __align__(16) double colB[COLS], rowA[RB];       // additive terms of columns / own rows
     __shared__ __align__(16) float vs[COLS];             // b v of all columns
     __shared__ __align__(16) float2 uas[RB];             // a u of own rows, in both halves
@@ -430,6 +451,8 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
     const int ob = L::owner_bits(NC), own = 1 << ob, share = COLS >> ob, tpb = ob - 2;
     double *xbuf = reinterpret_cast<double *>(smem_raw + L::PARTS);      // [2][NC][COLS] column parts of every block; TWO_STEP: [2][NC][share]
     double *tbuf = xbuf + (size_t)2 * NC * share;                        // TWO_STEP: [2][COLS] totals
+    double *sbuf = L::TWO_STEP ? tbuf + 2 * COLS : xbuf + (size_t)2 * NC * COLS;         // [2][COLS] what this block sends
+    double *ubuf = sbuf + 2 * COLS;                                      // TWO_STEP: [2][THREADS] totals it sends
     u64 *kstage = reinterpret_cast<u64 *>(smem_raw + L::PARTS + L::exchange(NC));   // K on its way into the registers
     int xch = 0;                                                         // exchanges so far: their buffer alternates
 
@@ -479,7 +502,7 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
         near_tot = (unsigned long long)fmin(t * 1.000001 * RSUM_SCALE, 1.0e18) + 2ull;
     }
     if (tid == 0) {
-        sflag = 0;
+        sflag = 0; vflag = 0;
         if constexpr (CLU) {
             for (int e = 0; e < 2; ++e) {
                 asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&xbar[e])) : "memory");
@@ -608,7 +631,7 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                 for (int q = 0; q < NQ; ++q) x[q] += y[q];
             }
 #pragma unroll
-            for (int q = 0; q < NQ; ++q) p[w][q] = (double)x[q];
+            for (int q = 0; q < NQ; ++q) p[w][q] = widen(x[q]);
         }
 #pragma unroll
         for (int step = 1; step < NP; step *= 2)
@@ -852,9 +875,10 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                     const double S = row_exchange<CL, L::FP32_COLS, true, 16, RW, float>(s, lane);
                     unew = rok ? rcp64(S) : 1.0;
                     const double term = rown ? a_fix * fabs(fma(us, S, -1.0)) : 0.0;
-                    const int flags = (out_of_band<SC_TAKE>(unew) ? SC_BAD : 0) | (out_of_band<SC_KEEP>(unew) ? SC_DRIFT : 0);
+                    const int flags = (rok && out_of_band<SC_SUMS>(S)) || out_of_band<SC_TAKE>(unew) ? SC_BAD | SC_DRIFT : (out_of_band<SC_KEEP>(unew) ? SC_DRIFT : 0);
+                    const unsigned long long fx = to_fixed(term);
                     if constexpr (LEG) {
-                        send_rows(to_fixed(term), flags);
+                        send_rows(fx, flags);
                         scaling_barrier<CLU>();
                         tot = recv_rows(all);
                         ++xch;
@@ -863,55 +887,55 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                     if (lane % SHARE == 0) { const float w = (float)(a_i * unew); uas[lr] = make_float2(w, w); }
                     __syncwarp();
                     col_parts();
-                    const unsigned long long word = rows_word(to_fixed(term), flags);
-                    if constexpr (CLU) {
-                        if (lane < NC) st_async(peer_addr(smem_addr(&xw[xch & 1][b * NW + warp]), lane), word, peer_addr(smem_addr(&xbar[xch & 1]), lane));
-                    } else if (lane == 0) xw[xch & 1][warp] = word;
+                    const unsigned long long word = rows_word(fx, flags);
+                    if (lane == 0) (CLU ? sw[xch & 1] : xw[xch & 1])[warp] = word;
                 }
                 __syncthreads();
                 block_cols(T);
                 if constexpr (CLU) {
-                    const unsigned bar = smem_addr(&xbar[xch & 1]);
+                    const int e = xch & 1;
+                    double *out = sbuf + e * COLS;
+                    if (cown) {
+                        if constexpr (NQ == 1) out[j0] = T[0];
+                        else {
+#pragma unroll
+                            for (int q = 0; q < NQ; q += 2) *reinterpret_cast<double2 *>(out + j0 + q) = make_double2(T[q], T[q + 1]);
+                        }
+                    }
+                    fence_for_copies();
                     if (tid == 0) {
-                        const int part_cols = !L::TWO_STEP ? COLS : (b < own ? share : 0);
-                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((unsigned)(NC * (part_cols + NW) * 8)) : "memory");
-                        if constexpr (L::TWO_STEP)
-                            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&tbar[xch & 1])), "r"((unsigned)(COLS * 8)) : "memory");
+                        expect_bytes(&xbar[e], (unsigned)(NC * ((!L::TWO_STEP ? COLS : (b < own ? share : 0)) + NW) * 8));
+                        if constexpr (L::TWO_STEP) expect_bytes(&tbar[e], (unsigned)(COLS * 8));
                     }
+                    __syncthreads();
+                    // a warp sends to the ranks warp, warp + NW, ...: one after the other from one warp they took 1000 clk
+                    for (int rk = warp; rk < NC; rk += NW) {
+                        if (lane == 0) {
+                            if constexpr (!L::TWO_STEP) copy_to_peer(xbuf + ((size_t)e * NC + b) * COLS, out, COLS * 8, &xbar[e], rk);
+                            else if (rk < own) copy_to_peer(xbuf + ((size_t)e * NC + b) * share, out + rk * share, share * 8, &xbar[e], rk);
+                            copy_to_peer(&xw[e][b * NW], sw[e], NW * 8, &xbar[e], rk);
+                        }
+                    }
+                    __syncwarp();
+                    const unsigned phase = (xphase >> e) & 1u;
+                    bool ok = bar_wait(smem_addr(&xbar[e]), phase);
                     if constexpr (L::TWO_STEP) {
-                        const unsigned dst = peer_addr(smem_addr(xbuf + ((size_t)(xch & 1) * NC + b) * share + j0 % share), j0 / share), pb = peer_addr(bar, j0 / share);
-#pragma unroll
-                        for (int q = 0; q < NQ; q += 2) st_async2(dst + 8 * q, (unsigned long long)__double_as_longlong(T[q]), (unsigned long long)__double_as_longlong(T[q + 1]), pb);
-                        const bool ok = bar_wait(bar, (xphase >> (xch & 1)) & 1u);
-                        const unsigned tb = smem_addr(&tbar[xch & 1]);
-                        if (b < own) {
+                        if (b < own) {                       // (the same for the whole block)
                             const double t = share_total(false);
-                            const unsigned tdst = smem_addr(tbuf + (size_t)(xch & 1) * COLS + b * share + (tid >> tpb));
-#pragma unroll
-                            for (int e = 0; e < L::RANKS / 2; ++e) {
-                                const int rk = (e << tpb) + (tid & ((1 << tpb) - 1));
-                                if (rk < NC) st_async(peer_addr(tdst, rk), (unsigned long long)__double_as_longlong(t), peer_addr(tb, rk));
-                            }
+                            if ((tid & ((1 << tpb) - 1)) == 0) ubuf[e * THREADS + (tid >> tpb)] = t;
+                            fence_for_copies();
+                            __syncthreads();
+                            for (int rk = warp; rk < NC; rk += NW)
+                                if (lane == 0) copy_to_peer(tbuf + (size_t)e * COLS + b * share, ubuf + e * THREADS, share * 8, &tbar[e], rk);
+                            __syncwarp();
                         }
-                        const bool ok2 = bar_wait(tb, (xphase >> (xch & 1)) & 1u);
-                        xphase ^= 1u << (xch & 1);
-                        if (__syncthreads_or(!ok || !ok2)) { dead = true; break; }
-                    } else {
-                        const unsigned dst = smem_addr(xbuf + ((size_t)(xch & 1) * NC + b) * COLS + j0);
-                        if (cown) {
-#pragma unroll
-                            for (int rk = 0; rk < MAX_CLUSTER_RANKS; ++rk) {
-                                if (rk >= NC) continue;
-                                if constexpr (NQ == 2) st_async2(peer_addr(dst, rk), (unsigned long long)__double_as_longlong(T[0]), (unsigned long long)__double_as_longlong(T[1]), peer_addr(bar, rk));
-                                else st_async(peer_addr(dst, rk), (unsigned long long)__double_as_longlong(T[0]), peer_addr(bar, rk));
-                            }
-                        }
-                        const bool ok = bar_wait(bar, (xphase >> (xch & 1)) & 1u);
-                        xphase ^= 1u << (xch & 1);
-                        if (__syncthreads_or(!ok)) { dead = true; break; }
+                        ok = bar_wait(smem_addr(&tbar[e]), phase) && ok;
                     }
+                    xphase ^= 1u << e;
+                    if (!ok) vflag = 2;
+                    __syncthreads();
+                    if (vflag) { dead = true; break; }
                 }
-                tot = recv_rows(all);
                 if constexpr (CLU && L::TWO_STEP) {
                     const double *src = tbuf + (size_t)(xch & 1) * COLS + j0;
 #pragma unroll
@@ -929,24 +953,28 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                         }
                     }
                 }
-                ++xch;
-                if (all || (tot <= near_tot && !frozen && !catch_up) || nf || (k - start >= P.max_iter && !catch_up) || (closing && it == todo)) break;
-                // g-leg
+                // g-leg, on its way while the words are added up
                 double vn[NQ];
                 int flags = 0;
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) {
-                    const int j = j0 + q;
                     vn[q] = 0.0;
-                    if (cown) {
-                        if (j < P.m) {
-                            vn[q] = rcp64(T[q]);
-                            flags |= out_of_band<SC_KEEP>(vn[q]);
-                        }
+                    if (cown && j0 + q < P.m) {
+                        vn[q] = rcp64(T[q]);
+                        flags |= out_of_band<SC_KEEP>(vn[q]) | out_of_band<SC_SUMS>(T[q]);
                     }
                 }
+                tot = recv_rows(all);
+                ++xch;
+                if (all || (tot <= near_tot && !frozen && !catch_up) || nf || (k - start >= P.max_iter && !catch_up) || (closing && it == todo)) break;
                 if (!frozen) put_vs(vn);
-                if (__syncthreads_or(flags)) break;
+                if (flags) vflag = 1;
+                __syncthreads();
+                if (vflag) {                             // (read by all before it is cleared, cleared before it is set again)
+                    __syncthreads();
+                    if (tid == 0) vflag = 0;
+                    break;
+                }
                 if (!frozen) {
                     us = unew;
 #pragma unroll
@@ -1172,7 +1200,7 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                 if (cown) {
                     if (j < P.m) {
                         vnew[q] = rcp64(T[q]);
-                        flags |= (out_of_band<SC_TAKE>(vnew[q]) ? SC_BAD : 0) | (out_of_band<SC_KEEP>(vnew[q]) ? SC_DRIFT : 0);
+                        flags |= out_of_band<SC_SUMS>(T[q]) || out_of_band<SC_TAKE>(vnew[q]) ? SC_BAD | SC_DRIFT : (out_of_band<SC_KEEP>(vnew[q]) ? SC_DRIFT : 0);
                     }
                     if (!frozen) vs[j] = (float)(bq[q] * vnew[q]);
                 }
