@@ -568,15 +568,25 @@ static bool cycles_in_one_launch(const skb_batch *h)
 static void enqueue_cycles_launch(skb_batch *h, int cycles)
 {
     const int w = h->known_width;
+    // A batch of more lanes than run at a time starts the ones with the smallest eps first: they need the most cycles
+    // as a rule, and one that starts last runs alone in the end (sweep workload: 10.8 -> 9.0 ms).  First launch only (the
+    // list lies where the planner keeps one later), and up to a width whose ranking is cheap.
+    h->dev.order = nullptr;
+    if (h->dev.phi0 && h->enqueued == 0 && w == h->cfg.W && w <= 4096 && (long long)w * scaling_blocks(h->dev) > 148) {
+        launch_order(h->dev, h->dev.fill_list, h->stream);
+        h->dev.order = h->dev.fill_list;
+        h->launches += 1;
+    }
     if (h->cfg.mode == SKB_STATIC) {
         launch_scaling(h->dev, SC_CYCLES, 0, cycles, w, h->stream);
+        h->dev.order = nullptr;
         launch_plan_static(h->dev, cycles, h->stream);
         launch_scaling(h->dev, SC_CATCH_UP, 0, 0, w, h->stream);
         h->enqueued += cycles;
         h->launches += 3;
         return;
     }
-    if (h->dev.phi0) launch_scaling(h->dev, SC_CYCLES, 0, cycles, w, h->stream);
+    if (h->dev.phi0) { launch_scaling(h->dev, SC_CYCLES, 0, cycles, w, h->stream); h->dev.order = nullptr; }
     else h->var->launch_cycles(h->dev, cycles, w, h->stream);
     int nk = 1;
     nk += launch_plan_cycles(h->dev, w, cycles, h->stream);

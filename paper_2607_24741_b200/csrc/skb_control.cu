@@ -1040,6 +1040,18 @@ void launch_apply_plan(const Dev &P, const void *x, const void *y, const float *
     launch_apply_tiled<P64_MAX_D>(P, x, y, eps, v, dv, out, lanes, st);
 }
 
+// Slots by falling scale (smallest eps first, equal ones as they come).
+__global__ void __launch_bounds__(128) order_kernel(const Dev P, int *order)
+{
+    const int s = blockIdx.x * 128 + threadIdx.x;
+    if (s >= P.W) return;
+    const double mine = P.scale[s];
+    int rank = 0;
+    for (int t = 0; t < P.W; ++t) { const double x = P.scale[t]; rank += x > mine || (x == mine && t < s); }
+    order[rank] = s;
+}
+void launch_order(const Dev &P, int *order, cudaStream_t st) { order_kernel<<<(P.W + 127) / 128, 128, 0, st>>>(P, order); }
+
 // ---------------------------------------------------------------- launchers
 void launch_lane_stats(const Dev &P, const void *x, const void *y, const float *eps, int slot0, int lane0, int count,
                        int cycle0, cudaStream_t st)

@@ -90,6 +90,7 @@ struct Dev {
     int *permx, *permy;
     float *boxx, *boxy, *topx[2], *topy;
     int nbx, nby;             // boxes of 32 points, padded to a multiple of 4
+    const int *order;         // scaling_kernel, a batch's first launch: the order in which slots are started (null: as they are)
     // per-slot scalars
     double *scale;            // s
     int *lane_id;

@@ -84,6 +84,8 @@ bool scaling_fits(bool dots, int n, int m);
 enum ScalingKind : int { SC_CYCLES, SC_CATCH_UP, SC_LEG };      // see scaling_kernel; `leg` counts for SC_LEG only
 void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int width, cudaStream_t st);
 int launch_plan_cycles(const Dev &P, int width, int cycles, cudaStream_t st);
+void launch_order(const Dev &P, int *order, cudaStream_t st);
+int scaling_blocks(const Dev &P);          // blocks of a lane
 void launch_plan_static(const Dev &P, int cycles, cudaStream_t st);
 void launch_gather(const Dev &P, void *f, void *g, bool f64, cudaStream_t st);
 void launch_gather_audit(const Dev &P, float *rrow, float *rcol, int *flagged, cudaStream_t st);

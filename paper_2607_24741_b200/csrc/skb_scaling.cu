@@ -36,6 +36,8 @@ static const ScalingVariant *scaling_variant(bool dots, int n, int m)
 
 bool scaling_fits(bool dots, int n, int m) { return scaling_variant(dots, n, m) != nullptr; }
 
+int scaling_blocks(const Dev &P) { return blocks_of(*scaling_variant(P.dots != nullptr, P.n, P.m), P.n); }
+
 void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int width, cudaStream_t st)
 {
     const ScalingVariant *v = scaling_variant(P.dots != nullptr, P.n, P.m);

@@ -421,7 +421,7 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
 
     pdl_enter();
     const Ctl c = *P.ctl;
-    const int slot = blockIdx.y;
+    const int slot = P.order ? P.order[blockIdx.y] : (int)blockIdx.y;
     // every exit here is taken by the whole cluster
     const int lane_id = P.lane_id[slot < c.n_phys ? slot : 0];
     if ((c.done && !catch_up) || slot >= c.n_phys) return;
