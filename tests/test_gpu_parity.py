@@ -1216,6 +1216,80 @@ def test_kernel_matrix_lanes_at_the_edges_of_their_tiles(oracle, n, m):
         sb.close()
 
 
+@pytest.mark.parametrize("n,m", [(40, 128), (129, 100), (128, 129), (257, 256), (130, 257), (600, 512), (64, 513), (193, 600),
+                                 (449, 1024), (1024, 520)])
+def test_deep_lanes_on_chip_at_the_edges_of_their_tiles(oracle, n, m):
+    # one block, clusters of 2 to 16 blocks, clusters with blocks that hold no rows, both ways of exchanging column sums;
+    # launches of many cycles, of one cycle, of one leg, and a logical mask must give the same bits
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("feature", W=3, n=n, m=m, d=64, max_iter=40)
+    r = run_gpu(w)
+    assert r["arith"] == "tensor"
+    check_against_oracle(oracle, w, r, range(3), pot_tol=POT_TOL_F32, exact_depth=False, floor=MARGIN_AUTO, max_iter=40,
+                         label=f"deep lanes on chip, {n} x {m}")
+    check_accounting(oracle, r, 3, "active")
+    rm = run_gpu(w, mode="masked")
+    np.testing.assert_array_equal(rm["f"], r["f"]); np.testing.assert_array_equal(rm["r_row"], r["r_row"])
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    for profiling in (False, True):
+        sb = B.SinkhornBatch(t(w.x).bfloat16(), t(w.y).bfloat16(), t(w.a), t(w.b), t(w.eps), w.tol, max_iter=40)
+        sb.set_profiling(profiling)
+        for _ in range(41):
+            sb.step(1)
+        assert sb.active() == 0
+        f, g = sb.potentials(f64=True)
+        np.testing.assert_array_equal(f.cpu().numpy(), r["f"]); np.testing.assert_array_equal(g.cpu().numpy(), r["g"])
+        assert sb.check_guards() == -1
+        sb.close()
+
+
+def test_last_audit_of_deep_lanes_follows_them_through_compaction():
+    # lanes that others' retirement has moved report their own audit, as lanes that stay in place do
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("feature", W=12, n=96, m=80, d=64)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    both = [B.SinkhornBatch(t(w.x).bfloat16(), t(w.y).bfloat16(), t(w.a), t(w.b), t(w.eps), w.tol, mode=m) for m in ("active", "masked")]
+    seen = set()
+    while both[0].active() > 0:
+        for sb in both:
+            sb.step(7)
+        seen.add(both[0].active())
+        running = (both[0].depths()[1] == 0).cpu().numpy()
+        (ra, ca, fa), (rm, cm, fm) = (tuple(v.cpu().numpy() for v in sb.last_audit()) for sb in both)
+        np.testing.assert_array_equal(ra[running], rm[running]); np.testing.assert_array_equal(fa[running], fm[running])
+    assert len(seen - {0, 12}) > 0                                # lanes really left one after the other
+    for sb in both:
+        sb.close()
+
+
+@pytest.mark.parametrize("light", [1.0, 2.0 ** -25, 2.0 ** -38, 2.0 ** -75])
+def test_lanes_that_start_with_their_costs_absorbed(oracle, light):
+    # four times the scaled squared radius on both sides of the 120 bits up to which a cold lane starts with zero potentials
+    # absorbed, weights on both sides of the 2^-40 from which it does (and of the 2^-80 below which it never absorbs)
+    rng = np.random.default_rng(11)
+    f32 = np.float32
+    W, n, m, d = 6, 70, 130, 5
+    x = rng.uniform(-1, 1, (W, n, d)).astype(f32); y = rng.uniform(-1, 1, (W, m, d)).astype(f32)
+    a = rng.uniform(0.5, 1.5, (W, n)); b = rng.uniform(0.5, 1.5, (W, m))
+    a[1::2, 4] *= light; b[::2, 9:12] *= light
+    rad = np.array([max(((x[t] - c) ** 2).sum(1).max(), ((y[t] - c) ** 2).sum(1).max())
+                    for t in range(W) for c in [np.concatenate([x[t], y[t]]).mean(0)]])
+    eps = (4.0 * 1.4426950408889634 * rad / np.array([20.0, 90.0, 118.0, 122.0, 200.0, 400.0])).astype(f32)
+    w = wl.Workload("cold", x, y, (a / a.sum(1, keepdims=True)).astype(f32), (b / b.sum(1, keepdims=True)).astype(f32), eps, 1e-3, 300)
+    for mode in ("active", "static"):
+        r = run_gpu(w, mode=mode)
+        if mode == "active":
+            assert r["arith"] == "f32"
+            check_against_oracle(oracle, w, r, range(W), pot_tol=POT_TOL_F32, exact_depth=False, floor=MARGIN_AUTO, max_iter=300,
+                                 label=f"cold lanes, weights down to {light:.0e}")
+    # a proposal replaces the zero potentials: two cycles, a restart from where they ended, and the rest
+    first = run_gpu(w, max_iter=2)
+    rest = run_gpu(w, warm=(first["f"], first["g"]))
+    np.testing.assert_array_equal(np.where(first["status"] == 1, first["depth"], rest["depth"] + 2), run_gpu(w)["depth"])
+
+
 @pytest.mark.parametrize("least", [2.0 ** -70, 2.0 ** -100, 2.0 ** -118])
 @pytest.mark.parametrize("n,m", [(60, 64), (150, 100), (300, 200)])
 def test_kernel_matrix_lanes_with_tiny_weights(oracle, n, m, least):
