@@ -65,6 +65,8 @@ typedef enum {
     SKB_COMPUTE_AUTO = 0,  /* F32 (TENSOR where eligible), or MIXED when some lane's cost/eps  */
                            /* range is beyond fp32 for the tolerance asked for: scaled squared */
                            /* radius log2(e)/eps * max|x - centre|^2 above 512 * min(1, tol/1e-3) */
+                           /* (F32 lanes of up to 512 columns whose kernel matrix stays on chip */
+                           /* have their exponents formed once, in float64)                     */
     SKB_COMPUTE_F32 = 1,   /* fp32 exponents and exponentials                                  */
     SKB_COMPUTE_MIXED = 2, /* float64 exponents (half-rate FP64 pipe), fp32 exponentials       */
     SKB_COMPUTE_F64 = 3,   /* float64 throughout, software exp2: the slow validation arithmetic */
