@@ -729,7 +729,7 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
         snap ^= 1;
         // grow the chunk every other round: cycles enqueued past completion are empty launches that
         // still have to drain, which matters for batches that finish within a dozen cycles
-        if (chunk < chunk_max && (scaling ? h->enqueued - h->enqueued_at_refill >= 16 * chunk : (++rounds & 1) == 0)) chunk *= 2;
+        if (chunk < chunk_max && (scaling ? h->enqueued - h->enqueued_at_refill >= 8 * chunk : (++rounds & 1) == 0)) chunk *= 2;
         if (h->enqueued - h->enqueued_at_refill > hard_cap + 64 + 2 * MAX_CYCLES_IN_LAUNCH) break;
     }
     if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "drain");

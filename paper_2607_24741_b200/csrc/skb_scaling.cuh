@@ -343,7 +343,71 @@ template <int NW>
 __device__ __noinline__ unsigned long long scaling_reeval(const Dev *P, const int slot, const int r0, const int r1, const double *pot,
                                                           unsigned long long *red, int *bad)
 {
-    return direct_rows_block<NW>(*P, slot, r0, NW, r1, pot, r0, red, bad);
+    // direct_rows_block, four rows of a warp side by side: the same terms in the same order, with the latencies of
+    // their distances, exponentials and shuffles shared (one row after the other 60 us a lane of 100 x 77)
+    constexpr int R = 4, U = 2;
+    const Dev &D = *P;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double s = D.scale[slot];
+    const double *gam = D.gam + (size_t)slot * D.mp;
+    const void *xl = (const char *)D.xraw + (size_t)slot * D.xraw_stride, *yl = (const char *)D.yraw + (size_t)slot * D.yraw_stride;
+    unsigned long long part = 0ull;
+    int nf = 0;
+    for (int i0 = r0 + warp; i0 < r1; i0 += R * NW) {
+        int row[R];
+        double phi[R], sum[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) { row[r] = min(i0 + r * NW, r1 - 1); phi[r] = pot[row[r] - r0]; sum[r] = 0.0; }
+        for (int j0 = lane; j0 < D.m; j0 += 32 * U) {
+            double c[R][U], gj[U];
+            size_t yb[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int j = j0 + 32 * u < D.m ? j0 + 32 * u : D.m - 1;
+                yb[u] = (size_t)j * D.d;
+                gj[u] = __ldcg(gam + j);
+#pragma unroll
+                for (int r = 0; r < R; ++r) c[r][u] = 0.0;
+            }
+            for (int k = 0; k < D.d; ++k) {
+                double y[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) y[u] = (double)load_raw(D, yl, yb[u] + k);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const double x = (double)load_raw(D, xl, (size_t)row[r] * D.d + k);
+#pragma unroll
+                    for (int u = 0; u < U; ++u) { const double t = x - y[u]; c[r][u] = fma(t, t, c[r][u]); }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const double v = exp2(phi[r] + gj[u] - s * c[r][u]);
+                    sum[r] += j0 + 32 * u < D.m ? v : 0.0;
+                }
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+            for (int r = 0; r < R; ++r) sum[r] += __shfl_xor_sync(0xffffffffu, sum[r], off);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (i0 + r * NW >= r1) continue;
+            const double term = fabs(sum[r] - D.wa[(size_t)slot * D.np + row[r]]);
+            if (!isfinite(term)) nf = 1;
+            else if (lane == 0) part += __double2ull_rn(fmin(term, RSUM_ROW_MAX) * RSUM_SCALE);
+        }
+    }
+    nf = __syncthreads_or(nf);
+    if (lane == 0) red[warp] = part;
+    __syncthreads();
+    unsigned long long all = 0ull;
+    if (threadIdx.x == 0) for (int w = 0; w < NW; ++w) all += red[w];
+    __syncthreads();
+    *bad = nf;
+    return all;
 }
 
 // Exchange between the blocks of a cluster without a cluster barrier: bulk copies from shared memory to shared memory
