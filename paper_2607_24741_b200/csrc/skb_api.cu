@@ -704,7 +704,7 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
     }
     // Lanes of the scaling kernel that finish inside a launch leave it (STATIC: wait for the second half), so the longest
     // launch costs nothing and saves forming the kernel matrices again; a mask's lanes work on until the launch
-    // ends, so its launches grow with what has been done and overshoot by an eighth at most.
+    // ends, so its launches grow to 64 cycles and beyond that only to an eighth of what has been done.
     const bool scaling = h->dev.phi0 && cycles_in_one_launch(h), masked = h->cfg.mode == SKB_MASKED;
     int chunk = scaling ? (masked ? 16 : MAX_CYCLES_IN_LAUNCH) : 2, snap = 0, rounds = 0;
     bool have_prev = false;
@@ -729,7 +729,7 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
         snap ^= 1;
         // grow the chunk every other round: cycles enqueued past completion are empty launches that
         // still have to drain, which matters for batches that finish within a dozen cycles
-        if (chunk < chunk_max && (scaling ? h->enqueued - h->enqueued_at_refill >= 8 * chunk : (++rounds & 1) == 0)) chunk *= 2;
+        if (chunk < chunk_max && (scaling && chunk >= 64 ? h->enqueued - h->enqueued_at_refill >= 8 * chunk : (++rounds & 1) == 0)) chunk *= 2;
         if (h->enqueued - h->enqueued_at_refill > hard_cap + 64 + 2 * MAX_CYCLES_IN_LAUNCH) break;
     }
     if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "drain");
