@@ -475,7 +475,10 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
     __shared__ __align__(16) unsigned long long sw[2][NW];          // ... what this block sends
     __shared__ __align__(16) unsigned long long xw[2][L::RANKS * NW];  // residual part and flags of every warp of the cluster
     __shared__ int sflag;                                // column flags
-    __shared__ volatile int vflag;                       // 1: a column has left the band, 2: a wait ran out
+    // Two words, because no block barrier lies between the last read of the one and the first write of the other within a
+    // cycle: a warp that reads late would take a column that has left the band, found by a warp ahead of it, for a wait that ran out.
+    __shared__ volatile int vflag;                       // a column has left the band
+    __shared__ volatile int wflag;                       // a wait ran out (never cleared)
     __shared__ __align__(16) double colB[COLS], rowA[RB];       // additive terms of columns / own rows
     __shared__ __align__(16) float vs[COLS];             // b v of all columns
     __shared__ __align__(16) float2 uas[RB];             // a u of own rows, in both halves
@@ -566,7 +569,7 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
         near_tot = (unsigned long long)fmin(t * 1.000001 * RSUM_SCALE, 1.0e18) + 2ull;
     }
     if (tid == 0) {
-        sflag = 0; vflag = 0;
+        sflag = 0; vflag = 0; wflag = 0;
         if constexpr (CLU) {
             for (int e = 0; e < 2; ++e) {
                 asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&xbar[e])) : "memory");
@@ -996,9 +999,9 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                         ok = bar_wait(smem_addr(&tbar[e]), phase) && ok;
                     }
                     xphase ^= 1u << e;
-                    if (!ok) vflag = 2;
+                    if (!ok) wflag = 1;
                     __syncthreads();
-                    if (vflag) { dead = true; break; }
+                    if (wflag) { dead = true; break; }
                 }
                 if constexpr (CLU && L::TWO_STEP) {
                     const double *src = tbuf + (size_t)(xch & 1) * COLS + j0;

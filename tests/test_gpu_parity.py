@@ -1331,6 +1331,45 @@ def test_kernel_matrix_lanes_whose_potentials_move_fast(oracle, cycles):
     assert err.max() <= 1e-6 * cycles + 2e-6, err
 
 
+@pytest.mark.parametrize("n,m,d", [(150, 60, 5), (130, 100, 5), (70, 200, 5), (300, 300, 5), (300, 200, 64), (300, 500, 64), (600, 520, 64)])
+def test_lanes_of_several_blocks_that_leave_the_band_again_and_again(oracle, n, m, d):
+    # clouds two apart per dimension: some scaling of a column leaves 2^+-30 every four to seven cycles (counted with numpy in
+    # float64), which one warp of one block finds first while others still look at the outcome of the exchange between blocks.
+    # No wait may be reported to have run out, and the bits may not depend on how the cycles are shared out among launches.
+    # (70 x 200 is a lane of one block, which has no exchange.)
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    rng = np.random.default_rng(n + m)
+    W, cycles = 24, 60
+    bf = lambda v: torch.from_numpy(v.astype(np.float32)).bfloat16().float().numpy()
+    x = rng.standard_normal((W, n, d)); y = rng.standard_normal((W, m, d))
+    if d == 64:
+        x /= np.linalg.norm(x, axis=2, keepdims=True); y /= np.linalg.norm(y, axis=2, keepdims=True)
+    x, y = (bf(x), bf(y + 2.0)) if d == 64 else (x.astype(np.float32), (y + 2.0).astype(np.float32))
+    a = rng.uniform(0.1, 1.0, (W, n)); b = rng.uniform(0.1, 1.0, (W, m))
+    eps = np.tile(np.float32([0.002, 0.01, 0.03, 0.05]), W // 4)
+    w = wl.Workload("far apart", x, y, (a / a.sum(1, keepdims=True)).astype(np.float32), (b / b.sum(1, keepdims=True)).astype(np.float32),
+                    eps, 1e-7, cycles, "bf16" if d == 64 else "f32")
+    compute = "tensor" if d == 64 else "mixed"
+    r = run_gpu(w, compute=compute)
+    ref = oracle.solve_batch(w.x[:4], w.y[:4], w.a[:4], w.b[:4], w.eps[:4], w.tol, max_iter=cycles)
+    err = np.maximum(np.abs(r["f"][:4] - ref.f).max(1), np.abs(r["g"][:4] - ref.g).max(1)) / w.eps[:4]
+    # in units of eps: 2^-22 per exponential and cycle remembered; stored products are sums of d fp32 terms, off by up to
+    # d 2^-24 |x| |y| each, twice that in the cost, which a leg (a soft minimum, so never more) hands on in every leg
+    dot = 0.0 if d == 5 else 2.0 * d * 2.0 ** -24 * np.linalg.norm(x[:4], axis=2).max(1) * np.linalg.norm(y[:4], axis=2).max(1) / w.eps[:4]
+    assert (err <= 1e-6 * cycles + 2e-6 + 2 * cycles * dot).all(), err
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    xs, ys = (t(w.x).bfloat16(), t(w.y).bfloat16()) if d == 64 else (t(w.x), t(w.y))
+    for run in (1, 7):
+        sb = B.SinkhornBatch(xs, ys, t(w.a), t(w.b), t(w.eps), w.tol, compute=compute, max_iter=cycles)
+        for _ in range(cycles // run + 1):
+            sb.step(run)
+        assert sb.active() == 0 and sb.check_guards() == -1
+        f, g = sb.potentials(f64=True)
+        np.testing.assert_array_equal(f.cpu().numpy(), r["f"]); np.testing.assert_array_equal(g.cpu().numpy(), r["g"])
+        sb.close()
+
+
 @pytest.mark.parametrize("kw", [dict(W=40, n=100, m=77, d=8), dict(W=24, n=64, m=64, d=2), dict(W=9, n=200, m=256, d=8), dict(W=5, n=300, m=500, d=8)])
 @pytest.mark.parametrize("every,guard", [(1, 0.0), (4, 0.3)])
 def test_static_batches_of_kernel_matrix_lanes_however_they_are_run(kw, every, guard):
