@@ -673,8 +673,8 @@ extern "C" skb_status sinkhorn_batch_step(skb_batch *h, int cycles)
     if (st != SKB_OK) return st;
     cudaError_t e;
     if (cycles_in_one_launch(h)) {
-        for (int left = cycles; left > 0 && !h->finished; left -= MAX_CYCLES_IN_LAUNCH)
-            enqueue_cycles_launch(h, left < MAX_CYCLES_IN_LAUNCH ? left : MAX_CYCLES_IN_LAUNCH);
+        const int longest = h->cfg.mode == SKB_MASKED ? MASK_CYCLES_IN_LAUNCH : MAX_CYCLES_IN_LAUNCH;
+        for (int left = cycles; left > 0 && !h->finished; left -= longest) enqueue_cycles_launch(h, left < longest ? left : longest);
     } else {
         for (int i = 0; i < cycles && !h->finished; ++i) {
             enqueue_cycle(h);
@@ -712,7 +712,7 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
     const long long hard_cap = (long long)h->cfg.max_iter + 4;
     while (!h->finished) {
         const bool multi = cycles_in_one_launch(h);      // may become true as the batch narrows
-        const int chunk_max = scaling ? (masked ? 256 : MAX_CYCLES_IN_LAUNCH) : (multi ? 32 : 16);
+        const int chunk_max = scaling ? (masked ? MASK_CYCLES_IN_LAUNCH : MAX_CYCLES_IN_LAUNCH) : (multi ? 32 : 16);
         NvtxRange nvtx_chunk(multi ? "skb:chunk (cycles in one launch)" : "skb:chunk (launch per leg)");
         if (multi) enqueue_cycles_launch(h, chunk);
         else for (int i = 0; i < chunk; ++i) enqueue_cycle(h);

@@ -47,6 +47,9 @@ constexpr int MAX_CLUSTER_BLOCKS = MAX_CLUSTER_RANKS;   // a lane needs at most 
 // Upper bound on the cycles one multi-cycle launch runs.  Lanes are independent and leave a launch when they pass, so a
 // long launch keeps the SMs full where a series of short ones waits for its slowest lanes after each.
 constexpr int MAX_CYCLES_IN_LAUNCH = 2048;
+// ... and under a logical mask, whose lanes work on until the launch ends, however early they pass: what a caller asks for
+// beyond the last lane's depth costs at most the rest of one launch (launches after it return at once).
+constexpr int MASK_CYCLES_IN_LAUNCH = 256;
 // Picks the variant for a shape (depends on the static shape only, so that every mode
 // and every run of the same batch uses the same reduction order).  Null if unsupported.
 const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_exp, int force_cs, bool spatial);

@@ -1435,6 +1435,24 @@ def test_last_audit_of_a_mask_does_not_depend_on_how_the_cycles_were_run():
 
 
 # ---- large low-dimensional lanes in spatial order ----------------------------------------------------
+def test_a_masks_launches_stay_short_however_many_cycles_are_asked_for():
+    # under a logical mask lanes work until their launch ends: of 4096 cycles asked for, those past the launch in which the last
+    # lane passes must be empty launches.  What a launch ran is not counted (Eq. 6-8 count to the last depth), so the launches are:
+    # one of cycles and its planner for every 256
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("tiny")
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    for mode, most in (("masked", 256), ("masked_exit", 2048), ("active", 2048)):
+        sb = B.SinkhornBatch(t(w.x), t(w.y), t(w.a), t(w.b), t(w.eps), w.tol, mode=mode, max_iter=w.max_iter)
+        before = sb.launch_count()
+        sb.step(4096)
+        assert sb.active() == 0
+        assert sb.launch_count() - before >= 2 * (4096 // most), mode
+        assert sb.stats()["cycles"] == int(sb.depths()[0].max())
+        sb.close()
+
+
 @pytest.mark.parametrize("n,m,d", [(1024, 1024, 3), (1023, 1025, 3), (1055, 64, 2), (31, 1100, 4), (1024, 33, 1), (8193, 40, 3)])
 def test_lanes_in_spatial_order(oracle, n, m, d):
     # sizes around the threshold, ragged boxes of 32, chunks of the ordering, every padded dimension; lanes of
