@@ -211,7 +211,8 @@ void launch_spatial_sort(const Dev &P, const void *x, const void *y, int slot0, 
 {
     const int mx = P.n > P.m ? P.n : P.m;
     const int smem = SORT_CHUNK * (8 + 4 * P.DP);
-    cudaFuncSetAttribute(spatial_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // (the limit for any dimension: another host thread may set it between this and the launch)
+    cudaFuncSetAttribute(spatial_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SORT_CHUNK * (8 + 4 * 4));
     spatial_sort_kernel<<<dim3((mx + SORT_CHUNK - 1) / SORT_CHUNK, count, 2), 1024, smem, st>>>(P, x, y, slot0);
 }
 

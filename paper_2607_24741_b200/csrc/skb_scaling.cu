@@ -48,18 +48,20 @@ void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int wid
     // memory; without a cluster they may wait, and ask for as much as keeps one block too many away.  (No more
     // than that: what is left is the cache that spilled registers live in; with all of it asked for, a solve of 64
     // lanes of 1024 x 1024, d = 512, takes 5.9 ms instead of 5.3.)
-    size_t smem = v->smem(nc);
+    size_t smem = v->smem(nc), most = v->smem(v->cluster ? v->max_blocks : nc);
     if (v->tm_cols && kind != SC_LEG) {
         cudaFuncAttributes fa;
         if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;        // (the caller looks at cudaGetLastError)
         const bool alone = (fa.numRegs + 7) / 8 * 8 * v->threads >= 65536;
         const size_t share = alone ? 0 : v->cluster ? (size_t)SMEM_PER_SM * v->tm_cols / 512 : (size_t)SMEM_PER_SM / (512 / v->tm_cols + 1) + 1024;
         if (share > fa.sharedSizeBytes + smem) smem = share - fa.sharedSizeBytes;
+        if (smem > most) most = smem;
     }
-    // (with the fixed arrays some variants are beyond the 48 KB that need no permission; the attribute belongs
-    // to the current device, so it is set with every launch)
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (nc > MAX_CLUSTER_RANKS) cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    // (with the fixed arrays some variants are beyond the 48 KB that need no permission; the attributes belong to the
+    // current device, so they are set with every launch, to the variant's limits whatever the lane: another
+    // host thread may launch the same variant for lanes of fewer blocks in between)
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (v->max_blocks > MAX_CLUSTER_RANKS) cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nc, width < 1 ? 1 : width);
     cfg.blockDim = dim3(v->threads);

@@ -900,7 +900,8 @@ void launch_gram(const Dev &P, const void *maps, int slot0, int count, cudaStrea
     constexpr int STAGES = 4;
     const auto kernel = update_tc_kernel<STAGES, 128, true>;
     const int smem = (P.d / TC_BK + STAGES) * (int)TC_CHUNK + 1024;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // (the limit for any d: another host thread may set it between this and the launch)
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (512 / TC_BK + STAGES) * (int)TC_CHUNK + 1024);
     const CUtensorMap *tm = reinterpret_cast<const CUtensorMap *>(maps);
     kernel<<<dim3((P.n + TC_BM - 1) / TC_BM, count), TC_THREADS, smem, st>>>(tm[0], tm[1], P, slot0);
 }

@@ -474,6 +474,51 @@ def test_four_batches_running_on_four_streams():
             sb.close()
 
 
+def test_host_threads_that_launch_the_same_kernels_for_different_shapes():
+    # shapes that run the same kernels with different amounts of shared memory (deep lanes by d, lanes of several blocks by
+    # their number, spatial order by the dimension), each from a host thread of its own, again and again: no thread's launch
+    # may fail for what another has set, and every batch ends with the bits it has alone
+    import threading
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    dev = torch.device("cuda:0")
+    t = lambda v: torch.from_numpy(v).to(dev)
+    kws = [dict(name="feature", W=2, n=40, m=100, d=64), dict(name="feature", W=2, n=40, m=100, d=512),
+           dict(name="feature", W=2, n=140, m=300, d=64), dict(name="feature", W=2, n=900, m=300, d=64),
+           dict(name="sensor", W=2, n=140, m=300), dict(name="sensor", W=2, n=1000, m=300),
+           dict(name="registration", W=1, n=1024), dict(name="registration", W=1, n=1024)]
+    work, alone = [], []
+    for i, kw in enumerate(kws):
+        w = wl.make(**kw, max_iter=10)
+        if i == len(kws) - 1:                                          # the same law in the plane
+            w.x, w.y = np.ascontiguousarray(w.x[:, :, :2]), np.ascontiguousarray(w.y[:, :, :2])
+        alone.append(run_gpu(w))
+        x, y = t(w.x), t(w.y)
+        work.append((x.bfloat16(), y.bfloat16(), t(w.a), t(w.b), t(w.eps)) if w.xy_dtype == "bf16" else (x, y, t(w.a), t(w.b), t(w.eps)))
+    torch.cuda.synchronize()
+    failed = []
+
+    def run(i):
+        try:
+            for _ in range(30):
+                sb = B.SinkhornBatch(*work[i], 1e-3, max_iter=10, stream=streams[i])
+                sb.drain()
+                with torch.cuda.stream(streams[i]):
+                    f, _g = sb.potentials(f64=True)
+                streams[i].synchronize()
+                np.testing.assert_array_equal(f.cpu().numpy(), alone[i]["f"])
+                sb.close()
+        except Exception as e:                                          # noqa: BLE001 (reported below, from the main thread)
+            failed.append((i, repr(e)[:300]))
+    streams = [torch.cuda.Stream(dev) for _ in work]
+    threads = [threading.Thread(target=run, args=(i,)) for i in range(len(work))]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not failed, failed
+
+
 # ---- the paper's guard: a stricter threshold inside, the reported tolerance outside ----------------
 @pytest.mark.parametrize("case", list(CASES))
 def test_guarded_thresholds_meet_the_reported_tolerance_without_slack(oracle, case):
