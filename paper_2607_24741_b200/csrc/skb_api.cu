@@ -122,7 +122,9 @@ static const double NEAR_SHARE = 0.75;
 static const double SPATIAL_TOL = 2.0e-3;
 
 // Deep lanes keep their dot products in the workspace and their kernel matrix on chip, up to this size of the
-// products (1024 lanes of 1024 x 1024, 2 % of the card's memory); wider batches form the products in every leg.
+// products (1024 lanes of 1024 x 1024, 2 % of the card's memory); beyond it they are formed in every leg, with other
+// roundings.  Counted over all lanes that the batch can take in, not over its slots: a queue of lanes through a few slots and
+// one batch of all of them run the same arithmetic, so a lane's bits do not depend on how it came in.
 static const size_t DOTS_LIMIT = (size_t)4 << 30;
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -235,7 +237,7 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
         d.boxx = (float *)take(W * 2 * DP * d.nbx * 4); d.boxy = (float *)take(W * 2 * DP * d.nby * 4);
         d.topx[0] = (float *)take(W * d.nbx * 4); d.topx[1] = (float *)take(W * d.nbx * 4); d.topy = (float *)take(W * d.nby * 4);
     }
-    if (tensor && scaling_fits(true, c->n, c->m) && W * np * mp * 4 <= DOTS_LIMIT) {
+    if (tensor && scaling_fits(true, c->n, c->m) && L * np * mp * 4 <= DOTS_LIMIT) {
         d.phi0 = (double *)take(W * np * 8); d.uu[0] = (double *)take(W * np * 8); d.uu[1] = (double *)take(W * np * 8);
         d.gam0 = (double *)take(W * mp * 8); d.vv = (double *)take(W * mp * 8);
         d.dots = (float *)take(W * np * mp * 4);

@@ -1130,6 +1130,46 @@ def test_refill_keeps_the_width_up_and_every_lane_its_own_result(oracle, compute
                              label=f"refilled lanes, {compute}")
 
 
+def _launches_per_step(sb):
+    # a step of one cycle (not a batch's first, which may rank its lanes) is three launches or fewer where the kernel matrix is on
+    # chip, four or more where legs are streamed
+    sb.step(1)
+    before = sb.launch_count()
+    sb.step(1)
+    return sb.launch_count() - before
+
+
+def test_a_deep_lane_has_the_same_bits_in_a_queue_and_in_one_batch_of_all_lanes():
+    # products of deep lanes are stored up to a size, counted over all lanes that a batch can take in: 1025 lanes of
+    # 1024 x 1024 are beyond it, in one batch and as a queue through eight slots
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    gen = torch.Generator(device="cuda:0"); gen.manual_seed(3)
+    W, n, d, S, given = 1025, 1024, 64, 8, 20
+    unit = lambda v: (v / v.norm(dim=2, keepdim=True)).bfloat16()
+    x, y = (unit(torch.randn(W, n, d, generator=gen, device="cuda:0")) for _ in range(2))
+    a = torch.full((W, n), 1.0 / n, device="cuda:0"); eps = torch.full((W,), 0.05, device="cuda:0")
+    kw = dict(max_iter=3, compute="tensor")
+    sb = B.SinkhornBatch(x, y, a, a, eps, 1e-7, **kw)
+    assert _launches_per_step(sb) > 3
+    sb.drain()
+    f, g = (v[:given].cpu().numpy() for v in sb.potentials(f64=True))
+    sb.close()
+    sb = B.SinkhornBatch(x[:S], y[:S], a[:S], a[:S], eps[:S], 1e-7, lane_capacity=W, **kw)
+    assert _launches_per_step(sb) > 3
+    nxt = S
+    while nxt < given:
+        sb.drain()
+        c = min(S, given - nxt)
+        assert sb.refill(x[nxt:nxt + c], y[nxt:nxt + c], a[:c], a[:c], eps[:c]) == nxt
+        nxt += c
+    sb.drain()
+    fq, gq = (v[:given].cpu().numpy() for v in sb.potentials(f64=True))
+    assert sb.check_guards() == -1
+    sb.close()
+    np.testing.assert_array_equal(fq, f); np.testing.assert_array_equal(gq, g)
+
+
 @pytest.mark.parametrize("options", [dict(guard_band=0.5), dict(audit_every=4, guard_band=0.5), dict(profiling=True),
                                      dict(compute="mixed", audit_every=3, guard_band=0.5)],
                          ids=["guard", "grid4_guard", "profiled", "mixed_grid3_guard"])
