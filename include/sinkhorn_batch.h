@@ -118,7 +118,14 @@ typedef struct {
 } skb_config;
 
 /* Bytes of device workspace a batch with this shape, dtype, mode and compute type
- * needs.  Returns 0 if the configuration is invalid. */
+ * needs.  Returns 0 if the configuration is invalid.
+ * Deep lanes on the tensor cores (TENSOR, or AUTO with bf16 inputs) of up to 1024 x 1024 points
+ * (up to 512 columns 1024 rows, up to 256 columns 2048 rows) are given room for their dot products
+ * x_i . y_j, W n m floats, as long as those of all lanes the batch can take in (W, or lane_capacity)
+ * are at most 4 GiB; they are formed once then, and in every leg otherwise.  Both ways agree to
+ * rounding, not bit for bit.  The choice depends on shape, lane count and workspace only: create
+ * also takes a workspace without that room (4 W n m and some 8 W (3 n + 2 m) bytes less, as far as
+ * an automatic batch, which may need float64 coordinates instead, does not need more anyway). */
 size_t sinkhorn_batch_workspace_bytes(const skb_config *cfg);
 
 /*

@@ -161,8 +161,8 @@ static double guard_width(const skb_config *c)
 // Lays the batch's arrays out in the workspace (base may be null: size query only).
 // Every array is followed by a guard strip (GUARD_STRIP_BYTES of a known pattern, see
 // sinkhorn_batch_check_guards); their offsets are listed in *guards.
-// spatial: the batch may keep its lanes in spatial order (SPATIAL_TOL).
-static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool spatial, char *base, Dev *D, size_t *zero_end_out = nullptr,
+// spatial: the batch may keep its lanes in spatial order (SPATIAL_TOL).  dots: there is room for the products of deep lanes.
+static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool spatial, bool dots, char *base, Dev *D, size_t *zero_end_out = nullptr,
                     GuardList *guards = nullptr)
 {
     size_t off = 0;
@@ -237,7 +237,7 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
         d.boxx = (float *)take(W * 2 * DP * d.nbx * 4); d.boxy = (float *)take(W * 2 * DP * d.nby * 4);
         d.topx[0] = (float *)take(W * d.nbx * 4); d.topx[1] = (float *)take(W * d.nbx * 4); d.topy = (float *)take(W * d.nby * 4);
     }
-    if (tensor && scaling_fits(true, c->n, c->m) && L * np * mp * 4 <= DOTS_LIMIT) {
+    if (tensor && dots && scaling_fits(true, c->n, c->m) && L * np * mp * 4 <= DOTS_LIMIT) {
         d.phi0 = (double *)take(W * np * 8); d.uu[0] = (double *)take(W * np * 8); d.uu[1] = (double *)take(W * np * 8);
         d.gam0 = (double *)take(W * mp * 8); d.vv = (double *)take(W * mp * 8);
         d.dots = (float *)take(W * np * mp * 4);
@@ -267,26 +267,31 @@ static const Variant *variant_for(const skb_config *c, int compute, bool spatial
     return choose_variant(c->W, c->n, c->m, c->d, f64, compute == SKB_COMPUTE_MIXED, c->column_split, spatial);
 }
 
-extern "C" size_t sinkhorn_batch_workspace_bytes(const skb_config *cfg)
+// dots = false: the least that create takes (deep lanes then form their products in every leg)
+static size_t workspace_need(const skb_config *cfg, bool dots)
 {
-    std::string why;
-    if (!config_ok(cfg, why)) return 0;
     // an automatic batch may end up with float64 coordinates: size for the larger layout
     if (cfg->compute == SKB_COMPUTE_TENSOR && !tc_eligible(cfg->d, cfg->xy_dtype == SKB_BF16)) return 0;
     const Variant *v = variant_for(cfg, cfg->compute == SKB_COMPUTE_AUTO ? SKB_COMPUTE_MIXED : cfg->compute, false);
     if (!v) return 0;
-    size_t need = carve(cfg, v, cfg->compute == SKB_COMPUTE_TENSOR, false, nullptr, nullptr);
+    size_t need = carve(cfg, v, cfg->compute == SKB_COMPUTE_TENSOR, false, dots, nullptr, nullptr);
     if (cfg->compute == SKB_COMPUTE_AUTO && tc_eligible(cfg->d, cfg->xy_dtype == SKB_BF16)) {
-        const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, false), true, false, nullptr, nullptr);
+        const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, false), true, false, dots, nullptr, nullptr);
         if (t > need) need = t;
     }
     if (cfg->compute == SKB_COMPUTE_AUTO || cfg->compute == SKB_COMPUTE_F32) {
         for (const bool spatial : {false, true}) {           // the tolerance, which decides, is not known here
-            const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, spatial), false, spatial, nullptr, nullptr);
+            const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, spatial), false, spatial, false, nullptr, nullptr);
             if (t > need) need = t;
         }
     }
     return need;
+}
+
+extern "C" size_t sinkhorn_batch_workspace_bytes(const skb_config *cfg)
+{
+    std::string why;
+    return config_ok(cfg, why) ? workspace_need(cfg, true) : 0;
 }
 
 static skb_status fail(skb_batch *h, skb_status st, const std::string &msg)
@@ -326,11 +331,12 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     if (cfg->compute == SKB_COMPUTE_TENSOR && !can_tensor)
         return fail(nullptr, SKB_ERR_SHAPE, "the tensor-core path needs bf16 x, y and d a multiple of 64 with 64 <= d <= 512");
     size_t zero_end = 0;
-    carve(cfg, var_big, false, false, nullptr, nullptr, &zero_end);
-    const size_t need = sinkhorn_batch_workspace_bytes(cfg);
+    carve(cfg, var_big, false, false, false, nullptr, nullptr, &zero_end);
+    const size_t need = workspace_need(cfg, true);
+    const bool dots = cfg->workspace_bytes >= need;
     if (!cfg->workspace) return fail(nullptr, SKB_ERR_WORKSPACE, "workspace is null");
     if (((uintptr_t)cfg->workspace & 255u) != 0) return fail(nullptr, SKB_ERR_WORKSPACE, "workspace must be 256-byte aligned");
-    if (cfg->workspace_bytes < need) {
+    if (!dots && cfg->workspace_bytes < workspace_need(cfg, false)) {
         char buf[128];
         snprintf(buf, sizeof(buf), "workspace too small: %zu bytes given, %zu needed", cfg->workspace_bytes, need);
         return fail(nullptr, SKB_ERR_WORKSPACE, buf);
@@ -345,7 +351,7 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     h->lanes_used = cfg->W; h->enqueued_at_refill = 0;
     for (int i = 0; i < SKB_N_PHASES; ++i) h->phase_ms[i] = 0.f;
     h->guards.count = 0;
-    carve(cfg, var, h->tensor, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+    carve(cfg, var, h->tensor, false, dots, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
     h->dev.tol_stop = (double)tol;
     h->dev.tol_screen = cfg->tol_screen > 0.0f ? (double)cfg->tol_screen : (double)tol;
     cudaError_t e;
@@ -394,13 +400,13 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
                          cfg->cost_form == 0 && cfg->column_split == 0;
         if (automatic && (wide_radius || h->f32_on_chip)) {
             h->var = var_big;
-            carve(cfg, var_big, false, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+            carve(cfg, var_big, false, false, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
         } else if (automatic && can_tensor) {
             h->tensor = true;
-            carve(cfg, var, true, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+            carve(cfg, var, true, false, dots, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
         } else if (near_shaped && radius <= FORM_DIFF_RADIUS && h->h_ctl[1].near_kept <= NEAR_SHARE * NEAR_PAIRS * cfg->W) {
             h->var = var_near;
-            carve(cfg, var_near, false, true, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+            carve(cfg, var_near, false, true, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
         }
         h->dev.tol_stop = ts; h->dev.tol_screen = tsc;
     }
@@ -961,9 +967,10 @@ extern "C" skb_status sinkhorn_batch_solve_host(const void *x, const void *y, co
                                                 float *r_row, float *r_col, long long *slots, int *cycles)
 {
     if (!x || !y || !a || !b || !eps || !cfg) return fail(nullptr, SKB_ERR_NULL, "x, y, a, b, eps and cfg are required");
-    const size_t core = sinkhorn_batch_workspace_bytes(cfg);
+    size_t core = sinkhorn_batch_workspace_bytes(cfg);
     if (core == 0) return fail(nullptr, SKB_ERR_SHAPE, "configuration rejected");
-    const HostStage s = host_stage(cfg, core);
+    HostStage s = host_stage(cfg, core);
+    if (cfg->workspace_bytes < s.end) { core = workspace_need(cfg, false); s = host_stage(cfg, core); }      // (as create)
     if (!cfg->workspace || cfg->workspace_bytes < s.end) return fail(nullptr, SKB_ERR_WORKSPACE, "workspace too small for the host-buffer call");
     char *base = (char *)cfg->workspace;
     cudaStream_t st = (cudaStream_t)cfg->stream;

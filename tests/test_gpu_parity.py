@@ -1170,6 +1170,61 @@ def test_a_deep_lane_has_the_same_bits_in_a_queue_and_in_one_batch_of_all_lanes(
     np.testing.assert_array_equal(fq, f); np.testing.assert_array_equal(gq, g)
 
 
+def test_deep_lanes_in_a_workspace_without_room_for_their_products(oracle):
+    # a workspace smaller by the products is taken, on device and host buffers (the products are formed in every leg then); one
+    # that lacks more is refused
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("feature", W=3, n=200, m=260, d=64)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    x, y, a, b, eps = t(w.x).bfloat16(), t(w.y).bfloat16(), t(w.a), t(w.b), t(w.eps)
+    dots, more = 4 * 3 * 200 * 260, 8 * 3 * (3 * 200 + 2 * 260)
+    stream = torch.cuda.current_stream().cuda_stream
+    cfg = B.make_config(3, 200, 260, 64, bf16=True, compute="tensor", stream=stream)
+    need = B.sinkhorn_batch_workspace_bytes(cfg)
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda:0")
+    cfg.workspace = ws.data_ptr()
+    cfg.workspace_bytes = need - dots - more - 8192
+    with pytest.raises(B.SkbError):
+        B.sinkhorn_batch_create(x, y, a, b, eps, w.tol, cfg)
+    full = run_gpu(w, compute="tensor")
+    out = {}
+    for room in (need, need - dots):
+        cfg.workspace_bytes = room
+        h = B.sinkhorn_batch_create(x, y, a, b, eps, w.tol, cfg)
+        before = ctypes.c_longlong(0); after = ctypes.c_longlong(0)
+        B.sinkhorn_batch_step(h, 1)
+        B.lib.sinkhorn_batch_launch_count(h, ctypes.byref(before))
+        B.sinkhorn_batch_step(h, 1)
+        B.lib.sinkhorn_batch_launch_count(h, ctypes.byref(after))
+        assert (after.value - before.value <= 3) == (room == need)
+        B.sinkhorn_batch_drain(h)
+        f = torch.zeros(3, 200, dtype=torch.float64, device="cuda:0"); g = torch.zeros(3, 260, dtype=torch.float64, device="cuda:0")
+        assert B.lib.sinkhorn_batch_potentials_f64(h, B._ptr(f), B._ptr(g)) == 0
+        depth = torch.zeros(3, dtype=torch.int32, device="cuda:0"); status = torch.zeros_like(depth)
+        assert B.lib.sinkhorn_batch_depths(h, B._ptr(depth), B._ptr(status)) == 0
+        bad = ctypes.c_int(-2)
+        assert B.lib.sinkhorn_batch_check_guards(h, ctypes.byref(bad)) == 0 and bad.value == -1
+        B.sinkhorn_batch_destroy(h)
+        out[room] = f.cpu().numpy(), g.cpu().numpy(), depth.cpu().numpy()
+    np.testing.assert_array_equal(out[need][0], full["f"]); np.testing.assert_array_equal(out[need][2], full["depth"])
+    np.testing.assert_array_equal(out[need - dots][2], full["depth"])
+    assert pot_err(*out[need - dots][:2], full["f"], full["g"], w.eps).max() <= 5e-6      # both within 3e-6 of the oracle's
+    # host buffers
+    host = B.sinkhorn_batch_host_workspace_bytes(cfg)
+    ws = torch.empty(host, dtype=torch.uint8, device="cuda:0")
+    cfg.workspace = ws.data_ptr()
+    hx, hy, ha, hb, he = (v.cpu().contiguous() for v in (x, y, a, b, eps))
+    ptr = lambda v: ctypes.c_void_p(v.data_ptr())
+    for room, want in ((host, out[need]), (host - dots, out[need - dots])):
+        cfg.workspace_bytes = room
+        f = torch.zeros(3, 200); g = torch.zeros(3, 260)
+        rc = B.lib.sinkhorn_batch_solve_host(ptr(hx), ptr(hy), ptr(ha), ptr(hb), ptr(he), ctypes.c_float(w.tol), ctypes.byref(cfg),
+                                             ptr(f), ptr(g), None, None, None, None, None, None)
+        assert rc == 0
+        np.testing.assert_array_equal(f.numpy(), want[0].astype(np.float32)); np.testing.assert_array_equal(g.numpy(), want[1].astype(np.float32))
+
+
 @pytest.mark.parametrize("options", [dict(guard_band=0.5), dict(audit_every=4, guard_band=0.5), dict(profiling=True),
                                      dict(compute="mixed", audit_every=3, guard_band=0.5)],
                          ids=["guard", "grid4_guard", "profiled", "mixed_grid3_guard"])
