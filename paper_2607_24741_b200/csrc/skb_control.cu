@@ -751,7 +751,10 @@ __device__ __forceinline__ void emit_move_one(const Dev &P, const Ctl &c, const 
             seg_end[ns++] = run;
         };
         const int np_ = ep ^ 1;   // buffer that holds the survivors' current row potentials
-        if (P.tensor) {
+        if (P.dots) {
+            // the tiled copies stay behind: nothing reads those of a lane whose products are stored
+            add(P.dots, (size_t)P.np * P.mp * 4);
+        } else if (P.tensor) {
             add(P.xb, (size_t)((P.n + 127) / 128) * P.d * 256);      // tiled copies: 128-point tiles x d bf16
             add(P.yb, (size_t)((P.m + 127) / 128) * P.d * 256);
         } else {
@@ -766,7 +769,6 @@ __device__ __forceinline__ void emit_move_one(const Dev &P, const Ctl &c, const 
         add(P.la2, (size_t)P.np * 8); add(P.lb2, (size_t)P.mp * 8);
         add(P.wa, (size_t)P.np * 8); add(P.wb, (size_t)P.mp * 8);
         add(P.phi[np_], (size_t)P.np * 8);
-        add(P.dots, (size_t)P.np * P.mp * 4);
         if (P.phi0) {                                                 // lanes on the scaling kernel have no streamed terms
             add(P.phi0, (size_t)P.np * 8); add(P.gam0, (size_t)P.mp * 8);
             add(P.uu[np_], (size_t)P.np * 8); add(P.vv, (size_t)P.mp * 8);
@@ -1087,9 +1089,8 @@ static size_t lane_state_bytes(const Dev &P)
 {
     const size_t ts = P.compute_f64 ? 8 : 4;
     size_t coords = (size_t)P.DP * (P.np + P.mp) * ts;
-    if (P.tensor) coords = ((size_t)((P.n + 127) / 128) + (size_t)((P.m + 127) / 128)) * P.d * 256;
+    if (P.tensor) coords = P.dots ? (size_t)P.np * P.mp * 4 : ((size_t)((P.n + 127) / 128) + (size_t)((P.m + 127) / 128)) * P.d * 256;
     if (P.guard > 0.0) coords += P.xraw_stride + P.yraw_stride;
-    if (P.dots) coords += (size_t)P.np * P.mp * 4;
     return coords + (size_t)(P.np + P.mp) * (4 * 8 + (P.phi0 ? 16 : 2 * ts) + 8);
 }
 // When even the retirement of every lane at once would move little (narrow batches of small

@@ -1225,6 +1225,49 @@ def test_deep_lanes_in_a_workspace_without_room_for_their_products(oracle):
         np.testing.assert_array_equal(f.numpy(), want[0].astype(np.float32)); np.testing.assert_array_equal(g.numpy(), want[1].astype(np.float32))
 
 
+@pytest.mark.parametrize("n,m,d,kw", [(101, 90, 64, {}), (140, 131, 64, {}), (250, 255, 128, {}), (300, 200, 320, {}), (333, 300, 64, {}), (300, 600, 64, {}),
+                                      (140, 131, 64, dict(guard_band=0.3, audit_every=3)), (333, 300, 64, dict(profiling=True))])
+def test_deep_lanes_refilled_after_compaction(oracle, n, m, d, kw):
+    # lanes with stored products come into slots that others have left or have been moved out of, in one block and in clusters
+    # of several: every lane must end as in one batch of all of them, bit for bit
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    W, S = 22, 7
+    w = wl.make("feature", W=W, n=n, m=m, d=d, max_iter=300)
+    w.eps = np.random.default_rng(5).permutation(np.geomspace(0.03, 0.5, W)).astype(np.float32)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    x, y, a, b, eps = t(w.x).bfloat16(), t(w.y).bfloat16(), t(w.a), t(w.b), t(w.eps)
+    profiling = kw.get("profiling", False)
+    kw = {k: v for k, v in kw.items() if k != "profiling"}
+    ref = run_gpu(w, **kw)
+    assert ref["arith"] == "tensor" and len(set(ref["depth"])) > 5
+    sb = B.SinkhornBatch(x[:S], y[:S], a[:S], b[:S], eps[:S], w.tol, max_iter=w.max_iter, lane_capacity=W, **kw)
+    sb.set_profiling(profiling)
+    nxt, partly = S, 0
+    while nxt < W:
+        sb.step(5)
+        left = sb.active()
+        c = min(S - left, W - nxt, 3)
+        if c > 0:
+            partly += left > 0
+            assert sb.refill(x[nxt:nxt + c], y[nxt:nxt + c], a[nxt:nxt + c], b[nxt:nxt + c], eps[nxt:nxt + c]) == nxt
+            nxt += c
+    assert partly >= 3                                                  # refills next to lanes that were still running
+    sb.drain()
+    f, g = sb.potentials(f64=True); depth, status = sb.depths(); rr, _ = sb.residuals()
+    assert sb.check_guards() == -1
+    sb.close()
+    if "audit_every" not in kw:                                         # (a lane's audits are on the batch's grid)
+        np.testing.assert_array_equal(depth.cpu().numpy(), ref["depth"]); np.testing.assert_array_equal(status.cpu().numpy(), ref["status"])
+        np.testing.assert_array_equal(f.cpu().numpy(), ref["f"]); np.testing.assert_array_equal(g.cpu().numpy(), ref["g"])
+        np.testing.assert_array_equal(rr.cpu().numpy(), ref["r_row"])
+        check_against_oracle(oracle, w, ref, range(0, W, 3), pot_tol=POT_TOL_F32, exact_depth=False, floor=MARGIN_AUTO,
+                             label=f"refilled deep lanes, {n} x {m}")
+    else:
+        late = depth.cpu().numpy() - ref["depth"]
+        assert (np.abs(late) < kw["audit_every"]).all() and (status.cpu().numpy() == ref["status"]).all(), late
+
+
 @pytest.mark.parametrize("options", [dict(guard_band=0.5), dict(audit_every=4, guard_band=0.5), dict(profiling=True),
                                      dict(compute="mixed", audit_every=3, guard_band=0.5)],
                          ids=["guard", "grid4_guard", "profiled", "mixed_grid3_guard"])
