@@ -569,11 +569,10 @@ def test_tensor_core_modes_and_compaction(oracle):
 
 @pytest.mark.parametrize("kw", [dict(W=5, n=300, m=520, d=320), dict(W=2, n=140, m=2400, d=512)])
 def test_tensor_core_pair_kernel_shapes_and_modes(oracle, kw):
-    # d > 256 runs the persistent CTA-pair kernel.  These shapes give it an odd number of row blocks
-    # (one CTA of the last pair has no rows), a ring shorter than six stages (d = 320), more column
-    # tiles than units (2400 columns) and, with so few lanes, row blocks whose column tiles are shared
-    # out among many clusters.  Whatever the split, the bits must not depend on it: ACTIVE (shrinking
-    # batch) and MASKED (fixed batch) must agree exactly.
+    # 140 x 2400 streams its legs through the persistent CTA-pair kernel (d > 256): an odd number of row blocks
+    # (one CTA of the last pair has no rows), more column tiles than units and, with so few lanes, row blocks whose
+    # column tiles are shared out among many clusters.  300 x 520 stores its products and runs on chip.
+    # Whatever the split, the bits must not depend on it: ACTIVE (shrinking batch) and MASKED (fixed batch) must agree exactly.
     w = wl.make("feature", **kw)
     W = w.shape[0]
     ra = run_gpu(w, mode="active", compute="tensor")
@@ -592,8 +591,8 @@ def test_tensor_core_pair_kernel_shapes_and_modes(oracle, kw):
 
 
 def test_tensor_core_pair_kernel_many_small_lanes(oracle):
-    # many more work units than clusters: every cluster walks several segments of different lanes,
-    # retirements move the tiled operand copies, and the column check visits a few flagged lanes
+    # many lanes with stored products, on chip: retirements move the products, and a few lanes are flagged at a time
+    # (the pair kernel on these shapes: test_tensor_core_legs_that_stream)
     w = wl.make("feature", W=150, n=130, m=140, d=320)
     r = run_gpu(w, mode="active", compute="tensor")
     lanes = [0, 1, 73, 74, 75, 148, 149] + list(range(9, 150, 29))
@@ -602,6 +601,47 @@ def test_tensor_core_pair_kernel_many_small_lanes(oracle):
     check_accounting(oracle, r, 150, "active")
     rm = run_gpu(w, mode="masked", compute="tensor")
     np.testing.assert_array_equal(rm["depth"], r["depth"]); np.testing.assert_array_equal(rm["f"], r["f"])
+
+
+# Deep lanes whose legs are streamed by the tensor-core kernels: lanes too large for their products to be stored, and small ones in
+# a workspace that has no room for those.  d <= 256: one CTA per row block; beyond: persistent CTA pairs, with an odd number of row
+# blocks (300, 40: a CTA of the last pair without rows), a ring shorter than six stages (d = 320), more column tiles than units
+# (2400 columns), few lanes (a row block's column tiles shared out among clusters) and many (every cluster walks several segments
+# of different lanes; retirements move the tiled operand copies; the column check visits a few flagged lanes).
+@pytest.mark.parametrize("roomy,kw", [
+    (True, dict(W=2, n=1100, m=1030, d=64)), (True, dict(W=2, n=70, m=1101, d=128)), (True, dict(W=2, n=1029, m=600, d=256)),
+    (True, dict(W=2, n=2049, m=90, d=192)), (True, dict(W=2, n=1300, m=1027, d=320)), (True, dict(W=3, n=40, m=2400, d=512)),
+    (False, dict(W=3, n=200, m=333, d=64)), (False, dict(W=6, n=256, m=256, d=128)), (False, dict(W=2, n=129, m=640, d=256)),
+    (False, dict(W=5, n=300, m=520, d=320)), (False, dict(W=3, n=1, m=129, d=64)), (False, dict(W=3, n=129, m=1, d=512)),
+    (False, dict(W=150, n=130, m=140, d=320)), (False, dict(W=150, n=130, m=140, d=128))])
+def test_tensor_core_legs_that_stream(oracle, monkeypatch, roomy, kw):
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    if not roomy:
+        whole = B.sinkhorn_batch_workspace_bytes
+        monkeypatch.setattr(B, "sinkhorn_batch_workspace_bytes", lambda cfg: whole(cfg) - 4 * cfg.W * cfg.n * cfg.m)
+    w = wl.make("feature", **kw, max_iter=150)
+    W = w.shape[0]
+    if W > 2:
+        w.eps = (w.eps * np.linspace(1.0, 3.0, W)).astype(np.float32)      # lanes leave at different depths
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    sb = B.SinkhornBatch(t(w.x).bfloat16(), t(w.y).bfloat16(), t(w.a), t(w.b), t(w.eps), w.tol, compute="tensor", max_iter=w.max_iter)
+    assert _launches_per_step(sb) > 3                                       # legs are streamed
+    sb.close()
+    ra = run_gpu(w, compute="tensor")
+    rm = run_gpu(w, mode="masked", compute="tensor")
+    np.testing.assert_array_equal(ra["depth"], rm["depth"])
+    np.testing.assert_array_equal(ra["f"], rm["f"]); np.testing.assert_array_equal(ra["g"], rm["g"])
+    lanes = range(W) if W < 10 else [0, 1, 73, 74, 75, 148, 149] + list(range(9, 150, 29))
+    check_against_oracle(oracle, w, ra, lanes, pot_tol=POT_TOL_F32, exact_depth=False, floor=MARGIN_AUTO,
+                         label=f"tensor cores, streamed, {kw}")
+    check_accounting(oracle, ra, W, "active")
+    rs = run_gpu(w, mode="static", compute="tensor")
+    np.testing.assert_array_equal(ra["depth"], rs["depth"])
+    check_accounting(oracle, rs, W, "static")
+    rx = run_gpu(w, mode="masked_exit", compute="tensor")                   # frozen lanes skipped, same bits
+    np.testing.assert_array_equal(rx["f"], rm["f"]); np.testing.assert_array_equal(rx["g"], rm["g"])
+    assert rx["stats"]["slots"] == ra["stats"]["slots"]
 
 
 def test_tensor_core_request_on_ineligible_input_is_refused():
