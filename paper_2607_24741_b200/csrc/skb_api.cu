@@ -571,16 +571,23 @@ static bool cycles_in_one_launch(const skb_batch *h)
     return narrow_lanes(h, h->var);
 }
 
+// Cycles of a launch from which on its lanes' order counts: depths of a batch differ by hundreds of cycles.
+static const int RANKED_CYCLES = 256;
 // `cycles` cycles in one launch (1 <= cycles <= MAX_CYCLES_IN_LAUNCH): lanes that pass inside it write their own
 // outputs; the planner accounts for every cycle of the launch and fills the holes.
 static void enqueue_cycles_launch(skb_batch *h, int cycles)
 {
     const int w = h->known_width;
-    // A batch of more lanes than run at a time starts the ones with the smallest eps first: they need the most cycles
-    // as a rule, and one that starts last runs alone in the end (sweep workload: 10.8 -> 9.0 ms).  First launch only (the
-    // list lies where the planner keeps one later), and up to a width whose ranking is cheap.
+    // A wide batch starts the lanes with the smallest eps first: they need the most cycles as a rule, and one that starts last
+    // runs alone in the end, or beside others as deep on its SM.  First launch only (the list lies where the planner
+    // keeps one later), if it is long enough for lanes to leave at different times: ranking takes 100 us for 4000 lanes, which
+    // a caller of one cycle would pay for nothing.  From one and a half blocks an SM on.  A solve without -> with, laws with
+    // eps spread over a factor of 5 to 25: 149 lanes of 64 x 128 1433 -> 1485 us, 10 of 1024 x 1024 (160 blocks) 849 -> 870,
+    // 200 of 256 x 256 1522 -> 1523, 64 of 512 x 512 (256 blocks) 2232 -> 1795, 300 of 64 x 64 896 -> 838, of 256 x 256 2212 -> 1624,
+    // 1200 of 128 x 128 2540 -> 1745, 4000 of 64 x 64 2617 -> 2255.
     h->dev.order = nullptr;
-    if (h->dev.phi0 && h->enqueued == 0 && w == h->cfg.W && w <= 4096 && (long long)w * scaling_blocks(h->dev) > 148) {
+    if (h->dev.phi0 && h->enqueued == 0 && w == h->cfg.W && w <= 4096 && cycles >= RANKED_CYCLES &&
+        2ll * w * scaling_blocks(h->dev) >= 3 * 148) {
         launch_order(h->dev, h->dev.fill_list, h->stream);
         h->dev.order = h->dev.fill_list;
         h->launches += 1;

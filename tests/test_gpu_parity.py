@@ -1658,6 +1658,27 @@ def test_last_audit_of_a_mask_does_not_depend_on_how_the_cycles_were_run():
 
 
 # ---- large low-dimensional lanes in spatial order ----------------------------------------------------
+def test_lanes_are_ranked_for_long_launches_of_wide_batches_only():
+    # the ranking is one launch more, before a batch's first cycles; the results do not depend on it
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    for W, ranked in ((221, 0), (222, 1)):
+        w = wl.make("sweep", W=W, n=20, m=30, d=4, max_iter=300)
+        out = []
+        for cycles, more in ((1, 0), (255, 0), (256, ranked)):
+            sb = B.SinkhornBatch(t(w.x), t(w.y), t(w.a), t(w.b), t(w.eps), w.tol, max_iter=w.max_iter)
+            count = [sb.launch_count()]
+            for k in (cycles, cycles):
+                sb.step(k)
+                count.append(sb.launch_count())
+            assert count[1] - count[0] - (count[2] - count[1]) == more, (W, cycles, count)
+            sb.drain()
+            out.append(sb.potentials(f64=True)[0].cpu().numpy())
+            sb.close()
+        np.testing.assert_array_equal(out[1], out[0]); np.testing.assert_array_equal(out[2], out[0])
+
+
 def test_a_masks_launches_stay_short_however_many_cycles_are_asked_for():
     # under a logical mask lanes work until their launch ends: of 4096 cycles asked for, those past the launch in which the last
     # lane passes must be empty launches.  What a launch ran is not counted (Eq. 6-8 count to the last depth), so the launches are:
