@@ -236,12 +236,15 @@ class Runner:
         g_ms = sb.profile_update(leg=1, reps=3)
         arith = sb.arithmetic()
         sb.close()
-        # which kernel the legs ran: lanes of up to about a thousand points keep their kernel matrix on chip; lanes in
-        # spatial order were put into it by a launch of their own at create, after one that estimated its worth
-        if arith == "tensor":
-            on_chip = n <= 1024 and m <= 1024 and W * n * m <= 1 << 30
-        else:
-            on_chip = (arith == "mixed" or (arith == "f32" and self.args.compute == "auto")) and d <= 32 and m <= 512 and n <= (1024 if m <= 128 or m > 256 else 512)
+        # which kernel the legs ran: under a logical mask only lanes whose kernel matrix stays on chip run a cycle in one
+        # launch beside the planner's; lanes in spatial order were put into it by a launch of their own at create, after
+        # one that estimated its worth
+        masked = self.batch("masked")
+        masked.step(1)
+        before = masked.launch_count()
+        masked.step(1)
+        on_chip = masked.launch_count() - before <= 2
+        masked.close()
         spatial = False
         if arith == "f32":
             plain = self.batch("static", column_split=1)
@@ -270,8 +273,7 @@ class Runner:
             for cycles in (64, 192):
                 best = None
                 for _ in range(4):
-                    sb = self.B.SinkhornBatch(self.x, self.y, self.a, self.b, self.eps, 1e-12, mode="active", max_iter=self.w.max_iter,
-                                              compute="tensor" if arith == "tensor" else self.args.compute)
+                    sb = self.batch("active", audit_every=1 << 20)
                     sb.step(64)
                     e0, e1 = self.torch.cuda.Event(enable_timing=True), self.torch.cuda.Event(enable_timing=True)
                     e0.record(); sb.step(cycles); e1.record()
