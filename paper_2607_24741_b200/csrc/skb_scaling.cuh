@@ -144,7 +144,12 @@ struct ScalingShape {
     __host__ __device__ static constexpr int owner_bits(int nc) { return nc >= 16 ? 4 : (nc >= 8 ? 3 : 2); }
     static constexpr int SHARE = 32 / RW;                            // threads that end up with the same row's sum
     static constexpr int BLOCKS = TM ? 512 / TM_COLS : (CL * RW >= 128 ? 256 : 512) / THREADS;   // registers: 255 / 128 a thread
-    static constexpr int LEG_BLOCKS = 512 / THREADS;                 // launches of one leg do not hold K: 128
+    // Launches of one leg do not hold K: 128 registers.  Lanes of 512 columns and more, whose G rows of distances are 64 registers
+    // and up, form their entries in a loop and take 255: unrolled, the entries' instructions run once and are
+    // fetched for longer, and at 128 registers they spill (f-leg of 64 lanes of 1024 x 1024 1224 -> 310 us, of 256 lanes of
+    // 512 x 512, d = 15, 344 -> 298 us; narrower lanes are faster unrolled: 1024 of 256 x 256 119 against 150 us).
+    static constexpr bool LEG_ROLLED = CL >= 16;
+    static constexpr int LEG_BLOCKS = (LEG_ROLLED ? 256 : 512) / THREADS;
     static constexpr int FP32_COLS = CL <= 4 ? 8 : 32;               // columns a row's sum holds before it becomes float64
     static constexpr int FP32_WARPS = CL >= 8 && RW <= 16 ? 2 : 1;   // warps' column parts added in fp32 (at most 32 rows)
     static_assert(RW >= 8 && RW <= 32 && CL >= 2 && CL <= 32, "unsupported tile");
@@ -467,7 +472,7 @@ __global__ void __launch_bounds__(32 * NW, (KIND == SC_LEG ? ScalingShape<NW, CL
 scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
 {
     typedef ScalingShape<NW, CL, RW, TMEM> L;
-    constexpr bool LEG = KIND == SC_LEG, catch_up = KIND == SC_CATCH_UP, TM = TMEM && !LEG;
+    constexpr bool LEG = KIND == SC_LEG, ROLLED = LEG && L::LEG_ROLLED, catch_up = KIND == SC_CATCH_UP, TM = TMEM && !LEG;
     constexpr int THREADS = L::THREADS, COLS = L::COLS, RB = L::RB, NQ = L::NQ, SHARE = L::SHARE;
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -637,6 +642,13 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                 pass(g + 1, rb);
                 if (g + 2 < NG) arrive(ra);
             }
+        } else if constexpr (ROLLED) {
+#pragma unroll 1
+            for (int r = 0; r < RW; r += L::G) {
+                u64 kk[L::G][CL / 2];
+                form(r / L::G, kk);
+                use(r, kk);
+            }
         } else {
 #pragma unroll
             for (int r = 0; r < RW; r += L::G) {
@@ -658,9 +670,14 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
     auto col_parts = [&]() {
         // (two sums of half the rows each where a warp has 32: shorter sums, smaller errors)
         constexpr int NA = RW > 16 ? 2 : 1;
+        static_assert(!ROLLED || NA == 1, "a rolled loop has one set of sums");
         u64 acc[NA][CL / 2];
+        if constexpr (ROLLED) {
+#pragma unroll
+            for (int h = 0; h < CL / 2; ++h) acc[0][h] = 0ull;
+        }
         each_rows([&](const int r, const u64 (&kk)[L::G][CL / 2]) {
-            const int e = r / (RW / NA), first = r % (RW / NA) == 0;
+            const int e = ROLLED ? 0 : r / (RW / NA), first = !ROLLED && r % (RW / NA) == 0;
 #pragma unroll
             for (int q = 0; q < L::G; q += 2) {
                 const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(uas + warp * RW + ((r + q) ^ perm));
