@@ -267,21 +267,26 @@ class Runner:
         dtype = {"f32": "f32", "mixed": "f64 exponents / f32 exp", "f64": "f64",
                  "tensor": "bf16 (f32 accumulate, f32 exp)"}[arith]
         if on_chip:
-            # a solve runs whole cycles in one launch: time per cycle at full width, from launches of 64 and 192
-            # cycles that no lane leaves; per pair and cycle one fp32 multiply-add in each leg
+            # a solve runs whole cycles in one launch: time per cycle at full width, from two launches of cycles that
+            # no lane leaves; per pair and cycle one fp32 multiply-add in each leg.  Without audits and far from its
+            # tolerance, where a lane would take the audit's path in every cycle; so no more cycles than a few times a
+            # solve's, whose fast lanes reach a residual of zero.  (The matrix of fp32 lanes is formed from float64
+            # coordinates, as in mixed arithmetic.)
+            short = 64 if self.solve("active", collect=True)["cycles"] >= 192 else 4
             ms = []
-            for cycles in (64, 192):
+            for cycles in (short, 3 * short):
                 best = None
                 for _ in range(4):
-                    sb = self.batch("active", audit_every=1 << 20)
-                    sb.step(64)
+                    sb = self.B.SinkhornBatch(self.x, self.y, self.a, self.b, self.eps, 1e-12, max_iter=self.w.max_iter,
+                                              compute="tensor" if arith == "tensor" else "mixed", guard_band=-1.0, audit_every=1 << 20)
+                    sb.step(2)
                     e0, e1 = self.torch.cuda.Event(enable_timing=True), self.torch.cuda.Event(enable_timing=True)
                     e0.record(); sb.step(cycles); e1.record()
                     self.torch.cuda.synchronize()
                     sb.close()
                     best = e0.elapsed_time(e1) if best is None else min(best, e0.elapsed_time(e1))
                 ms.append(best)
-            c_ms = (ms[1] - ms[0]) / 128
+            c_ms = (ms[1] - ms[0]) / (2 * short)
             fma_peak = SM_COUNT * FP32_LANES * f_hz
             fma = 2.0 * pairs / (c_ms * 1e-3)
             r = {"bound": "latency", "kernel": "scaling_kernel (one cycle of a launch of many, full width)", "arithmetic": arith,
