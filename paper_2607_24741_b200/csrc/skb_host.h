@@ -81,8 +81,8 @@ void launch_prep_near(const Dev &P, const void *x, const void *y, const float *a
 void launch_near_tops(const Dev &P, cudaStream_t st);
 int launch_near(const Dev &P, int leg, int width, cudaStream_t st);     // 1: the guard band's pool rode in a column-check launch
 int guard_pool_rows(int per_row, bool on, int lanes);
-// lanes of mixed arithmetic small enough for their kernel matrix to stay on chip: whole cycles, or one leg as a
-// launch of its own
+// lanes small enough for their kernel matrix to stay on chip (dots: deep lanes, formed from stored dot products): whole
+// cycles, or one leg as a launch of its own
 bool scaling_fits(bool dots, int n, int m);
 enum ScalingKind : int { SC_CYCLES, SC_CATCH_UP, SC_LEG };      // see scaling_kernel; `leg` counts for SC_LEG only
 void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int width, cudaStream_t st);

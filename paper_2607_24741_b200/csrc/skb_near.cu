@@ -28,7 +28,7 @@
 // What bounds it: instruction issue and the latency of a box's chain (load, offset, multiply-adds, ex2, sums); the
 // special-function unit is about half busy.  Registration workload at 32 lanes of 8192 points: a fifth of the
 // pairs is kept (an eighth would be with exact distances), f-leg 610 -> 213 us, g-leg 610 -> 230 us, solve
-// 376 -> 144 ms; one lane of 4096 points 22.7 -> 14.5 ms.  Steps on the way, f / g: Hilbert curve instead of the k-d
+// 376 -> 140 ms; one lane of 4096 points 22.7 -> 15 ms.  Steps on the way, f / g: Hilbert curve instead of the k-d
 // tree, tiles shared by the block, expanded form 280 / 300; a warp's own 16 rows, columns through L1 216 / 290 (groups
 // with outliers keep one warp of a block busy); all warps on every group 258 / 258; 32 rows to a group, four to a
 // thread, columns by cp.async 213 / 230.  Two loads ahead in registers, 16 rows at four to a thread: slower (307, 268).

@@ -1,4 +1,4 @@
-// Kernel matrices on chip: the variants for mixed arithmetic, the choice of a variant and the launch.
+// Kernel matrices on chip: the variants formed from float64 coordinates, the choice of a variant and the launch.
 #include "skb_scaling.cuh"
 
 namespace skb {

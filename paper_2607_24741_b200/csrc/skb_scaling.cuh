@@ -1,4 +1,5 @@
-// Small lanes in mixed arithmetic: the lane's kernel matrix is formed once and kept in registers.
+// Lanes whose kernel matrix stays on chip: formed once per launch, kept in registers or in tensor memory.  Lanes of mixed and,
+// under the automatic choice, fp32 arithmetic (exponents from float64 coordinates) and deep lanes (from stored dot products).
 //
 // With potentials (phi0, gam0) absorbed into the matrix,
 //     K_ij = 2^(phi0_i + gam0_j - s C_ij) / (a_i b_j),      phi = phi0 + log2 u,   gam = gam0 + log2 v,
@@ -18,8 +19,8 @@
 // of them: with a_i alone the column bound would carry a factor a_i / b_j).  The operands a u and b v stay normal
 // fp32 numbers, and K = P / (a_i b_j) <= 1 / a_i within its range, while no weight is below 2^-80: a lane with a
 // smaller one (SC_NO_MATRIX, found when its layout is written) stays in the log domain for all of its cycles.
-// The first cycle of a cold or
-// warm start is a log-domain cycle.  All of these decisions are taken per lane from the lane's own values, and K is a function of
+// A cold lane whose entries before any potential are above 2^-SC_COLD_BITS, with weights from SC_COLD_WEIGHT on, starts with zero
+// potentials absorbed; the first cycle of the others, and of a warm start, is a log-domain cycle.  All of these decisions are taken per lane from the lane's own values, and K is a function of
 // (phi0, gam0) alone, which are part of the lane's state: a lane's bits depend neither on how its cycles
 // were shared out among launches nor on the mode.
 //
@@ -28,9 +29,10 @@
 // lane would otherwise need several blocks, in tensor memory, which holds as much again as the register file and is
 // read as fast as the multiply-adds go (256 words of 256 threads: 770 clk alone, 1020 with one packed
 // multiply-add per pair of words, 960 for the multiply-adds alone).  Row
-// sums are reduced by a halving exchange over the 32 threads; column sums go through shared memory (and
-// to the other blocks through distributed shared memory), every block forming all of v by itself.  One
-// cluster barrier and two block barriers per cycle: the column sums of the next state are formed before
+// sums are reduced by a halving exchange over the 32 threads; column sums go through shared memory and, where a lane has
+// several blocks, by bulk copies between their shared memories that report to an mbarrier of the receiver.  Every block forms all
+// of v by itself.  A cycle takes two block barriers, four in a cluster, and one more in the blocks that add up a share
+// of the columns (two-step exchange); there is no cluster barrier in it.  The column sums of the next state are formed before
 // the row residual has been decided on, and dropped where the lane leaves.
 //
 // What bounds it: the chain of dependent steps of a cycle (two rounds of multiply-adds, the exchange of row
@@ -41,13 +43,15 @@
 // them 5.4 -> 1.55 us (four blocks of a cluster per SM waited for each other's exchanges); all 1024 of the sweep workload
 // 27 -> 10 us, 24 -> 10.9 ms per solve at tol 1e-3.  512 x 512, clusters of eight blocks, registers -> of four, tensor memory:
 // 5.6 -> 3.5 us.  16 warps of 16 rows instead of 8 of 32: 2.2 us.
-// Forming K costs 10 to 20 us per launch of one wave (latency: two warps per scheduler), so a caller that steps one cycle
-// per call pays mostly for that: 25 us on one lane of 256 x 256, 155 us on 1024.  The formation is a loop in every variant:
+// Forming K costs 10 to 35 us per wave of a launch (latency: two warps per scheduler), so a caller that steps one cycle per call
+// pays mostly for that: 28 us on one lane of 256 x 256, 156 us on 1024; 290 us on 256 lanes of 512 x 512, d = 15, and 295 us on 64 of
+// 1024 x 1024, d = 512, where two streamed legs take 120 and 130 us.  From three to four cycles per call on it is the faster way
+// (362 and 417 against 481 and 519 us), at 64 by 3 to 4 times.  The formation is a loop in every variant:
 // unrolled, as it has to be to index registers, it was 100 KB of instructions that ran once per launch, and
 // fetching them took longer than running them (256 x 256: 43 -> 25 us per call; 96 lanes of 100 x 77: 30 -> 20 us).
-// The exchange between blocks through remote stores that report to a barrier of the receiver, instead of a
-// cluster barrier: 2.9 -> 2.4 us; 128-thread blocks (two of different lanes per SM) instead of 256: 58 -> 47 us
-// per cycle of 1024 lanes, together with the rows' order that spares the selects of the exchange.
+// The exchange between blocks: a cluster barrier 2.9 us a cycle of 256 x 256 in four blocks, remote stores that report to a
+// barrier of the receiver 2.4; now bulk copies, see SC_WAIT_CLOCKS.  128-thread blocks (two of different lanes per SM)
+// instead of 256: 58 -> 47 us per cycle of 1024 lanes, together with the rows' order that spares the selects of the exchange.
 #pragma once
 #include "skb_update.cuh"
 #include "skb_host.h"
@@ -254,7 +258,7 @@ __device__ __forceinline__ double row_exchange(V (&s)[CNT], const int lane)
 
 // Log-domain row step for the RW rows of a warp: integer-valued reference M >= every argument - 1 and
 // S = sum_j 2^(arg_ij - M), arg_ij = colB_j + x_i . y_j, of row lane / SHARE.  Two passes over the
-// distances; runs in the first cycle and where an update leaves the range of K.
+// distances; runs in the first cycle of lanes that do not start absorbed and where an update leaves the range of K.
 template <int SRC, int NW, int CL, int RW>
 __device__ __noinline__ void log_rows(const ScalingOperand &o, const int i0,
                                       const double *colB, double *S, double *M)
