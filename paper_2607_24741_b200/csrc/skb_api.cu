@@ -127,6 +127,10 @@ static const double SPATIAL_TOL = 2.0e-3;
 // one batch of all of them run the same arithmetic, so a lane's bits do not depend on how it came in.
 static const size_t DOTS_LIMIT = (size_t)4 << 30;
 
+// Lanes in spatial order keep lists of the pairs that matter (n m / 8 bytes a lane), up to this size of all of them (250 lanes of 8192
+// points, 1 % of the card's memory); beyond it, and in a workspace without room for them, each leg chooses its pairs by itself.
+static const size_t NEAR_LISTS_LIMIT = (size_t)2 << 30;
+
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 static bool config_ok(const skb_config *c, std::string &why)
@@ -161,8 +165,9 @@ static double guard_width(const skb_config *c)
 // Lays the batch's arrays out in the workspace (base may be null: size query only).
 // Every array is followed by a guard strip (GUARD_STRIP_BYTES of a known pattern, see
 // sinkhorn_batch_check_guards); their offsets are listed in *guards.
-// spatial: the batch may keep its lanes in spatial order (SPATIAL_TOL).  dots: there is room for the products of deep lanes.
-static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool spatial, bool dots, char *base, Dev *D, size_t *zero_end_out = nullptr,
+// spatial: the batch may keep its lanes in spatial order (SPATIAL_TOL).  room: for the products of deep lanes, for the lists of
+// lanes in spatial order.
+static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool spatial, bool room, char *base, Dev *D, size_t *zero_end_out = nullptr,
                     GuardList *guards = nullptr)
 {
     size_t off = 0;
@@ -235,9 +240,26 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
         d.nbx = (int)align_up((n + BOX_COLS - 1) / BOX_COLS, 4); d.nby = (int)align_up((m + BOX_COLS - 1) / BOX_COLS, 4);
         d.permx = (int *)take(L * np * 4); d.permy = (int *)take(L * mp * 4);
         d.boxx = (float *)take(W * 2 * DP * d.nbx * 4); d.boxy = (float *)take(W * 2 * DP * d.nby * 4);
-        d.topx[0] = (float *)take(W * d.nbx * 4); d.topx[1] = (float *)take(W * d.nbx * 4); d.topy = (float *)take(W * d.nby * 4);
+        size_t halves = 1;       // (with lists the largest potentials of the source are kept for halves of a box)
+        const size_t groups = (n + GROUP_ROWS - 1) / GROUP_ROWS;
+        // (a warp's list holds its boxes' points and two steps of none)
+        d.list_cap = (int)(((m + BOX_COLS - 1) / BOX_COLS + GROUP_WARPS - 1) / GROUP_WARPS + 2) * BOX_COLS;
+        const size_t lists = W * groups * GROUP_WARPS * d.list_cap * 2;
+        const bool listed = room && lists <= NEAR_LISTS_LIMIT && mp < 65535 && W * (mp + 1) * 16 < ((size_t)1 << 32);
+        if (listed) halves = 2;
+        d.topx[0] = (float *)take(W * halves * d.nbx * 4); d.topx[1] = (float *)take(W * halves * d.nbx * 4); d.topy = (float *)take(W * d.nby * 4);
+        if (listed) {
+            d.home = (int *)take(W * 4);
+            d.boxx16 = (float *)take(W * 2 * DP * 2 * d.nbx * 4); d.groups = (GroupRecord *)take(W * 2 * d.nbx * sizeof(GroupRecord));
+            d.crdy = (float *)take(W * (mp + 1) * 16); d.gamy = DP == 4 ? (float *)take(W * (mp + 1) * 4) : nullptr;
+            d.ceny = (float *)take(W * (d.nby + 1) * 16); d.lby = (float *)take(W * d.nby * 4); d.unit_low = (float2 *)take(W * (mp + 1) * 8);
+            d.colacc[0] = (unsigned long long *)take(W * mp * 8); d.colacc[1] = (unsigned long long *)take(W * mp * 8);
+            d.lists = (unsigned short *)take(lists);
+            d.base_gam = (float *)take(W * mp * 4); d.base_top = (float *)take(W * d.nby * 4);
+            d.risen = (unsigned long long *)take(W * 8); d.based_at = (int *)take(W * 4); d.no_sums = (int *)take(W * 4);
+        }
     }
-    if (tensor && dots && scaling_fits(true, c->n, c->m) && L * np * mp * 4 <= DOTS_LIMIT) {
+    if (tensor && room && scaling_fits(true, c->n, c->m) && L * np * mp * 4 <= DOTS_LIMIT) {
         d.phi0 = (double *)take(W * np * 8); d.uu[0] = (double *)take(W * np * 8); d.uu[1] = (double *)take(W * np * 8);
         d.gam0 = (double *)take(W * mp * 8); d.vv = (double *)take(W * mp * 8);
         d.dots = (float *)take(W * np * mp * 4);
@@ -267,21 +289,22 @@ static const Variant *variant_for(const skb_config *c, int compute, bool spatial
     return choose_variant(c->W, c->n, c->m, c->d, f64, compute == SKB_COMPUTE_MIXED, c->column_split, spatial);
 }
 
-// dots = false: the least that create takes (deep lanes then form their products in every leg)
-static size_t workspace_need(const skb_config *cfg, bool dots)
+// room = false: the least that create takes (deep lanes then form their products in every leg, lanes in spatial order
+// choose their pairs in every leg)
+static size_t workspace_need(const skb_config *cfg, bool room)
 {
     // an automatic batch may end up with float64 coordinates: size for the larger layout
     if (cfg->compute == SKB_COMPUTE_TENSOR && !tc_eligible(cfg->d, cfg->xy_dtype == SKB_BF16)) return 0;
     const Variant *v = variant_for(cfg, cfg->compute == SKB_COMPUTE_AUTO ? SKB_COMPUTE_MIXED : cfg->compute, false);
     if (!v) return 0;
-    size_t need = carve(cfg, v, cfg->compute == SKB_COMPUTE_TENSOR, false, dots, nullptr, nullptr);
+    size_t need = carve(cfg, v, cfg->compute == SKB_COMPUTE_TENSOR, false, room, nullptr, nullptr);
     if (cfg->compute == SKB_COMPUTE_AUTO && tc_eligible(cfg->d, cfg->xy_dtype == SKB_BF16)) {
-        const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, false), true, false, dots, nullptr, nullptr);
+        const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, false), true, false, room, nullptr, nullptr);
         if (t > need) need = t;
     }
     if (cfg->compute == SKB_COMPUTE_AUTO || cfg->compute == SKB_COMPUTE_F32) {
         for (const bool spatial : {false, true}) {           // the tolerance, which decides, is not known here
-            const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, spatial), false, spatial, false, nullptr, nullptr);
+            const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, spatial), false, spatial, room, nullptr, nullptr);
             if (t > need) need = t;
         }
     }
@@ -333,10 +356,10 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     size_t zero_end = 0;
     carve(cfg, var_big, false, false, false, nullptr, nullptr, &zero_end);
     const size_t need = workspace_need(cfg, true);
-    const bool dots = cfg->workspace_bytes >= need;
+    const bool room = cfg->workspace_bytes >= need;
     if (!cfg->workspace) return fail(nullptr, SKB_ERR_WORKSPACE, "workspace is null");
     if (((uintptr_t)cfg->workspace & 255u) != 0) return fail(nullptr, SKB_ERR_WORKSPACE, "workspace must be 256-byte aligned");
-    if (!dots && cfg->workspace_bytes < workspace_need(cfg, false)) {
+    if (!room && cfg->workspace_bytes < workspace_need(cfg, false)) {
         char buf[128];
         snprintf(buf, sizeof(buf), "workspace too small: %zu bytes given, %zu needed", cfg->workspace_bytes, need);
         return fail(nullptr, SKB_ERR_WORKSPACE, buf);
@@ -351,7 +374,7 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     h->lanes_used = cfg->W; h->enqueued_at_refill = 0;
     for (int i = 0; i < SKB_N_PHASES; ++i) h->phase_ms[i] = 0.f;
     h->guards.count = 0;
-    carve(cfg, var, h->tensor, false, dots, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+    carve(cfg, var, h->tensor, false, room, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
     h->dev.tol_stop = (double)tol;
     h->dev.tol_screen = cfg->tol_screen > 0.0f ? (double)cfg->tol_screen : (double)tol;
     cudaError_t e;
@@ -403,10 +426,10 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
             carve(cfg, var_big, false, false, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
         } else if (automatic && can_tensor) {
             h->tensor = true;
-            carve(cfg, var, true, false, dots, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+            carve(cfg, var, true, false, room, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
         } else if (near_shaped && radius <= FORM_DIFF_RADIUS && h->h_ctl[1].near_kept <= NEAR_SHARE * NEAR_PAIRS * cfg->W) {
             h->var = var_near;
-            carve(cfg, var_near, false, true, false, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+            carve(cfg, var_near, false, true, room, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
         }
         h->dev.tol_stop = ts; h->dev.tol_screen = tsc;
     }

@@ -474,6 +474,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_kernel(const Dev P)
         P.form[dst] = P.form[src];
         P.absorbed[dst] = P.absorbed[src];
         P.cyc_log[dst] = P.cyc_log[src];
+        if (P.home) { const int t = P.home[dst]; P.home[dst] = P.home[src]; P.home[src] = t; }
         P.nonfinite[dst] = 0;
     }
     if (tid == 0) {
@@ -780,7 +781,7 @@ __device__ __forceinline__ void emit_move_one(const Dev &P, const Ctl &c, const 
         }
         if (P.topy) {                                                 // lanes in spatial order (the order itself is kept by lane)
             add(P.boxx, (size_t)2 * P.DP * P.nbx * 4); add(P.boxy, (size_t)2 * P.DP * P.nby * 4);
-            add(P.topx[np_], (size_t)P.nbx * 4); add(P.topy, (size_t)P.nby * 4);
+            add(P.topx[np_], (size_t)(P.lists ? 2 : 1) * P.nbx * 4); add(P.topy, (size_t)P.nby * 4);
         }
         seg_n = ns;
     }
@@ -1100,6 +1101,7 @@ static size_t lane_state_bytes(const Dev &P)
 static bool plan_fuses_move(const Dev &P, int width)
 {
     const int lanes = (P.mode == MODE_STATIC) ? P.W : (width < 1 ? 1 : width);
+    if (lanes == 1) return (size_t)(P.n + P.m) * 16 <= ((size_t)512 << 10);      // (a last lane is emitted, nothing moves)
     return (size_t)lanes * lane_state_bytes(P) <= ((size_t)512 << 10);
 }
 int launch_plan(const Dev &P, int width, cudaStream_t st)

@@ -34,11 +34,28 @@ constexpr float SC_MIN_WEIGHT = 0x1p-80f;
 constexpr double SC_COLD_BITS = 120.0;
 constexpr float SC_COLD_WEIGHT = 0x1p-40f;
 constexpr int BOX_COLS = 32;          // points per bounding box of lanes in spatial order
+constexpr int GROUP_ROWS = 16;        // ... source points of a block of near_rows_kernel
+constexpr int GROUP_WARPS = UPD_THREADS / 32;
 constexpr int TC_MAX_SPLIT = 8;      // a row block's columns go to at most this many clusters
 constexpr int MAX_CLUSTER_RANKS = 8;  // blocks per cluster (portable limit): row blocks of a lane in the multi-cycle kernels
 constexpr double RSUM_SCALE = 17592186044416.0;     // 2^44: unit of the fixed-point residual sums
 constexpr double RSUM_ROW_MAX = 4.0;                 // one row's term is clamped here (a whole L1 residual never exceeds 2 near
                                                      // convergence), so fewer than 2^18 rows cannot overflow 64 bits
+
+// What near_rows_kernel starts a group of GROUP_ROWS source points of a lane in spatial order from: reference (negated) and weight of
+// every row; the largest phi - log2 a and phi now and when the group's lists were made, the cycle of the target's
+// potentials that they were made from, their lengths; the centre of its box of 32 and the coordinates relative to it (negated).
+struct __align__(16) GroupRecord {
+    float2 row[GROUP_ROWS];
+    float prow, pcol, pad_[2];
+    float made_prow, made_pcol;
+    int made_from, pad2_;
+    int len[4];
+    float centre[4];
+    float crd[4][GROUP_ROWS];
+    float pad3_[16];
+};
+static_assert(sizeof(GroupRecord) == 512, "one 16-byte piece a thread of a warp");
 
 // Device-resident control block.  Written by the plan kernel (one CTA), read by all.
 struct Ctl {
@@ -90,6 +107,23 @@ struct Dev {
     int *permx, *permy;
     float *boxx, *boxy, *topx[2], *topy;
     int nbx, nby;             // boxes of 32 points, padded to a multiple of 4
+    // ... and where both legs share one pass over the pairs (near_rows_kernel; lists is null otherwise).  All by home[slot],
+    // which goes along when a lane moves.  Source: boxes of 16 points, a record for every group of 16 (GroupRecord).  Target
+    // (mp points and one of weight zero): coordinates and potentials as fp32 (four dimensions: potentials apart), powers
+    // of two next to 2^44 / b and the rest of the potentials, centres of the boxes of 32, the least log2 b in them, column
+    // sums in units of those powers (double-buffered by the cycle's parity).  For every group and warp the target points that matter to it; the target's potentials that the
+    // lists were made from, by point and the largest by box, how far they have risen since (high word: the cycle of
+    // `then`), that cycle, and the last cycle without column sums
+    int *home;
+    float *boxx16, *crdy, *gamy, *ceny, *lby;
+    float2 *unit_low;
+    GroupRecord *groups;
+    unsigned long long *colacc[2];
+    unsigned short *lists;
+    float *base_gam, *base_top;
+    unsigned long long *risen;
+    int *based_at, *no_sums;
+    int list_cap;             // entries of a warp's list
     const int *order;         // scaling_kernel, a batch's first launch: the order in which slots are started (null: as they are)
     // per-slot scalars
     double *scale;            // s

@@ -1787,6 +1787,57 @@ def test_spatial_order_is_taken_where_it_can_skip(oracle, law, n, m, d, eps, exp
         assert run(**kw)[2] == plain[2], kw
 
 
+# (law, n, m, d, eps): groups of 16 rows and lists by warp at their edges; lists longer than what tensor memory holds (a
+# large share of the pairs); outliers on both sides, whose potentials move by many bits in the first cycles
+ONE_PASS = [("sphere", 1040, 1025, 3, 0.02), ("sphere", 1100, 2049, 3, 0.05), ("cube", 1031, 97, 2, 0.002), ("cube", 40, 1025, 1, 0.002),
+            ("flat", 1500, 1100, 4, 0.004), ("outliers", 1300, 1300, 3, 0.01)]
+
+
+@pytest.mark.parametrize("law,n,m,d,eps", ONE_PASS)
+def test_both_legs_in_one_pass(oracle, monkeypatch, law, n, m, d, eps):
+    # lanes in spatial order whose g-legs take the column sums that the f-leg's pass has left, over enough cycles for lists to be
+    # kept and made again, against the oracle; in a workspace without room for the lists each leg goes over the pairs by itself, and
+    # lanes that come in later, move or stay under a mask have the bits of one batch
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    rng = np.random.default_rng(n + m + d)
+    W, cycles, f32 = 3, 30, np.float32
+    x, y = _cloud_pair("sphere" if law == "outliers" else law, W, n, m, d, rng)
+    if law == "outliers":
+        for c in (x, y):
+            far = rng.random(c.shape[:2]) < 0.05
+            c[far] = rng.uniform(-1.0, 1.0, (int(far.sum()), d))
+    a = rng.uniform(0.5, 1.5, (W, n)); b = rng.uniform(0.5, 1.5, (W, m))
+    w = wl.Workload(law, x.astype(f32), y.astype(f32), (a / a.sum(1, keepdims=True)).astype(f32),
+                    (b / b.sum(1, keepdims=True)).astype(f32), (eps * np.array([1.0, 1.15, 1.3])).astype(f32), 1e-3, cycles)
+    ref = oracle.solve_batch(w.x, w.y, w.a, w.b, w.eps, w.tol, max_iter=cycles)
+    e = w.eps.astype(np.float64)
+    r = run_gpu(w)
+    assert r["arith"] == "f32"
+    np.testing.assert_array_equal(r["depth"], ref.depth)
+    assert pot_err(r["f"], r["g"], ref.f, ref.g, e).max() <= POT_TOL_F32
+    rm = run_gpu(w, mode="masked")
+    np.testing.assert_array_equal(rm["f"], r["f"]); np.testing.assert_array_equal(rm["g"], r["g"])
+    # one slot after the other, then two at a time: later lanes in slots that others have used
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    sb = B.SinkhornBatch(t(w.x[:2]), t(w.y[:2]), t(w.a[:2]), t(w.b[:2]), t(w.eps[:2]), w.tol, max_iter=cycles, lane_capacity=W)
+    while sb.active() == 2:
+        sb.step(1)
+    sb.refill(t(w.x[2:]), t(w.y[2:]), t(w.a[2:]), t(w.b[2:]), t(w.eps[2:]))
+    sb.drain()
+    f, g = sb.potentials(f64=True)
+    np.testing.assert_array_equal(f.cpu().numpy(), r["f"]); np.testing.assert_array_equal(g.cpu().numpy(), r["g"])
+    assert sb.check_guards() == -1
+    sb.close()
+    if min(n, m) < 1000:                                  # (the lists are small beside what an automatic batch is sized for)
+        return
+    whole = B.sinkhorn_batch_workspace_bytes
+    monkeypatch.setattr(B, "sinkhorn_batch_workspace_bytes", lambda cfg: whole(cfg) - 256)
+    rs = run_gpu(w)
+    np.testing.assert_array_equal(rs["depth"], ref.depth)
+    assert pot_err(rs["f"], rs["g"], ref.f, ref.g, e).max() <= POT_TOL_F32
+
+
 @pytest.mark.parametrize("cost_form", [0, 1, 2])
 def test_large_radii_in_fp32_take_differences_whatever_the_size(oracle, cost_form):
     # scaled squared radius of 1000 to 3000, asked for in fp32: cost_form 0 and 2 must be the difference form with
