@@ -900,9 +900,9 @@ __global__ void __launch_bounds__(128) apply_plan_kernel(const Dev P, const void
         }
     }
 }
-// The wide tiles' part of R rows (skb_pairs64.cuh), by differences; this thread's quarter of the columns.  Out of line:
+// The wide tiles' part of R rows (skb_pairs64.cuh), by differences; every NC-th of the columns.  Out of line:
 // its registers would come off the tiled loop's.
-template <int DM, int DV, int R>
+template <int DM, int DV, int R, int NC>
 __device__ __noinline__ void apply_wide_tiles(const bool bf16, const int n, const int m, const int d, double *tile, const double *org, const void *x,
                                               const void *y, const float *v, const int i0, const double k2, const double *f,
                                               const double *g, const int dv, const int cs, const bool row_wide, double *out)
@@ -917,7 +917,7 @@ __device__ __noinline__ void apply_wide_tiles(const bool bf16, const int n, cons
         p64_fetch(part, j0, m, d, [&](int j, int k) { return raw(y, (size_t)j * d + k); }, [&](int j) { return g[j]; });
         const bool wide = p64_tile<DM, 128>(tile, org, j0, m, d, k2, part);
         if (!__syncthreads_or(wide || row_wide)) continue;
-        for (int j = j0 + cs; j < m && j < j0 + P64_TJ; j += 4)
+        for (int j = j0 + cs; j < m && j < j0 + P64_TJ; j += NC)
             for (int r = 0; r < R; ++r) {
                 const int i = i0 + r < n ? i0 + r : n - 1;
                 const double t = p64_entry(d, k2, f[i] + g[j], [&](int k) { return raw(x, (size_t)i * d + k); }, [&](int k) { return raw(y, (size_t)j * d + k); });
@@ -926,19 +926,22 @@ __device__ __noinline__ void apply_wide_tiles(const bool bf16, const int n, cons
     }
 }
 // The same for d <= 32 by column tiles in shared memory (skb_pairs64.cuh); DV: values per point, rounded up.
-// 8 lanes of 4096 x 4096 points, d = dv = 3: 966 us with one warp per row, 414 us so.
+// 8 lanes of 4096 x 4096 points, d = dv = 3: 966 us with one warp per row, 414 us so with CUDA's exp2 and two rows a thread,
+// 281 us with p64_exp2 and four.
+constexpr int P64_APPLY_ROWS = 32;                       // rows of a block (64: the last wave is emptier, 301 against 281 us)
 template <int DM, int DV>
-__global__ void __launch_bounds__(128) apply_plan_tiled_kernel(const Dev P, const void *x, const void *y, const float *eps,
+__global__ void __launch_bounds__(128, DM <= 4 && DV <= 3 ? 4 : 1) apply_plan_tiled_kernel(const Dev P, const void *x, const void *y, const float *eps,
                                                                const float *v, const int dv, float *out)
 {
-    constexpr int R = 2, RW = 16;
+    // (four rows to a thread halve what it reads from shared memory per pair; more values a point want the registers)
+    constexpr int R = DM <= 4 && DV <= 4 ? 4 : 2, RW = P64_APPLY_ROWS / 4, NC = 32 / (RW / R);
     __shared__ double tile[P64_TILE<DM, 128>];
     __shared__ double vals[DV * P64_TJ];                  // (a tile's values, float64)
     __shared__ double org[DM];
     const int lane_t = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (!P.emitted[lane_t]) return;
-    const int cs = lane >> 3, i0 = blockIdx.x * (4 * RW) + warp * RW + (lane & 7) * R;
-    const double k2 = 1.4426950408889634 / (double)eps[lane_t];
+    const int cs = lane / (RW / R), i0 = blockIdx.x * (4 * RW) + warp * RW + lane % (RW / R) * R;
+    const double k2 = 1.4426950408889634 / (double)eps[lane_t], entry = p64_table();
     const double *f = P.f_out + (size_t)lane_t * P.n, *g = P.g_out + (size_t)lane_t * P.m;
     const size_t xb = (size_t)lane_t * P.n * P.d, yb = (size_t)lane_t * P.m * P.d;
     if (threadIdx.x < DM) org[threadIdx.x] = threadIdx.x < P.d ? (double)load_raw(P, x, xb + (size_t)blockIdx.x * (4 * RW) * P.d + threadIdx.x) : 0.0;
@@ -959,7 +962,7 @@ __global__ void __launch_bounds__(128) apply_plan_tiled_kernel(const Dev P, cons
     bool any_wide = false;
     auto load = [&](int j, int k) { return load_raw(P, y, yb + (size_t)j * P.d + k); };
     auto pot = [&](int j) { return g[j]; };
-    constexpr int NV = P64_TJ * DV / 128;
+    constexpr int NV = (P64_TJ * DV + 127) / 128;
     float vn[NV];
     auto fetch_vals = [&](const int j0) {
 #pragma unroll
@@ -974,13 +977,14 @@ __global__ void __launch_bounds__(128) apply_plan_tiled_kernel(const Dev P, cons
         if (!P64_AHEAD<DM>) { p64_fetch(part, j0, P.m, P.d, load, pot); fetch_vals(j0); }
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < NV; ++q) vals[threadIdx.x + 128 * q] = (double)vn[q];
+        for (int q = 0; q < NV; ++q)
+            if (P64_TJ * DV % 128 == 0 || threadIdx.x + 128 * q < P64_TJ * DV) vals[threadIdx.x + 128 * q] = (double)vn[q];
         const bool wide = p64_tile<DM, 128>(tile, org, j0, P.m, P.d, k2, part);
         if (P64_AHEAD<DM>) { p64_fetch(part, j0 + P64_TJ, P.m, P.d, load, pot); fetch_vals(j0 + P64_TJ); }
         if (__syncthreads_or(wide || row_wide)) { any_wide = true; continue; }
-        const int end = P.m - j0 < P64_TJ ? P.m - j0 : P64_TJ;
+        const int end = P.m - j0 < P64_TJ ? P.m - j0 : P64_TJ;                 // (whole warps go on together past it)
 #pragma unroll 2
-        for (int jj = cs; jj < end; jj += 4) {
+        for (int jj = cs; jj < P64_TJ; jj += NC) {
             double t[R];
             const double c0 = tile[DM * P64_TJ + jj];
 #pragma unroll
@@ -991,8 +995,10 @@ __global__ void __launch_bounds__(128) apply_plan_tiled_kernel(const Dev P, cons
 #pragma unroll
                 for (int r = 0; r < R; ++r) t[r] = fma(xr[r][k], yk, t[r]);
             }
+            p64_exp2(t, entry);
+            if (end < P64_TJ && jj >= end)
 #pragma unroll
-            for (int r = 0; r < R; ++r) t[r] = exp2(t[r]);
+                for (int r = 0; r < R; ++r) t[r] = 0.0;
 #pragma unroll
             for (int c = 0; c < DV; ++c) {
                 const double vc = vals[c * P64_TJ + jj];
@@ -1004,7 +1010,7 @@ __global__ void __launch_bounds__(128) apply_plan_tiled_kernel(const Dev P, cons
     if (any_wide) {
         double more[R][DV];
         const size_t es = P.xy_bf16 ? 2 : 4;
-        apply_wide_tiles<DM, DV, R>(P.xy_bf16 != 0, P.n, P.m, P.d, tile, org, (const char *)x + xb * es, (const char *)y + yb * es,
+        apply_wide_tiles<DM, DV, R, NC>(P.xy_bf16 != 0, P.n, P.m, P.d, tile, org, (const char *)x + xb * es, (const char *)y + yb * es,
                                     v + (size_t)lane_t * P.m * dv, i0, k2, f, g, dv, cs, row_wide, &more[0][0]);
 #pragma unroll
         for (int r = 0; r < R; ++r)
@@ -1016,15 +1022,17 @@ __global__ void __launch_bounds__(128) apply_plan_tiled_kernel(const Dev P, cons
 #pragma unroll
         for (int c = 0; c < DV; ++c) {
             double a = acc[r][c];
-            a += __shfl_xor_sync(0xffffffffu, a, 8);
-            a += __shfl_xor_sync(0xffffffffu, a, 16);
+#pragma unroll
+            for (int off = RW / R; off < 32; off *= 2) a += __shfl_xor_sync(0xffffffffu, a, off);
             if (cs == 0 && i0 + r < P.n && c < dv) out[((size_t)lane_t * P.n + i0 + r) * dv + c] = (float)a;
         }
 }
 template <int DM>
 static void launch_apply_tiled(const Dev &P, const void *x, const void *y, const float *eps, const float *v, int dv, float *out, int lanes, cudaStream_t st)
 {
-    const dim3 grid((P.n + 63) / 64, lanes);
+    const dim3 grid((P.n + P64_APPLY_ROWS - 1) / P64_APPLY_ROWS, lanes);
+    if constexpr (DM <= 4)
+        if (dv <= 3) { apply_plan_tiled_kernel<DM, 3><<<grid, 128, 0, st>>>(P, x, y, eps, v, dv, out); return; }
     if (dv <= 4) apply_plan_tiled_kernel<DM, 4><<<grid, 128, 0, st>>>(P, x, y, eps, v, dv, out);
     else apply_plan_tiled_kernel<DM, APPLY_MAX_DV><<<grid, 128, 0, st>>>(P, x, y, eps, v, dv, out);
 }
@@ -1038,6 +1046,7 @@ void launch_apply_plan(const Dev &P, const void *x, const void *y, const float *
 {
     const bool narrow = (long long)((P.n + 63) / 64) * lanes <= (P.d <= 8 && dv <= 8 ? 80 : 8);
     if (P.d > P64_MAX_D || narrow) { apply_plan_kernel<<<dim3((P.n + 3) / 4, lanes), 128, 0, st>>>(P, x, y, eps, v, dv, out); return; }
+    if (P.d <= 3) { launch_apply_tiled<3>(P, x, y, eps, v, dv, out, lanes, st); return; }
     if (P.d <= 4) { launch_apply_tiled<4>(P, x, y, eps, v, dv, out, lanes, st); return; }
     if (P.d <= 16) { launch_apply_tiled<16>(P, x, y, eps, v, dv, out, lanes, st); return; }
     launch_apply_tiled<P64_MAX_D>(P, x, y, eps, v, dv, out, lanes, st);

@@ -89,9 +89,9 @@ __global__ void __launch_bounds__(NA_THREADS) row_residual_kernel(
     r_row[lane_id] = (float)tot;
 }
 
-// The wide tiles' part of a row's sum (skb_pairs64.cuh), by differences; this thread's quarter of the columns.
+// The wide tiles' part of a row's sum (skb_pairs64.cuh), by differences; every NC-th of the columns.
 // Out of line: its registers would come off the tiled loop's.
-template <int DM, int THREADS>
+template <int DM, int THREADS, int NC>
 __device__ __noinline__ double wide_tiles(double *tile, const double *org, const float *xi, const float *yl, const double fi, const double *gl,
                                           const int m, const int d, const double k2, const int cs, const bool row_wide)
 {
@@ -103,7 +103,7 @@ __device__ __noinline__ double wide_tiles(double *tile, const double *org, const
         p64_fetch(part, j0, m, d, [&](int j, int k) { return yl[(size_t)j * d + k]; }, [&](int j) { return gl[j]; });
         const bool wide = p64_tile<DM, THREADS>(tile, org, j0, m, d, k2, part);
         if (!__syncthreads_or(wide || row_wide)) continue;
-        for (int j = j0 + cs; j < m && j < j0 + P64_TJ; j += 4)
+        for (int j = j0 + cs; j < m && j < j0 + P64_TJ; j += NC)
             s += p64_entry(d, k2, fi + gl[j], [&](int k) { return xi[k]; }, [&](int k) { return yl[(size_t)j * d + k]; });
     }
     return s;
@@ -112,20 +112,20 @@ __device__ __noinline__ double wide_tiles(double *tile, const double *org, const
 // The same for d <= 32: a block of WPB warps takes 16 * WPB rows, column tiles come through shared memory
 // (skb_pairs64.cuh).  The entries are summed as they are; a row whose sum is not finite is redone the plain way,
 // so infinite potentials give what they always gave.  32 lanes of 1024 x 1000 points, d = 15: 1040 us with one
-// thread per row and the columns read from global memory, 145 us so.
-template <int DM, int WPB>
+// thread per row and the columns read from global memory, 145 us so with CUDA's exp2, 117 us with p64_exp2.
+template <int DM, int WPB, int RW>
 __global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
     Scratch *sc, const float *x, const float *y, const float *a, const double *f, const double *g,
     const float *eps, int n, int m, int d, float *r_row)
 {
     using namespace skb;
-    constexpr int R = 2, RW = 16;
+    constexpr int R = 2, NC = 32 / (RW / R);
     __shared__ double tile[P64_TILE<DM, 32 * WPB>];
     __shared__ double org[DM];
     __shared__ double red[WPB];
     __shared__ int is_last;
     const int lane_id = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int cs = lane >> 3, i0 = blockIdx.x * (RW * WPB) + warp * RW + (lane & 7) * R;
+    const int cs = lane / (RW / R), i0 = blockIdx.x * (RW * WPB) + warp * RW + lane % (RW / R) * R;
     const double inv_eps = 1.0 / (double)eps[lane_id], k2 = 1.4426950408889634 * inv_eps;
     const float *xl = x + (size_t)lane_id * n * d, *yl = y + (size_t)lane_id * m * d;
     const double *fl = f + (size_t)lane_id * n, *gl = g + (size_t)lane_id * m;
@@ -144,6 +144,7 @@ __global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
         s[r] = 0.0;
     }
     bool any_wide = false;
+    const double entry = p64_table();
     auto load = [&](int j, int k) { return yl[(size_t)j * d + k]; };
     auto pot = [&](int j) { return gl[j]; };
     P64Part<DM, 32 * WPB> part;
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
         if (P64_AHEAD<DM>) p64_fetch(part, j0 + P64_TJ, m, d, load, pot);
         if (__syncthreads_or(wide || row_wide)) { any_wide = true; continue; }
 #pragma unroll 2
-        for (int jj = cs; jj < P64_TJ; jj += 4) {
+        for (int jj = cs; jj < P64_TJ; jj += NC) {
             double v[R];
             const double c = tile[DM * P64_TJ + jj];
 #pragma unroll
@@ -166,20 +167,21 @@ __global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[r] = fma(xr[r][k], yk, v[r]);
             }
+            p64_exp2(v, entry);
 #pragma unroll
-            for (int r = 0; r < R; ++r) s[r] += exp2(v[r]);
+            for (int r = 0; r < R; ++r) s[r] += v[r];
         }
     }
     if (any_wide)
         for (int r = 0; r < R; ++r) {
             const int i = i0 + r < n ? i0 + r : n - 1;
-            s[r] += wide_tiles<DM, 32 * WPB>(tile, org, xl + (size_t)i * d, yl, fl[i], gl, m, d, k2, cs, row_wide);
+            s[r] += wide_tiles<DM, 32 * WPB, NC>(tile, org, xl + (size_t)i * d, yl, fl[i], gl, m, d, k2, cs, row_wide);
         }
     double term = 0.0;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        s[r] += __shfl_xor_sync(0xffffffffu, s[r], 8);
-        s[r] += __shfl_xor_sync(0xffffffffu, s[r], 16);
+#pragma unroll
+        for (int off = RW / R; off < 32; off *= 2) s[r] += __shfl_xor_sync(0xffffffffu, s[r], off);
         if (cs == 0 && i0 + r < n) {
             if (!isfinite(s[r])) {
                 // the plain sum, with its running maximum
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
             term += fabs(s[r] - (double)a[(size_t)lane_id * n + i0 + r]);
         }
     }
-    for (int off = 4; off > 0; off >>= 1) term += __shfl_down_sync(0xffffffffu, term, off);
+    for (int off = RW / R / 2; off > 0; off >>= 1) term += __shfl_down_sync(0xffffffffu, term, off);
     if (lane == 0) red[warp] = term;
     __syncthreads();
     if (tid == 0) {
@@ -215,13 +217,14 @@ __global__ void __launch_bounds__(32 * WPB) row_residual_tiled_kernel(
     r_row[lane_id] = (float)tot;
 }
 
-// 64 rows to a block while the scratch has a slot for every block (n <= 4096), 128 beyond
+// 32 rows to a block while the scratch has a slot for every block (n <= 2048), 64 and 128 beyond
 template <int DM>
 void launch_tiled(Scratch *sc, const float *x, const float *y, const float *a, const double *f, const double *g, const float *eps,
                   int W, int n, int m, int d, float *r_row, cudaStream_t st)
 {
-    if (n <= 64 * NA_MAX_BLOCKS) row_residual_tiled_kernel<DM, 4><<<dim3((n + 63) / 64, W), 128, 0, st>>>(sc, x, y, a, f, g, eps, n, m, d, r_row);
-    else row_residual_tiled_kernel<DM, 8><<<dim3((n + 127) / 128, W), 256, 0, st>>>(sc, x, y, a, f, g, eps, n, m, d, r_row);
+    if (n <= 32 * NA_MAX_BLOCKS) row_residual_tiled_kernel<DM, 4, 8><<<dim3((n + 31) / 32, W), 128, 0, st>>>(sc, x, y, a, f, g, eps, n, m, d, r_row);
+    else if (n <= 64 * NA_MAX_BLOCKS) row_residual_tiled_kernel<DM, 4, 16><<<dim3((n + 63) / 64, W), 128, 0, st>>>(sc, x, y, a, f, g, eps, n, m, d, r_row);
+    else row_residual_tiled_kernel<DM, 8, 16><<<dim3((n + 127) / 128, W), 256, 0, st>>>(sc, x, y, a, f, g, eps, n, m, d, r_row);
 }
 
 skb_status fail(skb_status st, const std::string &msg)

@@ -9,11 +9,11 @@
 // k |y - org|^2 instead of with the cost itself: a tile in which one of them is above P64_WIDE is summed by
 // differences, term by term (the caller's own loop).  Below it the terms are at most 2^17 and the d + 2 roundings
 // of an argument add up to less than 2^-32 (d = 32), 2^-8 of the rounding of an fp32 result.
-// A warp holds 16 rows, two to a thread; its four quarters take every fourth column, so a quarter-warp reads one
-// shared-memory address.  The partial sums of the quarters are added by xor-shuffles.
+// A warp holds 8 or 16 rows, two or four to a thread; the threads that hold the same rows share the columns out, and their partial
+// sums are added by xor-shuffles.
 //
-// What bounds it: the latency of dependent float64 operations (d + 1 and exp2 per pair) at 3.3 warps a scheduler; the float64
-// pipe is busy half of the time (52 % at d = 3, 49 % at d = 15).  The next tile's coordinates are fetched into registers
+// What bounds it: issue and the latency of dependent float64 operations at 3.2 warps a scheduler.  Plan application at d = 3: 17 float64
+// operations of 38 instructions a pair, the float64 pipe and the issue slots both half busy.  The next tile's coordinates are fetched into registers
 // before the pair loop of the present one (up to eight dimensions: beyond, the rows' own coordinates need the registers).
 #pragma once
 #include <cuda_runtime.h>
@@ -28,6 +28,44 @@ constexpr double P64_WIDE = 32768.0;
 
 // k |p - org|^2 is too large for the expanded form (NaN and infinity included)
 __device__ __forceinline__ bool p64_wide(const double k2, const double sq) { return !(k2 * sq <= P64_WIDE); }
+
+// 2^t for R arguments of every thread of a warp, good to about an ulp: t = k / 32 + r, |r| <= 1/64, 2^(k mod 32 / 32) from a table of
+// one entry a thread (`entry`: 2^(lane / 32)), 2^r from its Taylor series (degree 6: truncation 4e-18); the table method of
+// P. Tang, ACM TOMS 15, 1989, with the table read by shuffles.  Ten float64 operations, some twenty in CUDA's exp2, which
+// takes the arguments that leave [-1022, 1022], except that those below -1080 are zero.  Called by whole warps.
+__device__ __forceinline__ double p64_table() { return exp2((double)(threadIdx.x & 31) / 32.0); }
+template <int R>
+__device__ __forceinline__ void p64_exp2(double (&t)[R], const double entry)
+{
+    bool odd = false;
+#pragma unroll
+    for (int r = 0; r < R; ++r) odd = odd || ((unsigned)__double2hiint(t[r]) & 0x7fffffffu) >= 0x408ff000u;         // |t| >= 1022 or NaN
+    double v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const double magic = 211106232532992.0;          // 1.5 * 2^47: the sum's low word is k
+        const double m = t[r] + magic, x = t[r] - (m - magic);
+        const int k = __double2loint(m);
+        const int lo = __shfl_sync(0xffffffffu, __double2loint(entry), k), hi = __shfl_sync(0xffffffffu, __double2hiint(entry), k);
+        const double s = __hiloint2double(hi + (k >> 5 << 20), lo);
+        double q = 1.5403530393381609e-4;                // ln(2)^6 / 720 ...
+        q = fma(q, x, 1.3333558146428443e-3);
+        q = fma(q, x, 9.6181291076284772e-3);
+        q = fma(q, x, 5.5504108664821580e-2);
+        q = fma(q, x, 2.4022650695910072e-1);
+        q = fma(q, x, 6.9314718055994531e-1);
+        v[r] = fma(s, q * x, s);
+    }
+    if (odd) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const unsigned h = (unsigned)__double2hiint(t[r]);
+            if ((h & 0x7fffffffu) >= 0x408ff000u) v[r] = h >= 0xc090e000u && h <= 0xfff00000u ? 0.0 : exp2(t[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) t[r] = v[r];
+}
 
 // One entry of a wide tile, from coordinate differences.
 template <typename LoadX, typename LoadY>
