@@ -1657,6 +1657,54 @@ def test_last_audit_of_a_mask_does_not_depend_on_how_the_cycles_were_run():
                 np.testing.assert_array_equal(rc, out[0][1]); np.testing.assert_array_equal(fl, out[0][2])
 
 
+@pytest.mark.parametrize("n,m,d", [(1, 1, 1), (31, 65, 3), (2048, 64, 15), (2049, 63, 4), (4097, 65, 3), (100, 130, 17)])
+def test_row_residual_over_the_whole_range_of_exponents(n, m, d):
+    # blocks of 32, 64 and 128 rows at their edges, ragged tiles; entries from 2^-5000 to 2^40, a column of no weight
+    # (g = -inf).  float64 sums stored as fp32: 2^-24 of the value, and m + d + 4 roundings of 2^-53 of an argument of up to 5000
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    rng = np.random.default_rng(n + 7 * m + d)
+    x = rng.standard_normal((2, n, d)).astype(np.float32); y = rng.standard_normal((2, m, d)).astype(np.float32)
+    a = rng.uniform(0.5, 1.5, (2, n)).astype(np.float32) / n
+    eps = np.array([0.02, 0.5], np.float32)
+    f = eps[:, None] * rng.uniform(-10.0, 10.0, (2, n)); g = eps[:, None] * rng.uniform(-10.0, 10.0, (2, m))
+    cost = ((x.astype(np.float64)[:, :, None] - y.astype(np.float64)[:, None]) ** 2).sum(3)
+    f += np.where(rng.random((2, n)) < 0.1, cost.min(2), 0.0)                # some rows with entries of the order of one
+    if m > 1:
+        g[:, m // 2] = -np.inf
+    with np.errstate(under="ignore"):
+        p = np.exp((f[:, :, None] + g[:, None] - cost) / eps.astype(np.float64)[:, None, None])
+        ref = np.abs(p.sum(2) - a.astype(np.float64)).sum(1)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    r = B.sinkhorn_row_residual_static(t(x), t(y), t(a), t(f), t(g), t(eps)).cpu().numpy().astype(np.float64)
+    np.testing.assert_allclose(r, ref, rtol=2.0 ** -24 + (m + d + 4) * 5000 * 2.0 ** -53 + 1e-11)
+
+
+@pytest.mark.parametrize("n,d,dv", [(2700, 3, 3), (2600, 2, 1), (2600, 4, 4), (2600, 3, 5), (2564, 8, 3)])
+def test_plan_application_by_tiles(oracle, n, d, dv):
+    # enough row blocks for the tiles (81 of 32 and 64 rows), ragged ones, the widths of the values around those that the tiles are
+    # made for; against the sums in float64.  fp32 results: 2^-24 of the value's own scale, 64-bit sums of m terms below that
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    rng = np.random.default_rng(n + d + dv)
+    W, m = 2, 333
+    x = rng.standard_normal((W, n, d)).astype(np.float32); y = (1.1 * rng.standard_normal((W, m, d))).astype(np.float32)
+    a = np.full((W, n), 1.0 / n, np.float32); b = np.full((W, m), 1.0 / m, np.float32)
+    eps = np.array([0.3, 0.6], np.float32)
+    v = rng.standard_normal((W, m, dv)).astype(np.float32)
+    t = lambda q: torch.from_numpy(q).to("cuda:0")
+    sb = B.SinkhornBatch(t(x), t(y), t(a), t(b), t(eps), 1e-2, max_iter=40)
+    sb.drain()
+    f, g = (q.cpu().numpy() for q in sb.potentials(f64=True))
+    out = sb.apply_plan(t(v)).cpu().numpy().astype(np.float64)
+    sb.close()
+    for k in range(W):
+        cost = ((x[k].astype(np.float64)[:, None] - y[k].astype(np.float64)[None]) ** 2).sum(2)
+        p = np.exp((f[k][:, None] + g[k][None] - cost) / float(eps[k]))
+        want, size = p @ v[k].astype(np.float64), p @ np.abs(v[k]).astype(np.float64)
+        assert (np.abs(out[k] - want) <= 2.0 ** -24 * np.abs(want) + 1e-11 * size).all()
+
+
 # ---- large low-dimensional lanes in spatial order ----------------------------------------------------
 def test_lanes_are_ranked_for_long_launches_of_wide_batches_only():
     # the ranking is one launch more, before a batch's first cycles; the results do not depend on it
