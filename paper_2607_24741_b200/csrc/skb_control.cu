@@ -631,6 +631,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
         g->n_retire = FUSE ? 0 : nholes;
         g->slots += slots;
         g->pair_terms += terms;
+        g->mask_left = g->mask_last = 0;
         if (c.n_running == nret) g->done = 1;
     }
     if (FUSE && nholes > 0) {

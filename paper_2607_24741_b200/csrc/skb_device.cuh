@@ -74,6 +74,7 @@ struct Ctl {
     unsigned long long max_radius_bits;   // largest scaled squared radius over lanes (double bits)
     long long slots;       // lane-cycles physically executed
     long long pair_terms;  // n * m per lane and pass of the update launches
+    int mask_left, mask_last;   // MASKED, launches of whole cycles: lanes that have passed in the launch, the latest cycle at which one has
 };
 
 struct Dev {

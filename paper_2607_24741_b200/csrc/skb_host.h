@@ -47,7 +47,8 @@ constexpr int MAX_CLUSTER_BLOCKS = MAX_CLUSTER_RANKS;   // a lane needs at most 
 // Upper bound on the cycles one multi-cycle launch runs.  Lanes are independent and leave a launch when they pass, so a
 // long launch keeps the SMs full where a series of short ones waits for its slowest lanes after each.
 constexpr int MAX_CYCLES_IN_LAUNCH = 2048;
-// ... and under a logical mask, whose lanes work on until the launch ends, however early they pass: what a caller asks for
+// ... and under a logical mask, whose lanes work on until the last one has passed, however early they do.  Lanes that wait for a
+// place on the GPU cannot pass, so a launch of more lanes than fit works on to its end: what a caller asks for
 // beyond the last lane's depth costs at most the rest of one launch (launches after it return at once).
 constexpr int MASK_CYCLES_IN_LAUNCH = 256;
 // Picks the variant for a shape (depends on the static shape only, so that every mode
@@ -89,6 +90,7 @@ void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int wid
 int launch_plan_cycles(const Dev &P, int width, int cycles, cudaStream_t st);
 void launch_order(const Dev &P, int *order, cudaStream_t st);
 int scaling_blocks(const Dev &P);          // blocks of a lane
+int scaling_resident(const Dev &P);        // lanes that are on the GPU at the same time, at least
 void launch_plan_static(const Dev &P, int cycles, cudaStream_t st);
 void launch_gather(const Dev &P, void *f, void *g, bool f64, cudaStream_t st);
 void launch_gather_audit(const Dev &P, float *rrow, float *rcol, int *flagged, cudaStream_t st);

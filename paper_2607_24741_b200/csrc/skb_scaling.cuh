@@ -60,7 +60,7 @@
 namespace skb {
 
 constexpr int SC_TAKE = 45, SC_KEEP = 30;               // bands of log2 u and log2 v: update taken / K kept
-constexpr int SC_BAD = 1, SC_DRIFT = 2, SC_NF = 4;
+constexpr int SC_BAD = 1, SC_DRIFT = 2, SC_NF = 4, SC_LEAVE = 8;
 
 // 2^arg for a float64 argument: integer part split off in float64, the remainder (|.| <= 1/2) rounded
 // to fp32 and put through the Taylor series of e^(x ln 2) (degree 7: truncation 5e-9), so the result is
@@ -778,6 +778,15 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
             return (unsigned long long)lo + ((unsigned long long)hi << CUT);
         }
     };
+    // Logical mask: a frozen lane works on until the batch is over, which is when the last lane has passed and this one has
+    // run as many cycles.  Asked by one thread of the lane, every sixteenth cycle, and told to the others with the flags.
+    auto mask_over = [&](const int k) -> int {
+        if (KIND != SC_CYCLES || !frozen || b != 0 || tid != 0 || (k & 15) != 0) return 0;
+        const volatile Ctl *now = P.ctl;
+        if (now->mask_left < c.n_running) return 0;
+        __threadfence();
+        return k >= now->mask_last ? SC_LEAVE : 0;
+    };
     // TWO_STEP: this thread's column of the block's share, its total (or maximum) from the parts in xbuf
     auto share_total = [&](const bool is_max) -> double {
         const double *src = xbuf + (size_t)(xch & 1) * NC * share + (tid >> tpb);
@@ -957,7 +966,7 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                     const double S = row_exchange<CL, L::FP32_COLS, true, 16, RW, float>(s, lane);
                     unew = rok ? rcp64(S) : 1.0;
                     const double term = rown ? a_fix * fabs(fma(us, S, -1.0)) : 0.0;
-                    const int flags = (rok && out_of_band<SC_SUMS>(S)) || out_of_band<SC_TAKE>(unew) ? SC_BAD | SC_DRIFT : (out_of_band<SC_KEEP>(unew) ? SC_DRIFT : 0);
+                    const int flags = mask_over(k) | ((rok && out_of_band<SC_SUMS>(S)) || out_of_band<SC_TAKE>(unew) ? SC_BAD | SC_DRIFT : (out_of_band<SC_KEEP>(unew) ? SC_DRIFT : 0));
                     const unsigned long long fx = to_fixed(term);
                     if constexpr (LEG) {
                         send_rows(fx, flags);
@@ -1071,6 +1080,13 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
             if (tid == 0) atomicOr(&P.ctl->error, ERR_WAIT);
             break;
         }
+        if (all & SC_LEAVE) {
+            rr = (double)tot * (1.0 / RSUM_SCALE);           // (the state has been the same since it froze)
+            rc = 0.0;
+            fl = 0;
+            par = c.parity ^ (todo & 1);                     // where the lanes that go on have theirs
+            break;
+        }
         if (done) {
             // (the last audit was that of the state before this launch's last cycle, and it flagged nothing)
             rr = (double)tot * (1.0 / RSUM_SCALE);
@@ -1095,10 +1111,17 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                 unew = 0.0;
                 if (rok) row_math((int)FORM_DOT, true, P.la2[ro], P.sqx[ro], a_i, row_phi(us), (float)M, S, 0.f, unew, term);
                 const int flags = !isfinite(unew) || !isfinite(term) ? SC_NF : 0;
-                send_rows(rown && !flags ? to_fixed(term * RSUM_SCALE) : 0ull, flags);
+                send_rows(rown && !flags ? to_fixed(term * RSUM_SCALE) : 0ull, flags | mask_over(k));
                 scaling_barrier<CLU>();
                 tot = recv_rows(all);
                 ++xch;
+                if (all & SC_LEAVE) {
+                    rr = (double)tot * (1.0 / RSUM_SCALE);
+                    rc = 0.0;
+                    fl = 0;
+                    par = c.parity ^ (todo & 1);
+                    break;
+                }
             }
             if (all & SC_NF) nf = 1;
             near = tot <= near_tot;
@@ -1239,7 +1262,12 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                         P.depth[lane_id] = (limit && st != LANE_DONE) ? P.max_iter : k - start;
                         P.status[lane_id] = st;
                         P.emitted[lane_id] = 1;
-                        if (P.mode == MODE_MASKED) P.state[slot] = 1;
+                        if (P.mode == MODE_MASKED) {
+                            P.state[slot] = 1;
+                            atomicMax(&P.ctl->mask_last, k);
+                            __threadfence();
+                            atomicAdd(&P.ctl->mask_left, 1);
+                        }
                     }
                 }
                 retired_at = k + 1;

@@ -1727,6 +1727,38 @@ def test_lanes_are_ranked_for_long_launches_of_wide_batches_only():
         np.testing.assert_array_equal(out[1], out[0]); np.testing.assert_array_equal(out[2], out[0])
 
 
+@pytest.mark.parametrize("W,n,m,light", [(5, 20, 30, False), (6, 200, 256, False), (5, 300, 500, False), (160, 20, 30, False), (5, 20, 30, True)])
+def test_a_masks_launch_ends_when_its_last_lane_has_passed(W, n, m, light):
+    # drained lanes under a mask leave their launch together, in one block or in clusters, with lanes that stay in the log domain
+    # (a weight below 2^-80) and with more lanes than are on the GPU at a time (whose launches stay short); same bits and
+    # counts as without a mask, and what the last audit saw of lanes that froze long before it
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("sweep", W=W, n=n, m=m, d=8, max_iter=700, tol=3e-3)
+    if light:
+        w.a[0, 3] = 2.0 ** -90
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    out = []
+    for mode in ("active", "masked"):
+        sb = B.SinkhornBatch(t(w.x), t(w.y), t(w.a), t(w.b), t(w.eps), w.tol, mode=mode, max_iter=w.max_iter)
+        before = sb.launch_count()
+        sb.drain()
+        launches = sb.launch_count() - before
+        f, g = (v.cpu().numpy() for v in sb.potentials(f64=True))
+        depth, status = (v.cpu().numpy() for v in sb.depths())
+        assert sb.check_guards() == -1
+        out.append((f, g, depth, status, launches, sb.stats()["cycles"]))
+        if mode == "masked":
+            rr, rc, fl = (v.cpu().numpy() for v in sb.last_audit())
+            early = depth < depth.max()
+            assert (rr[early] <= w.tol * 1.01).all() and not fl[early].any()
+        sb.close()
+    for a, b in zip(out[0][:4], out[1][:4]):
+        np.testing.assert_array_equal(a, b)
+    assert out[1][5] == out[0][5] == out[0][2].max()
+    assert (out[1][4] <= 2 * 2 + 1) == (W < 148)           # two launches at most, each with its planner (and the ranking)
+
+
 def test_a_masks_launches_stay_short_however_many_cycles_are_asked_for():
     # under a logical mask lanes work until their launch ends: of 4096 cycles asked for, those past the launch in which the last
     # lane passes must be empty launches.  What a launch ran is not counted (Eq. 6-8 count to the last depth), so the launches are:
