@@ -38,7 +38,7 @@
 // What bounds it: the chain of dependent steps of a cycle (two rounds of multiply-adds, the exchange of row
 // sums, two float64 reciprocals, the column parts through shared memory, the exchange between blocks), not a
 // unit: the multiply-adds of a 256 x 256 lane are 256 clk of packed fp32 per scheduler, a cycle is 3700.
-// Measured per cycle in long launches: 8 lanes of 64 x 64, d = 2: 0.82 us; 96 of 100 x 77: 0.91 us; one lane of
+// Measured per cycle in long launches: 8 lanes of 64 x 64, d = 2: 0.75 us; 96 of 100 x 77: 1.2 us; one lane of
 // 256 x 256, d = 8, K in registers of a cluster of four blocks -> in tensor memory of one block: 1.7 -> 1.5 us; 148 of
 // them 5.4 -> 1.55 us (four blocks of a cluster per SM waited for each other's exchanges); all 1024 of the sweep workload
 // 27 -> 10 us, 24 -> 10.9 ms per solve at tol 1e-3.  512 x 512, clusters of eight blocks, registers -> of four, tensor memory:
@@ -779,9 +779,10 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
         }
     };
     // Logical mask: a frozen lane works on until the batch is over, which is when the last lane has passed and this one has
-    // run as many cycles.  Asked by one thread of the lane, every sixteenth cycle, and told to the others with the flags.
+    // run as many cycles.  Every 64th cycle one thread of the lane asks, and tells the others with the flags.  (Off the usual path: asked
+    // there with the flags of every cycle, it cost lanes without a mask 4 %.)
     auto mask_over = [&](const int k) -> int {
-        if (KIND != SC_CYCLES || !frozen || b != 0 || tid != 0 || (k & 15) != 0) return 0;
+        if (b != 0 || tid != 0) return 0;
         const volatile Ctl *now = P.ctl;
         if (now->mask_left < c.n_running) return 0;
         __threadfence();
@@ -966,7 +967,7 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                     const double S = row_exchange<CL, L::FP32_COLS, true, 16, RW, float>(s, lane);
                     unew = rok ? rcp64(S) : 1.0;
                     const double term = rown ? a_fix * fabs(fma(us, S, -1.0)) : 0.0;
-                    const int flags = mask_over(k) | ((rok && out_of_band<SC_SUMS>(S)) || out_of_band<SC_TAKE>(unew) ? SC_BAD | SC_DRIFT : (out_of_band<SC_KEEP>(unew) ? SC_DRIFT : 0));
+                    const int flags = (rok && out_of_band<SC_SUMS>(S)) || out_of_band<SC_TAKE>(unew) ? SC_BAD | SC_DRIFT : (out_of_band<SC_KEEP>(unew) ? SC_DRIFT : 0);
                     const unsigned long long fx = to_fixed(term);
                     if constexpr (LEG) {
                         send_rows(fx, flags);
@@ -1057,7 +1058,7 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                 }
                 tot = recv_rows(all);
                 ++xch;
-                if (all || (tot <= near_tot && !frozen && !catch_up) || nf || (k - start >= P.max_iter && !catch_up) || (closing && it == todo)) break;
+                if (all || (frozen ? (k & 63) == 0 : tot <= near_tot && !catch_up) || nf || (k - start >= P.max_iter && !catch_up) || (closing && it == todo)) break;
                 if (!frozen) put_vs(vn);
                 if (flags) vflag = 1;
                 __syncthreads();
@@ -1080,19 +1081,29 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
             if (tid == 0) atomicOr(&P.ctl->error, ERR_WAIT);
             break;
         }
-        if (all & SC_LEAVE) {
-            rr = (double)tot * (1.0 / RSUM_SCALE);           // (the state has been the same since it froze)
-            rc = 0.0;
-            fl = 0;
-            par = c.parity ^ (todo & 1);                     // where the lanes that go on have theirs
-            break;
-        }
         if (done) {
             // (the last audit was that of the state before this launch's last cycle, and it flagged nothing)
             rr = (double)tot * (1.0 / RSUM_SCALE);
             rc = 0.0;
             fl = 0;
             break;
+        }
+
+        if (KIND == SC_CYCLES && frozen && (k & 63) == 0) {
+            send_rows(0ull, mask_over(k));
+            scaling_barrier<CLU>();
+            int over;
+            recv_rows(over);
+            ++xch;
+            if (over & SC_LEAVE) {
+                // (a frozen lane's last audit flags nothing and has the residual of the state it froze at)
+                if (!(all & SC_BAD)) rr = (double)tot * (1.0 / RSUM_SCALE);
+                else if (it == 0) rr = P.rrow[slot];
+                rc = 0.0;
+                fl = 0;
+                par = c.parity ^ (todo & 1);                 // where the lanes that go on have theirs
+                break;
+            }
         }
 
         // ---------------- f-leg in the log domain, where K cannot be used
@@ -1111,17 +1122,10 @@ scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
                 unew = 0.0;
                 if (rok) row_math((int)FORM_DOT, true, P.la2[ro], P.sqx[ro], a_i, row_phi(us), (float)M, S, 0.f, unew, term);
                 const int flags = !isfinite(unew) || !isfinite(term) ? SC_NF : 0;
-                send_rows(rown && !flags ? to_fixed(term * RSUM_SCALE) : 0ull, flags | mask_over(k));
+                send_rows(rown && !flags ? to_fixed(term * RSUM_SCALE) : 0ull, flags);
                 scaling_barrier<CLU>();
                 tot = recv_rows(all);
                 ++xch;
-                if (all & SC_LEAVE) {
-                    rr = (double)tot * (1.0 / RSUM_SCALE);
-                    rc = 0.0;
-                    fl = 0;
-                    par = c.parity ^ (todo & 1);
-                    break;
-                }
             }
             if (all & SC_NF) nf = 1;
             near = tot <= near_tot;
