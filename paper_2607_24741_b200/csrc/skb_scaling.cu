@@ -49,6 +49,10 @@ void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int wid
     const ScalingVariant *v = scaling_variant(P.dots != nullptr, P.n, P.m);
     const void *kernel = v->kernel[kind];
     const int nc = blocks_of(*v, P.n);
+    // Lanes in half of the tensor memory: alone on their SM with all of its registers while that makes two rounds at most.  Drain
+    // of lanes of 128 x 160, d = 8, two blocks an SM -> one: 1 lane 994 -> 887 us, 148 1003 -> 905, 256 1105 -> 900, 400 1290 <- 1365,
+    // 1200 3073 <- 3519.
+    if (kind == SC_CYCLES && nc * width <= 2 * 148) kernel = v->roomy;
     // No block may take its place on an SM and then wait there for tensor memory while blocks of its cluster hold theirs.
     // Blocks that take the whole register file are alone anyway.  Others ask for shared memory in proportion to their tensor
     // memory; without a cluster they may wait, and ask for as much as keeps one block too many away.  (No more
