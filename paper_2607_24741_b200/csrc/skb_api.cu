@@ -760,7 +760,15 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
         if ((e = cudaMemcpyAsync(&h->h_ctl[snap], h->dev.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess)
             return cuda_fail(h, e, "drain");
         if ((e = cudaEventRecord(h->ev[snap], h->stream)) != cudaSuccess) return cuda_fail(h, e, "drain");
-        if (have_prev) {
+        // Launches of up to 2048 cycles are waited for one by one: a second one enqueued beside a first that finishes the batch is
+        // three empty kernels, and the control block that comes back with the first is the last (some 20 us of a solve).
+        // Shorter chunks: one is enqueued while the one before it runs.
+        if (scaling && !masked) {
+            if ((e = cudaEventSynchronize(h->ev[snap])) != cudaSuccess) return cuda_fail(h, e, "drain");
+            skb_status st = absorb(h, h->h_ctl[snap]);
+            if (st != SKB_OK) return st;
+            if (h->finished) { if (cycles_run) *cycles_run = h->h_ctl[snap].cycle; return SKB_OK; }
+        } else if (have_prev) {
             if ((e = cudaEventSynchronize(h->ev[snap ^ 1])) != cudaSuccess) return cuda_fail(h, e, "drain");
             skb_status st = absorb(h, h->h_ctl[snap ^ 1]);
             if (st != SKB_OK) { cudaStreamSynchronize(h->stream); return st; }
@@ -772,23 +780,24 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
         if (chunk < chunk_max && (scaling && chunk >= 64 ? h->enqueued - h->enqueued_at_refill >= 8 * chunk : (++rounds & 1) == 0)) chunk *= 2;
         if (h->enqueued - h->enqueued_at_refill > hard_cap + 64 + 2 * MAX_CYCLES_IN_LAUNCH) break;
     }
-    if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "drain");
-    if ((e = cudaMemcpy(&h->h_ctl[0], h->dev.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost)) != cudaSuccess)
-        return cuda_fail(h, e, "drain");
-    skb_status st = absorb(h, h->h_ctl[0]);
+    Ctl last;
+    skb_status st = read_ctl(h, &last);
     if (st != SKB_OK) return st;
     if (!h->finished) return fail(h, SKB_ERR_STATE, "drain ended with lanes still running");
-    if (cycles_run) *cycles_run = h->h_ctl[0].cycle;
+    if (cycles_run) *cycles_run = last.cycle;
     return SKB_OK;
 }
 
+// The control block when everything enqueued so far has run: one wait, for the copy behind it.  (A snapshot that step() has left in
+// flight lies in one of the two pinned blocks, and is absorbed later if it is not yet.)
 static skb_status read_ctl(skb_batch *h, Ctl *c)
 {
     cudaError_t e;
-    if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "sync");
-    if ((e = cudaMemcpy(&h->h_ctl[0], h->dev.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost)) != cudaSuccess)
+    Ctl *dst = &h->h_ctl[h->snap_pending ? h->snap_idx ^ 1 : 0];
+    if ((e = cudaMemcpyAsync(dst, h->dev.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess)
         return cuda_fail(h, e, "read control block");
-    *c = h->h_ctl[0];
+    if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "sync");
+    *c = *dst;
     return absorb(h, *c);
 }
 
@@ -1023,8 +1032,10 @@ extern "C" skb_status sinkhorn_batch_solve_host(const void *x, const void *y, co
     int cyc = 0;
     rc = sinkhorn_batch_drain(h, &cyc);
     if (rc == SKB_OK) rc = sinkhorn_batch_potentials(h, f ? (float *)(base + s.f) : nullptr, g ? (float *)(base + s.g) : nullptr);
-    if (rc == SKB_OK) rc = sinkhorn_batch_depths(h, (int *)(base + s.depth), (int *)(base + s.status));
-    if (rc == SKB_OK) rc = sinkhorn_batch_residuals(h, (float *)(base + s.rrow), (float *)(base + s.rcol));
+    if (rc == SKB_OK) {
+        launch_gather_small(h->dev, (int *)(base + s.depth), (int *)(base + s.status), (float *)(base + s.rrow), (float *)(base + s.rcol), h->stream);
+        if ((e = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(h, e, "solve_host (read-back)");
+    }
     if (rc == SKB_OK) {
         e = cudaSuccess;
         if (f) e = cudaMemcpyAsync(f, base + s.f, W * n * 4, cudaMemcpyDeviceToHost, st);
