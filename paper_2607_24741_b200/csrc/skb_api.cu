@@ -116,6 +116,10 @@ static double mixed_radius(double tol)
 // 747 us at 0.1 (all kept); 4 lanes of 4096 points 37 -> 16 us at 0.01, 35 -> 22 us at 0.03 (share 0.6), 35 -> 27 us at
 // 0.05 (0.8), 34 -> 34 us at 0.1.  (With few blocks in flight it still wins at 0.8, with many it loses from 0.75.)
 static const double NEAR_SHARE = 0.75;
+// With lists a pair is formed once per cycle instead of twice, and a list is shorter than the boxes that the estimate counts.  Plain -> one
+// pass, us a cycle: 16 lanes of 1024 points, share 0.82 33 -> 27, 1.0 37 -> 27; 4 of 2048, 0.88, 47 -> 24; 4 of 4096, 0.83, 63 -> 37; 32 of
+// 4096 293 -> 215; 8 of 600, 1.0, 27 -> 20.  Clouds of which next to nothing can be left out keep the plain kernel.
+static const double NEAR_SHARE_LISTS = 0.95;
 // ... and up to this tolerance: plans applied from looser solves agree with those of the plain kernel's potentials to
 // the rounding of its expanded cost, 1.2e-6 on the registration workload at tol 1e-2, and callers hold such results to
 // 1e-6 of earlier ones.  It costs those solves the 624 against 212 us a leg.
@@ -183,7 +187,7 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
     const size_t W = c->W, n = c->n, m = c->m;
     const size_t L = c->lane_capacity > c->W ? c->lane_capacity : c->W;      // lanes the result buffers hold
     const size_t DP = var->DP ? var->DP : padded_dim(c->d);
-    const bool near = spatial && !tensor && near_shape(var->f64, var->DP, var->CS, c->n, c->m);      // lanes in spatial order: whole boxes
+    const bool near = spatial && !tensor && near_shape(var->f64, var->DP, var->CS, c->n, c->m, room ? c->W : 1);      // lanes in spatial order: whole boxes
     const size_t np = align_up(n, near ? BOX_COLS : 4), mp = align_up(m, near ? BOX_COLS : 4);
     const size_t ts = var->f64 ? 8 : 4;
     Dev d;
@@ -403,7 +407,7 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     // spatial order: never for a cost form the caller named, nor for radii at which the plain kernels take differences
     const Variant *var_near = variant_for(cfg, SKB_COMPUTE_F32, true);
     const bool near_shaped = var_near && (automatic || cfg->compute == SKB_COMPUTE_F32) && (double)tol <= SPATIAL_TOL && cfg->cost_form == 0 &&
-                             near_shape(var_near->f64, var_near->DP, var_near->CS, cfg->n, cfg->m);
+                             near_shape(var_near->f64, var_near->DP, var_near->CS, cfg->n, cfg->m, room ? cfg->W : 1);
     if (near_shaped) { launch_near_estimate(h->dev, x, y, cfg->W, h->stream); h->launches += 1; }
     if (automatic || near_shaped) {
         // read the largest scaled radius back and pick the arithmetic and the layout for the whole batch
@@ -427,9 +431,14 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
         } else if (automatic && can_tensor) {
             h->tensor = true;
             carve(cfg, var, true, false, room, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
-        } else if (near_shaped && radius <= FORM_DIFF_RADIUS && h->h_ctl[1].near_kept <= NEAR_SHARE * NEAR_PAIRS * cfg->W) {
-            h->var = var_near;
-            carve(cfg, var_near, false, true, room, (char *)cfg->workspace, &h->dev, nullptr, &h->guards);
+        } else if (near_shaped && radius <= FORM_DIFF_RADIUS) {
+            Dev near;
+            GuardList strips;
+            carve(cfg, var_near, false, true, room, (char *)cfg->workspace, &near, nullptr, &strips);
+            const bool large = near_shape(var_near->f64, var_near->DP, var_near->CS, cfg->n, cfg->m, 1);
+            if ((near.lists || large) && h->h_ctl[1].near_kept <= (near.lists ? NEAR_SHARE_LISTS : NEAR_SHARE) * NEAR_PAIRS * cfg->W) {
+                h->var = var_near; h->dev = near; h->guards = strips;
+            }
         }
         h->dev.tol_stop = ts; h->dev.tol_screen = tsc;
     }

@@ -1037,15 +1037,16 @@ static void launch_apply_tiled(const Dev &P, const void *x, const void *y, const
     if (dv <= 4) apply_plan_tiled_kernel<DM, 4><<<grid, 128, 0, st>>>(P, x, y, eps, v, dv, out);
     else apply_plan_tiled_kernel<DM, APPLY_MAX_DV><<<grid, 128, 0, st>>>(P, x, y, eps, v, dv, out);
 }
-// Few blocks of 64 rows leave SMs empty while the threads of the tiled kernel walk 16 times the columns: up to the
-// counts below a warp per row is faster (us, tiled -> warp per row, d = dv = 3: one lane of 1000 points 82 -> 55; of
-// 4096, 64 blocks, 257 -> 168; of 5000, 79 blocks, 340 -> 333; of 6000, 94 blocks, 404 <- 415; d = 8, dv = 1, 32 blocks
-// 152 -> 114; d = 12, 8 blocks 56 -> 46; d = 30, 5 blocks 68 -> 58).  Wide values (dv = 16, d = 4, 64 blocks 265 <- 560)
-// and more dimensions (d = dv = 15, 16 blocks 102 <- 109) want the tiles earlier.
+// Few blocks of rows leave SMs empty while the threads of the tiled kernel walk 16 times the columns: up to the counts of blocks of 64
+// below a warp per row is faster (us, tiled <-> warp per row; d = 8, dv = 1: 500 points 43 <- 39, 1000 64 <- 58, 1300 75 <- 73, 1600 82 -> 83,
+// 2000 101 -> 112; wide values, d = dv = 5, two lanes of 1000 72 <- 56; dv = 12, d = 3, 500 points 42 <- 39).  Not where the tiles hold four
+// rows a thread (d = dv = 3: one lane of 500 points 35 -> 39, of 4096 100 -> 165, of 5000 139 -> 345), nor for narrow values of
+// more dimensions (d = 30, dv = 3, 8 blocks 61 -> 78).
 void launch_apply_plan(const Dev &P, const void *x, const void *y, const float *eps, const float *v, int dv, float *out,
                        int lanes, cudaStream_t st)
 {
-    const bool narrow = (long long)((P.n + 63) / 64) * lanes <= (P.d <= 8 && dv <= 8 ? 80 : 8);
+    const long long blocks = (long long)((P.n + 63) / 64) * lanes;
+    const bool narrow = dv <= 4 ? P.d > 4 && P.d <= 8 && blocks <= 24 : blocks <= (P.d <= 8 && dv <= 8 ? 80 : 8);
     if (P.d > P64_MAX_D || narrow) { apply_plan_kernel<<<dim3((P.n + 3) / 4, lanes), 128, 0, st>>>(P, x, y, eps, v, dv, out); return; }
     if (P.d <= 3) { launch_apply_tiled<3>(P, x, y, eps, v, dv, out, lanes, st); return; }
     if (P.d <= 4) { launch_apply_tiled<4>(P, x, y, eps, v, dv, out, lanes, st); return; }

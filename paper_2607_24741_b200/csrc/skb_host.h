@@ -74,7 +74,7 @@ void launch_update_tc(const Dev &P, const void *maps, int leg, int width, cudaSt
 void launch_gram(const Dev &P, const void *maps, int slot0, int count, cudaStream_t st);
 int launch_emit_move(const Dev &P, int width, cudaStream_t st);
 // lanes kept in spatial order, whose legs skip the boxes of columns that are too far away to matter
-bool near_shape(int f64, int DP, int CS, int n, int m);
+bool near_shape(int f64, int DP, int CS, int n, int m, int lanes);    // lanes: of a batch that has room for lists, else 1
 constexpr int NEAR_PAIRS = 4096;        // pairs per lane that launch_near_estimate counts into Ctl::near_kept
 void launch_near_estimate(const Dev &P, const void *x, const void *y, int lanes, cudaStream_t st);
 void launch_spatial_sort(const Dev &P, const void *x, const void *y, int slot0, int count, cudaStream_t st);

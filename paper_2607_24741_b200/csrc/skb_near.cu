@@ -50,11 +50,16 @@ constexpr double NEAR_FLOOR = 0x1p-6;
 // Points of the larger cloud from which the order pays: at 1024 points (16 lanes, eps 0.01) a leg is 13.7 -> 10.3 us and
 // a solve of 60 cycles 2.5 -> 2.3 ms, ordering included; the boxes of smaller clouds are too wide to skip much.
 constexpr int NEAR_MIN = 1024;
+// ... and with lists of single points (both legs in one pass) for clouds that are too large for the on-chip kernels, beside one another:
+// registration lanes, eps 0.01, a solve plain -> one pass: 32 of 520 points 17.9 -> 12.6 ms, 4 of 700 9.4 -> 8.3, 8 of 900 14.1 -> 9.6,
+// 32 of 900 21.6 -> 14.9; one lane of 600 (a cycle 17.2 <- 20.8 us) is better off where its blocks run many cycles in a launch.
+constexpr int NEAR_MIN_LISTS = 513;
 constexpr int NEAR_BLOCKS = 4;                      // blocks per SM (127 registers); five and six spill: 225 and 224 us a leg
 
-bool near_shape(int f64, int DP, int CS, int n, int m)
+bool near_shape(int f64, int DP, int CS, int n, int m, int lanes)
 {
-    return !f64 && DP > 0 && DP <= 4 && CS == 4 && (n > m ? n : m) >= NEAR_MIN;
+    const int mx = n > m ? n : m;
+    return !f64 && DP > 0 && DP <= 4 && CS == 4 && (mx >= NEAR_MIN || (lanes >= 2 && mx >= NEAR_MIN_LISTS));
 }
 
 // ---------------------------------------------------------------- is the order worth it

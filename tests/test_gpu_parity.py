@@ -1870,7 +1870,7 @@ def test_spatial_order_is_taken_where_it_can_skip(oracle, law, n, m, d, eps, exp
 # (law, n, m, d, eps): groups of 16 rows and lists by warp at their edges; lists longer than what tensor memory holds (a
 # large share of the pairs); outliers on both sides, whose potentials move by many bits in the first cycles
 ONE_PASS = [("sphere", 1040, 1025, 3, 0.02), ("sphere", 1100, 2049, 3, 0.05), ("cube", 1031, 97, 2, 0.002), ("cube", 40, 1025, 1, 0.002),
-            ("flat", 1500, 1100, 4, 0.004), ("outliers", 1300, 1300, 3, 0.01)]
+            ("flat", 1500, 1100, 4, 0.004), ("outliers", 1300, 1300, 3, 0.01), ("sphere", 600, 513, 3, 0.01), ("cube", 530, 90, 2, 0.01)]
 
 
 @pytest.mark.parametrize("law,n,m,d,eps", ONE_PASS)
