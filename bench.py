@@ -300,8 +300,8 @@ class Runner:
         elif spatial:
             # boxes of far columns are skipped, so the pairs a launch covers are not exponentials evaluated: no
             # fraction of a unit's rate can be formed from them
-            r = {"bound": "issue", "kernel": "update_near_kernel (f-leg, full width)", "arithmetic": arith,
-                 "binding_unit": "instruction issue and the latency of a box's chain", "achieved": achieved_exp / 1e12, "peak": None,
+            r = {"bound": "issue", "kernel": "near_rows_kernel (f-leg and column sums, full width)", "arithmetic": arith,
+                 "binding_unit": "instruction issue at the 16 warps an SM that tensor memory allows", "achieved": achieved_exp / 1e12, "peak": None,
                  "unit": "T pairs covered/s (far ones skipped)", "frac": None, "exp_frac": None, "pipe_frac": None,
                  "ms_per_launch": k_ms, "g_leg_ms_per_launch": g_ms, "pairs_per_launch": pairs,
                  "peak_clock_mhz": pk["sm_max_mhz"], "traffic": None}
