@@ -873,11 +873,7 @@ extern "C" skb_status sinkhorn_batch_last_audit(skb_batch *h, float *r_row, floa
     if (!h) return SKB_ERR_NULL;
     // (lanes that the streaming kernels would run a leg at a time have them on chip too: the planner moves them along)
     const bool streamed = h->tensor || (h->f32_on_chip && !narrow_lanes(h, h->var_stream));
-    // (small lanes in spatial order run a leg at a time; whether they keep these values is decided as for the kernels they would run
-    // whole cycles with otherwise)
-    const bool small = h->dev.permx && !near_shape(h->dev.compute_f64, h->dev.DP, 4, h->cfg.n, h->cfg.m, 1) && !h->profiling && !h->no_multi_cycle &&
-                       h->var_stream->launch_cycles && narrow_lanes(h, h->var_stream);
-    if ((cycles_in_one_launch(h) || small) && h->cfg.mode == SKB_ACTIVE && !streamed) return fail(h, SKB_ERR_STATE, "per-audit values are kept by the one-launch-per-leg path only (MASKED, STATIC, tensor or profiled batches)");
+    if (cycles_in_one_launch(h) && h->cfg.mode == SKB_ACTIVE && !streamed) return fail(h, SKB_ERR_STATE, "per-audit values are kept by the one-launch-per-leg path only (MASKED, STATIC, tensor or profiled batches)");
     launch_gather_audit(h->dev, r_row, r_col, flagged, h->stream);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? SKB_OK : cuda_fail(h, e, "last_audit");

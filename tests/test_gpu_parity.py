@@ -1898,14 +1898,10 @@ def test_both_legs_in_one_pass(oracle, monkeypatch, law, n, m, d, eps):
     assert pot_err(r["f"], r["g"], ref.f, ref.g, e).max() <= POT_TOL_F32
     rm = run_gpu(w, mode="masked")
     np.testing.assert_array_equal(rm["f"], r["f"]); np.testing.assert_array_equal(rm["g"], r["g"])
-    # values of the last audit: not of lanes small enough for the kernels that keep none, whatever they run here
+    # values of the last audit
     sb = B.SinkhornBatch(*(torch.from_numpy(v).to("cuda:0") for v in (w.x, w.y, w.a, w.b, w.eps)), w.tol, max_iter=cycles)
     sb.step(2)
-    if max(n, m) < 1024:
-        with pytest.raises(B.SkbError):
-            sb.last_audit()
-    else:
-        assert (sb.last_audit()[0] > 0).all()
+    assert (sb.last_audit()[0] > 0).all()
     sb.close()
     # one slot after the other, then two at a time: later lanes in slots that others have used
     t = lambda v: torch.from_numpy(v).to("cuda:0")
