@@ -231,7 +231,7 @@ class Runner:
         W, n, m, d = w.shape
         sb = self.batch("static")
         launches = sb.launch_count()
-        sb.step(12 if n >= 1024 and d <= 4 else 2)          # (lanes in spatial order: which columns count has settled by then)
+        sb.step(48 if n >= 1024 and d <= 4 else 2)          # (lanes in spatial order: which columns count has settled by then)
         k_ms = sb.profile_update(leg=0, reps=20 if W * n * m < (1 << 30) else 8)
         g_ms = sb.profile_update(leg=1, reps=3)
         arith = sb.arithmetic()

@@ -574,7 +574,7 @@ __device__ __forceinline__ void stream_near(const float *colc, const float *colt
 // and walks its own boxes, so there is one block barrier a group, for the row sums; the next group's record and the
 // heads of its lists are on their way meanwhile.  A thread has four rows and four of a step's 32 points.
 // What bounds it: instruction issue (half of the slots; 190 instructions a step of 16 pairs a thread, 86 of them multiply-adds, sums and
-// exponentials, and 640 a warp and group) at the 14 warps that tensor memory allows; the special-function unit is a quarter busy.
+// exponentials, and 640 a warp and group) at the 16 warps an SM that tensor memory allows; the special-function unit is a quarter busy.
 // Registration workload, f-leg and g-leg -> one pass and g-leg: 32 lanes of 8192 points 212 + 233 -> 200 + 9 us, solve 139 -> 76 ms;
 // one lane of 4096 points 14 + 24 -> 7 + 4 us, solve 12.8 -> 6.4 ms.  Steps on the way, 32 lanes: boxes of 8 points tested in every
 // cycle 423 us; lists of single points kept over cycles 247 us; persistent blocks, records ahead 234 us; a step's points
