@@ -980,7 +980,6 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) near_rows_kernel(con
         }
         __syncwarp();
         const float4 wr = *reinterpret_cast<const float4 *>(wsm[warp] + 4 * rq);
-        float most = 0.f;
         auto add_part = [&](const uint32_t (&w)[16], const unsigned id, const float sc) {
             auto col = [&](const int q) -> float {
                 return fmaf(__uint_as_float(w[12 + q]), wr.w, fmaf(__uint_as_float(w[8 + q]), wr.z, fmaf(__uint_as_float(w[4 + q]), wr.y, __uint_as_float(w[q]) * wr.x)));
@@ -989,10 +988,11 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) near_rows_kernel(con
             // halving exchange over the four threads that have the other rows
             const float k0 = (u1 ? s2 : s0) + __shfl_xor_sync(0xffffffffu, u1 ? s0 : s2, 1), k1 = (u1 ? s3 : s1) + __shfl_xor_sync(0xffffffffu, u1 ? s1 : s3, 1);
             const float v = ((u2 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, u2 ? k0 : k1, 2)) * sc;
-            most = fmaxf(most, v);
-            // (a total that something above the limit has gone into is not used)
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u64 p, %1, 0;\n\t@p red.global.add.u64 [%0], %1;\n\t}"
-                         ::"l"(at_bytes(acc, 8u * (ha + id))), "l"(__float2ull_rn(v)) : "memory");
+            useless = useless || !(v <= limit);          // (NaN, too)
+            // What rounds to nothing is not added.  Nor is a NaN, which the point of weight zero has, too, where a lane is not finite: its
+            // number is that of the next lane's first total.  (A total that something above the limit has gone into is not used.)
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %2, 0f3f000000;\n\t@p red.global.add.u64 [%0], %1;\n\t}"
+                         ::"l"(at_bytes(acc, 8u * (ha + id))), "l"(__float2ull_rn(v)), "f"(v) : "memory");
         };
         tc_st_wait();
         {
@@ -1023,7 +1023,7 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) near_rows_kernel(con
                     add_part(x, id, P.unit_low[hy + id].x);
                 });
         }
-        useless = useless || __any_sync(0xffffffffu, !(most <= limit));
+        useless = __any_sync(0xffffffffu, useless);
         if (useless && lane == 0 && !P.dry_run) P.no_sums[home] = c.cycle + 1;
 
         // ---- the rows' epilogue: one warp's, while the others go on
@@ -1081,7 +1081,7 @@ __device__ __forceinline__ bool columns_from_sums(const Dev &P, const Ctl &c, co
     if (has) {
         t = P.colacc[c.parity ^ 1][(size_t)home * P.mp + j];
         sq = P.sqy[o]; lb = P.lb2[o]; sc = P.unit_low[ho].x; before = P.gam[o];
-        low = !((double)t >= (double)CY_LOW * P.wb[o] * (double)sc) || t < (1ull << 36);
+        low = !((double)t >= (double)CY_LOW * P.wb[o] * (double)sc) || t < (1ull << 36) || t >= (1ull << 62);
     }
     if (__syncthreads_or(low)) return false;
     const bool frozen = (P.mode == MODE_MASKED) && P.state[slot] != 0;

@@ -1923,6 +1923,53 @@ def test_both_legs_in_one_pass(oracle, monkeypatch, law, n, m, d, eps):
     assert pot_err(rs["f"], rs["g"], ref.f, ref.g, e).max() <= POT_TOL_F32
 
 
+def _sphere_lanes(W, n, m, eps, cycles, seed=5):
+    # lanes on a noisy unit sphere, uneven weights: at eps 0.01 to 0.03 they go into spatial order
+    rng, f32 = np.random.default_rng(seed), np.float32
+    x, y = _cloud_pair("sphere", W, n, m, 3, rng)
+    a = rng.uniform(0.5, 1.5, (W, n)); b = rng.uniform(0.5, 1.5, (W, m))
+    return wl.Workload("sphere", x.astype(f32), y.astype(f32), (a / a.sum(1, keepdims=True)).astype(f32),
+                       (b / b.sum(1, keepdims=True)).astype(f32), np.asarray(eps, f32), 1e-3, cycles)
+
+
+def _parts(w, lanes):
+    import torch
+    return [torch.from_numpy(np.ascontiguousarray(v[lanes])).to("cuda:0") for v in (w.x, w.y, w.a, w.b, w.eps)]
+
+
+@pytest.mark.parametrize("first", [0, 3])
+def test_a_lane_that_is_not_finite_leaves_its_neighbours_alone(first):
+    # one pass: a lane whose points are finite but too far apart for fp32 comes in through a queue (create's radius test does not
+    # see it) and takes the place of lane `first`, before another's arrays or before the end of all.  Its sums are NaN in the second cycle; no
+    # part of them may go into another lane's totals or beyond the last one's, so the others' bits are those they have beside
+    # a lane that is fine
+    from paper_2607_24741_b200 import binding as B
+    eps = np.full(5, 0.01, np.float32)
+    eps[first] = 0.06
+    w = _sphere_lanes(5, 1040, 1050, eps, 150)
+    out = []
+    for broken in (False, True):
+        late = _parts(w, slice(4, 5))
+        if broken:
+            late[1][0, 5] = 1.0e20
+            late[1][0, 6] = -1.0e20
+        sb = B.SinkhornBatch(*_parts(w, slice(0, 4)), w.tol, max_iter=w.max_iter, lane_capacity=5)
+        while sb.active() == 4:
+            sb.step(1)
+        assert sb.active() == 3
+        sb.refill(*late)
+        sb.drain()
+        f, g = (v.cpu().numpy() for v in sb.potentials(f64=True))
+        depth, status = (v.cpu().numpy() for v in sb.depths())
+        assert sb.check_guards() == -1
+        sb.close()
+        assert depth[first] < depth[[k for k in range(4) if k != first]].min()
+        assert status[4] == (B.LANE_NONFINITE if broken else B.LANE_ITER_LIMIT)
+        out.append((f[:4], g[:4], depth[:4]))
+    for p, q in zip(*out):
+        np.testing.assert_array_equal(p, q)
+
+
 @pytest.mark.parametrize("cost_form", [0, 1, 2])
 def test_large_radii_in_fp32_take_differences_whatever_the_size(oracle, cost_form):
     # scaled squared radius of 1000 to 3000, asked for in fp32: cost_form 0 and 2 must be the difference form with
