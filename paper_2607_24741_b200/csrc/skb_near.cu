@@ -1064,14 +1064,19 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) near_rows_kernel(con
     if (warp == 0) { tc_fence_after(); tc_dealloc<CY_TM>(tm_holder); }
 }
 
-// The g-leg of RB columns from the totals that near_rows_kernel left.  False where they cannot be used: the caller
-// then goes over the pairs.  (All threads of the block take the same way.)
+// The g-leg of RB columns from the totals that near_rows_kernel left.  Returns, a bit for each box of 32, where they cannot be used: the
+// caller then goes over the pairs of those.  (By box, not by block: what a column is formed from must not depend on how many
+// a launch gives to a block.)
 template <int RB>
-__device__ __forceinline__ bool columns_from_sums(const Dev &P, const Ctl &c, const int slot, const int base)
+__device__ __forceinline__ unsigned columns_from_sums(const Dev &P, const Ctl &c, const int slot, const int base)
 {
+    constexpr unsigned ALL = (1u << RB / BOX_COLS) - 1u;
+    __shared__ unsigned left;
     const int home = P.home[slot];
-    if (P.no_sums[home] == c.cycle) return false;
+    if (P.no_sums[home] == c.cycle) return ALL;
     const int tid = threadIdx.x, j = base + tid;
+    if (tid == 0) left = 0u;
+    __syncthreads();
     const bool has = tid < RB && j < P.m;
     const size_t o = (size_t)slot * P.mp + (has ? j : 0), ho = (size_t)home * (P.mp + 1) + (has ? j : 0);
     unsigned long long t = 0ull;
@@ -1083,9 +1088,10 @@ __device__ __forceinline__ bool columns_from_sums(const Dev &P, const Ctl &c, co
         sq = P.sqy[o]; lb = P.lb2[o]; sc = P.unit_low[ho].x; before = P.gam[o];
         low = !((double)t >= (double)CY_LOW * P.wb[o] * (double)sc) || t < (1ull << 36) || t >= (1ull << 62);
     }
-    if (__syncthreads_or(low)) return false;
+    low = __any_sync(0xffffffffu, low);
+    if (low && (tid & 31) == 0) atomicOr(&left, 1u << tid / BOX_COLS);
     const bool frozen = (P.mode == MODE_MASKED) && P.state[slot] != 0;
-    if (tid < RB && !frozen && !P.dry_run) {             // whole warps
+    if (tid < RB && !low && !frozen && !P.dry_run) {     // whole warps
         double pot = -1.0e300;
         if (has) {
             const int e = (int)(__float_as_uint(sc) >> 23) - 127;
@@ -1103,7 +1109,8 @@ __device__ __forceinline__ bool columns_from_sums(const Dev &P, const Ctl &c, co
         if ((tid & 31) == 0 && has) P.topy[(size_t)slot * P.nby + j / BOX_COLS] = top;
         note_rise(P, c, slot, j, before, pot);
     }
-    return true;
+    __syncthreads();
+    return left;
 }
 
 // A block takes NG groups of 32 rows; its four warps share every group's boxes (box J goes to warp J mod 4), so
@@ -1148,8 +1155,10 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) update_near_kernel(c
     const float *cbox = (rows_x ? P.boxy : P.boxx) + (size_t)slot * 2 * DP * nbc;
     const float *ctop = rows_x ? P.topy + (size_t)slot * nbc : P.topx[c.parity] + (size_t)slot * (P.lists ? 2 : 1) * nbc;
     double before = 0.0;                                 // this thread's potential
+    unsigned own = (1u << NG) - 1u;                      // the groups that go over the pairs
     if (leg == LEG_G && P.lists) {
-        if (columns_from_sums<RB>(P, c, slot, row_base)) return;
+        own = columns_from_sums<RB>(P, c, slot, row_base);
+        if (!own) return;
         if (threadIdx.x < RB && row_base + (int)threadIdx.x < nrows) before = P.gam[(size_t)slot * rp + row_base + threadIdx.x];
     }
     const int nbox = (ncols + BOX_COLS - 1) / BOX_COLS;
@@ -1187,7 +1196,7 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) update_near_kernel(c
 #pragma unroll 1
         for (int g = 0; g < NG; ++g) {
             if (row_base + BOX_COLS * g >= nrows) break;
-            if (pass == 1 && !redo[g]) continue;
+            if (pass == 1 ? !redo[g] : !(own >> g & 1u)) continue;
             float mx[R];
             double sd[R];
             stream_near<DP, RB>(colc, colt, cp, nbox, cbox, ctop, !rows_x && P.lists, nbc, rows, g, cut, pass == 1, warp, lane, ring[warp], list[warp], mx, sd);
@@ -1201,7 +1210,7 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) update_near_kernel(c
         // the warps' parts, in warp order; rows far below their estimate start over, from "minus infinity" and over
         // all columns (rows that were fine keep the first pass's result, whatever their group needed)
         int low = 0;
-        if (tid < RB && (pass == 0 || sc.row_h[tid] != 0.f)) {
+        if (tid < RB && (own >> warp & 1u) && (pass == 0 || sc.row_h[tid] != 0.f)) {
             float m = part_m[0][tid];
             double t = part_s[0][tid];
 #pragma unroll
@@ -1219,8 +1228,8 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) update_near_kernel(c
         if (!__syncthreads_or(low)) break;
     }
     // (row_h is the shift of difference-form rows, which these lanes do not have: all zero by now)
-    finish_rows<float, RB, UPD_THREADS, true>(P, c, leg, slot, (int)FORM_DOT, sc.row_m, sc.row_s, sc.row_h, sc.red, row_base);
-    if (leg == LEG_G && P.lists && tid < RB) {
+    finish_rows<float, RB, UPD_THREADS, true>(P, c, leg, slot, (int)FORM_DOT, sc.row_m, sc.row_s, sc.row_h, sc.red, row_base, own);
+    if (leg == LEG_G && P.lists && tid < RB && (own >> warp & 1u)) {
         const int j = row_base + tid;
         if (j < nrows) home_potential(P, P.home[slot], j, P.gam[(size_t)slot * rp + j]);
         note_rise(P, c, slot, j, before, j < nrows ? P.gam[(size_t)slot * rp + j] : 0.0);

@@ -557,11 +557,11 @@ __device__ __forceinline__ void finish_lane_residual(const Dev &P, const int leg
 // Float64 epilogue of a CTA's RB rows (one thread per row) and the fused residual reduction.
 // row_m / row_s hold, per CTA-local row, the integer-valued maximum and the sum of
 // 2^(arg - max) over ALL columns; row_h the fp32 shift a difference-form row carried.
-// BOX: lanes in spatial order also keep the largest potential of every BOX_COLS points.
+// BOX: lanes in spatial order also keep the largest potential of every BOX_COLS points; only those of `boxes` (one bit each).
 template <typename T, int RB, int THREADS = UPD_THREADS, bool BOX = false>
 __device__ __forceinline__ void finish_rows(const Dev &P, const Ctl &c, const int leg, const int slot,
                                             const int form, const float *row_m, const double *row_s,
-                                            const float *row_h, double *red, const int row_base)
+                                            const float *row_h, double *red, const int row_base, const unsigned boxes = ~0u)
 {
     constexpr int NWARP = THREADS / 32;
     const int nrows = (leg == LEG_F) ? P.n : P.m;
@@ -573,6 +573,7 @@ __device__ __forceinline__ void finish_rows(const Dev &P, const Ctl &c, const in
         const int i = row_base + lr;
         if constexpr (BOX) {
             static_assert(RB % BOX_COLS == 0 && BOX_COLS == 32, "a warp's rows are one box");
+            if (!(boxes >> lr / BOX_COLS & 1u)) continue;
             double pot = -1.0e300, term = 0.0;
             if (i < nrows) term = finish_one_row<T>(P, c, leg, slot, form, i, row_m[lr], row_s[lr], row_h[lr], writes, &pot);
             if (writes) {

@@ -1970,6 +1970,35 @@ def test_a_lane_that_is_not_finite_leaves_its_neighbours_alone(first):
         np.testing.assert_array_equal(p, q)
 
 
+def test_a_lanes_bits_do_not_depend_on_the_width_of_its_launches():
+    # one pass: column launches of ten lanes have blocks of 64 columns, those of three lanes blocks of 32; in the first cycles some columns
+    # are low and go over the pairs, which must leave their neighbours in a block to the totals.  Outliers on both sides, a
+    # ragged last box; one batch, a queue through three slots, lanes by themselves
+    from paper_2607_24741_b200 import binding as B
+    W, n, m = 10, 1030, 4001
+    assert (m + 63) // 64 * 3 < 592 <= (m + 63) // 64 * W          # (the rule of the launch)
+    w = _sphere_lanes(W, n, m, np.linspace(0.01, 0.02, W), 16)
+    rng = np.random.default_rng(2)
+    for c in (w.x, w.y):
+        far = rng.random(c.shape[:2]) < 0.05
+        c[far] = rng.uniform(-1.0, 1.0, (int(far.sum()), 3))
+    whole = run_gpu(w)
+    assert whole["arith"] == "f32"
+    sb = B.SinkhornBatch(*_parts(w, slice(0, 3)), w.tol, max_iter=w.max_iter, lane_capacity=W)
+    for k in range(3, W, 3):
+        while sb.active():
+            sb.step(4)
+        sb.refill(*_parts(w, slice(k, min(k + 3, W))))
+    sb.drain()
+    f, g = (v.cpu().numpy() for v in sb.potentials(f64=True))
+    assert sb.check_guards() == -1
+    sb.close()
+    np.testing.assert_array_equal(f, whole["f"]); np.testing.assert_array_equal(g, whole["g"])
+    for k in (0, W - 1):
+        one = run_gpu(wl.Workload("one", *(np.ascontiguousarray(v[k:k + 1]) for v in (w.x, w.y, w.a, w.b, w.eps)), w.tol, w.max_iter))
+        np.testing.assert_array_equal(one["f"][0], whole["f"][k]); np.testing.assert_array_equal(one["g"][0], whole["g"][k])
+
+
 @pytest.mark.parametrize("cost_form", [0, 1, 2])
 def test_large_radii_in_fp32_take_differences_whatever_the_size(oracle, cost_form):
     # scaled squared radius of 1000 to 3000, asked for in fp32: cost_form 0 and 2 must be the difference form with
