@@ -720,7 +720,7 @@ extern "C" skb_status sinkhorn_batch_step(skb_batch *h, int cycles)
     if (st != SKB_OK) return st;
     cudaError_t e;
     if (cycles_in_one_launch(h)) {
-        const int longest = h->cfg.mode == SKB_MASKED ? MASK_CYCLES_IN_LAUNCH : MAX_CYCLES_IN_LAUNCH;
+        const int longest = h->cfg.mode == SKB_MASKED ? MASK_CYCLES_IN_LAUNCH : STEP_CYCLES_IN_LAUNCH;
         for (int left = cycles; left > 0 && !h->finished; left -= longest) enqueue_cycles_launch(h, left < longest ? left : longest);
     } else {
         for (int i = 0; i < cycles && !h->finished; ++i) {
@@ -753,7 +753,7 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
     // on until the last one has passed), so the longest launch costs nothing and saves forming the kernel matrices again.  Not
     // so for a mask with more lanes than are on the GPU at a time: those work until the launch ends, so its launches
     // grow to 64 cycles and beyond that only to an eighth of what has been done.  96 lanes of 100 x 77 (deepest 2970 cycles),
-    // launches that grow -> launches of 2048: 5.0 -> 3.9 ms a solve.
+    // launches that grow -> long launches: 5.0 -> 3.9 ms a solve.
     const bool scaling = h->dev.phi0 && cycles_in_one_launch(h), masked = h->cfg.mode == SKB_MASKED && scaling && h->cfg.W > scaling_resident(h->dev);
     int chunk = scaling ? (masked ? 16 : MAX_CYCLES_IN_LAUNCH) : 2, snap = 0, rounds = 0;
     bool have_prev = false;
@@ -769,8 +769,9 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
         if ((e = cudaMemcpyAsync(&h->h_ctl[snap], h->dev.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess)
             return cuda_fail(h, e, "drain");
         if ((e = cudaEventRecord(h->ev[snap], h->stream)) != cudaSuccess) return cuda_fail(h, e, "drain");
-        // Launches of up to 2048 cycles are waited for one by one: a second one enqueued beside a first that finishes the batch is
-        // three empty kernels, and the control block that comes back with the first is the last (some 20 us of a solve).
+        // Long launches are waited for one by one: a second one enqueued beside a first that finishes the batch is
+        // three empty kernels, and the control block that comes back with the first is the last (some 20 us of a solve).  They are
+        // as long as the planner takes, for the wait between two of them is as much again.
         // Shorter chunks: one is enqueued while the one before it runs.
         if (scaling && !masked) {
             if ((e = cudaEventSynchronize(h->ev[snap])) != cudaSuccess) return cuda_fail(h, e, "drain");

@@ -522,7 +522,9 @@ template <typename T, bool FUSE>
 __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, const int K)
 {
     __shared__ int wsum[PLAN_THREADS / 32][3];
-    __shared__ int left_at[MAX_CYCLES_IN_LAUNCH];   // lanes that left at the audit of the state after k0 + j cycles
+    // lanes that left at the audit of the state after k0 + j cycles (a word between 32 of them: threads read runs of a power of two)
+    __shared__ int left_[MAX_CYCLES_IN_LAUNCH + MAX_CYCLES_IN_LAUNCH / 32];
+    auto left_at = [&](const int j) -> int & { return left_[j + (j >> 5)]; };
     __shared__ int checks_s, nret_s, last_s, ran_s;
     __shared__ unsigned long long slots_s, terms_s;
     pdl_enter();
@@ -530,13 +532,13 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
     const int tid = threadIdx.x, NT = blockDim.x;
     if (c.done) { if (tid == 0) P.ctl->n_retire = 0; return; }
     const int k0 = c.cycle, A = c.n_phys;
-    for (int j = tid; j < K; j += NT) left_at[j] = 0;
+    for (int j = tid; j < K; j += NT) left_at(j) = 0;
     if (tid == 0) { checks_s = nret_s = ran_s = 0; last_s = 0; slots_s = terms_s = 0ull; }
     __syncthreads();
     int nchk = 0;
     for (int s = tid; s < A; s += NT) {
         const int r = P.ret_at[s];
-        if (r > 0) { atomicAdd(&left_at[r - 1 - k0], 1); atomicAdd(&nret_s, 1); atomicMax(&last_s, r - 1 - k0); }
+        if (r > 0) { atomicAdd(&left_at(r - 1 - k0), 1); atomicAdd(&nret_s, 1); atomicMax(&last_s, r - 1 - k0); }
         nchk += P.n_checks[s];
         P.rsum_row[s] = 0ull; P.rsum_col[s] = 0ull;      // between launches the residual sums are zero
         P.rsum_row64[s] = 0ull; P.esc[s] = 0;
@@ -598,7 +600,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
         const bool full = P.mode == MODE_MASKED && !P.early_exit;
         const int per = (K + NT - 1) / NT, j0 = tid * per, j1 = min(K, j0 + per);
         int mine = 0;
-        for (int j = j0; j < j1; ++j) mine += left_at[j];
+        for (int j = j0; j < j1; ++j) mine += left_at(j);
         int incl = mine;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) { const int o = __shfl_up_sync(0xffffffffu, incl, off); if ((tid & 31) >= off) incl += o; }
@@ -609,7 +611,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_cycles_kernel(const Dev P, 
         unsigned long long slots = 0ull, legs = 0ull;
         for (int j = j0; j < j1 && w > 0; ++j) {
             legs += full ? A : w;                        // the f-leg whose epilogue screened the state after k0 + j cycles
-            w -= left_at[j];
+            w -= left_at(j);
             if (w == 0) break;
             const int width = full ? A : w;              // the launch's width is the running lanes', or W under a mask
             if (k0 + j < P.widths_cap) P.widths[k0 + j] = width;      // cycle k0 + j + 1 ran at this width

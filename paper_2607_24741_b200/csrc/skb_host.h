@@ -45,8 +45,11 @@ struct Variant {
 };
 constexpr int MAX_CLUSTER_BLOCKS = MAX_CLUSTER_RANKS;   // a lane needs at most this many row blocks
 // Upper bound on the cycles one multi-cycle launch runs.  Lanes are independent and leave a launch when they pass, so a
-// long launch keeps the SMs full where a series of short ones waits for its slowest lanes after each.
-constexpr int MAX_CYCLES_IN_LAUNCH = 2048;
+// long launch keeps the SMs full where a series of short ones waits for its slowest lanes after each.  A drain waits for every launch
+// before it enqueues the next, 12 to 17 us with an idle GPU, which lanes deeper than this pay.
+constexpr int MAX_CYCLES_IN_LAUNCH = 8192;
+// ... of those that a caller's number of cycles is cut into (enqueued one behind the other)
+constexpr int STEP_CYCLES_IN_LAUNCH = 2048;
 // ... and under a logical mask, whose lanes work on until the last one has passed, however early they do.  Lanes that wait for a
 // place on the GPU cannot pass, so a launch of more lanes than fit works on to its end: what a caller asks for
 // beyond the last lane's depth costs at most the rest of one launch (launches after it return at once).

@@ -1759,6 +1759,32 @@ def test_a_masks_launch_ends_when_its_last_lane_has_passed(W, n, m, light):
     assert (out[1][4] <= 2 * 2 + 1) == (W < 148)           # two launches at most, each with its planner (and the ranking)
 
 
+@pytest.mark.parametrize("mode", ["active", "static", "masked"])
+def test_a_drain_of_deep_lanes_waits_once_in_8192_cycles(mode):
+    # a drain waits for a launch before it enqueues the next, so lanes of thousands of cycles must not be cut into many launches;
+    # however they are cut, a lane's bits and the accounting are those of single steps.  (No lane passes: depth = max_iter.)
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("sweep", W=3, n=30, m=20, d=4, max_iter=8300, tol=1e-12)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    out = []
+    for step in (0, 700):
+        sb = B.SinkhornBatch(t(w.x), t(w.y), t(w.a), t(w.b), t(w.eps), w.tol, mode=mode, max_iter=w.max_iter)
+        before = sb.launch_count()
+        while step and sb.active():
+            sb.step(step)
+        sb.drain()
+        launches = sb.launch_count() - before
+        f, g = (v.cpu().numpy() for v in sb.potentials(f64=True))
+        s = sb.stats(widths_cap=9000)
+        assert s["cycles"] == 8300 and s["slots"] == 3 * 8300 and list(s["widths"]) == [3] * 8300
+        assert (sb.depths()[0] == 8300).all() and sb.check_guards() == -1
+        out.append((f, g, launches))
+        sb.close()
+    assert out[0][2] <= 2 * 3
+    np.testing.assert_array_equal(out[0][0], out[1][0]); np.testing.assert_array_equal(out[0][1], out[1][1])
+
+
 def test_a_masks_launches_stay_short_however_many_cycles_are_asked_for():
     # under a logical mask lanes work until their launch ends: of 4096 cycles asked for, those past the launch in which the last
     # lane passes must be empty launches.  What a launch ran is not counted (Eq. 6-8 count to the last depth), so the launches are:
