@@ -584,10 +584,11 @@ constexpr int CY_TM = 16 * CY_STEPS;                     // ... columns of it: f
 constexpr float CY_MARGIN = 2.f;
 constexpr float CY_LOW = 0x1p-6f, CY_HIGH = 0x1p60f;
 
-// How far the potentials of 32 target points (a warp's) have risen since their base, or their new base.
+// How far the potentials of 32 target points (a warp's) have risen since their base, or their new base.  Those of a frozen lane, too, whose
+// potentials stay: a lane that froze in the cycle of a new base would go without and make its lists in every cycle from then on.
 __device__ __forceinline__ void note_rise(const Dev &P, const Ctl &c, const int slot, const int j, const double before, const double now)
 {
-    if (P.dry_run || ((P.mode == MODE_MASKED) && P.state[slot] != 0)) return;      // (whole warps)
+    if (P.dry_run) return;
     const int home = P.home[slot], at = P.based_at[home];
     const bool has = j < P.m;
     float base = -3.0e38f, rise = 0.f;
@@ -1091,9 +1092,9 @@ __device__ __forceinline__ unsigned columns_from_sums(const Dev &P, const Ctl &c
     low = __any_sync(0xffffffffu, low);
     if (low && (tid & 31) == 0) atomicOr(&left, 1u << tid / BOX_COLS);
     const bool frozen = (P.mode == MODE_MASKED) && P.state[slot] != 0;
-    if (tid < RB && !low && !frozen && !P.dry_run) {     // whole warps
-        double pot = -1.0e300;
-        if (has) {
+    if (tid < RB && !low && !P.dry_run) {                // whole warps
+        double pot = frozen ? before : -1.0e300;
+        if (has && !frozen) {
             const int e = (int)(__float_as_uint(sc) >> 23) - 127;
             pot = before + lb - (log2((double)t) - (double)e);
             float hi, lo;
@@ -1106,7 +1107,7 @@ __device__ __forceinline__ unsigned columns_from_sums(const Dev &P, const Ctl &c
         float top = __double2float_ru(pot);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, off));
-        if ((tid & 31) == 0 && has) P.topy[(size_t)slot * P.nby + j / BOX_COLS] = top;
+        if ((tid & 31) == 0 && has && !frozen) P.topy[(size_t)slot * P.nby + j / BOX_COLS] = top;
         note_rise(P, c, slot, j, before, pot);
     }
     __syncthreads();

@@ -1996,6 +1996,32 @@ def test_a_lane_that_is_not_finite_leaves_its_neighbours_alone(first):
         np.testing.assert_array_equal(p, q)
 
 
+@pytest.mark.parametrize("mode", ["masked", "static"])
+def test_a_frozen_lane_keeps_its_lists(mode):
+    # one pass: the first lane (a flat kernel) passes after one cycle, in which the potentials of its heavy targets rise by three bits, so
+    # that the pass which finds it done calls for new lists.  It works on under a mask, and must not make them again in
+    # every cycle.  What a group's lists were made from is kept as a count of cycles, so
+    # a lane that makes its lists in cycle k writes the number k once for every group of 16 points
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    n, cycles = 2048, range(98, 118)                       # (lengths of lists are multiples of 32)
+    w = _sphere_lanes(3, n, 2048, [400.0, 0.01, 0.01], 200)
+    w.b[0, ::16] *= 8.0
+    w.b[0] /= w.b[0].astype(np.float64).sum()
+    sb = B.SinkhornBatch(*_parts(w, slice(0, 3)), w.tol, mode=mode, max_iter=w.max_iter)
+    sb.step(cycles[0] - 1)
+    depth = sb.depths()[0].cpu().numpy()
+    assert depth[0] == 1 and (mode == "static" or not depth[1:].any())
+    made = []
+    for k in cycles:
+        sb.step(1)
+        assert sb.stats()["cycles"] == k
+        words = sb.workspace[:sb.workspace.numel() // 4 * 4].view(torch.int32)
+        made.append(int((words == k).sum()) >= n // 16)
+    sb.close()
+    assert sum(made) <= 4, made                            # (the other lanes' lists hold for a dozen cycles and more by then)
+
+
 def test_a_lanes_bits_do_not_depend_on_the_width_of_its_launches():
     # one pass: column launches of ten lanes have blocks of 64 columns, those of three lanes blocks of 32; in the first cycles some columns
     # are low and go over the pairs, which must leave their neighbours in a block to the totals.  Outliers on both sides, a
