@@ -228,11 +228,12 @@ void launch_spatial_sort(const Dev &P, const void *x, const void *y, int slot0, 
     spatial_sort_kernel<<<dim3((mx + SORT_CHUNK - 1) / SORT_CHUNK, count, 2), 1024, smem, st>>>(P, x, y, slot0);
 }
 
-// The largest potential of a box of the source (with lists: of its halves).
+// The largest potential of a box of the source (with lists: of its halves; one without points keeps this minus infinity, for
+// near_rows_kernel writes the others only).
 __device__ __forceinline__ void top_x(const Dev &P, const int parity, const int slot, const int box, const float top)
 {
     const size_t o = (size_t)slot * P.nbx + box;
-    if (P.lists) reinterpret_cast<float2 *>(P.topx[parity])[o] = make_float2(top, top);
+    if (P.lists) reinterpret_cast<float2 *>(P.topx[parity])[o] = make_float2(top, BOX_COLS * box + GROUP_ROWS < P.n ? top : -3.0e38f);
     else P.topx[parity][o] = top;
 }
 __device__ __forceinline__ GroupRecord &group_record(const Dev &P, const int home, const int group)

@@ -1996,6 +1996,30 @@ def test_a_lane_that_is_not_finite_leaves_its_neighbours_alone(first):
         np.testing.assert_array_equal(p, q)
 
 
+def test_a_half_box_without_points_has_no_largest_potential(monkeypatch):
+    # one pass: the source's largest potentials are kept for halves of a box of 32; that of the last box is empty where n mod 32 is 1 to 16,
+    # and must not hold its box's pairs up with what was there before.  Its value is minus infinity (-3e38) in both buffers, as
+    # are the two of an empty half's record and the upper corner of its box: seven words a lane of a workspace that was zero
+    import torch
+    from paper_2607_24741_b200 import binding as B
+
+    class Zeros:
+        empty = staticmethod(torch.zeros)
+        __getattr__ = staticmethod(lambda name: getattr(torch, name))
+    monkeypatch.setattr(B, "torch", Zeros())
+    w = _sphere_lanes(3, 1040, 1056, [0.01, 0.01, 0.01], 50)
+    warm = [torch.zeros(3, k, dtype=torch.float64, device="cuda:0") for k in (1040, 1056)]
+    for cycles, first in ((0, None), (0, warm), (7, None)):
+        sb = B.SinkhornBatch(*_parts(w, slice(0, 3)), w.tol, max_iter=w.max_iter)
+        if first:
+            sb.warm_start(*first)
+        sb.step(cycles)
+        torch.cuda.synchronize()
+        words = sb.workspace[:sb.workspace.numel() // 4 * 4].view(torch.float32)
+        assert int((words == torch.tensor(-3.0e38, device="cuda:0")).sum()) == 3 * 7
+        sb.close()
+
+
 @pytest.mark.parametrize("mode", ["masked", "static"])
 def test_a_frozen_lane_keeps_its_lists(mode):
     # one pass: the first lane (a flat kernel) passes after one cycle, in which the potentials of its heavy targets rise by three bits, so
