@@ -260,7 +260,7 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
             d.colacc[0] = (unsigned long long *)take(W * mp * 8); d.colacc[1] = (unsigned long long *)take(W * mp * 8);
             d.lists = (unsigned short *)take(lists);
             d.base_gam = (float *)take(W * mp * 4); d.base_top = (float *)take(W * d.nby * 4);
-            d.risen = (unsigned long long *)take(W * 8); d.based_at = (int *)take(W * 4); d.no_sums = (int *)take(W * 4);
+            d.risen = (unsigned long long *)take(W * 8); d.based_at = (int *)take(W * 4); d.overrun = (unsigned *)take(W * 8);
         }
     }
     if (tensor && room && scaling_fits(true, c->n, c->m) && L * np * mp * 4 <= DOTS_LIMIT) {

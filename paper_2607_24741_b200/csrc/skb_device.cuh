@@ -114,7 +114,7 @@ struct Dev {
     // of two next to 2^44 / b and the rest of the potentials, centres of the boxes of 32, the least log2 b in them, column
     // sums in units of those powers (double-buffered by the cycle's parity).  For every group and warp the target points that matter to it; the target's potentials that the
     // lists were made from, by point and the largest by box, how far they have risen since (high word: the cycle of
-    // `then`), that cycle, and the last cycle without column sums
+    // `then`), that cycle, and what phi has risen by beyond what the lists have room for (two buffers of W)
     int *home;
     float *boxx16, *crdy, *gamy, *ceny, *lby;
     float2 *unit_low;
@@ -123,7 +123,8 @@ struct Dev {
     unsigned short *lists;
     float *base_gam, *base_top;
     unsigned long long *risen;
-    int *based_at, *no_sums;
+    int *based_at;
+    unsigned *overrun;
     int list_cap;             // entries of a warp's list
     const int *order;         // scaling_kernel, a batch's first launch: the order in which slots are started (null: as they are)
     // per-slot scalars

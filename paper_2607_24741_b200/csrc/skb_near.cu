@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(128) prep_near_kernel(const Dev P, const void 
                 P.unit_low[(size_t)home * (pp + 1) + pp].x = 0.f;
                 home_potential(P, home, pp, (double)NEG_BIG);
             }
-            if (i == 0) { P.home[slot] = home; P.risen[home] = 0ull; P.based_at[home] = 0; P.no_sums[home] = 0; }
+            if (i == 0) { P.home[slot] = home; P.risen[home] = 0ull; P.based_at[home] = 0; P.overrun[home] = P.overrun[P.W + home] = 0u; }
         }
     } else {
         for (int e = 0; e < 2; ++e) {
@@ -566,6 +566,11 @@ __device__ __forceinline__ void stream_near(const float *colc, const float *colt
 // most of them among the first 50.)  All of it follows from the lane's own values, cycle by cycle.
 // Rows whose sum comes out below 2^-6 of the estimate, or above 2^60, start over with the largest argument over all columns as
 // their reference.  Columns whose total comes out below 2^-6 of b_j (or beyond its range) are left to the g-leg's own pass.
+// What is left out is below 2^-32 of a row's estimated sum, so below 2^-26 of any row sum that is taken.  A column's part is
+// bounded with pcol, from before the f-leg, which may raise phi by up to six bits: where it raises group g's beyond what
+// its lists have room for, by r_g bits, up to 2^-32 of b_j times the mean of 2^r_g over the groups is missing, and columns are left to
+// their own pass below 2^-6 of b_j times that mean already (`overrun`), so that less than 2^-26 of any total that is taken is missing, too.
+// (With the largest r_g in place of the mean, which outliers set: registration 76.4 -> 77.1 ms.)
 //
 // Arguments.  E_j is formed as ((gam_j - ref) - |c_j|^2 / 2), the potential as the sum of two fp32 numbers, c_j relative to the centre of
 // the group's box of 32 and ref one row's reference, so what is rounded is small where an entry matters.  Against 64 bits, 16
@@ -609,6 +614,12 @@ __device__ __forceinline__ void note_rise(const Dev &P, const Ctl &c, const int 
     if ((threadIdx.x & 31) == 0) atomicMax(P.risen + home, ((unsigned long long)(unsigned)at << 32) | __float_as_uint(rise));
 }
 
+// 2^r of a group whose phi has risen by r bits more than its lists have room for, added up by lane as integers (any order), double-buffered
+// like the column totals (the planner zeroes the next cycle's: beside the totals that store cost 5 of 245 us a cycle, in the g-leg 1 of 9);
+// OVERRUN_ALL: those cannot be used.
+constexpr float OVERRUN_UNIT = 64.f;
+constexpr unsigned OVERRUN_ALL = 1u << 31;               // (2^14 groups, the most that 262 143 points make, of 2^14 + 1 units stay below)
+
 // base + off bytes: a base that is the same for the whole launch and a 32-bit offset (the layout keeps these arrays below 4 GiB)
 template <typename T>
 __device__ __forceinline__ T *at_bytes(T *base, const unsigned off)
@@ -629,6 +640,7 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) near_rows_kernel(con
     __shared__ float partm[NW][GR];
     __shared__ __align__(16) float wsm[NW][GR];
     __shared__ float redo_ref[GR];
+    __shared__ float allowed[2];                         // the largest phi that the group's lists have room for
     __shared__ uint32_t tm_holder;
 
     // (programmatic dependent launch as in update_kernel)
@@ -700,6 +712,7 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) near_rows_kernel(con
         const float wt = R.row[rr].y;
         bool stale = rebase || R.made_from != based || !(prow - R.made_prow <= CY_MARGIN - rise && pcol - R.made_pcol <= CY_MARGIN - rise);
         int len = stale ? 0 : R.len[warp];
+        if (tid == 0 && !stale) allowed[b] = R.made_pcol + (CY_MARGIN - rise);
         float gcen[DP], gref = R.row[0].x > NEG_BIG ? -R.row[0].x : 0.f;          // a reference for the whole group
         u64 xn[4][DP], nref[4];
 #pragma unroll
@@ -772,7 +785,10 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) near_rows_kernel(con
             for (int at = cnt + lane; at < len + 64; at += 32) { list[at] = (unsigned short)P.mp; if (at < HEAD + 64) id0[at] = (unsigned short)P.mp; }
             GroupRecord &g = group_record(P, home, group);
             if (lane == 0) g.len[warp] = len;
-            if (tid == 0) { g.made_prow = prow; g.made_pcol = pcol; g.made_from = rebase ? c.cycle + 1 : based; }
+            if (tid == 0) {
+                g.made_prow = prow; g.made_pcol = pcol; g.made_from = rebase ? c.cycle + 1 : based;
+                allowed[b] = pcol + (rebase ? CY_MARGIN : CY_MARGIN - rise);
+            }
             __syncwarp();
         };
         // A step is 32 listed points.  They are shifted to the group's centre once, by the lane they fall to, and go through shared
@@ -1026,12 +1042,13 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) near_rows_kernel(con
                 });
         }
         useless = __any_sync(0xffffffffu, useless);
-        if (useless && lane == 0 && !P.dry_run) P.no_sums[home] = c.cycle + 1;
+        if (useless && lane == 0 && !P.dry_run) atomicOr(P.overrun + (size_t)c.parity * P.W + home, OVERRUN_ALL);
 
         // ---- the rows' epilogue: one warp's, while the others go on
         if (warp == (turn++ & (NW - 1))) {
             const bool frozen = (P.mode == MODE_MASKED) && P.state[slot] != 0, writes = !frozen && !P.dry_run;
             const bool in = wt > 0.f;
+            const float most = allowed[b];
             const int ri = group * GR + rr;
             const size_t ro = (size_t)slot * P.np + (in ? ri : 0);
             const double p0 = P.phi[c.parity][ro], lw = P.la2[ro], sq = P.sqx[ro];
@@ -1056,6 +1073,9 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) near_rows_kernel(con
                 for (int off = GR / 2; off > 0; off >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, off));
                 if (lane == 0) P.topx[c.parity ^ 1][(size_t)slot * 2 * P.nbx + group] = top;
                 row_record(P, home, ri, in, pot, lw, sq, wt);                   // (both halves of the warp write the same)
+                // (the whole warp asks; at most six bits, or the rows have started over)
+                if (top > most && lane == 0)
+                    atomicAdd(P.overrun + (size_t)c.parity * P.W + home, (unsigned)(OVERRUN_UNIT * ex2_fast(fminf(top - most, 8.f))) + 1u);
             }
             if (lane == 0 && !P.dry_run) finish_lane_residual(P, LEG_F, slot, fixed);
         }
@@ -1076,7 +1096,7 @@ __device__ __forceinline__ unsigned columns_from_sums(const Dev &P, const Ctl &c
     constexpr int NB = RB / BOX_COLS;
     __shared__ int low_box[NB];
     const int home = P.home[slot];
-    const bool none = P.no_sums[home] == c.cycle;
+    const unsigned over = P.overrun[(size_t)(c.parity ^ 1) * P.W + home];
     const int tid = threadIdx.x, j = base + tid;
     const bool has = tid < RB && j < P.m;
     const size_t o = (size_t)slot * P.mp + (has ? j : 0), ho = (size_t)home * (P.mp + 1) + (has ? j : 0);
@@ -1087,7 +1107,10 @@ __device__ __forceinline__ unsigned columns_from_sums(const Dev &P, const Ctl &c
     if (has) {
         t = P.colacc[c.parity ^ 1][(size_t)home * P.mp + j];
         sq = P.sqy[o]; lb = P.lb2[o]; sc = P.unit_low[ho].x; before = P.gam[o];
-        low = none || !((double)t >= (double)CY_LOW * P.wb[o] * (double)sc) || t < (1ull << 36) || t >= (1ull << 62);
+        double least = (double)CY_LOW;                   // of b_j
+        if (over)
+            least = over >= OVERRUN_ALL ? 1.0e300 : least * (double)(1.f + (float)over / (OVERRUN_UNIT * (float)((P.n + GROUP_ROWS - 1) / GROUP_ROWS)));
+        low = !((double)t >= least * P.wb[o] * (double)sc) || t < (1ull << 36) || t >= (1ull << 62);
     }
     low = __any_sync(0xffffffffu, low);
     if (tid < RB && (tid & 31) == 0) low_box[tid / BOX_COLS] = low;
