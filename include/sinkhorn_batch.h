@@ -95,8 +95,9 @@ typedef struct {
     int cost_form;         /* fp32 arithmetic: 0 = chosen from the lanes' scaled radii; 1 = */
                            /* expanded |x|^2+|y|^2-2x.y everywhere; 2 = difference |x-y|^2  */
                            /* everywhere.  With 0, lanes of at most four dimensions and at  */
-                           /* least 1024 points (513 in batches of two and more, where the  */
-                           /* workspace has room for lists) may be kept in spatial order,   */
+                           /* least 1024 points (513 where the batch can take in two lanes  */
+                           /* and more and the workspace has room for lists) may be kept in */
+                           /* spatial order,                                                */
                            /* coordinates relative to local boxes, where create finds that  */
                            /* it pays                                                       */
     void *stream;          /* cudaStream_t (0 = legacy default stream)                     */
@@ -129,7 +130,8 @@ typedef struct {
  * also takes a workspace without that room (4 W n m and some 8 W (3 n + 2 m) bytes less, as far as
  * an automatic batch, which may need float64 coordinates instead, does not need more anyway).
  * fp32 lanes of at most four dimensions that may be kept in spatial order are given room for lists of the
- * pairs that matter to them, some W n m / 8 bytes, as long as those are at most 2 GiB (and m below 65 535).  With them
+ * pairs that matter to them, some W n m / 8 bytes, as long as n m / 8 bytes for every lane that the batch can take in (W, or
+ * lane_capacity if that is more) are at most 8 GiB (and m below 65 535).  With them
  * a cycle takes one pass over those pairs (32 lanes of 8192 points: 0.24 ms), without two passes over
  * more of them (0.5 ms); create takes a workspace without that room, too.  Both ways agree to rounding. */
 size_t sinkhorn_batch_workspace_bytes(const skb_config *cfg);

@@ -131,11 +131,15 @@ static const double SPATIAL_TOL = 2.0e-3;
 // one batch of all of them run the same arithmetic, so a lane's bits do not depend on how it came in.
 static const size_t DOTS_LIMIT = (size_t)4 << 30;
 
-// Lanes in spatial order keep lists of the pairs that matter (n m / 8 bytes a lane), up to this size of all of them (250 lanes of 8192
-// points, 1 % of the card's memory); beyond it, and in a workspace without room for them, each leg chooses its pairs by itself.
-static const size_t NEAR_LISTS_LIMIT = (size_t)2 << 30;
+// Lanes in spatial order keep lists of the pairs that matter (n m / 8 bytes a slot), up to this size for all lanes that the batch can take in
+// (1000 lanes of 8192 points; as for the products above, a queue and one batch must run the same arithmetic, so lanes count and
+// not slots).  Beyond it, and in a workspace without room for them, each leg chooses its pairs by itself.
+static const size_t NEAR_LISTS_LIMIT = (size_t)8 << 30;
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+// Lanes that a batch can take in: its slots' and those that replace them.
+static int lanes_of(const skb_config *c) { return c->lane_capacity > c->W ? c->lane_capacity : c->W; }
 
 static bool config_ok(const skb_config *c, std::string &why)
 {
@@ -185,9 +189,9 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
         return p;
     };
     const size_t W = c->W, n = c->n, m = c->m;
-    const size_t L = c->lane_capacity > c->W ? c->lane_capacity : c->W;      // lanes the result buffers hold
+    const size_t L = lanes_of(c);                        // lanes the result buffers hold
     const size_t DP = var->DP ? var->DP : padded_dim(c->d);
-    const bool near = spatial && !tensor && near_shape(var->f64, var->DP, var->CS, c->n, c->m, room ? c->W : 1);      // lanes in spatial order: whole boxes
+    const bool near = spatial && !tensor && near_shape(var->f64, var->DP, var->CS, c->n, c->m, room ? lanes_of(c) : 1);      // lanes in spatial order: whole boxes
     const size_t np = align_up(n, near ? BOX_COLS : 4), mp = align_up(m, near ? BOX_COLS : 4);
     const size_t ts = var->f64 ? 8 : 4;
     Dev d;
@@ -248,8 +252,8 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
         const size_t groups = (n + GROUP_ROWS - 1) / GROUP_ROWS;
         // (a warp's list holds its boxes' points and two steps of none)
         d.list_cap = (int)(((m + BOX_COLS - 1) / BOX_COLS + GROUP_WARPS - 1) / GROUP_WARPS + 2) * BOX_COLS;
-        const size_t lists = W * groups * GROUP_WARPS * d.list_cap * 2;
-        const bool listed = room && lists <= NEAR_LISTS_LIMIT && mp < 65535 && W * (mp + 1) * 16 < ((size_t)1 << 32);
+        const size_t lists = groups * GROUP_WARPS * d.list_cap * 2;        // of a lane
+        const bool listed = room && L * lists <= NEAR_LISTS_LIMIT && mp < 65535 && L * (mp + 1) * 16 < ((size_t)1 << 32);
         if (listed) halves = 2;
         d.topx[0] = (float *)take(W * halves * d.nbx * 4); d.topx[1] = (float *)take(W * halves * d.nbx * 4); d.topy = (float *)take(W * d.nby * 4);
         if (listed) {
@@ -258,7 +262,7 @@ static size_t carve(const skb_config *c, const Variant *var, bool tensor, bool s
             d.crdy = (float *)take(W * (mp + 1) * 16); d.gamy = DP == 4 ? (float *)take(W * (mp + 1) * 4) : nullptr;
             d.ceny = (float *)take(W * (d.nby + 1) * 16); d.lby = (float *)take(W * d.nby * 4); d.unit_low = (float2 *)take(W * (mp + 1) * 8);
             d.colacc[0] = (unsigned long long *)take(W * mp * 8); d.colacc[1] = (unsigned long long *)take(W * mp * 8);
-            d.lists = (unsigned short *)take(lists);
+            d.lists = (unsigned short *)take(W * lists);
             d.base_gam = (float *)take(W * mp * 4); d.base_top = (float *)take(W * d.nby * 4);
             d.risen = (unsigned long long *)take(W * 8); d.based_at = (int *)take(W * 4); d.overrun = (unsigned *)take(W * 8);
         }
@@ -290,7 +294,7 @@ static const Variant *variant_for(const skb_config *c, int compute, bool spatial
 {
     if (compute == SKB_COMPUTE_TENSOR) compute = SKB_COMPUTE_F32;     // fp32 epilogue, same scratch shapes
     const bool f64 = compute == SKB_COMPUTE_F64 || compute == SKB_COMPUTE_MIXED;
-    return choose_variant(c->W, c->n, c->m, c->d, f64, compute == SKB_COMPUTE_MIXED, c->column_split, spatial);
+    return choose_variant(c->W, lanes_of(c), c->n, c->m, c->d, f64, compute == SKB_COMPUTE_MIXED, c->column_split, spatial);
 }
 
 // room = false: the least that create takes (deep lanes then form their products in every leg, lanes in spatial order
@@ -407,7 +411,7 @@ extern "C" skb_status sinkhorn_batch_create(const void *x, const void *y, const 
     // spatial order: never for a cost form the caller named, nor for radii at which the plain kernels take differences
     const Variant *var_near = variant_for(cfg, SKB_COMPUTE_F32, true);
     const bool near_shaped = var_near && (automatic || cfg->compute == SKB_COMPUTE_F32) && (double)tol <= SPATIAL_TOL && cfg->cost_form == 0 &&
-                             near_shape(var_near->f64, var_near->DP, var_near->CS, cfg->n, cfg->m, room ? cfg->W : 1);
+                             near_shape(var_near->f64, var_near->DP, var_near->CS, cfg->n, cfg->m, room ? lanes_of(cfg) : 1);
     if (near_shaped) { launch_near_estimate(h->dev, x, y, cfg->W, h->stream); h->launches += 1; }
     if (automatic || near_shaped) {
         // read the largest scaled radius back and pick the arithmetic and the layout for the whole batch

@@ -56,7 +56,8 @@ constexpr int STEP_CYCLES_IN_LAUNCH = 2048;
 constexpr int MASK_CYCLES_IN_LAUNCH = 256;
 // Picks the variant for a shape (depends on the static shape only, so that every mode
 // and every run of the same batch uses the same reduction order).  Null if unsupported.
-const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_exp, int force_cs, bool spatial);
+// (lanes: those that the batch can take in, which decides about the spatial order)
+const Variant *choose_variant(int W, int lanes, int n, int m, int d, bool f64, bool fast_exp, int force_cs, bool spatial);
 int padded_dim(int d);
 
 void launch_lane_stats(const Dev &P, const void *x, const void *y, const float *eps, int slot0, int lane0, int count,
@@ -77,7 +78,7 @@ void launch_update_tc(const Dev &P, const void *maps, int leg, int width, cudaSt
 void launch_gram(const Dev &P, const void *maps, int slot0, int count, cudaStream_t st);
 int launch_emit_move(const Dev &P, int width, cudaStream_t st);
 // lanes kept in spatial order, whose legs skip the boxes of columns that are too far away to matter
-bool near_shape(int f64, int DP, int CS, int n, int m, int lanes);    // lanes: of a batch that has room for lists, else 1
+bool near_shape(int f64, int DP, int CS, int n, int m, int lanes);    // lanes: that a batch with room for lists can take in, else 1
 constexpr int NEAR_PAIRS = 4096;        // pairs per lane that launch_near_estimate counts into Ctl::near_kept
 void launch_near_estimate(const Dev &P, const void *x, const void *y, int lanes, cudaStream_t st);
 void launch_spatial_sort(const Dev &P, const void *x, const void *y, int slot0, int count, cudaStream_t st);

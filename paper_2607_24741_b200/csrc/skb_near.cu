@@ -53,7 +53,8 @@ constexpr int NEAR_MIN = 1024;
 // ... and with lists of single points (both legs in one pass) for clouds that are too large for the on-chip kernels, beside one another:
 // registration lanes, eps 0.01, a solve plain -> one pass: 32 of 520 points 17.9 -> 12.6 ms, 4 of 700 9.4 -> 8.3, 8 of 900 14.1 -> 9.6,
 // 32 of 900 21.6 -> 14.9; one lane of 600 (a cycle 17.2 <- 20.8 us) has too few groups and is better off
-// with its columns split over more blocks.
+// with its columns split over more blocks.  (Counted are the lanes a batch can take in: a queue through one slot
+// has the arithmetic, and so the bits, of one batch.)
 constexpr int NEAR_MIN_LISTS = 513;
 constexpr int NEAR_BLOCKS = 4;                      // blocks per SM (127 registers); five and six spill: 225 and 224 us a leg
 

@@ -153,7 +153,7 @@ int padded_dim(int d)
     return -1;
 }
 
-const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_exp, int force_cs, bool spatial)
+const Variant *choose_variant(int W, int lanes, int n, int m, int d, bool f64, bool fast_exp, int force_cs, bool spatial)
 {
     const int DP = padded_dim(d);
     if (DP < 0) return nullptr;
@@ -184,7 +184,7 @@ const Variant *choose_variant(int W, int n, int m, int d, bool f64, bool fast_ex
         const double score = (util_n < util_m ? util_n : util_m) * fill * (c == 32 ? 0.6 : (c == 1 ? 0.85 : 1.0));
         if (score > best + 1e-9) { best = score; cs = c; }
     }
-    if (spatial && near_shape(f64 ? 1 : 0, DP, 4, n, m, W)) cs = 4;             // far columns are skipped: few steps are left to split
+    if (spatial && near_shape(f64 ? 1 : 0, DP, 4, n, m, lanes)) cs = 4;             // far columns are skipped: few steps are left to split
     if (force_cs == 1 || force_cs == 4 || force_cs == 32) cs = force_cs;
     for (const Variant &v : g_variants)
         if (v.f64 == (f64 ? 1 : 0) && v.xf == ((f64 && fast_exp) ? 1 : 0) && v.DP == DP && v.CS == cs) return &v;

@@ -1996,6 +1996,39 @@ def test_a_lane_that_is_not_finite_leaves_its_neighbours_alone(first):
         np.testing.assert_array_equal(p, q)
 
 
+@pytest.mark.parametrize("W,slots,n,m,cycles", [(3, 1, 600, 530, 40), (264, 66, 8192, 8192, 2)])
+def test_a_queue_of_lanes_in_spatial_order_has_the_bits_of_one_batch(W, slots, n, m, cycles):
+    # whether lanes of 513 to 1023 points are in spatial order, and whether there are lists, must not depend on the slots: a queue
+    # through one slot, and one whose slots' lists are small where those of all its lanes are 2.2 GiB
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    if W < 100:
+        w = _sphere_lanes(W, n, m, np.full(W, 0.01), cycles)
+        parts = lambda a, b: _parts(w, slice(a, b))
+    else:                                                  # (made on the GPU: 50 MB of points)
+        gen = torch.Generator("cuda:0").manual_seed(1)
+        c = torch.randn(2, W, n, 3, device="cuda:0", generator=gen)
+        c /= c.norm(dim=3, keepdim=True)
+        flat = torch.full((W, n), 1.0 / n, device="cuda:0")
+        every = (c[0], c[1], flat, flat, torch.full((W,), 0.01, device="cuda:0"))
+        parts = lambda a, b: [v[a:b].contiguous() for v in every]
+    sb = B.SinkhornBatch(*parts(0, W), 1e-3, max_iter=cycles)
+    sb.drain()
+    whole = sb.potentials(f64=True)
+    sb.close()
+    del sb
+    sb = B.SinkhornBatch(*parts(0, slots), 1e-3, max_iter=cycles, lane_capacity=W)
+    for k in range(slots, W, slots):
+        while sb.active():
+            sb.step(4)
+        sb.refill(*parts(k, min(k + slots, W)))
+    sb.drain()
+    queue = sb.potentials(f64=True)
+    assert sb.check_guards() == -1
+    sb.close()
+    assert torch.equal(queue[0], whole[0]) and torch.equal(queue[1], whole[1])
+
+
 class _ZeroedWorkspace:
     # stands in for torch in the binding: workspaces start as zeros
     def __getattr__(self, name):
