@@ -312,6 +312,7 @@ static size_t workspace_need(const skb_config *cfg, bool room)
     }
     if (cfg->compute == SKB_COMPUTE_AUTO || cfg->compute == SKB_COMPUTE_F32) {
         for (const bool spatial : {false, true}) {           // the tolerance, which decides, is not known here
+            if (spatial && cfg->cost_form != 0) continue;    // (a named cost form rules it out)
             const size_t t = carve(cfg, variant_for(cfg, SKB_COMPUTE_F32, spatial), false, spatial, room, nullptr, nullptr);
             if (t > need) need = t;
         }

@@ -72,6 +72,24 @@ def test_guard_band_and_lane_capacity_show_in_the_workspace(B):
     assert grow >= 2 * W * (n + m) * 8 and grow < 2 * W * (n + m) * 8 + 64 * 1024
 
 
+def test_lists_of_lanes_in_spatial_order_show_in_the_workspace_where_they_can_be_used(B):
+    # some n m / 8 bytes a slot, for batches that may go into spatial order: not with a cost form, a column split that rules it out,
+    # five dimensions, one lane below 1024 points; by all lanes that a batch can take in up to 8 GiB, and by its slots in size
+    ws = lambda W, n, d=3, **kw: B.sinkhorn_batch_workspace_bytes(B.make_config(W, n, n, d, compute="f32", **kw))
+    lists = lambda W, n: W * n * n // 8
+    for W, n in ((4, 4096), (2, 600), (1, 1024), (250, 8192), (900, 8192)):
+        plain = ws(W, n, cost_form=1)
+        assert ws(W, n, cost_form=2) == plain and ws(W, n, column_split=32) == plain
+        assert ws(W, n) - plain >= lists(W, n), (W, n)
+    assert ws(1, 600) - ws(1, 600, cost_form=1) < lists(1, 600)
+    assert ws(4, 4096, d=5) == ws(4, 4096, d=5, cost_form=1)
+    assert ws(1100, 8192) - ws(1100, 8192, cost_form=1) < lists(1100, 8192)
+    for cap, listed in ((900, True), (1100, False)):
+        more = ws(50, 8192, lane_capacity=cap) - ws(50, 8192, lane_capacity=cap, cost_form=1)
+        assert (more >= lists(50, 8192)) == listed and more < 2 * lists(50, 8192)
+    assert ws(1, 600, lane_capacity=2) - ws(1, 600, lane_capacity=2, cost_form=1) >= lists(1, 600)
+
+
 def test_create_rejects_bad_arguments_without_touching_the_gpu(B):
     cfg = B.make_config(8, 64, 64, 2)
     h = ctypes.c_void_p()
