@@ -1895,8 +1895,8 @@ def test_spatial_order_is_taken_where_it_can_skip(oracle, law, n, m, d, eps, exp
 
 # (law, n, m, d, eps): groups of 16 rows and lists by warp at their edges; lists longer than what tensor memory holds (a
 # large share of the pairs); outliers on both sides, whose potentials move by many bits in the first cycles
-ONE_PASS = [("sphere", 1040, 1025, 3, 0.02), ("sphere", 1100, 2049, 3, 0.05), ("cube", 1031, 97, 2, 0.002), ("cube", 40, 1025, 1, 0.002),
-            ("flat", 1500, 1100, 4, 0.004), ("outliers", 1300, 1300, 3, 0.01), ("sphere", 600, 513, 3, 0.01), ("cube", 530, 90, 2, 0.01)]
+ONE_PASS = [("sphere", 1040, 1025, 3, 0.02), ("sphere", 1100, 2049, 3, 0.04), ("cube", 1031, 97, 2, 0.002), ("cube", 40, 1025, 1, 0.002),
+            ("flat", 1500, 1100, 4, 0.004), ("outliers", 1300, 1300, 3, 0.01), ("sphere", 600, 513, 3, 0.01), ("cube", 530, 520, 2, 0.005)]
 
 
 @pytest.mark.parametrize("law,n,m,d,eps", ONE_PASS)
@@ -1920,6 +1920,25 @@ def test_both_legs_in_one_pass(oracle, monkeypatch, law, n, m, d, eps):
     e = w.eps.astype(np.float64)
     r = run_gpu(w)
     assert r["arith"] == "f32"
+    # these kernels did run: lanes in spatial order are ordered by one more launch at create, and groups of 16 have their lists (a
+    # record of 512 bytes: the cycle they are from, in word 38, and the lengths for four warps, whole steps of 32, in words 40 to 43)
+    t = lambda v: torch.from_numpy(v).to("cuda:0")
+    at_create = []
+    monkeypatch.setattr(B, "torch", _ZeroedWorkspace())
+    for kw in ({}, dict(column_split=1)):
+        sb = B.SinkhornBatch(t(w.x), t(w.y), t(w.a), t(w.b), t(w.eps), w.tol, max_iter=cycles, **kw)
+        at_create.append(sb.launch_count())
+        if not kw:
+            sb.step(1)
+            torch.cuda.synchronize()
+            words = sb.workspace[:sb.workspace.numel() // 256 * 256].view(torch.int32).view(-1, 64)
+            length = words[(words[:, 38] == 1) & (words[:, 40:44] % 32 == 0).all(1) & (words[:, 40:44] <= m + 96).all(1) & (words[:, 40:44] >= 0).all(1), 40:44]
+            assert len(length) >= W * ((n + 15) // 16)
+            if (n, m) == (1100, 2049):
+                assert int(length.max()) > 256               # more than what tensor memory holds
+        sb.close()
+    monkeypatch.undo()
+    assert at_create[0] - at_create[1] == 2                  # the estimate, the ordering
     np.testing.assert_array_equal(r["depth"], ref.depth)
     assert pot_err(r["f"], r["g"], ref.f, ref.g, e).max() <= POT_TOL_F32
     rm = run_gpu(w, mode="masked")
@@ -1930,7 +1949,6 @@ def test_both_legs_in_one_pass(oracle, monkeypatch, law, n, m, d, eps):
     assert (sb.last_audit()[0] > 0).all()
     sb.close()
     # one slot after the other, then two at a time: later lanes in slots that others have used
-    t = lambda v: torch.from_numpy(v).to("cuda:0")
     sb = B.SinkhornBatch(t(w.x[:2]), t(w.y[:2]), t(w.a[:2]), t(w.b[:2]), t(w.eps[:2]), w.tol, max_iter=cycles, lane_capacity=W)
     while sb.active() == 2:
         sb.step(1)
@@ -1947,6 +1965,40 @@ def test_both_legs_in_one_pass(oracle, monkeypatch, law, n, m, d, eps):
     rs = run_gpu(w)
     np.testing.assert_array_equal(rs["depth"], ref.depth)
     assert pot_err(rs["f"], rs["g"], ref.f, ref.g, e).max() <= POT_TOL_F32
+    assert not np.array_equal(rs["f"], r["f"])               # (other arithmetic, to rounding)
+
+
+def test_one_pass_under_the_other_modes_and_between_its_cycles(oracle):
+    # STATIC over more than the first cycles, the mask that skips frozen lanes, audits on a grid, and timed dry launches between
+    # cycles (whose lists are thrown away or the same): the bits, depths and audits of one plain solve
+    from paper_2607_24741_b200 import binding as B
+    n, m, cycles = 1300, 1100, 90
+    w = _sphere_lanes(4, n, m, [0.05, 0.03, 0.012, 0.01], cycles)
+    r = run_gpu(w)
+    assert r["arith"] == "f32" and (r["depth"] < cycles).any() and (r["depth"] == cycles).any()
+    rx = run_gpu(w, mode="masked_exit")
+    for k in ("f", "g", "depth", "status", "r_row"):
+        np.testing.assert_array_equal(rx[k], r[k])
+    # (12 cycles: no lane has passed, so STATIC's common cycle is max_iter)
+    few, static = run_gpu(w, max_iter=12), run_gpu(w, mode="static", max_iter=12)
+    assert (few["depth"] == 12).all()
+    np.testing.assert_array_equal(static["f"], few["f"]); np.testing.assert_array_equal(static["g"], few["g"])
+    ref = oracle.solve_batch(w.x, w.y, w.a, w.b, w.eps, w.tol, max_iter=cycles, audit_every=7)
+    grid = run_gpu(w, audit_every=7)
+    np.testing.assert_array_equal(grid["depth"], ref.depth)
+    assert pot_err(grid["f"], grid["g"], ref.f, ref.g, w.eps.astype(np.float64)).max() <= POT_TOL_F32
+    for when in (0, 1, 2, 9):
+        sb = B.SinkhornBatch(*_parts(w, slice(0, 4)), w.tol, max_iter=cycles)
+        for k in range(12):
+            if k % 10 == when:
+                sb.profile_update(leg=0, reps=2); sb.profile_update(leg=1, reps=2)
+            sb.step(1)
+        sb.drain()
+        f, g = (v.cpu().numpy() for v in sb.potentials(f64=True))
+        np.testing.assert_array_equal(f, r["f"]); np.testing.assert_array_equal(g, r["g"])
+        np.testing.assert_array_equal(sb.residuals()[0].cpu().numpy(), r["r_row"])
+        assert sb.check_guards() == -1
+        sb.close()
 
 
 def _sphere_lanes(W, n, m, eps, cycles, seed=5):
