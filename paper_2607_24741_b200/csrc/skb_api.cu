@@ -118,7 +118,9 @@ static double mixed_radius(double tol)
 static const double NEAR_SHARE = 0.75;
 // With lists a pair is formed once per cycle instead of twice, and a list is shorter than the boxes that the estimate counts.  Plain -> one
 // pass, us a cycle: 16 lanes of 1024 points, share 0.82 33 -> 27, 1.0 37 -> 27; 4 of 2048, 0.88, 47 -> 24; 4 of 4096, 0.83, 63 -> 37; 32 of
-// 4096 293 -> 215; 8 of 600, 1.0, 27 -> 20.  Clouds of which next to nothing can be left out keep the plain kernel.
+// 4096 293 -> 215; 8 of 600, 1.0, 27 -> 20.  One lane, a solve in ms: 1024 points, share 0.82 3.41 -> 3.40, 0.89 2.82 -> 2.81, 1.0 2.06 -> 2.18;
+// 1100, 0.89, 3.36 -> 3.12; 2048, 0.76, 3.89 -> 3.00, 0.98 2.48 -> 2.13; 8192, 0.89, 5.85 -> 3.77.  Clouds of which next to nothing can be left
+// out keep the plain kernel: at a share of 1 one lane of 1024 to 1500 points and batches of 8192 lose with lists.
 static const double NEAR_SHARE_LISTS = 0.95;
 // ... and up to this tolerance: plans applied from looser solves agree with those of the plain kernel's potentials to
 // the rounding of its expanded cost, 1.2e-6 on the registration workload at tol 1e-2, and callers hold such results to

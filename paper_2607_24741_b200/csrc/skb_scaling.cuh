@@ -93,6 +93,12 @@ __device__ __forceinline__ float exp2_split(const double arg)
     }
 }
 
+__device__ __forceinline__ u64 mul2(u64 a, u64 b)
+{
+    u64 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 // fp32 -> float64 and back (towards zero) by integers, for positive normal fp32 numbers: the conversion unit is slow and
 // far away.  Zero and subnormal numbers become something below 2^-125, infinities and NaN something from 2^128 on.
 __device__ __forceinline__ double widen(const float x)
