@@ -506,8 +506,6 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_kernel(const Dev P)
             g->done = 1;
         }
     }
-    if (P.overrun)                                       // (the next f-leg's; behind what the g-leg waits for)
-        for (int s = tid; s < P.W; s += NT) P.overrun[(size_t)(c.parity ^ 1) * P.W + s] = 0u;
     if (FUSE && P.mode != MODE_STATIC && nret > 0) {
         __syncthreads();                                  // the lists and per-slot scalars above are this block's own writes
         Ctl cc = c;

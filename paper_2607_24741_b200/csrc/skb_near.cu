@@ -616,8 +616,8 @@ __device__ __forceinline__ void note_rise(const Dev &P, const Ctl &c, const int 
 }
 
 // 2^r of a group whose phi has risen by r bits more than its lists have room for, added up by lane as integers (any order), double-buffered
-// like the column totals (the planner zeroes the next cycle's: beside the totals that store cost 5 of 245 us a cycle, in the g-leg 1 of 9);
-// OVERRUN_ALL: those cannot be used.
+// like the column totals (the column check's launch zeroes the next cycle's: beside the totals that store cost 5 of 245 us a cycle, in the
+// g-leg 1 of 9, in the planner 0.1 us of every batch's cycle); OVERRUN_ALL: those cannot be used.
 constexpr float OVERRUN_UNIT = 64.f;
 constexpr unsigned OVERRUN_ALL = 1u << 31;               // (2^14 groups, the most that 262 143 points make, of 2^14 + 1 units stay below)
 
@@ -1164,6 +1164,8 @@ __global__ void __launch_bounds__(UPD_THREADS, NEAR_BLOCKS) update_near_kernel(c
     const Ctl c = *P.ctl;
     if (leg == LEG_V) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int slot = blockIdx.y, row_base = (int)blockIdx.x * RB;
+    if (leg == LEG_V && P.lists && row_base == 0 && slot < c.n_phys && slot < nlanes && threadIdx.x == 0)
+        P.overrun[(size_t)(c.parity ^ 1) * P.W + P.home[slot]] = 0u;
     if (leg == LEG_V && (int)blockIdx.y >= nlanes) {
         guard_pool(P, c, nlanes, reinterpret_cast<unsigned long long *>(sc.red));
         return;
