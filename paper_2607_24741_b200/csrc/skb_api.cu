@@ -769,6 +769,11 @@ extern "C" skb_status sinkhorn_batch_drain(skb_batch *h, int *cycles_run)
     while (!h->finished) {
         const bool multi = cycles_in_one_launch(h);      // may become true as the batch narrows
         const int chunk_max = scaling ? (masked ? MASK_CYCLES_IN_LAUNCH : MAX_CYCLES_IN_LAUNCH) : (multi ? 32 : 16);
+        // ... not where the lanes left after some cycles get an SM each, and its registers, from a launch of their own (350 lanes of 128 x 160, a
+        // solve in launches of 2048 -> 8192: 4142 -> 4175 us, 4790 -> 4852); nor under STATIC, whose lanes wait for the others in the middle of each
+        // launch (400 of them: 14.4 -> 15.2 ms)
+        if (scaling && !masked)
+            chunk = h->cfg.mode == SKB_STATIC || (h->cfg.mode == SKB_ACTIVE && scaling_shares_sm(h->dev, h->known_width)) ? STEP_CYCLES_IN_LAUNCH : MAX_CYCLES_IN_LAUNCH;
         NvtxRange nvtx_chunk(multi ? "skb:chunk (cycles in one launch)" : "skb:chunk (launch per leg)");
         if (multi) enqueue_cycles_launch(h, chunk);
         else for (int i = 0; i < chunk; ++i) enqueue_cycle(h);

@@ -93,6 +93,7 @@ enum ScalingKind : int { SC_CYCLES, SC_CATCH_UP, SC_LEG };      // see scaling_k
 void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int width, cudaStream_t st);
 int launch_plan_cycles(const Dev &P, int width, int cycles, cudaStream_t st);
 void launch_order(const Dev &P, int *order, cudaStream_t st);
+bool scaling_shares_sm(const Dev &P, int width);       // lanes that fewer of them would not
 int scaling_blocks(const Dev &P);          // blocks of a lane
 int scaling_resident(const Dev &P);        // lanes that are on the GPU at the same time, at least
 void launch_plan_static(const Dev &P, int cycles, cudaStream_t st);

@@ -42,17 +42,36 @@ int scaling_resident(const Dev &P)
     const int nc = scaling_blocks(P);
     return nc <= 1 ? 148 : (nc <= 2 ? 74 : (nc <= 4 ? 33 : (nc <= 8 ? 15 : 7)));
 }
+// The kernel with 128 or the one with 255 registers a thread, for `blocks` blocks.
+static const void *cycles_kernel(const ScalingVariant *v, ScalingKind kind, const Dev &P, long long blocks)
+{
+    if (kind == SC_LEG) return v->kernel[kind];
+    const bool mask = P.mode == MODE_MASKED && !P.early_exit;
+    // Lanes in half of the tensor memory: alone on their SM with all of its registers while that makes two rounds at most.  Drain
+    // of lanes of 128 x 160, d = 8, two blocks an SM -> one: 1 lane 994 -> 887 us, 148 1003 -> 905, 256 1105 -> 900, 400 1290 <- 1365,
+    // 1200 3073 <- 3519.  One round under a mask, whose lanes all work to the end: 149 3822 <- 4128, 220 4532 <- 4749, 296 4608 <- 5143.
+    if (v->tm_cols) return blocks <= (mask ? 148 : 2 * 148) ? v->roomy[kind] : v->kernel[kind];
+    // K in 32 registers: 255 wherever lanes leave.  Where all work to the end (STATIC) or launches end together (a mask), what
+    // counts beyond one round of 296 blocks is how full the last one is.  60 x 60 and 30 x 30, 128 -> 255, STATIC: 296 lanes 2033 -> 1718, 320
+    // 2310 -> 2204 and 2103 <-> 2102, 360 2326 <- 2419, 592 2579 <- 2733, 1500 4715 <- 5243; mask: 296 1988 -> 1618, 320 2400 <- 2596,
+    // 400 2498 <- 2687, 450 2846 -> 2718, 700 3981 -> 3722, 1500 6761 -> 6701.
+    const long long places = 148 * 256 / v->threads;
+    const bool shared = P.mode == MODE_STATIC ? blocks > places + places / 8 : mask && blocks > places && blocks <= places + 2 * places / 5;
+    return shared ? v->kernel[kind] : v->roomy[kind];
+}
+// Does a launch of `width` lanes take the kernel that shares an SM, where one of fewer lanes would take the one that has it alone?
+bool scaling_shares_sm(const Dev &P, int width)
+{
+    const ScalingVariant *v = scaling_variant(P.dots != nullptr, P.n, P.m);
+    return cycles_kernel(v, SC_CYCLES, P, (long long)blocks_of(*v, P.n) * width) != v->roomy[SC_CYCLES];
+}
 int scaling_blocks(const Dev &P) { return blocks_of(*scaling_variant(P.dots != nullptr, P.n, P.m), P.n); }
 
 void launch_scaling(const Dev &P, ScalingKind kind, int leg, int cycles, int width, cudaStream_t st)
 {
     const ScalingVariant *v = scaling_variant(P.dots != nullptr, P.n, P.m);
-    const void *kernel = v->kernel[kind];
     const int nc = blocks_of(*v, P.n);
-    // Lanes in half of the tensor memory: alone on their SM with all of its registers while that makes two rounds at most.  Drain
-    // of lanes of 128 x 160, d = 8, two blocks an SM -> one: 1 lane 994 -> 887 us, 148 1003 -> 905, 256 1105 -> 900, 400 1290 <- 1365,
-    // 1200 3073 <- 3519.
-    if (kind == SC_CYCLES && nc * width <= 2 * 148) kernel = v->roomy;
+    const void *kernel = cycles_kernel(v, kind, P, (long long)nc * width);
     // No block may take its place on an SM and then wait there for tensor memory while blocks of its cluster hold theirs.
     // Blocks that take the whole register file are alone anyway.  Others ask for shared memory in proportion to their tensor
     // memory; without a cluster they may wait, and ask for as much as keeps one block too many away.  (No more

@@ -150,9 +150,11 @@ struct ScalingShape {
     // K in registers: 255 of them a thread for the narrow tiles, too, which spill in every cycle with 128 although the entries
     // are 32 or 64 of those (drain of lanes of 64 x 64, d = 2, 128 -> 255: one lane 573 -> 460 us, 256 602 -> 493, 1200
     // 1054 -> 736; of 100 x 60 870 -> 674, 993 -> 750, 2169 -> 1681; 168 registers lie between).
-    // K in 256 columns of tensor memory: two blocks an SM with 128 registers, or one that does not spill (ROOMY).
-    static constexpr int BLOCKS = TM ? 512 / TM_COLS : 256 / THREADS;
-    static constexpr bool HAS_ROOMY = TM && BLOCKS * THREADS > 256;
+    // K in 256 columns of tensor memory, or in 32 registers: two kernels, BLOCKS an SM with 128 registers a thread and half as many
+    // that do not spill (ROOMY); cycles_kernel has the rule.
+    static constexpr int BLOCKS = TM ? 512 / TM_COLS : (CL * RW == 32 ? 512 : 256) / THREADS;
+    static constexpr bool HAS_ROOMY = BLOCKS * THREADS > 256;
+    static constexpr int ROOMY_BLOCKS = TM ? 1 : 256 / THREADS;
     // Launches of one leg do not hold K: 128 registers.  Lanes of 512 columns and more, whose G rows of distances are 64 registers
     // and up, form their entries in a loop and take 255: unrolled, the entries' instructions run once and are
     // fetched for longer, and at 128 registers they spill (f-leg of 64 lanes of 1024 x 1024 1224 -> 310 us, of 256 lanes of
@@ -476,9 +478,9 @@ __device__ __forceinline__ void scaling_barrier()
 // the cycle that the others have reached (plan_static_kernel).  SC_LEG: leg = LEG_F / LEG_V / LEG_G as a launch of its
 // own, for phase timing and dry runs: an entry of K is formed where it is used, with the same bits, and never kept.
 // CLU = 0: a lane has one block (its rows fit), and nothing of the cluster machinery is in the way.
-// ROOMY: one block an SM, with all of its registers (same arithmetic).
+// ROOMY: with 255 registers a thread where there is a kernel with 128, too (same arithmetic).
 template <int SRC, int NW, int CL, int RW, bool CLU, bool TMEM, int KIND, bool ROOMY = false>
-__global__ void __launch_bounds__(32 * NW, (KIND == SC_LEG ? ScalingShape<NW, CL, RW, TMEM>::LEG_BLOCKS : (ROOMY ? 1 : ScalingShape<NW, CL, RW, TMEM>::BLOCKS)))
+__global__ void __launch_bounds__(32 * NW, (KIND == SC_LEG ? ScalingShape<NW, CL, RW, TMEM>::LEG_BLOCKS : (ROOMY ? ScalingShape<NW, CL, RW, TMEM>::ROOMY_BLOCKS : ScalingShape<NW, CL, RW, TMEM>::BLOCKS)))
 scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
 {
     typedef ScalingShape<NW, CL, RW, TMEM> L;
@@ -1431,14 +1433,15 @@ struct ScalingVariant {
     int threads, cols, rb;
     bool cluster;                                        // lanes of several blocks
     int min_blocks, max_blocks;
-    const void *kernel[3], *roomy;                       // by ScalingKind; of SC_CYCLES, where there is one
+    const void *kernel[3], *roomy[2];                    // by ScalingKind; of SC_CYCLES and SC_CATCH_UP, where there are any
     int tm_cols;                                         // tensor memory columns (0: K in registers)
     size_t (*smem)(int nc);
 };
 #define SKB_SC(SRC, NW, CL, RW, CLU, TM) { 32 * NW, 32 * CL, NW * RW, CLU, ScalingShape<NW, CL, RW, TM>::MIN_BLOCKS, ScalingShape<NW, CL, RW, TM>::RANKS, \
     {(const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CYCLES>, (const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CATCH_UP>, \
      (const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_LEG>}, \
-    (const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CYCLES, ScalingShape<NW, CL, RW, TM>::HAS_ROOMY>, TM ? ScalingShape<NW, CL, RW, TM>::TM_COLS : 0, &ScalingShape<NW, CL, RW, TM>::smem }
+    {(const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CYCLES, ScalingShape<NW, CL, RW, TM>::HAS_ROOMY>, \
+     (const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CATCH_UP, !TM && ScalingShape<NW, CL, RW, TM>::HAS_ROOMY>}, TM ? ScalingShape<NW, CL, RW, TM>::TM_COLS : 0, &ScalingShape<NW, CL, RW, TM>::smem }
 
 // Variants by the source of their exponents, narrowest column count first, then fewest rows per block.
 struct ScalingTable { const ScalingVariant *v; int count; };

@@ -1759,6 +1759,27 @@ def test_a_masks_launch_ends_when_its_last_lane_has_passed(W, n, m, light):
     assert (out[1][4] <= 2 * 2 + 1) == (W < 148)           # two launches at most, each with its planner (and the ranking)
 
 
+@pytest.mark.parametrize("n,m,Ws", [(40, 50, (330, 340, 400)), (100, 140, (140, 150, 300))])
+def test_kernels_of_128_and_255_registers_have_the_same_bits(n, m, Ws):
+    # lanes whose matrix is in 32 registers a thread, or in half of the tensor memory, have two kernels, chosen by the mode and the number
+    # of blocks; on both sides of each line STATIC, a mask and the plain batch give a lane the same bits
+    import torch
+    from paper_2607_24741_b200 import binding as B
+    w = wl.make("sweep", W=max(Ws), n=n, m=m, d=4, max_iter=40)
+    first = None
+    for W in Ws:
+        part = [torch.from_numpy(v[:W]).to("cuda:0") for v in (w.x, w.y, w.a, w.b, w.eps)]
+        for mode in ("active", "static", "masked"):
+            sb = B.SinkhornBatch(*part, 1e-9, mode=mode, max_iter=w.max_iter)      # (no lane passes: the common cycle of STATIC is theirs)
+            sb.drain()
+            f, g = (v.cpu().numpy() for v in sb.potentials(f64=True))
+            assert (sb.depths()[0] == w.max_iter).all() and sb.check_guards() == -1
+            sb.close()
+            first = first or (f, g)
+            k = len(first[0])
+            np.testing.assert_array_equal(f[:k], first[0]); np.testing.assert_array_equal(g[:k], first[1])
+
+
 @pytest.mark.parametrize("mode", ["active", "static", "masked"])
 def test_a_drain_of_deep_lanes_waits_once_in_8192_cycles(mode):
     # a drain waits for a launch before it enqueues the next, so lanes of thousands of cycles must not be cut into many launches;
@@ -1781,7 +1802,7 @@ def test_a_drain_of_deep_lanes_waits_once_in_8192_cycles(mode):
         assert (sb.depths()[0] == 8300).all() and sb.check_guards() == -1
         out.append((f, g, launches))
         sb.close()
-    assert out[0][2] <= 2 * 3
+    assert out[0][2] <= (5 * 3 if mode == "static" else 2 * 3)      # (STATIC: 2048 cycles and three kernels a launch)
     np.testing.assert_array_equal(out[0][0], out[1][0]); np.testing.assert_array_equal(out[0][1], out[1][1])
 
 
