@@ -280,7 +280,7 @@ typedef enum {
  * Lanes whose kernel matrix stays on chip form its entries anew in every leg of such a solve, which a
  * plain one does once per launch of many cycles, and one cycle is five launches: theirs takes 6 to 50 times the
  * plain solve (256 lanes of 512 x 512, d = 15: 5.2 ms against 0.8; 64 bf16 lanes of 1024 x 1024: 267 against 14.3; 1024 of
- * 256 x 256, d = 8: 401 against 8.6).
+ * 256 x 256, d = 8: 401 against 7.5).
  */
 skb_status sinkhorn_batch_set_profiling(skb_batch *h, int on);
 
