@@ -55,7 +55,10 @@ static const void *cycles_kernel(const ScalingVariant *v, ScalingKind kind, cons
     // counts beyond one round of 296 blocks is how full the last one is.  60 x 60 and 30 x 30, 128 -> 255, STATIC: 296 lanes 2033 -> 1718, 320
     // 2310 -> 2204 and 2103 <-> 2102, 360 2326 <- 2419, 592 2579 <- 2733, 1500 4715 <- 5243; mask: 296 1988 -> 1618, 320 2400 <- 2596,
     // 400 2498 <- 2687, 450 2846 -> 2718, 700 3981 -> 3722, 1500 6761 -> 6701.
+    // Clusters of 64 registers, 250 x 60, 128 -> 255: STATIC 296 lanes 7632 -> 7387, 512 11.3 -> 10.8 ms, 750 14.1 -> 14.0 and 15.1 <- 15.3, 900 15.1 <- 16.5,
+    // 1200 20.0 <- 23.2; a mask 27.4 -> 21.2 at 900.
     const long long places = 148 * 256 / v->threads;
+    if (v->cluster) return P.mode == MODE_STATIC && blocks > 5 * places ? v->kernel[kind] : v->roomy[kind];
     const bool shared = P.mode == MODE_STATIC ? blocks > places + places / 8 : mask && blocks > places && blocks <= places + 2 * places / 5;
     return shared ? v->kernel[kind] : v->roomy[kind];
 }

@@ -150,10 +150,10 @@ struct ScalingShape {
     // K in registers: 255 of them a thread for the narrow tiles, too, which spill in every cycle with 128 although the entries
     // are 32 or 64 of those (drain of lanes of 64 x 64, d = 2, 128 -> 255: one lane 573 -> 460 us, 256 602 -> 493, 1200
     // 1054 -> 736; of 100 x 60 870 -> 674, 993 -> 750, 2169 -> 1681; 168 registers lie between).
-    // K in 256 columns of tensor memory, or in 32 registers: two kernels, BLOCKS an SM with 128 registers a thread and half as many
-    // that do not spill (ROOMY); cycles_kernel has the rule.
-    static constexpr int BLOCKS = TM ? 512 / TM_COLS : (CL * RW == 32 ? 512 : 256) / THREADS;
-    static constexpr bool HAS_ROOMY = BLOCKS * THREADS > 256;
+    // K in 256 columns of tensor memory, in 32 registers, or in 64 of clusters of two columns a thread: two kernels, blocks() an SM with 128
+    // registers a thread and half as many that do not spill (ROOMY); cycles_kernel has the rule.
+    static constexpr int blocks(bool cluster) { return TM ? 512 / TM_COLS : (CL * RW == 32 || (cluster && CL == 2) ? 512 : 256) / THREADS; }
+    static constexpr bool has_roomy(bool cluster) { return blocks(cluster) * THREADS > 256; }
     static constexpr int ROOMY_BLOCKS = TM ? 1 : 256 / THREADS;
     // Launches of one leg do not hold K: 128 registers.  Lanes of 512 columns and more, whose G rows of distances are 64 registers
     // and up, form their entries in a loop and take 255: unrolled, the entries' instructions run once and are
@@ -164,7 +164,7 @@ struct ScalingShape {
     static constexpr int FP32_COLS = CL <= 4 ? 8 : 32;               // columns a row's sum holds before it becomes float64
     static constexpr int FP32_WARPS = CL >= 8 && RW <= 16 ? 2 : 1;   // warps' column parts added in fp32 (at most 32 rows)
     static_assert(RW >= 8 && RW <= 32 && CL >= 2 && CL <= 32, "unsupported tile");
-    static_assert(!TM || (NW % 4 == 0 && GW % 32 == 0 && TM_COLS <= 512 && BLOCKS <= 4), "unsupported tile in tensor memory");
+    static_assert(!TM || (NW % 4 == 0 && GW % 32 == 0 && TM_COLS <= 512 && 512 / TM_COLS <= 4), "unsupported tile in tensor memory");
     static_assert(!TWO_STEP || COLS == 4 * THREADS, "the two-step exchange has one thread to a column where four blocks share them");
     // dynamic shared memory: column parts of every warp; the exchange buffers: what goes out, what comes in (TWO_STEP: parts
     // of the own columns, totals of all; totals that go out); where K is in registers, the words it is formed in
@@ -480,7 +480,7 @@ __device__ __forceinline__ void scaling_barrier()
 // CLU = 0: a lane has one block (its rows fit), and nothing of the cluster machinery is in the way.
 // ROOMY: with 255 registers a thread where there is a kernel with 128, too (same arithmetic).
 template <int SRC, int NW, int CL, int RW, bool CLU, bool TMEM, int KIND, bool ROOMY = false>
-__global__ void __launch_bounds__(32 * NW, (KIND == SC_LEG ? ScalingShape<NW, CL, RW, TMEM>::LEG_BLOCKS : (ROOMY ? ScalingShape<NW, CL, RW, TMEM>::ROOMY_BLOCKS : ScalingShape<NW, CL, RW, TMEM>::BLOCKS)))
+__global__ void __launch_bounds__(32 * NW, (KIND == SC_LEG ? ScalingShape<NW, CL, RW, TMEM>::LEG_BLOCKS : (ROOMY ? ScalingShape<NW, CL, RW, TMEM>::ROOMY_BLOCKS : ScalingShape<NW, CL, RW, TMEM>::blocks(CLU))))
 scaling_kernel(const __grid_constant__ Dev P, const int leg, const int cycles)
 {
     typedef ScalingShape<NW, CL, RW, TMEM> L;
@@ -1440,8 +1440,8 @@ struct ScalingVariant {
 #define SKB_SC(SRC, NW, CL, RW, CLU, TM) { 32 * NW, 32 * CL, NW * RW, CLU, ScalingShape<NW, CL, RW, TM>::MIN_BLOCKS, ScalingShape<NW, CL, RW, TM>::RANKS, \
     {(const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CYCLES>, (const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CATCH_UP>, \
      (const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_LEG>}, \
-    {(const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CYCLES, ScalingShape<NW, CL, RW, TM>::HAS_ROOMY>, \
-     (const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CATCH_UP, !TM && ScalingShape<NW, CL, RW, TM>::HAS_ROOMY>}, TM ? ScalingShape<NW, CL, RW, TM>::TM_COLS : 0, &ScalingShape<NW, CL, RW, TM>::smem }
+    {(const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CYCLES, ScalingShape<NW, CL, RW, TM>::has_roomy(CLU)>, \
+     (const void *)&scaling_kernel<SRC, NW, CL, RW, CLU, TM, SC_CATCH_UP, !TM && ScalingShape<NW, CL, RW, TM>::has_roomy(CLU)>}, TM ? ScalingShape<NW, CL, RW, TM>::TM_COLS : 0, &ScalingShape<NW, CL, RW, TM>::smem }
 
 // Variants by the source of their exponents, narrowest column count first, then fewest rows per block.
 struct ScalingTable { const ScalingVariant *v; int count; };

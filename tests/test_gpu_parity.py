@@ -1759,7 +1759,7 @@ def test_a_masks_launch_ends_when_its_last_lane_has_passed(W, n, m, light):
     assert (out[1][4] <= 2 * 2 + 1) == (W < 148)           # two launches at most, each with its planner (and the ranking)
 
 
-@pytest.mark.parametrize("n,m,Ws", [(40, 50, (330, 340, 400)), (100, 140, (140, 150, 300))])
+@pytest.mark.parametrize("n,m,Ws", [(40, 50, (330, 340, 400)), (100, 140, (140, 150, 300)), (140, 20, (735, 745))])
 def test_kernels_of_128_and_255_registers_have_the_same_bits(n, m, Ws):
     # lanes whose matrix is in 32 registers a thread, or in half of the tensor memory, have two kernels, chosen by the mode and the number
     # of blocks; on both sides of each line STATIC, a mask and the plain batch give a lane the same bits
